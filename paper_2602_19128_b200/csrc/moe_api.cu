@@ -89,7 +89,9 @@ void fill_layout(int T, int H, int I, int E, int k, moe_workspace_layout_t *L) {
 int layer_token_tile_bound(int T, int H, int I, int E, int k, unsigned flags, bool fp8w) {
     const bool pinned = fp8w || (flags & (MOE_FLAG_SINGLE_CTA_GEMM | MOE_FLAG_TWO_SLAB_GEMM | MOE_FLAG_NARROW_TILES)) != 0;
     const bool wide_ok = !pinned && I % 128 == 0 && H % 256 == 0;
-    return choose_nt_max(T, E, k, wide_ok);
+    const int bound = choose_nt_max(T, E, k, wide_ok);
+    // FP8 weights: 192 rows are the most that leave tensor memory room for converted weights beside two accumulators.
+    return fp8w && bound > 192 ? 192 : bound;
 }
 
 int forward_impl(const void *x, const float *logits, const void *w13, const void *w2, int T, int H, int I, int E, int k,
@@ -161,6 +163,15 @@ int forward_impl(const void *x, const float *logits, const void *w13, const void
         g1.gather_top_k = k;
     }
 
+    // Hand-over: the down GEMM starts expert by expert as the gate/up GEMM finishes them (not with the opt-in
+    // two-slab tiles, whose epilogue counts differently).
+    const bool dense_tiles = (flags & MOE_FLAG_TWO_SLAB_GEMM) != 0;
+    if (!dense_tiles && !(flags & MOE_FLAG_VALIDATION_GEMM)) {
+        g1.handover_role = 1;
+        g2.handover_role = 2;
+        g1.handover = g2.handover = status;
+        g2.handover_per_token_tile = handover_counts_per_token_tile(I);
+    }
     if (fp8w) {
         g1.w_scale = w13_scale;
         g2.w_scale = w2_scale;
@@ -179,15 +190,6 @@ int forward_impl(const void *x, const float *logits, const void *w13, const void
         // skewed workloads they are 5 % resp. 25 % slower than one slab, because the accumulators then
         // fill TMEM and the epilogue no longer overlaps the next tile's MMAs.
         const bool single = (flags & MOE_FLAG_SINGLE_CTA_GEMM) != 0;
-        const bool dense_tiles = (flags & MOE_FLAG_TWO_SLAB_GEMM) != 0;
-        // Hand-over: the down GEMM starts expert by expert as the gate/up GEMM finishes them (not with the opt-in
-        // two-slab tiles, whose epilogue counts differently).
-        if (!dense_tiles) {
-            g1.handover_role = 1;
-            g2.handover_role = 2;
-            g1.handover = g2.handover = status;
-            g2.handover_per_token_tile = handover_counts_per_token_tile(I);
-        }
         auto run = [&](const GroupedGemmArgs &g, bool allow_two_slabs) {
             if (!single && grouped_gemm_tc_ring_applies(g)) return launch_grouped_gemm_tc_ring(g, stream);
             int slabs = single ? 0 : grouped_gemm_tc_pair_slabs(g);

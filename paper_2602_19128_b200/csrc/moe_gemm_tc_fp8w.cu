@@ -3,22 +3,28 @@
 // Paper: the workload is an "FP8 MoE" (Table 2; Sec. 4.5) and the paper's kernel feeds 16-bit
 // tensor-core tiles, so stored FP8 weights are converted and rescaled on their way to the MMA.  Here
 // the weights stay FP8 in HBM (half the bytes of the bf16 layer, which is what bounds the decode- and
-// Mixtral-sized workloads) and the conversion happens in shared memory:
+// Mixtral-sized workloads) and the conversion happens between shared memory and tensor memory:
 //
-//   warp 0      TMA: per ring slot (128 K-elements = one scale block) the 128 x 128 tile of FP8 codes
-//               (16 KiB, unswizzled) and the bf16 token tile as two 128-byte-swizzled 64-wide chunks,
-//               each with ONE copy (a copy has a fixed cost, so slots are as large as the bf16 kernel's)
-//   warps 6..9  converters: wait for the slot, turn the codes into bf16 * block scale and write them in
-//               the 128-byte-swizzled K-major layout the MMA reads (two 32 KiB buffers),
-//               fence towards the tensor core's proxy, signal
-//   warp 1      MMA: A operand from the converted buffer, B operand straight from the slot
-//   warps 2..5  epilogue (unchanged: SwiGLU or plain, double-buffered TMEM)
+//   warp 0       weight TMA: per ring slot (128 K-elements = one scale block) the 128 x 128 tile of codes (16 KiB)
+//                in the 128-byte swizzle, which a warp reads by rows without bank conflicts
+//   warp 6       token TMA: the bf16 token tile of a slot as two 128-byte-swizzled 64-wide chunks, one copy, a ring of
+//                its own (weights come from HBM and want a deep ring, tokens from L2)
+//   warps 8..    converters: a thread owns one weight row (= its lane of tensor memory), turns 64 of the slot's 128
+//                codes into bf16 * block scale and stores them to tensor memory, the MMA's A operand
+//   warp 1       MMA: A from tensor memory, B straight from the token slot
+//   warps 2..5   epilogue (SwiGLU or plain, two accumulators)
+//
+// What bounds it and why A sits in tensor memory: with A rebuilt in shared memory a slot of 96 token rows moved 144 KiB
+// through shared memory (codes in, codes out, 32 KiB of bf16 in and out again, tokens in and out), 1150 cycles at 128
+// bytes per cycle, above the 700 cycles a slot takes at the HBM rate, and the conversion issued 2.5 ALU instructions
+// per weight.  Now a slot moves 80 KiB and the conversion is two ALU instructions and one multiply per TWO weights
+// (one more for the byte permute).
 //
 // A weight is decode(code) * scale[row/128][k/128].  A CTA's 128 weight rows lie in one scale block
 // (down projection) or in one gate block and one up block (gate/up), and a slot is one 128-wide K
 // block, so a slot needs one or two scalar scales.  Conversion: the code's exponent and
-// mantissa bits are moved into a bf16 bit pattern worth value * 2^-120 (two byte permutes and three
-// logic operations per four codes), then one bf16x2 multiply by scale * 2^120 per pair.  The scale is
+// mantissa bits are moved into a bf16 bit pattern worth value * 2^-120, then one bf16x2 multiply by
+// scale * 2^120 per pair.  The scale is
 // rounded to bf16 once per slot and the product once per weight: at most 2^-8 relative on a weight, an
 // order of magnitude inside the layer's tolerance.  Scales must stay below 2^7 for scale * 2^120 to be finite.
 #include "moe_tc_common.cuh"
@@ -28,86 +34,100 @@ namespace {
 
 using namespace tc;
 
-constexpr int kConvWarps = 16;  // four per scheduler: the conversion is ALU work (2.5 instructions per weight) and
-                                // needs the issue slots; measured 4 / 8 / 16 warps: 2.79 / 2.20 / 2.05 ms on the
-                                // decode-sized gate/up GEMM
-constexpr int kFp8Threads = (6 + kConvWarps) * 32;
-constexpr int kSlotK = 128;                         // K elements per ring slot: one scale block, two MMA K-chunks of 64
+constexpr int kGroupWarps = 4;                     // converter warps per slot: one per quarter of tensor memory's lanes
+constexpr int kFirstConvWarp = 8;
+constexpr int kTokenWarp = 6;
+constexpr int kSlotK = 128;                        // K elements per ring slot: one scale block, two MMA K-chunks of 64
 constexpr int kSlotQBytes = kTileM * kSlotK;       // 16 KiB of codes
-constexpr int kConvBytes = 2 * kSlotABytes;        // 32 KiB: two 128-byte-swizzled bf16 tiles (K 0..63 | 64..127)
+constexpr int kConvCols = kSlotK / 2;              // tensor-memory columns of a converted slot (two bf16 per column)
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
+// D[tmem] (+)= A[tmem] * B[smem]^T, bf16 inputs, fp32 accumulate, issued by one thread.
+__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                             uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// Four E4M3 codes (one 32-bit word, lowest byte first) -> four bf16 values times the block scale.
-// A code byte placed in the high byte of a 16-bit lane and shifted so that its 4 exponent and 3 mantissa
-// bits sit at the top of bf16's exponent-low/mantissa-high positions is a bf16 number equal to the
-// code's value times 2^-120, for normal AND subnormal codes alike (E4M3's bias is 7, bf16's 127, and a
-// zero exponent field means "no hidden one" in both); one bf16x2 multiply by scale * 2^120 finishes it.
-__device__ __forceinline__ void convert_four(uint32_t codes, __nv_bfloat162 scale2, uint32_t &lo, uint32_t &hi) {
-    const uint32_t t0 = __byte_perm(codes, 0u, 0x1404);  // bytes 0,1 -> high bytes of the two 16-bit lanes
-    const uint32_t t1 = __byte_perm(codes, 0u, 0x3424);  // bytes 2,3
-    const uint32_t r0 = ((t0 & 0x7F007F00u) >> 4) | (t0 & 0x80008000u);
-    const uint32_t r1 = ((t1 & 0x7F007F00u) >> 4) | (t1 & 0x80008000u);
-    __nv_bfloat162 v0, v1;
-    *reinterpret_cast<uint32_t *>(&v0) = r0;
-    *reinterpret_cast<uint32_t *>(&v1) = r1;
-    v0 = __hmul2(v0, scale2);
-    v1 = __hmul2(v1, scale2);
-    lo = *reinterpret_cast<uint32_t *>(&v0);
-    hi = *reinterpret_cast<uint32_t *>(&v1);
+// 32 consecutive 32-bit columns of this thread's tensor-memory lane (tcgen05.wait::st completes it).
+__device__ __forceinline__ void tmem_store_32(uint32_t taddr, const uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+        ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
+          "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]),
+          "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]),
+          "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+        : "memory");
 }
 
-template <int NT_MAX, int STAGES, int CONV>
+// Two E4M3 codes (bytes `kSel` of a word) -> two bf16 values times the block scale.  The permute puts each code in the
+// low byte of a 16-bit lane under its replicated sign bit; shifted left by four, exponent and mantissa sit at the top of
+// bf16's exponent-low / mantissa-high positions, and the mask keeps them and the sign.  That bit pattern is a bf16
+// number equal to the code's value times 2^-120, for normal AND subnormal codes alike (E4M3's bias is 7, bf16's 127, and
+// a zero exponent field means "no hidden one" in both); one bf16x2 multiply by scale * 2^120 finishes it.
+template <uint32_t kSel>
+__device__ __forceinline__ uint32_t convert_two(uint32_t codes, __nv_bfloat162 scale2) {
+    uint32_t x;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(x) : "r"(codes), "n"(kSel));
+    const uint32_t bits = (x << 4) & 0x87F087F0u;
+    __nv_bfloat162 v;
+    *reinterpret_cast<uint32_t *>(&v) = bits;
+    v = __hmul2(v, scale2);
+    return *reinterpret_cast<uint32_t *>(&v);
+}
+
+template <int NT_MAX, int STAGES_Q>
 struct Fp8Smem {
+    // converted slots in tensor memory (beside two accumulators), token tiles in shared memory, and converter groups
+    static constexpr int kConv = NT_MAX > 128 ? 2 : NT_MAX > 64 ? 3 : 4;
+    static constexpr int kThreads = (kFirstConvWarp + kConv * kGroupWarps) * 32;
     static constexpr int kSlotBBytes = 2 * NT_MAX * kRowBytes;       // two swizzled token tiles (K 0..63 | 64..127)
-    static constexpr int kConv = 0;                                  // CONV x 32 KiB bf16 operand buffers (1024-aligned)
-    static constexpr int kB = CONV * kConvBytes;                     // STAGES token-tile pairs
-    static constexpr int kQ = kB + STAGES * kSlotBBytes;             // STAGES code tiles
-    static constexpr int kBars = kQ + STAGES * kSlotQBytes;          // raw_full[S], raw_empty[S], conv_full[C], conv_empty[C], acc_full[2], acc_empty[2]
-    static constexpr int kTmemSlot = kBars + (2 * STAGES + 2 * CONV + 4) * 8;
+    static constexpr int kB = 0;                                     // kConv token-tile pairs
+    static constexpr int kQ = kB + kConv * kSlotBBytes;           // STAGES_Q code tiles
+    // q_full[SQ], q_empty[SQ], op_full[C], op_empty[C], acc_full[2], acc_empty[2]
+    static constexpr int kBars = kQ + STAGES_Q * kSlotQBytes;
+    static constexpr int kTmemSlot = kBars + (2 * STAGES_Q + 2 * kConv + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
 
-template <int NT_MAX, int STAGES, int CONV, bool SWIGLU>
-__global__ void __launch_bounds__(kFp8Threads, 1)
+template <int NT_MAX, int STAGES_Q, bool SWIGLU>
+__global__ void __launch_bounds__((Fp8Smem<NT_MAX, STAGES_Q>::kThreads), 1)
 grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
-    using L = Fp8Smem<NT_MAX, STAGES, CONV>;
-    constexpr int kTmemCols = 2 * NT_MAX;
-    static_assert(kTmemCols >= 32 && kTmemCols <= 512 && (kTmemCols & (kTmemCols - 1)) == 0,
-                  "a tensor-memory allocation must be a power of two between 32 and 512 columns");
+    using L = Fp8Smem<NT_MAX, STAGES_Q>;
+    constexpr int kConv = L::kConv;
+    constexpr int kColsUsed = 2 * NT_MAX + kConv * kConvCols;
+    constexpr int kTmemCols = kColsUsed <= 256 ? 256 : 512;  // (a power of two)
+    static_assert(kColsUsed <= 512 && kConv * kConvCols <= 256, "accumulators and converted slots exceed tensor memory");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
     chain_release();  // the next kernel of the forward call may be scheduled; it waits for this grid to finish
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
-    const uint32_t bar_raw_full = base + L::kBars, bar_raw_empty = bar_raw_full + STAGES * 8;
-    const uint32_t bar_conv_full = bar_raw_empty + STAGES * 8, bar_conv_empty = bar_conv_full + CONV * 8;
-    const uint32_t bar_acc_full = bar_conv_empty + CONV * 8, bar_acc_empty = bar_acc_full + 16;
+    const uint32_t bar_q_full = base + L::kBars, bar_q_empty = bar_q_full + STAGES_Q * 8;
+    const uint32_t bar_op_full = bar_q_empty + STAGES_Q * 8, bar_op_empty = bar_op_full + kConv * 8;
+    const uint32_t bar_acc_full = bar_op_empty + kConv * 8, bar_acc_empty = bar_acc_full + 16;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(base_ptr + L::kTmemSlot);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(bar_raw_full + s * 8, 1);
-            mbar_init(bar_raw_empty + s * 8, 1);
+        for (int s = 0; s < STAGES_Q; ++s) {
+            mbar_init(bar_q_full + s * 8, 1);
+            mbar_init(bar_q_empty + s * 8, kGroupWarps);
         }
-        for (int c = 0; c < CONV; ++c) {
-            mbar_init(bar_conv_full + c * 8, kConvWarps);
-            mbar_init(bar_conv_empty + c * 8, 1);
+        for (int c = 0; c < kConv; ++c) {
+            mbar_init(bar_op_full + c * 8, kGroupWarps + 1);  // the converter warps, and the token tile's bytes
+            mbar_init(bar_op_empty + c * 8, 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(bar_acc_full + a * 8, 1);
@@ -127,11 +147,12 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     __syncthreads();
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    chain_wait();  // everything above overlapped the previous kernel; its results are read from here on
-    const int total_tiles = p.tile_prefix[p.E] * p.n_feature_tiles;
+    // everything above overlapped the previous kernel; its results are read from here on
+    const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
+    const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
 
     if (warp == 0) {
-        // ---------------- TMA producer ----------------
+        // ---------------- weight TMA ----------------
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true;
@@ -139,129 +160,170 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p);
-            const int n_mma = (t.n_valid + 15) & ~15;
             const int w_row = t.e * p.w_rows + t.f * kTileM;
-            const uint32_t tx_bytes = kSlotQBytes + 2 * n_mma * kRowBytes;
             for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                ok = mbar_wait_warp(bar_raw_empty + stage * 8, phase ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                ok = mbar_wait_warp(bar_q_empty + stage * 8, phase ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
                 if (!ok) break;
                 if (elect_one()) {
-                    const uint32_t full = bar_raw_full + stage * 8;
-                    mbar_expect_tx(full, tx_bytes);
+                    const uint32_t full = bar_q_full + stage * 8;
+                    mbar_expect_tx(full, kSlotQBytes);
                     const uint32_t sq = base + L::kQ + stage * kSlotQBytes;
-                    const uint32_t sb = base + L::kB + stage * L::kSlotBBytes;
                     const int k0 = kb * kSlotK;
                     if (SWIGLU)
                         tma_load_5d(sq, &maps.w, k0, 0, 0, t.f * 4, t.e, full);
                     else
                         tma_load_2d(sq, &maps.w, k0, w_row, full);
-                    // one copy: rows x (two 64-wide K chunks), each chunk landing as its own swizzled tile of n_mma rows
-                    tma_load_3d(sb, act_map<16>(maps, n_mma), 0, t.row0, 2 * kb, full);
                 }
                 __syncwarp();
-                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                if (++stage == STAGES_Q) { stage = 0; phase ^= 1u; }
+            }
+        }
+    } else if (warp == kTokenWarp) {
+        // ---------------- token TMA ----------------
+        int stage = 0;
+        uint32_t phase = 0;
+        bool ok = true, gate_up_done = false;
+        for (int round = 0; ok; ++round) {
+            const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
+            if (tile >= total_tiles) break;
+            const Tile t = decode_tile(tile, p);
+            const int n_mma = (t.n_valid + 15) & ~15;
+            ok = handover_wait_expert(p.handover_role, p.handover, t.e, t.n_tok_tiles, p.handover_per_token_tile,
+                                      p.tile_prefix[p.E], gate_up_done, abort_flag, p.status, lane);
+            if (!ok) break;
+            for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                ok = mbar_wait_warp(bar_op_empty + stage * 8, phase ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                if (!ok) break;
+                if (elect_one()) {
+                    const uint32_t full = bar_op_full + stage * 8;
+                    mbar_expect_tx(full, 2 * n_mma * kRowBytes);
+                    // one copy: rows x (two 64-wide K chunks), each chunk landing as its own swizzled tile of n_mma rows
+                    tma_load_3d(base + L::kB + stage * L::kSlotBBytes, act_map<16>(maps, n_mma), 0, t.row0, 2 * kb, full);
+                }
+                __syncwarp();
+                if (++stage == kConv) { stage = 0; phase ^= 1u; }
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        int stage = 0, conv = 0, acc = 0;
-        uint32_t phase = 0, conv_phase = 0, acc_phase = 0;
+        // One elected thread walks a whole tile's slots.  With the election, the vote and the warp barrier inside the
+        // K loop a slot took 560 cycles to issue beside busy converter warps, more than its MMAs take (N/2 + 10 each with
+        // A in tensor memory, measured): 0.400 against 0.379 ms on the 333-token layer, 0.291 against 0.267 on 32 tokens.
+        int op = 0, acc = 0;
+        uint32_t op_phase = 0, acc_phase = 0;
         bool ok = true;
+        const uint64_t b_desc0 = smem_desc_k_major_sw128(base + L::kB);
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p);
-            const uint32_t idesc = instr_desc_bf16(kTileM, (t.n_valid + 15) & ~15);
+            const int n_mma = (t.n_valid + 15) & ~15;
+            const uint32_t idesc = instr_desc_bf16(kTileM, n_mma);
             ok = mbar_wait_warp(bar_acc_empty + acc * 8, acc_phase ^ 1u, abort_flag, p.status, kSiteMmaTmemEmpty + kSiteOffset);
             if (!ok) break;
-            tcgen05_fence_after();
             const uint32_t d_tmem = tmem_base + acc * NT_MAX;
-            for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                // the converted weights imply the slot has landed; the token tile is read from the slot itself
-                ok = mbar_wait_warp(bar_conv_full + conv * 8, conv_phase, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
-                if (ok) ok = mbar_wait_warp(bar_raw_full + stage * 8, phase, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
-                if (!ok) break;
-                tcgen05_fence_after();
-                if (elect_one()) {
-                    const int n_mma = (t.n_valid + 15) & ~15;
+            if (elect_one()) {
+                int o = op;
+                uint32_t ph = op_phase;
+                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                    ok = mbar_wait(bar_op_full + o * 8, ph, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
+                    if (!ok) break;
+                    tcgen05_fence_after();
+                    const uint32_t a_tmem = tmem_base + 2 * NT_MAX + o * kConvCols;
+                    const uint64_t b_desc = b_desc0 + (uint32_t)(o * (L::kSlotBBytes >> 4));
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {  // the slot's two 64-wide K chunks
-                        const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kConv + conv * kConvBytes + j * kSlotABytes);
-                        const uint64_t b_desc =
-                            smem_desc_k_major_sw128(base + L::kB + stage * L::kSlotBBytes + j * n_mma * kRowBytes);
+                    for (int j = 0; j < 2; ++j)  // the slot's two 64-wide K chunks
 #pragma unroll
-                        for (int kk = 0; kk < kBlockK / 16; ++kk)
-                            umma_bf16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | j | kk) != 0);
-                    }
-                    umma_commit(bar_conv_empty + conv * 8);
-                    umma_commit(bar_raw_empty + stage * 8);
-                    if (kb == p.n_k_blocks - 1) umma_commit(bar_acc_full + acc * 8);
+                        for (int kk = 0; kk < kBlockK / 16; ++kk)  // 16 K-elements = 8 columns of A, 2 descriptor units of B
+                            umma_bf16_ts(d_tmem, a_tmem + (j * (kBlockK / 16) + kk) * 8,
+                                         b_desc + (uint32_t)(j * (n_mma * kRowBytes >> 4)) + 2 * kk, idesc, (kb | j | kk) != 0);
+                    umma_commit(bar_op_empty + o * 8);
+                    if (++o == kConv) { o = 0; ph ^= 1u; }
                 }
-                __syncwarp();
-                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                if (++conv == CONV) { conv = 0; conv_phase ^= 1u; }
+                if (ok) umma_commit(bar_acc_full + acc * 8);
             }
+            __syncwarp();
+            ok = __all_sync(0xffffffffu, ok);
+            const int uses = op + p.n_k_blocks;
+            op_phase ^= (uint32_t)(uses / kConv) & 1u;
+            op = uses % kConv;
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-    } else if (warp >= 6) {
-        // ---------------- converters: FP8 codes -> scaled bf16 in the MMA's swizzled layout ----------------
-        // A slot holds 128 rows x 128 codes.  Warp cw owns rows (128/kConvWarps)*cw ..; per iteration lanes
-        // 8m..8m+7 take the eight 16-byte pieces of row base + 4i + m (512 contiguous bytes per
-        // instruction), and each lane writes its 16 weights as two 16-byte chunks of the bf16 row in
-        // K-chunk tile (piece / 4): chunk c of row r at r*128 + ((c ^ (r & 7)) * 16).
-        const int cw = warp - 6, piece = lane & 7, sub_row = lane >> 3;
-        constexpr int kRowsPerWarp = kTileM / kConvWarps;
-        int stage = 0, conv = 0;
-        uint32_t phase = 0, conv_phase = 0;
+    } else if (warp >= kFirstConvWarp) {
+        // ---------------- converters: FP8 codes -> scaled bf16 in tensor memory ----------------
+        // Group g (four warps) takes the ring slots g, g + kConv, ... of the CTA's whole sequence and always converts
+        // into operand buffer g.  A warp may only touch lanes 32 * (warp % 4) .. +31 of tensor memory: its threads own
+        // rows 32 * (warp % 4) + lane and convert the row's 128 codes, eight 16-byte pieces of the swizzled row.
+        // A stage of the weight ring belongs to one group: a wait on its parity is only valid for a warp that has seen the
+        // stage's previous use complete.
+        static_assert(STAGES_Q % kConv == 0, "a stage of the weight ring must always go to the same converter group");
+        static_assert(kFirstConvWarp % 4 == 0 && kGroupWarps == 4, "converter lane mapping");
+        const int q = warp & 3, group = (warp - kFirstConvWarp) / kGroupWarps, row = q * 32 + lane;
+        const uint32_t a_tmem = tmem_base + ((uint32_t)(q * 32) << 16) + 2 * NT_MAX + group * kConvCols;
+        const uint32_t full = bar_op_full + group * 8, empty = bar_op_empty + group * 8;
+        const uint8_t *my_row = base_ptr + L::kQ + row * kSlotK;
+        const int swz = row & 7;
+        int stage = group, turn = 0;
+        uint32_t phase = 0, op_phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p);
-            // scale rows: the tile's gate block and up block (gate/up), or its single block (down)
+            // this row's scales: its tile's gate block or up block (gate/up: 16 gate rows, 16 up rows in turn), or the
+            // tile's single block (down)
             const int row_blocks = p.w_rows >> 7;
-            const float *scale_a = p.w_scale + ((size_t)t.e * row_blocks + (SWIGLU ? (t.f * 64) >> 7 : t.f)) * p.n_k_blocks;
-            const float *scale_b = SWIGLU ? p.w_scale + ((size_t)t.e * row_blocks + ((p.n_out + t.f * 64) >> 7)) * p.n_k_blocks
-                                          : scale_a;
-            float next_a = __ldg(scale_a), next_b = __ldg(scale_b);
-            for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                const float two120 = 1329227995784915872903807060280344576.0f;  // 2^120
-                const __nv_bfloat162 sa = __float2bfloat162_rn(next_a * two120);
-                const __nv_bfloat162 sb = SWIGLU ? __float2bfloat162_rn(next_b * two120) : sa;
-                if (kb + 1 < p.n_k_blocks) {  // next slot's scales, off the critical path
-                    next_a = __ldg(scale_a + kb + 1);
-                    next_b = __ldg(scale_b + kb + 1);
-                }
-                ok = mbar_wait_warp(bar_raw_full + stage * 8, phase, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
-                if (ok) ok = mbar_wait_warp(bar_conv_empty + conv * 8, conv_phase ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+            const int block = !SWIGLU ? t.f : ((row & 16) ? (p.n_out + t.f * 64) >> 7 : (t.f * 64) >> 7);
+            const float *scale = p.w_scale + ((size_t)t.e * row_blocks + block) * p.n_k_blocks;
+            int kb = (group - turn + kConv) % kConv;  // first slot of this tile that is this group's
+            turn = (turn + p.n_k_blocks) % kConv;
+            float next = kb < p.n_k_blocks ? __ldg(scale + kb) : 0.f;
+            for (; kb < p.n_k_blocks; kb += kConv) {
+                const __nv_bfloat162 s2 = __float2bfloat162_rn(next * 1329227995784915872903807060280344576.0f);  // 2^120
+                if (kb + kConv < p.n_k_blocks) next = __ldg(scale + kb + kConv);  // off the critical path
+                ok = mbar_wait_warp(bar_q_full + stage * 8, phase, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
                 if (!ok) break;
-                const uint8_t *src = base_ptr + L::kQ + stage * kSlotQBytes;
-                uint8_t *dst = base_ptr + L::kConv + conv * kConvBytes + (piece >> 2) * kSlotABytes;
-                const int chunk = 2 * (piece & 3);
+                const uint8_t *src = my_row + stage * kSlotQBytes;
 #pragma unroll
-                for (int i = 0; i < kRowsPerWarp / 4; ++i) {
-                    const int row = cw * kRowsPerWarp + i * 4 + sub_row;
-                    // gate/up slots interleave 16 gate rows and 16 up rows
-                    const __nv_bfloat162 s2 = (SWIGLU && (row & 16)) ? sb : sa;
-                    const uint4 q = *reinterpret_cast<const uint4 *>(src + row * kSlotK + piece * 16);
-                    uint4 lo, hi;
-                    convert_four(q.x, s2, lo.x, lo.y);
-                    convert_four(q.y, s2, lo.z, lo.w);
-                    convert_four(q.z, s2, hi.x, hi.y);
-                    convert_four(q.w, s2, hi.z, hi.w);
-                    uint8_t *drow = dst + row * kRowBytes;
-                    *reinterpret_cast<uint4 *>(drow + ((chunk ^ (row & 7)) << 4)) = lo;
-                    *reinterpret_cast<uint4 *>(drow + (((chunk + 1) ^ (row & 7)) << 4)) = hi;
+                for (int half = 0; half < 2; ++half) {
+                    uint4 codes[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        codes[i] = *reinterpret_cast<const uint4 *>(src + (((half * 4 + i) ^ swz) << 4));
+                    uint32_t v[32];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t w[4] = {codes[i].x, codes[i].y, codes[i].z, codes[i].w};
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            v[i * 8 + c * 2] = convert_two<0x9180>(w[c], s2);
+                            v[i * 8 + c * 2 + 1] = convert_two<0xB3A2>(w[c], s2);
+                        }
+                    }
+                    if (half == 0) {  // the MMAs that read the buffer's previous contents are complete
+                        ok = mbar_wait_warp(empty, op_phase ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                        if (!ok) break;
+                        tcgen05_fence_after();
+                    }
+                    __syncwarp();  // (the store is an aligned warp instruction)
+                    tmem_store_32(a_tmem + half * (kConvCols / 2), v);
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy stores -> visible to the MMA
+                if (!ok) break;
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tcgen05_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar_conv_full + conv * 8);
-                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                if (++conv == CONV) { conv = 0; conv_phase ^= 1u; }
+                if (lane == 0) {
+                    mbar_arrive(full);
+                    mbar_arrive(bar_q_empty + stage * 8);
+                }
+                __syncwarp();
+                op_phase ^= 1u;
+                stage += kConv;
+                if (stage >= STAGES_Q) { stage = group; phase ^= 1u; }
             }
         }
-    } else {
+    } else if (warp < kTokenWarp) {
         // ---------------- epilogue: TMEM -> registers -> global ----------------
         const int q = warp & 3;
         int acc = 0;
@@ -304,11 +366,13 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty + acc * 8);
+            handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
     }
 
     // ---------------- teardown ----------------
+    gemm_chain_finish(p.handover_role);
     tcgen05_fence_before();
     __syncthreads();
     if (*abort_flag) {
@@ -320,23 +384,23 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     }
 }
 
-template <int NT_MAX, int STAGES, int CONV, bool SWIGLU>
+template <int NT_MAX, int STAGES_Q, bool SWIGLU>
 int launch_fp8_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
-    using L = Fp8Smem<NT_MAX, STAGES, CONV>;
+    using L = Fp8Smem<NT_MAX, STAGES_Q>;
     static_assert(L::kDynamicBytes <= 232448, "rings do not fit in shared memory");
-    auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES, CONV, SWIGLU>;
+    auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES_Q, SWIGLU>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, kFp8Threads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+    return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }
 
 template <bool SWIGLU>
 int dispatch_fp8(int nt_max, const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t s) {
     switch (nt_max) {
-        case 32: return launch_fp8_instance<32, 5, 2, SWIGLU>(maps, p, grid, s);
-        case 64: return launch_fp8_instance<64, 4, 2, SWIGLU>(maps, p, grid, s);
-        case 128: return launch_fp8_instance<128, 3, 2, SWIGLU>(maps, p, grid, s);
-        case 256: return launch_fp8_instance<256, 2, 2, SWIGLU>(maps, p, grid, s);
+        case 32: return launch_fp8_instance<32, 12, SWIGLU>(maps, p, grid, s);
+        case 64: return launch_fp8_instance<64, 8, SWIGLU>(maps, p, grid, s);
+        case 128: return launch_fp8_instance<128, 6, SWIGLU>(maps, p, grid, s);
+        case 192: return launch_fp8_instance<192, 8, SWIGLU>(maps, p, grid, s);
         default: return MOE_ERR_UNSUPPORTED;
     }
 }
@@ -349,8 +413,8 @@ int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &a, cudaStream_t stream) {
     if (a.n_out % 128 != 0) return MOE_ERR_UNSUPPORTED;  // gate and up halves must both start on a scale block
 
     TensorMaps maps;
-    const bool ok_w = a.swiglu ? encode_weight_map_gate_up_fp8(&maps.w, a.w, a.E, a.n_out, a.K)
-                               : encode_weight_map_2d_fp8(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
+    const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
+                               : encode_mx_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
     if (!ok_w || !encode_act_maps_k128(maps.act, a.act, a.A, a.K, 16)) return MOE_ERR_CUDA;
 
     KernelParams p;
@@ -366,9 +430,9 @@ int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &a, cudaStream_t stream) {
     p.w_rows = a.w_rows;
     p.n_feature_tiles = a.n_out / features_per_tile;
     p.w_scale = a.w_scale;
-    p.handover_role = 0;
-    p.handover = nullptr;
-    p.handover_per_token_tile = 0;
+    p.handover_role = a.handover_role;
+    p.handover = a.handover;
+    p.handover_per_token_tile = a.handover_per_token_tile;
 
     const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
     const long long max_tiles = max_token_tiles * p.n_feature_tiles;

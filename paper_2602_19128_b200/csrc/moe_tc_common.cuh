@@ -336,9 +336,7 @@ __device__ __forceinline__ float swiglu(float g, float u) { return __fdividef(g,
 // ---- host side ----------------------------------------------------------------------------------
 bool encode_weight_map_2d(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K);
 bool encode_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int I, int H);
-bool encode_weight_map_2d_fp8(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K);
 bool encode_act_maps_k128(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum);
-bool encode_weight_map_gate_up_fp8(CUtensorMap *map, const void *w13, int E, int I, int H);
 bool encode_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int count = kNumActMaps);
 bool encode_row_map(CUtensorMap *map, const void *act, uint64_t rows, uint64_t K);
 bool encode_mx_weight_map_2d(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K);

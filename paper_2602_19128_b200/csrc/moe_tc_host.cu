@@ -98,15 +98,14 @@ bool encode_cached(CUtensorMap *map, CUtensorMapDataType dtype, int rank, const 
     return true;
 }
 
-// bf16 operands and MX codes land in the 128-byte-swizzled layout the MMA reads; the FP8 codes of the
-// dequantising kernel are staged unswizzled for its converter warps.
-enum class Operand { kBf16, kCodesForConverter, kCodesForMma };
+// All operands land in the 128-byte swizzle: the layout the MMA reads, and the one a converter warp reads by rows
+// without bank conflicts.
+enum class Operand { kBf16, kCodes };
 
 bool encode(CUtensorMap *map, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
             const cuuint32_t *box, Operand kind = Operand::kBf16) {
     return encode_cached(map, kind == Operand::kBf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8,
-                         rank, base, dims, strides, box,
-                         kind == Operand::kCodesForConverter ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B);
+                         rank, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 }  // namespace
@@ -149,30 +148,12 @@ bool encode_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int I, 
     return encode(map, w13, 5, dims, strides, box);
 }
 
-// The same two weight maps over FP8 codes (one byte per element): [rows, K] with a 128-row x 64-byte box,
-// and the gate/up view [E][I/16][2][16][H] with the {64,16,2,4,1} box.
-// (FP8 slots are 128 K-elements wide: 128-byte rows of codes.)
-bool encode_weight_map_2d_fp8(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K) {
-    const cuuint64_t dims[2] = {K, rows};
-    const cuuint64_t strides[1] = {K};
-    const cuuint32_t box[2] = {128, (cuuint32_t)kTileM};
-    return encode(map, w, 2, dims, strides, box, Operand::kCodesForConverter);
-}
-
-bool encode_weight_map_gate_up_fp8(CUtensorMap *map, const void *w13, int E, int I, int H) {
-    const cuuint64_t row_bytes = (cuuint64_t)H;
-    const cuuint64_t dims[5] = {(cuuint64_t)H, 16, 2, (cuuint64_t)(I / 16), (cuuint64_t)E};
-    const cuuint64_t strides[4] = {row_bytes, (cuuint64_t)I * row_bytes, 16 * row_bytes, 2 * (cuuint64_t)I * row_bytes};
-    const cuuint32_t box[5] = {128, 16, 2, 4, 1};
-    return encode(map, w13, 5, dims, strides, box, Operand::kCodesForConverter);
-}
-
-// MX operands: one byte per element, 128 K-elements (one 128-byte swizzle row) per ring slot.
+// MX operands and FP8 weights: one byte per element, 128 K-elements (one 128-byte swizzle row) per ring slot.
 bool encode_mx_weight_map_2d(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K) {
     const cuuint64_t dims[2] = {K, rows};
     const cuuint64_t strides[1] = {K};
     const cuuint32_t box[2] = {128, (cuuint32_t)kTileM};
-    return encode(map, w, 2, dims, strides, box, Operand::kCodesForMma);
+    return encode(map, w, 2, dims, strides, box, Operand::kCodes);
 }
 
 bool encode_mx_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int I, int H) {
@@ -180,7 +161,7 @@ bool encode_mx_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int 
     const cuuint64_t dims[5] = {(cuuint64_t)H, 16, 2, (cuuint64_t)(I / 16), (cuuint64_t)E};
     const cuuint64_t strides[4] = {row_bytes, (cuuint64_t)I * row_bytes, 16 * row_bytes, 2 * (cuuint64_t)I * row_bytes};
     const cuuint32_t box[5] = {128, 16, 2, 4, 1};
-    return encode(map, w13, 5, dims, strides, box, Operand::kCodesForMma);
+    return encode(map, w13, 5, dims, strides, box, Operand::kCodes);
 }
 
 bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum) {
@@ -188,7 +169,7 @@ bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint6
         const cuuint64_t dims[2] = {K, rows};
         const cuuint64_t strides[1] = {K};
         const cuuint32_t box[2] = {128, (cuuint32_t)row_quantum * (cuuint32_t)(i + 1)};
-        if (!encode(&maps[i], act, 2, dims, strides, box, Operand::kCodesForMma)) return false;
+        if (!encode(&maps[i], act, 2, dims, strides, box, Operand::kCodes)) return false;
     }
     return true;
 }

@@ -57,6 +57,19 @@ def test_fp8w_forward_matches_oracle(T, H, I, E, k, skew):
     assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k", [(8, 2048, 1408, 2, 2),    # tiles of up to 32 rows, 16 and 11 slots of K
+                                       (31, 1920, 1152, 2, 2),   # 64: 15 and 9 slots
+                                       (75, 1408, 2048, 2, 2),   # 128
+                                       (190, 1664, 1280, 2, 2),  # 192, one tile per expert
+                                       (193, 896, 1152, 2, 2)])  # 192, two ragged tiles per expert
+def test_fp8w_long_rows_wrap_the_rings(T, H, I, E, k):
+    """K longer than the weight ring and the operand buffers, slot counts that are no multiple of either: every buffer
+    is reused across tiles in another phase."""
+    inp = make_fp8w_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=3, device="cuda")
+    out, _ = run_fp8w(inp)
+    assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
+
+
 def test_fp8w_with_unit_scales_equals_the_bf16_layer_bit_for_bit():
     """All E4M3 values are bf16 values, and a scale of 1 is exact in bf16: both paths see the same operands."""
     g = torch.Generator().manual_seed(0)
