@@ -244,9 +244,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            const int uses = op + p.n_k_blocks;
-            op_phase ^= (uint32_t)(uses / kConv) & 1u;
-            op = uses % kConv;
+            ring_advance<kConv>(op, op_phase, p.n_k_blocks);
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }

@@ -129,30 +129,34 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             ok = handover_wait_expert(p.handover_role, p.handover, t.e, t.n_tok_tiles, p.handover_per_token_tile,
                                       p.tile_prefix[p.E], gate_up_done, abort_flag, p.status, lane);
             if (!ok) break;
-            for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                ok = mbar_wait_warp(bar_empty + stage * 8, phase ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
-                if (!ok) break;
-                if (elect_one()) {
-                    const uint32_t full = bar_full + stage * 8;
+            if (elect_one()) {
+                int slot = stage;
+                uint32_t ph = phase;
+                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                    ok = mbar_wait(bar_empty + slot * 8, ph ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                    if (!ok) break;
+                    const uint32_t full = bar_full + slot * 8;
                     mbar_expect_tx(full, tx_bytes);
-                    const uint32_t sa = base + L::kA + stage * kMxSlotABytes;
-                    const uint32_t sb = base + L::kB + stage * L::kSlotBBytes;
+                    const uint32_t sa = base + L::kA + slot * kMxSlotABytes;
+                    const uint32_t sb = base + L::kB + slot * L::kSlotBBytes;
                     const int k0 = kb * kMxSlotK;
                     if (SWIGLU)
                         tma_load_5d(sa, &maps.w, k0, 0, 0, t.f * 4, t.e, full);
                     else
                         tma_load_2d(sa, &maps.w, k0, w_row, full);
                     tma_load_2d(sb, act_map<16>(maps, n_mma), k0, t.row0, full);
-                    bulk_load(base + L::kSfA + stage * kMxSfAtomBytes, w_sf + (size_t)kb * kMxSfAtomBytes, kMxSfAtomBytes, full);
-                    bulk_load(base + L::kSfB + stage * kMxSfBBytes, a_sf + (size_t)kb * p.n_atoms * kMxSfAtomBytes,
+                    bulk_load(base + L::kSfA + slot * kMxSfAtomBytes, w_sf + (size_t)kb * kMxSfAtomBytes, kMxSfAtomBytes, full);
+                    bulk_load(base + L::kSfB + slot * kMxSfBBytes, a_sf + (size_t)kb * p.n_atoms * kMxSfAtomBytes,
                               kMxSfBBytes, full);
+                    if (++slot == STAGES) { slot = 0; ph ^= 1u; }
                 }
-                __syncwarp();
-                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             }
+            __syncwarp();
+            ok = __all_sync(0xffffffffu, ok);
+            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
+        // ---------------- MMA issuer: one elected thread walks a whole tile's slots ----------------
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool ok = true;
@@ -166,27 +170,29 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             if (!ok) break;
             tcgen05_fence_after();
             const uint32_t d_tmem = tmem_base + acc * NT_MAX;
-            for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                ok = mbar_wait_warp(bar_full + stage * 8, phase, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
-                if (!ok) break;
-                tcgen05_fence_after();
-                if (elect_one()) {
-                    const uint32_t sfa_smem = base + L::kSfA + stage * kMxSfAtomBytes;
-                    const uint32_t sfb_smem = base + L::kSfB + stage * kMxSfBBytes;
-                    tmem_copy_sf_atom(sfa_tmem, smem_desc_sf_atom(sfa_smem));
-                    tmem_copy_sf_atom(sfb_tmem, smem_desc_sf_atom(sfb_smem));
-                    const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + stage * kMxSlotABytes);
-                    const uint64_t b_desc = smem_desc_k_major_sw128(base + L::kB + stage * L::kSlotBBytes);
+            if (elect_one()) {
+                int s = stage;
+                uint32_t ph = phase;
+                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                    ok = mbar_wait(bar_full + s * 8, ph, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
+                    if (!ok) break;
+                    tcgen05_fence_after();
+                    tmem_copy_sf_atom(sfa_tmem, smem_desc_sf_atom(base + L::kSfA + s * kMxSfAtomBytes));
+                    tmem_copy_sf_atom(sfb_tmem, smem_desc_sf_atom(base + L::kSfB + s * kMxSfBBytes));
+                    const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + s * kMxSlotABytes);
+                    const uint64_t b_desc = smem_desc_k_major_sw128(base + L::kB + s * L::kSlotBBytes);
 #pragma unroll
                     for (int kk = 0; kk < kMxSlotK / 32; ++kk)  // 32 K-elements = 32 bytes = 2 descriptor units
                         umma_mx(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, instr_desc_mx(kTileM, n_mma, kk), (kb | kk) != 0,
                                 sfa_tmem, sfb_tmem);
-                    umma_commit(bar_empty + stage * 8);
-                    if (kb == p.n_k_blocks - 1) umma_commit(bar_acc_full + acc * 8);
+                    umma_commit(bar_empty + s * 8);
+                    if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
-                __syncwarp();
-                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                if (ok) umma_commit(bar_acc_full + acc * 8);
             }
+            __syncwarp();
+            ok = __all_sync(0xffffffffu, ok);
+            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }

@@ -172,7 +172,7 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
     } else if (warp == kPairThreads / 32 - 1) {
         producer_loop(false, true);
     } else if (warp == 1) {
-        // ---------------- MMA issuer (leader CTA only) ----------------
+        // ---------------- MMA issuer (leader CTA only): one elected thread walks a whole tile's slots ----------------
         if (rank == 0) {
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
@@ -188,29 +188,32 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
                 if (!ok) break;
                 tcgen05_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * NT_MAX;
-                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                    ok = __all_sync(0xffffffffu, pair_wait(bar_full + stage * 8, phase, abort_flag, peer_abort, p.status,
-                                                           kSiteMmaFull + kSiteOffset));
-                    if (!ok) break;
-                    tcgen05_fence_after();
-                    if (elect_one()) {
-                        tmem_copy_sf_atom_pair(sfa_tmem, smem_desc_sf_atom(base + L::kSfA + stage * kMxSfAtomBytes));
+                if (elect_one()) {
+                    int s = stage;
+                    uint32_t ph = phase;
+                    for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                        ok = pair_wait(bar_full + s * 8, ph, abort_flag, peer_abort, p.status, kSiteMmaFull + kSiteOffset);
+                        if (!ok) break;
+                        tcgen05_fence_after();
+                        tmem_copy_sf_atom_pair(sfa_tmem, smem_desc_sf_atom(base + L::kSfA + s * kMxSfAtomBytes));
 #pragma unroll
                         for (int a = 0; a < L::kAtomsB; ++a)
                             tmem_copy_sf_atom_pair(sfb_tmem + 4 * a,
-                                                   smem_desc_sf_atom(base + L::kSfB + stage * L::kSfBBytes + a * kMxSfAtomBytes));
-                        const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + stage * kMxSlotABytes);
-                        const uint64_t b_desc = smem_desc_k_major_sw128(base + L::kB + stage * L::kSlotBBytes);
+                                                   smem_desc_sf_atom(base + L::kSfB + s * L::kSfBBytes + a * kMxSfAtomBytes));
+                        const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + s * kMxSlotABytes);
+                        const uint64_t b_desc = smem_desc_k_major_sw128(base + L::kB + s * L::kSlotBBytes);
 #pragma unroll
                         for (int kk = 0; kk < kMxSlotK / 32; ++kk)
                             umma_mx_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, instr_desc_mx(2 * kTileM, n_mma, kk),
                                          (kb | kk) != 0, sfa_tmem, sfb_tmem);
-                        umma_commit_pair(bar_empty + stage * 8);
-                        if (kb == p.n_k_blocks - 1) umma_commit_pair(bar_acc_full + acc * 8);
+                        umma_commit_pair(bar_empty + s * 8);
+                        if (++s == STAGES) { s = 0; ph ^= 1u; }
                     }
-                    __syncwarp();
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    if (ok) umma_commit_pair(bar_acc_full + acc * 8);
                 }
+                __syncwarp();
+                ok = __all_sync(0xffffffffu, ok);
+                ring_advance<STAGES>(stage, phase, p.n_k_blocks);
                 if (!ok) break;
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }

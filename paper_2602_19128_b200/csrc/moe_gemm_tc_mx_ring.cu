@@ -213,7 +213,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
     } else if (warp == kMxRingThreads / 32 - 1) {
         producer_loop(false, true);
     } else if (warp == 1) {
-        // ---------------- MMA issuer (leader CTA only): the warp walks the ring, one elected lane issues ----------------
+        // ---------------- MMA issuer (leader CTA only): one elected thread walks a whole tile's slots ----------------
         if (rank == 0) {
             int stage = 0, seq = 0;
             uint32_t phase = 0, chunk_phase = 0;  // bit c: parity of chunk c's next hand-back
@@ -222,37 +222,39 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
             for (int round = 0; ok; ++round, ++seq) {
                 const int tile = tile_of_round(round, pair, n_pairs);
                 if (tile >= total_tiles) break;
-                MxParts parts;
-                parts.n = 0;
-                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                    ok = __all_sync(0xffffffffu, pair_wait(bar_full + stage * 8, phase, abort_flag, peer_abort, p.status,
-                                                           kSiteMmaFull + kSiteOffset));
-                    if (!ok) break;
-                    if (kb == 0) {
-                        // the tile's width, then its chunks of the accumulator ring, each free of its last occupant
-                        const int n_mma = queue[seq & (kTileQueue - 1)];
-                        const int n_chunks = n_mma / kChunkCols;
-                        parts = split_mx_tile(seq, n_mma);
-                        {   // lane c waits for the tile's c-th chunk (a tile has at most 24)
-                            const int first = parts.first_col / kChunkCols, chunk = first + lane;
-                            bool mine = true;
-                            if (lane < n_chunks)
-                                mine = pair_wait(bar_acc_empty + chunk * 8, ((chunk_phase >> chunk) & 1u) ^ 1u, abort_flag, peer_abort,
-                                                 p.status, kSiteMmaTmemEmpty + kSiteOffset);
-                            ok = __all_sync(0xffffffffu, mine);
-                            chunk_phase ^= ((1u << n_chunks) - 1u) << first;
+                ok = __all_sync(0xffffffffu, pair_wait(bar_full + stage * 8, phase, abort_flag, peer_abort, p.status,
+                                                       kSiteMmaFull + kSiteOffset));
+                if (!ok) break;
+                // the tile's width, then its chunks of the accumulator ring, each free of its last occupant
+                const int n_mma = queue[seq & (kTileQueue - 1)];
+                const int n_chunks = n_mma / kChunkCols;
+                const MxParts parts = split_mx_tile(seq, n_mma);
+                {   // lane c waits for the tile's c-th chunk (a tile has at most 24)
+                    const int first = parts.first_col / kChunkCols, chunk = first + lane;
+                    bool mine = true;
+                    if (lane < n_chunks)
+                        mine = pair_wait(bar_acc_empty + chunk * 8, ((chunk_phase >> chunk) & 1u) ^ 1u, abort_flag, peer_abort,
+                                         p.status, kSiteMmaTmemEmpty + kSiteOffset);
+                    ok = __all_sync(0xffffffffu, mine);
+                    chunk_phase ^= ((1u << n_chunks) - 1u) << first;
+                }
+                if (!ok) break;
+                if (elect_one()) {
+                    int st = stage;
+                    uint32_t ph = phase;
+                    for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                        if (kb > 0) {
+                            ok = pair_wait(bar_full + st * 8, ph, abort_flag, peer_abort, p.status, kSiteMmaFull + kSiteOffset);
+                            if (!ok) break;
                         }
-                        if (!ok) break;
-                    }
-                    tcgen05_fence_after();
-                    if (elect_one()) {
-                        tmem_copy_sf_atom_pair(sfa_tmem, smem_desc_sf_atom(base + L::kSfA + stage * kMxSfAtomBytes));
+                        tcgen05_fence_after();
+                        tmem_copy_sf_atom_pair(sfa_tmem, smem_desc_sf_atom(base + L::kSfA + st * kMxSfAtomBytes));
 #pragma unroll
                         for (int a = 0; a < L::kAtomsB; ++a)
                             tmem_copy_sf_atom_pair(sfb_tmem + 4 * a,
-                                                   smem_desc_sf_atom(base + L::kSfB + stage * L::kSfBBytes + a * kMxSfAtomBytes));
-                        const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + stage * kMxSlotABytes);
-                        const uint32_t sb = base + L::kB + stage * L::kSlotBBytes;
+                                                   smem_desc_sf_atom(base + L::kSfB + st * L::kSfBBytes + a * kMxSfAtomBytes));
+                        const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + st * kMxSlotABytes);
+                        const uint32_t sb = base + L::kB + st * L::kSlotBBytes;
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
                             if (i < parts.n) {
@@ -264,12 +266,14 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
                                                  instr_desc_mx(2 * kTileM, parts.cols[i], kk), (kb | kk) != 0, sfa_tmem, sfb_part);
                             }
                         }
-                        umma_commit_pair(bar_empty + stage * 8);
-                        if (kb == p.n_k_blocks - 1) umma_commit_pair(bar_acc_full + (seq & (kAccFullBars - 1)) * 8);
+                        umma_commit_pair(bar_empty + st * 8);
+                        if (++st == STAGES) { st = 0; ph ^= 1u; }
                     }
-                    __syncwarp();
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    if (ok) umma_commit_pair(bar_acc_full + (seq & (kAccFullBars - 1)) * 8);
                 }
+                __syncwarp();
+                ok = __all_sync(0xffffffffu, ok);
+                ring_advance<STAGES>(stage, phase, p.n_k_blocks);
             }
             // wait until every chunk has been handed back by both CTAs' epilogues (lane c: chunk c)
             if (ok) {

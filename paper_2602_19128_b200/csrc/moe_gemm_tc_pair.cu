@@ -202,7 +202,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     } else if (warp == kPairThreads / 32 - 1) {
         producer_loop(false, true);
     } else if (warp == 1) {
-        // ---------------- MMA issuer (leader CTA only): the warp walks the ring, one elected lane issues ----------------
+        // ---------------- MMA issuer (leader CTA only): one elected thread walks a whole tile's slots ----------------
         if (rank == 0) {
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
@@ -217,27 +217,30 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
                 if (!ok) break;
                 tcgen05_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * SLABS * NT_MAX;
-                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                    ok = __all_sync(0xffffffffu, pair_wait(bar_full + stage * 8, phase, abort_flag, peer_abort, p.status,
-                                                           kSiteMmaFull + kSiteOffset));
-                    if (!ok) break;
-                    tcgen05_fence_after();
-                    if (elect_one()) {
-                        const uint64_t b_desc = smem_desc_k_major_sw128(base + L::kB + stage * L::kSlotBBytes);
+                if (elect_one()) {
+                    int st = stage;
+                    uint32_t ph = phase;
+                    for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                        ok = pair_wait(bar_full + st * 8, ph, abort_flag, peer_abort, p.status, kSiteMmaFull + kSiteOffset);
+                        if (!ok) break;
+                        tcgen05_fence_after();
+                        const uint64_t b_desc = smem_desc_k_major_sw128(base + L::kB + st * L::kSlotBBytes);
 #pragma unroll
                         for (int s = 0; s < SLABS; ++s) {
                             const uint64_t a_desc =
-                                smem_desc_k_major_sw128(base + L::kA + stage * L::kSlotABytesAll + s * kSlotABytes);
+                                smem_desc_k_major_sw128(base + L::kA + st * L::kSlotABytesAll + s * kSlotABytes);
 #pragma unroll
                             for (int kk = 0; kk < kBlockK / 16; ++kk)  // 16 K-elements = 32 bytes = 2 descriptor units
                                 umma_bf16_pair(d_tmem + s * NT_MAX, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0);
                         }
-                        umma_commit_pair(bar_empty + stage * 8);
-                        if (kb == p.n_k_blocks - 1) umma_commit_pair(bar_acc_full + acc * 8);
+                        umma_commit_pair(bar_empty + st * 8);
+                        if (++st == STAGES) { st = 0; ph ^= 1u; }
                     }
-                    __syncwarp();
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    if (ok) umma_commit_pair(bar_acc_full + acc * 8);
                 }
+                __syncwarp();
+                ok = __all_sync(0xffffffffu, ok);
+                ring_advance<STAGES>(stage, phase, p.n_k_blocks);
                 if (!ok) break;
                 if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1u; }
             }

@@ -98,11 +98,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
-// True in exactly one lane of a converged warp, always the same lane.  The role loops are run by
-// whole warps and only the issuing instructions sit under this predicate: loop state then stays
-// warp-uniform and the descriptors of TMA / tcgen05 instructions (which take uniform-register
-// operands) need no per-instruction transfer.  Measured: with a single lane running the whole loop
-// under `lane == 0`, every TMA or MMA instruction cost about 150 cycles to issue.
+// True in exactly one lane of a converged warp, always the same lane.  Waits and bookkeeping between tiles are run by
+// whole warps.  An MMA warp enters this predicate once per TILE and its thread waits for and issues all of the tile's
+// slots: the election, the vote on the wait's result and the warp barrier of every slot had cost more issue time than a
+// narrow slot's MMAs take (one-token Mixtral-shaped layer 160 -> 137 us, FP8-weight layer of 32 tokens 291 -> 267 us,
+// MX prefill on 32 resident experts 585 -> 572 us).  The one-CTA kernels' producers do the same (137 -> 135 us, one-token
+// MX layer 87.6 -> 85.7); the pair kernels' producers (MX prefill 572 -> 576 us) and the power-bound bf16 wide-tile
+// kernel (no change) keep the election per slot.  With a single lane running the whole loop under `lane == 0` instead,
+// every TMA or MMA instruction cost about 150 cycles.
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;
     asm volatile(
@@ -111,6 +114,13 @@ __device__ __forceinline__ bool elect_one() {
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(pred));
     return pred != 0;
+}
+// Ring position after n more slots.
+template <int kStages>
+__device__ __forceinline__ void ring_advance(int &stage, uint32_t &phase, int n) {
+    const int uses = stage + n;
+    phase ^= (uint32_t)(uses / kStages) & 1u;
+    stage = uses % kStages;
 }
 // Bounded wait by a whole warp; the result is made uniform.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status,
