@@ -61,6 +61,18 @@ def test_grouped_route_matches_oracle(T, E, k, n_group, topk_group):
     assert np.array_equal(off, want_off) and np.array_equal(s2f, want_s2f) and np.array_equal(f2s, want_f2s)
 
 
+@pytest.mark.parametrize("n_group,topk_group", [(8, 1), (8, 8), (7, 3), (5, 2), (2, 1)])
+def test_groups_of_32_match_oracle(n_group, topk_group):
+    """The folded reduction over groups of exactly 32 experts, full and partly used, with tied group scores."""
+    E, T, k = 32 * n_group, 70, 8
+    g = torch.Generator().manual_seed(E)
+    logits = (torch.randn((T, E), generator=g) * 1.5).cuda()
+    logits[::4] = torch.randint(-1, 2, (len(logits[::4]), E), generator=g).float().cuda()
+    ids, w, *_ = run_route(logits, k, n_group, topk_group, None, 1.5)
+    want_ids, want_w = moe_oracle.get("f32").route_grouped(logits.cpu().numpy(), k, n_group, topk_group, scale=1.5)
+    assert np.array_equal(ids, want_ids) and np.array_equal(w, want_w)
+
+
 def test_grouped_route_without_bias_and_with_ties():
     logits = torch.zeros((40, 64), device="cuda")
     logits[:, 37] = 1.0

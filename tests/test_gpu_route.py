@@ -81,6 +81,18 @@ def test_route_all_tokens_to_one_expert_and_empty_experts():
     check_against_oracle(logits, k)
 
 
+@pytest.mark.parametrize("T,E,k", [(16, 256, 8), (17, 64, 2), (256, 40, 8), (257, 256, 8), (1023, 97, 6), (1024, 256, 32),
+                                   (1025, 65, 8), (1600, 256, 1)])
+def test_route_at_the_limits_of_its_launch_forms(T, E, k):
+    """One block, several blocks, spans longer than a warp's registers, the three-kernel form; a third of the logits take
+    few distinct values, so that ties cross the selection bound and some tokens have more than 32 candidates."""
+    g = torch.Generator().manual_seed(T)
+    logits = torch.randn(T, E, generator=g)
+    logits[::3] = torch.randint(0, 4, (len(logits[::3]), E), generator=g).float() - 1.0
+    logits[1::6, E // 3:] = 2.0
+    check_against_oracle(logits, k)
+
+
 def test_route_empty_batch_and_argument_errors():
     dev = "cuda"
     E, k = 8, 2
