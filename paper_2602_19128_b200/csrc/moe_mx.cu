@@ -67,48 +67,61 @@ mx_quantize_rows_kernel(const uint4 *__restrict__ x, const int *__restrict__ fla
     const long long w = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int r = (int)(w / warps_per_row), first_seg = (int)(w % warps_per_row);
     if (r >= n_rows) return;
-    // kScatter: lane j holds rank j's destination row and where its scale bytes go inside one K-slot's atoms
-    int my_row = -1;
-    long long my_sf_base = 0;
-    if (kScatter && lane < k) {
-        my_row = flat_to_sorted[(size_t)r * k + lane];
-        if (my_row >= 0) {
-            const int e = topk_ids[(size_t)r * k + lane] - local_offset;  // resident, or the row would be -1
-            const int begin = expert_offsets[e], i = my_row - begin;
-            // row tr of token tile i / rows of this expert, whose tiles all have `rows` rows (the schedule's choice)
-            const int rows = tile_rows[e], stride = tile > 256 ? 256 : tile;
-            const int atoms_per_tile = (tile + 127) / 128, tr = i % rows;
-            my_sf_base = (long long)((begin / stride + e + i / rows) * atoms_per_tile + tr / 128) * kMxSfAtomBytes +
-                         mx_atom_byte(tr % 128, 0);
-        }
-    }
-    (void)n_local;
-    if (kScatter && !__any_sync(0xffffffffu, my_row >= 0)) return;  // none of the token's experts is resident here
+    int my_row = -1;  // kScatter: lane j holds rank j's destination row ...
+    if (kScatter && lane < k) my_row = flat_to_sorted[(size_t)r * k + lane];
+    const unsigned live = kScatter ? __ballot_sync(0xffffffffu, my_row >= 0) : 1u;
+    if (!live) return;  // none of the token's experts is resident here
     const uint4 *src = x + (size_t)r * vec_per_row;
     constexpr int kInFlight = 4;  // independent 16-byte loads per lane before the first is used
     const int n_segs = (vec_per_row + 31) / 32;
-    for (int s0 = first_seg; s0 < n_segs; s0 += kInFlight * warps_per_row) {  // uniform over the warp
-        uint4 in[kInFlight];
+    uint4 in[kInFlight];
+    auto fetch = [&](int s0) {
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u) {
             const int v = (s0 + u * warps_per_row) * 32 + lane;
             in[u] = (s0 + u * warps_per_row < n_segs && v < vec_per_row) ? src[v] : make_uint4(0, 0, 0, 0);
         }
+    };
+    // The first segments are on their way while the chain of loads below runs (rank -> expert -> its rows and tiles);
+    // after it they started two round trips later.  With the ranks without a row skipped and a slot's scale bytes stored
+    // as one word: 41 -> 33 us for 8192 tokens of 7168 features, one resident rank per token on average.
+    if (kScatter) fetch(first_seg);
+    long long my_sf_base = 0;  // ... and where its scale bytes go inside one K-slot's atoms
+    if (kScatter && my_row >= 0) {
+        const int e = topk_ids[(size_t)r * k + lane] - local_offset;  // resident, or the row would be -1
+        const int begin = expert_offsets[e], i = my_row - begin;
+        // row tr of token tile i / rows of this expert, whose tiles all have `rows` rows (the schedule's choice)
+        const int rows = tile_rows[e], stride = tile > 256 ? 256 : tile;
+        const int atoms_per_tile = (tile + 127) / 128, tr = i % rows;
+        my_sf_base = (long long)((begin / stride + e + i / rows) * atoms_per_tile + tr / 128) * kMxSfAtomBytes +
+                     mx_atom_byte(tr % 128, 0);
+    }
+    for (int s0 = first_seg; s0 < n_segs; s0 += kInFlight * warps_per_row) {  // uniform over the warp
+        if (!kScatter) fetch(s0);
+        uint4 cur[kInFlight];
+#pragma unroll
+        for (int u = 0; u < kInFlight; ++u) cur[u] = in[u];
+        if (kScatter && s0 + kInFlight * warps_per_row < n_segs) fetch(s0 + kInFlight * warps_per_row);
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u) {
             if (s0 + u * warps_per_row >= n_segs) break;  // uniform
             const int v = (s0 + u * warps_per_row) * 32 + lane;
             uint32_t sb;
-            const uint2 q = quantize_8_of_32(in[u], sb);  // every lane takes part in the shuffles
+            const uint2 q = quantize_8_of_32(cur[u], sb);  // every lane takes part in the shuffles
             const int block = v >> 2;  // 32-element block along the row; 4 blocks per 128-element slot
             if (kScatter) {
-                for (int j = 0; j < k; ++j) {
+                // the four scale bytes of a slot in one word, in the first lane of its sixteen
+                uint32_t four = sb << (8 * (block & 3));
+                four |= __shfl_xor_sync(0xffffffffu, four, 4);
+                four |= __shfl_xor_sync(0xffffffffu, four, 8);
+                uint8_t *slot = scales + (size_t)(block >> 2) * n_atoms * kMxSfAtomBytes;
+                for (unsigned rest = live; rest; rest &= rest - 1) {  // the ranks with a row here
+                    const int j = __ffs(rest) - 1;
                     const int row = __shfl_sync(0xffffffffu, my_row, j);
                     const long long sf_base = __shfl_sync(0xffffffffu, my_sf_base, j);
-                    if (row < 0 || v >= vec_per_row) continue;
+                    if (v >= vec_per_row) continue;
                     __stcs(codes + (size_t)row * vec_per_row + v, q);  // streaming: the GEMM reads it from memory anyway
-                    if ((lane & 3) == 0)
-                        scales[(size_t)(block >> 2) * n_atoms * kMxSfAtomBytes + sf_base + (block & 3)] = (uint8_t)sb;
+                    if ((lane & 15) == 0) *reinterpret_cast<uint32_t *>(slot + sf_base) = four;
                 }
             } else if (v < vec_per_row) {
                 codes[(size_t)r * vec_per_row + v] = q;

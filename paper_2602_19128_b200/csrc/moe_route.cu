@@ -781,38 +781,46 @@ combine_kernel(const uint4 *__restrict__ y, const float *__restrict__ topk_w, co
 // The same sum for a layer with a resident subset of the experts, where most ranks of most tokens have no row here
 // (the paper's 32 of 256: one live rank per token on average).  There the kernel above has one 16-byte load in flight
 // per thread and is bound by the latency of that load (3.1 TB/s alone on the machine, 0.09 ms for 8192 tokens).
-// Here a block takes kSparseTokens consecutive tokens, lists their live (token, rank) pairs in order, and every
+// Here a block takes kTokens consecutive tokens, lists their live (token, rank) pairs in order, and every
 // thread fetches up to kSparseBatch rows at once before it sums them, token after token, rank after rank: the
-// same order of summation, the same result, sixteen loads in flight.
-constexpr int kSparseTokens = 16, kSparseBatch = 16;
+// same order of summation, the same result, kSparseBatch loads in flight.  All threads build the list, one pair each,
+// in one round trip (one warp took four, and its block waited): 60 -> 40 us for 8192 tokens of 7168 features, 0.23 GB, 5.9
+// TB/s.  Below 2048 tokens a block takes four: with sixteen, 128 tokens make 56 blocks and a chain of two batches each
+// (11 -> 5 us).
+constexpr int kSparseBatch = 16;
+template <int kTokens>
 __global__ void __launch_bounds__(kCombineThreads)
 combine_sparse_kernel(const uint4 *__restrict__ y, const float *__restrict__ topk_w, const int *__restrict__ flat_to_sorted,
                       int T, int k, int vec_per_row, int blocks_per_group, uint4 *__restrict__ out) {
-    __shared__ int live_row[kSparseTokens * kMaxTopK], live_tok[kSparseTokens * kMaxTopK];
-    __shared__ float live_w[kSparseTokens * kMaxTopK];
-    __shared__ int n_live;
+    __shared__ int live_row[kTokens * kMaxTopK], live_tok[kTokens * kMaxTopK];
+    __shared__ float live_w[kTokens * kMaxTopK];
+    __shared__ int warp_live[kCombineThreads / 32];
     chain_release();
     chain_wait();
     const int group = blockIdx.x / blocks_per_group;
-    const int t0 = group * kSparseTokens, i = (blockIdx.x - group * blocks_per_group) * kCombineThreads + threadIdx.x;
-    const int n_tok = min(kSparseTokens, T - t0);
-    if (threadIdx.x < 32) {  // warp 0 compacts the live pairs, in (token, rank) order
-        int count = 0;
-        for (int e0 = 0; e0 < n_tok * k; e0 += 32) {
-            const int e = e0 + threadIdx.x;
-            const int row = e < n_tok * k ? flat_to_sorted[(size_t)t0 * k + e] : -1;
-            const unsigned mask = __ballot_sync(kFullMask, row >= 0);
-            if (row >= 0) {
-                const int at = count + __popc(mask & ((1u << threadIdx.x) - 1u));
-                live_row[at] = row;
-                live_tok[at] = e / k;
-                live_w[at] = topk_w[(size_t)t0 * k + e];
-            }
-            count += __popc(mask);
+    const int t0 = group * kTokens, i = (blockIdx.x - group * blocks_per_group) * kCombineThreads + threadIdx.x;
+    const int n_tok = min(kTokens, T - t0);
+    int n_live = 0;
+    for (int e0 = 0; e0 < n_tok * k; e0 += kCombineThreads) {  // the live pairs, in (token, rank) order
+        const int e = e0 + threadIdx.x, warp = threadIdx.x >> 5;
+        const int row = e < n_tok * k ? flat_to_sorted[(size_t)t0 * k + e] : -1;
+        const float w = e < n_tok * k ? topk_w[(size_t)t0 * k + e] : 0.f;
+        const unsigned mask = __ballot_sync(kFullMask, row >= 0);
+        if ((threadIdx.x & 31) == 0) warp_live[warp] = __popc(mask);
+        __syncthreads();
+        int at = n_live + __popc(mask & ((1u << (threadIdx.x & 31)) - 1u));
+#pragma unroll
+        for (int q = 0; q < kCombineThreads / 32; ++q) {
+            if (q < warp) at += warp_live[q];
+            n_live += warp_live[q];
         }
-        if (threadIdx.x == 0) n_live = count;
+        if (row >= 0) {
+            live_row[at] = row;
+            live_tok[at] = e / k;
+            live_w[at] = w;
+        }
+        __syncthreads();  // (warp_live is written again)
     }
-    __syncthreads();
     if (i >= vec_per_row) return;
     const int L = n_live;
     float acc[8];
@@ -915,8 +923,10 @@ cudaError_t launch_combine(const __nv_bfloat16 *y, const float *topk_w, const in
                            int H, __nv_bfloat16 *out, cudaStream_t stream, bool resident_subset) {
     const int vec_per_row = H / 8, blocks_per_token = (vec_per_row + kCombineThreads - 1) / kCombineThreads;
     if (resident_subset) {
-        const long long groups = ((long long)T + kSparseTokens - 1) / kSparseTokens;
-        return launch_chained(combine_sparse_kernel, (unsigned)(groups * blocks_per_token), kCombineThreads, 0, stream,
+        const int tokens = T >= 2048 ? 16 : 4;
+        const long long groups = ((long long)T + tokens - 1) / tokens;
+        return launch_chained(tokens == 16 ? combine_sparse_kernel<16> : combine_sparse_kernel<4>,
+                              (unsigned)(groups * blocks_per_token), kCombineThreads, 0, stream,
                               reinterpret_cast<const uint4 *>(y), topk_w, flat_to_sorted, T, k, vec_per_row, blocks_per_token,
                               reinterpret_cast<uint4 *>(out));
     }
