@@ -23,7 +23,8 @@
  * read from memory once per group, streams its tokens through a pipeline of TMA copies that follow the page table
  * (one tile per page for page sizes that are powers of two of at least 8, one 256-byte row copy per token otherwise),
  * and the last block of each (item, key-value head) merges the partial results.  Results do not depend on which block
- * is last.
+ * is last.  For tiled page sizes, a batch whose blocks fill the machine at most twice and whose lengths differ enough is cut
+ * into equal pieces, one per resident block, instead (a piece: the end of one sequence, whole ones, the start of another).
  */
 #ifndef GQA_DECODE_B200_H_
 #define GQA_DECODE_B200_H_
@@ -73,7 +74,9 @@ MOE_API int gqa_paged_decode(const void *q, const void *k_cache, const void *v_c
  * (its first 256 bytes are overwritten). */
 MOE_API int gqa_selftest_wait_timeout(void *workspace, size_t workspace_bytes, void *stream);
 
-/* Host-only, pure.  Tokens per sequence split and number of splits the call above uses for these sizes (reporting). */
+/* Host-only, pure.  Tokens per sequence split the workspace above is sized for (reporting): the finest the call above may
+ * use; it cuts sequences less finely where its blocks fill the machine without.  A workspace that holds the partial results
+ * of the splits in use is accepted too. */
 MOE_API int gqa_decode_split_tokens(int B, int Hq, int Hkv, int D, int max_kv_len);
 
 #ifdef __cplusplus

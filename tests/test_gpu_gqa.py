@@ -82,6 +82,25 @@ def test_decode_matches_oracle(B, Hq, Hkv, P, lengths):
     check(inp)
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,P,long,short", [
+    (24, 64, 8, 16, [8000, 0, 4100, 64], 65),     # one sequence in dozens of parts, empty items, pieces of whole sequences
+    (24, 8, 8, 8, [0, 0, 8191], 1),               # groups of one head, the line starts behind empty items
+    (140, 32, 2, 64, [6000, 2049, 0], 63),        # groups of 16 heads, more items than the 128 ranges they are summed in
+    (300, 2, 1, 32, [9000, 128], 0),              # nearly everything empty: fewer pieces than blocks
+])
+def test_equal_pieces_of_a_ragged_batch_match_oracle(B, Hq, Hkv, P, long, short):
+    """Lengths ragged enough for the balanced form: sequences cut by the blocks' pieces at any chunk."""
+    lengths = [short] * B
+    for i, n in enumerate(long):
+        lengths[(i * 7 + (0 if i % 2 else B - 1)) % B] = n
+    inp = make_gqa_inputs(dict(B=B, Hq=Hq, Hkv=Hkv, D=128, page_size=P, lengths=lengths), seed=B, device="cuda")
+    full = check(inp)
+    # a workspace that holds only as many partial results as fixed splits need, whatever the lengths: the same answer
+    check(inp, max_kv_len=64)
+    again, _ = run_gpu(inp)
+    assert torch.equal(full.view(torch.int16), again.view(torch.int16))   # the merge order does not depend on arrival
+
+
 @pytest.mark.parametrize("P", [16, 12, 64, 128])
 def test_slots_past_the_end_of_a_sequence_are_never_used(P):
     """The cache behind the last token of a sequence, and every page no sequence owns, holds NaN: the tiled gather
