@@ -199,6 +199,9 @@ __device__ __forceinline__ void attend_16_tokens(const uint32_t (&qa)[kD / 16][4
                 asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};"
                              ::"r"(v_tile + tile_offset<true>(row_base + r, i & 15, sh)), "r"(0) : "memory");
         }
+        // A block that goes on to another sequence hands this stage back, and the next copy into it is an async-proxy
+        // write: without a proxy fence by the lanes that stored, the barrier alone does not order the two.
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
     }
     // S = Q K^T for 16 tokens: two n-tiles of 8 tokens, 8 K-steps.  A warp is one of one to three on its

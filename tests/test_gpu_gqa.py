@@ -101,6 +101,17 @@ def test_equal_pieces_of_a_ragged_batch_match_oracle(B, Hq, Hkv, P, long, short)
     assert torch.equal(full.view(torch.int16), again.view(torch.int16))   # the merge order does not depend on arrival
 
 
+def test_stages_refilled_behind_a_zeroed_tail_hold_the_next_sequence():
+    """Equal pieces of many short sequences with ragged ends: nearly every stage whose last value rows were zeroed is
+    filled again by the same block.  A zero that lands on the next sequence's values would change a result."""
+    lengths = [6100] + [64 * (i % 3 + 1) + (7 * i) % 63 + 1 for i in range(47)]
+    inp = make_gqa_inputs(dict(B=48, Hq=32, Hkv=4, D=128, page_size=16, lengths=lengths), seed=1, device="cuda")
+    first = check(inp)
+    for _ in range(10):
+        again, _ = run_gpu(inp)
+        assert torch.equal(first.view(torch.int16), again.view(torch.int16))
+
+
 @pytest.mark.parametrize("P", [16, 12, 64, 128])
 def test_slots_past_the_end_of_a_sequence_are_never_used(P):
     """The cache behind the last token of a sequence, and every page no sequence owns, holds NaN: the tiled gather

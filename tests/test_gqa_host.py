@@ -2,6 +2,8 @@
 sequence splits and the workspace size.  No GPU: only the pure host functions are called, plus the argument checks
 of gqa_paged_decode that come before any CUDA call."""
 import ctypes
+import re
+from pathlib import Path
 
 import pytest
 
@@ -69,3 +71,15 @@ def test_argument_checks_come_before_any_cuda_call():
     assert call(ptrs=[0x1000] * 3 + [0x1002] + [0x1000] * 2) == ERR_ALIGN
     assert call(out_ws=(0x2000, None, 0x4010, 1 << 30, None)) == ERR_ALIGN
     assert call(out_ws=(0x2000, None, 0x4000, 16, None)) == ERR_WORKSPACE
+
+
+def test_zeroed_value_rows_are_fenced_before_a_copy_may_refill_their_stage():
+    """The rows past a sequence's end are zeroed with ordinary stores; the stage is then handed back on an mbarrier and a
+    TMA copy (the async proxy) overwrites it.  A missing proxy fence is a race that no run is sure to show, so the
+    source is read: in the function that zeroes, every lane fences between its last such store and the warp barrier."""
+    source = (Path(moe.__file__).parent / "csrc" / "gqa_decode.cu").read_text()
+    body = source[source.index("attend_16_tokens("):]
+    body = re.sub(r"//[^\n]*", "", body[:body.index("\n}\n")])
+    behind_stores = body[body.rindex("st.shared"):]
+    barrier = behind_stores.index("__syncwarp()")
+    assert "fence.proxy.async.shared::cta" in behind_stores[:barrier]
