@@ -444,17 +444,18 @@ __device__ __forceinline__ void merge_parts(const Params &p, const Segment &seg,
     };
     fetch_ml(0);
     fetch(0, 0);
+    // Weight of a sum taken relative to the maximum `from` in one relative to `to`.  No difference is taken of equal maxima:
+    // parts whose scores are all NaN have a maximum of -inf and a NaN sum, which must reach lse as a NaN.
+    auto factor_of = [](float from, float to) { return from == to ? 1.f : exp2f(from - to); };
     float m = -INFINITY, l = 0.f;
     for (int base = 0;;) {
         float m_new = m;
 #pragma unroll
         for (int u = 0; u < kMergeDeep; ++u) m_new = fmaxf(m_new, ml[u].x);
-        if (m_new != -INFINITY) {
-            l *= exp2f(m - m_new);
+        l *= factor_of(m, m_new);
 #pragma unroll
-            for (int u = 0; u < kMergeDeep; ++u) l += ml[u].y * exp2f(ml[u].x - m_new);
-            m = m_new;
-        }
+        for (int u = 0; u < kMergeDeep; ++u) l += ml[u].y * factor_of(ml[u].x, m_new);
+        m = m_new;
         base += kMergeBatch;
         if (base >= n_parts) break;
         fetch_ml(base);
@@ -463,7 +464,7 @@ __device__ __forceinline__ void merge_parts(const Params &p, const Segment &seg,
     for (int off = 4; off > 0; off >>= 1) {  // (a fixed tree)
         const float om = __shfl_xor_sync(0xffffffffu, m, off), ol = __shfl_xor_sync(0xffffffffu, l, off);
         const float mm = fmaxf(m, om);
-        l = mm == -INFINITY ? 0.f : l * exp2f(m - mm) + ol * exp2f(om - mm);
+        l = l * factor_of(m, mm) + ol * factor_of(om, mm);
         m = mm;
     }
     sync_compute();  // (the buffers' previous readers are done)

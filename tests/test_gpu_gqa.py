@@ -130,6 +130,32 @@ def test_slots_past_the_end_of_a_sequence_are_never_used(P):
     check(inp)
 
 
+@pytest.mark.parametrize("P,lengths", [
+    (16, [300, 5]),                        # one part per sequence
+    (16, [20000, 9000]),                   # fixed splits, merged
+    (12, [20000, 9000]),                   # the same from the row gather
+    (16, [8000, 3000] + [70] * 22),        # equal pieces
+])
+def test_nan_scores_reach_out_and_lse(P, lengths):
+    """A query head of NaN, and a run of NaN keys long enough to be whole parts of the sequence: out and lse are NaN
+    for the heads that saw them, whether a sequence was merged from parts or not.  (lse = -inf would say that nothing
+    is cached: a caller that combines attention states by lse would drop the NaN.)"""
+    inp = make_gqa_inputs(dict(B=len(lengths), Hq=32, Hkv=4, D=128, page_size=P, lengths=lengths), seed=P, device="cuda")
+    expect_out, expect_lse = oracle(inp)
+    nan = np.zeros(expect_lse.shape, dtype=bool)
+    inp["q"][0, 3] = float("nan")
+    nan[0, 3] = True
+    n_pages = min(lengths[0] // P, 6000 // P)           # the first tokens of item 0, as whole pages, key-value head 2
+    inp["k_cache"][inp["kv_indices"][:n_pages].long(), :, 2] = float("nan")
+    nan[0, 16:24] = True
+    out, lse = run_gpu(inp)
+    got, got_lse = out.float().cpu().numpy(), lse.cpu().numpy()
+    assert np.array_equal(np.isnan(got_lse), nan), got_lse[0]
+    assert np.isnan(got[nan]).all()
+    assert (np.abs(got - expect_out) <= OUT_TOL * (1 + np.abs(expect_out)))[~nan].all()
+    assert (np.abs(got_lse - expect_lse) <= LSE_TOL)[~nan].all()
+
+
 def test_the_workspace_status_word_reports_success():
     inp = make_gqa_inputs(dict(B=2, Hq=32, Hkv=4, D=128, page_size=16, lengths=[5000, 300]), seed=3, device="cuda")
     ws = moe.alloc_workspace(moe.gqa_decode_workspace_bytes(2, 32, 4, 128, 5000), "cuda")
