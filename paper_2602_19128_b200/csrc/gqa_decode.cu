@@ -29,7 +29,7 @@
 //     fetches the parts' outputs together with their (max, sum) pairs: one sequence of 65 536 tokens in 49 parts 42 -> 37 us.
 // The merge is a fixed-order sum over parts, so results do not depend on which block arrives last.
 // Every wait on a stage's barrier is bounded: a block that gives up records MOE_ERR_DEVICE_TIMEOUT in the
-// workspace's status word (read it with moe_last_status) and leaves without writing a result.
+// workspace's status word (read it with moe_last_status) and leaves without writing a result for the segment it was in.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -157,19 +157,6 @@ __device__ __forceinline__ bool bounded_wait(uint32_t bar, uint32_t parity, int 
     *gave_up = 1;
     if (atomicCAS(status, 0, (int)MOE_ERR_DEVICE_TIMEOUT) == 0) { status[1] = 12; status[2] = blockIdx.x; }
     return false;
-}
-
-// Self-test of that error path: one warp waits, with a small bound, on a barrier at which nothing arrives.
-__global__ void gqa_wait_timeout_selftest_kernel(int *status) {
-    __shared__ __align__(8) unsigned long long bar;
-    __shared__ int gave_up;
-    if (threadIdx.x == 0) {
-        mbar_init(smem_u32(&bar), 1);
-        gave_up = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    bounded_wait(smem_u32(&bar), 0, 1 << 14, &gave_up, status);
 }
 
 // Byte offset, inside a 64-token tile, of 16-byte piece `piece` (0..15) of token row `row`.
@@ -305,6 +292,33 @@ __device__ __forceinline__ void attend_16_tokens(const uint32_t (&qa)[kD / 16][4
 
 // ---- shared by the two kernels ----------------------------------------------------------------------------------
 __device__ __forceinline__ void sync_compute() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
+// The same barrier, and whether any of the 128 threads passed true: what they do next, they do together.
+__device__ __forceinline__ bool any_compute(bool flag) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "bar.red.or.pred p, 1, %2, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(any) : "r"((uint32_t)flag), "n"(kThreads) : "memory");
+    return any != 0;
+}
+
+// Self-test of the error path: one of the four compute warps waits, with a small bound, on a barrier at which nothing
+// arrives.  All four must come to the same answer, that the block has no result, and count themselves in the fourth word.
+__global__ void __launch_bounds__(kThreads) gqa_wait_timeout_selftest_kernel(int *status) {
+    __shared__ __align__(8) unsigned long long bar;
+    __shared__ int gave_up;
+    if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&bar), 1);
+        gave_up = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const bool ok = threadIdx.x >= 32 || bounded_wait(smem_u32(&bar), 0, 1 << 14, &gave_up, status);
+    __syncwarp();
+    if (any_compute(!ok) && (threadIdx.x & 31) == 0) atomicAdd(status + 3, 1);
+}
 
 __device__ __forceinline__ int cached_tokens(const Params &p, int b) {
     const int pages = __ldg(&p.kv_indptr[b + 1]) - __ldg(&p.kv_indptr[b]);
@@ -347,7 +361,7 @@ constexpr int kMergeFloats = kWarps * (kWarps - 1) * 4 * 32 * 2, kMergeBytes = (
 
 // End of a segment, by the 128 compute threads: the four warps' (max, sum, O) are merged -- warp w ends up with dims 32 w ..
 // 32 w + 31 of every head, eight heads per pass, summed in warp order -- and written to out / lse, or, for a part of a
-// sequence, to the part's slot.
+// sequence, to the part's slot.  The caller has passed a barrier of these threads since the buffer was last read.
 __device__ __forceinline__ void store_segment(const Params &p, const Segment &seg, const float (&o_acc)[kD / 8][4],
                                               const float (&m_run)[2], const float (&l_run)[2], float *merge, int warp, int lane) {
     float2 *foreign = reinterpret_cast<float2 *>(merge);                        // [to warp][from][4 n-tiles][32 lanes]
@@ -358,7 +372,7 @@ __device__ __forceinline__ void store_segment(const Params &p, const Segment &se
 #pragma unroll
     for (int pass = 0; pass < 2; ++pass) {  // heads 8 pass .. 8 pass + 7
         if (pass * 8 >= p.group) break;
-        sync_compute();                     // (the buffer's previous readers are done)
+        if (pass > 0) sync_compute();       // (the buffer's previous readers are done)
         if ((lane & 3) == 0) ml_w[warp * kRows + pass * 8 + r0] = make_float2(m_run[pass], l_run[pass]);
 #pragma unroll
         for (int to = 0; to < kWarps; ++to)
@@ -880,7 +894,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         int tok_base = c * kChunk + warp * 16;
         for (int i = run; i > 0; --i, tok_base += kChunk) {
             if (ok) ok = __all_sync(0xffffffffu, bounded_wait(full_base + stage * 8, parity, kWaitLimit, &gave_up, p.status));
-            if (!ok) break;  // (the warp still takes part in every barrier below; the status word says that out is incomplete)
+            if (!ok) break;
             const uint32_t k_tile = smem_base + stage * kTiledStageBytes;
             if (tok_base < L)  // (uniform over the warp)
                 attend_16_tokens<true>(qa, o_acc, m_run, l_run, k_tile, k_tile + kTiledTileBytes, warp * 16, tok_base, L, sh,
@@ -889,6 +903,8 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
             if (lane == 0) mbar_arrive(empty_base + stage * 8);
             if (++stage == kTiledStages) { stage = 0; parity ^= 1u; }
         }
+        // A block one of whose warps gave up stores and counts nothing more: what it would store is not the whole segment.
+        if (any_compute(!ok)) { ok = false; break; }
         Segment seg;
         seg.b = b; seg.kvh = kvh;
         bool first = true;
@@ -1012,7 +1028,7 @@ int gqa_selftest_wait_timeout(void *workspace, size_t workspace_bytes, void *str
     if (arch != MOE_OK) return arch;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(workspace, 0, 256, st) != cudaSuccess) return MOE_ERR_CUDA;
-    gqa_wait_timeout_selftest_kernel<<<1, 32, 0, st>>>(static_cast<int *>(workspace));
+    gqa_wait_timeout_selftest_kernel<<<1, kThreads, 0, st>>>(static_cast<int *>(workspace));
     return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }
 

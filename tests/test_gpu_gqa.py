@@ -181,6 +181,15 @@ def test_an_expired_barrier_wait_is_reported_and_leaves_the_device_usable():
     assert moe.moe_last_status(ws) == 0
 
 
+def test_warps_of_a_block_whose_wait_ran_out_leave_together():
+    """One warp's wait runs out while the other three have what they waited for: all four come to the answer that the
+    block has no result to store.  (What three of four warps have would overwrite out with an incomplete sum.)"""
+    ws = moe.alloc_workspace(256, "cuda")
+    moe.gqa_selftest_wait_timeout(ws)
+    assert moe.moe_last_status(ws) == -7
+    assert ws[:16].view(torch.int32)[3].item() == 4
+
+
 def test_a_sequence_longer_than_the_hint_is_still_computed_in_full():
     inp = make_gqa_inputs(dict(B=2, Hq=32, Hkv=4, D=128, page_size=16, lengths=[3000, 500]), seed=2, device="cuda")
     check(inp, max_kv_len=1024)     # the last split runs to the end of the sequence
