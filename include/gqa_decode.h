@@ -39,7 +39,8 @@ extern "C" {
 #endif
 
 /* Host-only, pure.  Bytes of workspace gqa_paged_decode needs (a status word, block counters and the partial results
- * of the sequence splits); 0 outside the supported envelope.  max_kv_len: an upper bound of the cached lengths, used to size
+ * of the sequence splits or, where there may be more of those, of the equal pieces: two per resident block; a workspace
+ * that holds the splits' alone is accepted, and the batch is then never cut into pieces); 0 outside the supported envelope.  max_kv_len: an upper bound of the cached lengths, used to size
  * the split of the sequence (a longer sequence is still computed correctly, by its last block).
  * Envelope: D == 128; Hq a multiple of Hkv with 1 <= Hq / Hkv <= 16; B >= 0; max_kv_len >= 0. */
 MOE_API size_t gqa_decode_workspace_bytes(int B, int Hq, int Hkv, int D, int max_kv_len);
@@ -75,9 +76,8 @@ MOE_API int gqa_paged_decode(const void *q, const void *k_cache, const void *v_c
  * (its first 256 bytes are overwritten). */
 MOE_API int gqa_selftest_wait_timeout(void *workspace, size_t workspace_bytes, void *stream);
 
-/* Host-only, pure.  Tokens per sequence split the workspace above is sized for (reporting): the finest the call above may
- * use; it cuts sequences less finely where its blocks fill the machine without.  A workspace that holds the partial results
- * of the splits in use is accepted too. */
+/* Host-only, pure.  Tokens per sequence split the call above uses for these sizes (reporting), except for a batch that it
+ * cuts into equal pieces: those depend on the lengths, which only the device knows. */
 MOE_API int gqa_decode_split_tokens(int B, int Hq, int Hkv, int D, int max_kv_len);
 
 #ifdef __cplusplus

@@ -980,30 +980,27 @@ void choose_fixed_split(int B, int Hkv, int max_kv_len, int *split_tokens, int *
     *n_splits = (int)((chunks + per_block - 1) / per_block);
 }
 
-// The split the workspace is sized for and the reporting function names: the fixed one, cut finer where a long
-// sequence's batch would otherwise have fewer slots than the balanced blocks need, two each.  Sequences of up to 32 chunks
-// keep the fixed split: there the batch either has slots enough or its blocks are short anyway.
-void choose_split(int B, int Hkv, int max_kv_len, int *split_tokens, int *n_splits) {
-    choose_fixed_split(B, Hkv, max_kv_len, split_tokens, n_splits);
+// Slots per (item, key-value head) the workspace is sized for: the fixed splits, or more where a long sequence's batch would
+// otherwise have fewer slots than the balanced blocks need, two each.  Sequences of up to 32 chunks keep the fixed
+// split's: there the batch either has slots enough or its blocks are short anyway.
+int choose_slots(int B, int Hkv, int max_kv_len, int fixed_splits) {
     const long long base = (long long)B * Hkv, chunks = ((long long)max_kv_len + kChunk - 1) / kChunk;
-    if (base < 1 || chunks <= 32 || base * *n_splits >= 2 * kBalancedBlocks) return;
+    if (base < 1 || chunks <= 32 || base * fixed_splits >= 2 * kBalancedBlocks) return fixed_splits;
     long long n = (2 * kBalancedBlocks + base - 1) / base;
     if (n > chunks / 4) n = chunks / 4;
     if (n > kMaxSplits) n = kMaxSplits;
-    if (n <= *n_splits) return;
-    const long long per_block = chunks / n;  // (rounded down: at least n splits)
-    const long long splits = (chunks + per_block - 1) / per_block;
-    if (splits > kMaxSplits) return;
-    *split_tokens = (int)(per_block * kChunk);
-    *n_splits = (int)splits;
+    if (n <= fixed_splits) return fixed_splits;
+    const long long per_slot = chunks / n;  // (rounded down: at least n slots, in whole runs of chunks)
+    const long long slots = (chunks + per_slot - 1) / per_slot;
+    return slots > kMaxSplits ? fixed_splits : (int)slots;
 }
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-size_t workspace_bytes_for(int B, int Hq, int Hkv, int n_splits) {
+size_t workspace_bytes_for(int B, int Hq, int Hkv, int slots) {
     const size_t bh = (size_t)B * Hkv, group = Hq / Hkv;
-    return 256 + align_up(bh * sizeof(int), 256) + align_up(bh * n_splits * group * 2 * sizeof(float), 256) +
-           align_up(bh * n_splits * group * kD * sizeof(float), 256) + 256;
+    return 256 + align_up(bh * sizeof(int), 256) + align_up(bh * slots * group * 2 * sizeof(float), 256) +
+           align_up(bh * slots * group * kD * sizeof(float), 256) + 256;
 }
 
 }  // namespace
@@ -1015,8 +1012,8 @@ size_t gqa_decode_workspace_bytes(int B, int Hq, int Hkv, int D, int max_kv_len)
     using namespace gqa;
     if (!envelope_ok(B, Hq, Hkv, D, max_kv_len)) return 0;
     int st, ns;
-    choose_split(B, Hkv, max_kv_len, &st, &ns);
-    return workspace_bytes_for(B, Hq, Hkv, ns);
+    choose_fixed_split(B, Hkv, max_kv_len, &st, &ns);
+    return workspace_bytes_for(B, Hq, Hkv, choose_slots(B, Hkv, max_kv_len, ns));
 }
 
 int gqa_selftest_wait_timeout(void *workspace, size_t workspace_bytes, void *stream) {
@@ -1036,7 +1033,7 @@ int gqa_decode_split_tokens(int B, int Hq, int Hkv, int D, int max_kv_len) {
     using namespace gqa;
     if (!envelope_ok(B, Hq, Hkv, D, max_kv_len)) return 0;
     int st, ns;
-    choose_split(B, Hkv, max_kv_len, &st, &ns);
+    choose_fixed_split(B, Hkv, max_kv_len, &st, &ns);
     return st;
 }
 
@@ -1056,11 +1053,11 @@ int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, co
         misaligned(workspace, 256))
         return MOE_ERR_ALIGN;
     // A workspace that holds the fixed splits' results only is enough too: the fixed form then.
-    int fixed_tokens, fixed_splits, slot_tokens, slot_splits;
+    int fixed_tokens, fixed_splits;
     choose_fixed_split(B, Hkv, max_kv_len, &fixed_tokens, &fixed_splits);
-    choose_split(B, Hkv, max_kv_len, &slot_tokens, &slot_splits);
-    if (workspace_bytes < workspace_bytes_for(B, Hq, Hkv, slot_splits)) slot_splits = fixed_splits;
-    if (workspace_bytes < workspace_bytes_for(B, Hq, Hkv, slot_splits)) return MOE_ERR_WORKSPACE;
+    int slots = choose_slots(B, Hkv, max_kv_len, fixed_splits);
+    if (workspace_bytes < workspace_bytes_for(B, Hq, Hkv, slots)) slots = fixed_splits;
+    if (workspace_bytes < workspace_bytes_for(B, Hq, Hkv, slots)) return MOE_ERR_WORKSPACE;
     const int arch = moe::check_device();
     if (arch != MOE_OK) return arch;
 
@@ -1083,7 +1080,7 @@ int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, co
     p.counters = reinterpret_cast<int *>(ws + 256);
     ws += 256 + align_up(bh * sizeof(int), 256);
     p.part_ml = reinterpret_cast<float *>(ws);
-    ws += align_up(bh * slot_splits * p.group * 2 * sizeof(float), 256);
+    ws += align_up(bh * slots * p.group * 2 * sizeof(float), 256);
     p.part_o = reinterpret_cast<float *>(ws);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1106,7 +1103,7 @@ int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, co
     if (!tiled) {
         if (!ready(gqa_row_decode_kernel, kSmemBytes)) return MOE_ERR_CUDA;
         gqa_row_decode_kernel<<<dim3(p.n_splits, Hkv, B), kThreads, kSmemBytes, st>>>(p);
-    } else if (bh * slot_splits >= 2 * kBalancedBlocks && bh * p.n_splits <= 2 * kBalancedBlocks) {
+    } else if (bh * slots >= 2 * kBalancedBlocks && bh * p.n_splits <= 2 * kBalancedBlocks) {
         if (!ready(gqa_tiled_decode_kernel<true>, kSmemBytesTiled)) return MOE_ERR_CUDA;
         gqa_tiled_decode_kernel<true><<<shares > kBalancedBlocks ? shares : kBalancedBlocks, kThreads + 32, kSmemBytesTiled, st>>>(p, k_map, v_map);
     } else {
