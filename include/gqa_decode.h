@@ -57,7 +57,8 @@ MOE_API size_t gqa_decode_workspace_bytes(int B, int Hq, int Hkv, int D, int max
  *   workspace        at least gqa_decode_workspace_bytes(...) bytes, 256-byte aligned; concurrent calls need distinct
  *                    workspaces.  Afterwards its first int32 is the call's device status, which
  *                    moe_last_status(workspace, stream) reads: MOE_OK, or MOE_ERR_DEVICE_TIMEOUT when a block's bounded
- *                    wait for its copies ran out (out is then incomplete); the rest is undefined
+ *                    wait for its copies ran out (out is then incomplete); its fourth is 1 if the batch was cut into
+ *                    equal pieces, else 0 (reporting); the rest is undefined
  * Pointers of q, the caches and out must be 16-byte aligned, the int arrays and lse 4-byte aligned.
  * B == 0 succeeds without a launch.  Page numbers and lengths are NOT validated (they live on the device); page
  * numbers outside [0, num_pages) are outside the contract.  num_pages * page_size must be below 2^31

@@ -734,6 +734,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         if (tid < kThreads)
             for (int i = tid * per; i < min(p.B, (tid + 1) * per); ++i) {
                 const int n = (cached_tokens(p, i) + kChunk - 1) / kChunk;
+                if (n <= 0) continue;  // an item without tokens has no share
                 const int parts_of = min(p.n_splits, (n + split_chunks - 1) / split_chunks);
                 sum += n;
                 sequence = max(sequence, n);
@@ -784,6 +785,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
             w = divide(total * blockIdx.x, n_blocks);
             w_end = divide(total * (blockIdx.x + 1), n_blocks);
             if (tid == 0) { line.total = total; line.begin = w; line.end = w_end; line.n_blocks = n_blocks; line.balanced = true; }
+            if (blockIdx.x == 0 && tid == 0) p.status[3] = 1;  // (reporting: the batch was cut into equal pieces)
             const int x = (int)divide(w, p.Hkv);
             int r = 0;  // the last range that starts at or before chunk x of the items
 #pragma unroll

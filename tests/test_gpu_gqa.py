@@ -101,6 +101,29 @@ def test_equal_pieces_of_a_ragged_batch_match_oracle(B, Hq, Hkv, P, long, short)
     assert torch.equal(full.view(torch.int16), again.view(torch.int16))   # the merge order does not depend on arrival
 
 
+def ran_equal_pieces(inp, max_kv_len=None, workspace_bytes=None):
+    """Whether the call cut the batch into equal pieces (the workspace's fourth word); its result is checked."""
+    B, Hq, Hkv, D = inp["B"], inp["Hq"], inp["Hkv"], inp["D"]
+    max_kv_len = max(inp["kv_len"]) if max_kv_len is None else max_kv_len
+    wg = Guarded(moe.gqa_decode_workspace_bytes(B, Hq, Hkv, D, max_kv_len) if workspace_bytes is None else workspace_bytes, "cuda")
+    out = torch.empty((B, Hq, D), dtype=torch.bfloat16, device="cuda")
+    moe.gqa_paged_decode(inp["q"], inp["k_cache"], inp["v_cache"], inp["kv_indptr"], inp["kv_indices"],
+                         inp["kv_last_page_len"], max_kv_len, inp["sm_scale"], out, wg.inner)
+    assert moe.moe_last_status(wg.inner) == 0
+    wg.assert_bands_intact("gqa_paged_decode workspace")
+    ref, _ = oracle(inp)
+    assert (np.abs(out.float().cpu().numpy() - ref) <= OUT_TOL * (1 + np.abs(ref))).all()
+    return bool(wg.inner[12:16].view(torch.int32).item())
+
+
+@pytest.mark.parametrize("B,Hkv,n,max_kv_len", [(16, 4, 1000, 16000), (30, 4, 500, 2500), (24, 8, 1000, 2500)])
+def test_an_item_without_tokens_does_not_change_the_form(B, Hkv, n, max_kv_len):
+    """Equal lengths keep the fixed shares, however far below the hint; so do they with one empty item among them."""
+    for lengths in ([n] * B, [n] * (B - 1) + [0]):
+        inp = make_gqa_inputs(dict(B=B, Hq=8 * Hkv, Hkv=Hkv, D=128, page_size=16, lengths=lengths), seed=B, device="cuda")
+        assert not ran_equal_pieces(inp, max_kv_len)
+
+
 def test_stages_refilled_behind_a_zeroed_tail_hold_the_next_sequence():
     """Equal pieces of many short sequences with ragged ends: nearly every stage whose last value rows were zeroed is
     filled again by the same block.  A zero that lands on the next sequence's values would change a result."""
