@@ -25,9 +25,11 @@ namespace moe {
 namespace {
 
 constexpr unsigned kFullMask = 0xffffffffu;
-// A chunk's block has 16 warps of two tokens each: at 64 registers two such blocks fit on an SM, and the 256 blocks of an
-// 8192-token batch run in one wave (one block of 32 warps per SM: two waves).
-constexpr int kRouteThreads = 512;
+// A chunk's block has a warp per token while every block has an SM of its own, and 16 warps of two tokens each beyond: at
+// 64 registers two such blocks fit on an SM, and the 256 blocks of an 8192-token batch run in one wave, not in two.
+// Router and sort of 64 experts, top 2, a warp per token / two tokens: 4096 tokens 16.4 / 16.4 us, 1025 14.4 / 15.4; 8192
+// 19.5 / 18.4.
+constexpr int kRouteThreads = 1024, kRouteThreadsManyChunks = 512, kRouteSms = 148;
 constexpr int kLogitsPerLane = kMaxExperts / 32;
 
 // Order-preserving map from float to unsigned: a > b  <=>  ordered_key(a) > ordered_key(b) (for non-NaN values;
@@ -75,9 +77,22 @@ struct Candidates {
 // counts the candidates before it.  More than 32 candidates (many equal logits, k near 32) fall back to select_top_k.
 // About half the warp instructions, at E = 256 and k = 8, of k rounds of a full arg-max over eight registers, and a chain
 // of k short reductions instead of k long ones (8192 tokens: router and sort 43 -> 25 us, grouped 56 -> 33 us).
+// k = 1 is a single arg-max (route_topk_kernel, 1500 tokens of 32 experts: 5.8 -> 5.1 us).
 // Lane j < k returns rank j's expert with its key and score.
 __device__ __forceinline__ void select_candidates(const unsigned (&key)[kLogitsPerLane], const float (&score)[kLogitsPerLane], int E,
                                                   int k, int lane, Candidates *c, int &my_id, unsigned &my_key, float &my_score) {
+    if (k == 1) {  // one arg-max
+        unsigned best = key[0];
+        int e = lane;
+        float v = score[0];
+#pragma unroll
+        for (int i = 1; i < kLogitsPerLane; ++i)
+            if (key[i] > best) { best = key[i]; e = i * 32 + lane; v = score[i]; }
+        my_key = __reduce_max_sync(kFullMask, lane < E ? best : 0u);
+        my_id = (int)__reduce_min_sync(kFullMask, lane < E && best == my_key ? (unsigned)e : (unsigned)INT_MAX);
+        my_score = __shfl_sync(kFullMask, v, my_id & 31);
+        return;
+    }
     int n;
     unsigned cand_key = key[0];
     int cand_e = lane;
@@ -351,20 +366,21 @@ __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, i
     }
 }
 
-__global__ void __launch_bounds__(kRouteThreads, 2)
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 route_topk_kernel(const float *__restrict__ logits, int T, int E, int k, int local_offset, int n_local,
                   const RouterParams rp, int *__restrict__ topk_ids, float *__restrict__ topk_w,
                   int *__restrict__ chunk_counts) {
     __shared__ int hist[kMaxExperts];  // indexed by local expert (expert id - local_offset)
-    __shared__ Candidates cand[kRouteThreads / 32];
+    __shared__ Candidates cand[kThreads / 32];
     chain_release();
-    for (int e = threadIdx.x; e < n_local; e += kRouteThreads) hist[e] = 0;
+    for (int e = threadIdx.x; e < n_local; e += kThreads) hist[e] = 0;
     __syncthreads();
     chain_wait();
     const int t0 = blockIdx.x * kRouteTokensPerBlock;
     route_tokens(logits, t0, min(T, t0 + kRouteTokensPerBlock), E, k, local_offset, n_local, rp, topk_ids, topk_w, cand, hist);
     __syncthreads();
-    for (int e = threadIdx.x; e < n_local; e += kRouteThreads) chunk_counts[(size_t)blockIdx.x * n_local + e] = hist[e];
+    for (int e = threadIdx.x; e < n_local; e += kThreads) chunk_counts[(size_t)blockIdx.x * n_local + e] = hist[e];
 }
 
 // Exclusive scan over threads 0..255 of the block (wider blocks may call it; their other threads pass 0
@@ -467,23 +483,35 @@ __device__ __forceinline__ int schedule_phase(int count, int E, int nt_max, int 
     return row_start;
 }
 
-// Scan over the chunks, 32 experts per block: warp w takes a contiguous share of the chunks and lane l expert 32 b + l,
-// so that a load is one 128-byte line and up to kScanBatch of them are in flight per thread.  The counts are replaced by
-// the rows of all earlier chunks.  The block that finishes last (a counter zeroed by the call's memset) then has every
-// expert's total and runs the schedule phase.  One block for everything took 17-24 us at 256 chunks (of 32 to 256 experts,
-// up to 256 KB in and out of one SM); now 9-10 us.
-constexpr int kScanWarps = kScanThreads / 32, kScanBatch = 16;
+// Scan over the chunks, in groups of 32 experts: a warp takes a contiguous share of the chunks for one group, lane l its
+// l-th expert, so that a load is one 128-byte line and up to kScanBatch of them are in flight per thread.  The counts are
+// replaced by the rows of all earlier chunks.  Either one block takes all groups, a share of its warps each, and goes
+// straight on to the schedule phase; or every block takes a group, and the one that finishes last (a counter zeroed by the
+// call's memset) has every expert's total and runs the schedule phase.  Several blocks share the traffic of many chunks
+// (256 chunks, up to 256 KB in and out of one SM: 17-24 us by one block, 9-10 us by eight), but their hand-over costs 2 us:
+// one block while its threads hold all their counts in registers (kScanBatch).  Router and sort, one block / several:
+// 1500 tokens, 64 experts, top 2 14.4 / 16.5 us; 4096, 128, 8 18.5 / 20.5; 2400, 256, 8 22.6 / 20.5; 8192, 256, 8 32.8 /
+// 24.6.  A share has at least four chunks: the block's threads add up the shares one after the other (1500 tokens of 8
+// experts 14.3 -> 12.3 us).
+constexpr int kScanWarps = kScanThreads / 32, kScanBatch = 16, kScanLeast = 4;
+__host__ __device__ inline int scan_warps_per_group(int n_chunks, int groups) {
+    const int most = kScanWarps / groups, useful = (n_chunks + kScanLeast - 1) / kScanLeast;
+    return useful < most ? useful : most;
+}
 __global__ void __launch_bounds__(kScanThreads)
 route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_quantum, int *expert_offsets,
                   int *tile_prefix, int *tile_order, int *tile_rows, int *totals, int *done_counter) {
-    __shared__ int partial[kScanWarps][32];
+    __shared__ int partial[kScanWarps][32], all_totals[kMaxExperts];
     __shared__ ScheduleShared sh;
     __shared__ int is_last;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+    const bool one_block = gridDim.x == 1;
+    const int groups = one_block ? (E + 31) / 32 : 1, warps_per_group = scan_warps_per_group(n_chunks, groups);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / warps_per_group, share = warp - group * warps_per_group;
+    const int e = group < groups ? ((one_block ? group : (int)blockIdx.x) * 32 + lane) : E;  // (warps left over: no expert)
     chain_release();
     chain_wait();
-    const int per = (n_chunks + kScanWarps - 1) / kScanWarps;
-    const int b_begin = min(n_chunks, warp * per), b_end = min(n_chunks, b_begin + per);
+    const int per = (n_chunks + warps_per_group - 1) / warps_per_group;
+    const int b_begin = min(n_chunks, share * per), b_end = min(n_chunks, b_begin + per);
     const bool one_batch = per <= kScanBatch;  // then the counts stay in registers between the passes
     int first[kScanBatch];
     int sum = 0;
@@ -500,11 +528,13 @@ route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_qu
     partial[warp][lane] = sum;
     __syncthreads();
     int run = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < kScanWarps; ++w) {
-        const int v = partial[w][lane];
-        if (w < warp) run += v;
-        total += v;
+    if (e < E) {
+#pragma unroll 4
+        for (int w = 0; w < warps_per_group; ++w) {
+            const int v = partial[group * warps_per_group + w][lane];
+            if (w < share) run += v;
+            total += v;
+        }
     }
     if (e < E) {
         for (int b0 = b_begin; b0 < b_end; b0 += kScanBatch) {
@@ -518,16 +548,24 @@ route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_qu
                 run += c[i];
             }
         }
-        if (warp == 0) totals[e] = total;
+        if (share == 0) {
+            if (one_block) all_totals[e] = total; else totals[e] = total;
+        }
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(done_counter, 1) == (int)gridDim.x - 1;
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    const int count = (int)threadIdx.x < E ? __ldcg(&totals[threadIdx.x]) : 0;
-    __syncthreads();  // (the totals may sit where the schedule is written)
+    int count = 0;
+    if (one_block) {
+        __syncthreads();
+        if ((int)threadIdx.x < E) count = all_totals[threadIdx.x];
+    } else {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) is_last = atomicAdd(done_counter, 1) == (int)gridDim.x - 1;
+        __syncthreads();
+        if (!is_last) return;
+        __threadfence();
+        if ((int)threadIdx.x < E) count = __ldcg(&totals[threadIdx.x]);
+        __syncthreads();  // (the totals may sit where the schedule is written)
+    }
     schedule_phase(count, E, nt_max, row_quantum, expert_offsets, tile_prefix, tile_order, tile_rows, sh);
 }
 
@@ -890,11 +928,15 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
                               scratch.tile_prefix, scratch.tile_order, scratch.tile_rows, sorted_to_flat, flat_to_sorted,
                               status + kDoneCounterInt);
     }
-    err = launch_chained(route_topk_kernel, scratch.n_chunks, kRouteThreads, 0, stream, logits, T, E, k, local.offset,
-                         local.count, router, topk_ids, topk_w, scratch.chunk_counts);
+    const bool many = scratch.n_chunks > kRouteSms;
+    err = launch_chained(many ? route_topk_kernel<kRouteThreadsManyChunks> : route_topk_kernel<kRouteThreads>, scratch.n_chunks,
+                         many ? kRouteThreadsManyChunks : kRouteThreads, 0, stream, logits, T, E, k, local.offset, local.count,
+                         router, topk_ids, topk_w, scratch.chunk_counts);
     if (err != cudaSuccess) return err;
     // (the blocks' totals per expert sit where the last block then writes the tile rows)
-    err = launch_chained(route_scan_kernel, (local.count + 31) / 32, kScanThreads, 0, stream, scratch.chunk_counts, scratch.n_chunks,
+    const int groups = (local.count + 31) / 32, warps_per_group = scan_warps_per_group(scratch.n_chunks, groups);
+    const int scan_blocks = (scratch.n_chunks + warps_per_group - 1) / warps_per_group <= kScanBatch ? 1 : groups;
+    err = launch_chained(route_scan_kernel, scan_blocks, kScanThreads, 0, stream, scratch.chunk_counts, scratch.n_chunks,
                          local.count, nt_max, row_quantum, expert_offsets, scratch.tile_prefix, scratch.tile_order,
                          scratch.tile_rows, scratch.tile_rows, status + kDoneCounterInt);
     if (err != cudaSuccess) return err;

@@ -93,6 +93,21 @@ def test_route_at_the_limits_of_its_launch_forms(T, E, k):
     check_against_oracle(logits, k)
 
 
+@pytest.mark.parametrize("T,E,k", [(1056, 256, 1), (2048, 256, 4),    # the most chunks one block scans of 256 experts
+                                   (2049, 256, 1), (2081, 225, 8),    # one more: eight blocks
+                                   (1100, 160, 2), (3072, 161, 3),    # five groups of six warps, two left over; six of five
+                                   (4096, 128, 2), (4097, 100, 1),
+                                   (4736, 8, 1), (4737, 8, 2),        # a chunk per SM, and one more
+                                   (16384, 32, 1), (16385, 32, 4), (1025, 1, 1), (20000, 33, 1)])
+def test_route_at_the_limits_of_its_scan(T, E, k):
+    """One block for all experts' counts or one per 32 of them, shares of at least four chunks, a warp per token or per
+    two tokens, and the single arg-max of k = 1, with many ties among the logits."""
+    g = torch.Generator().manual_seed(T + E)
+    logits = torch.randn(T, E, generator=g)
+    logits[::3] = torch.randint(0, 4, (len(logits[::3]), E), generator=g).float() - 1.0
+    check_against_oracle(logits, k)
+
+
 def test_route_empty_batch_and_argument_errors():
     dev = "cuda"
     E, k = 8, 2
