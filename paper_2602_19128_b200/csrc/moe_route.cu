@@ -823,8 +823,9 @@ combine_kernel(const uint4 *__restrict__ y, const float *__restrict__ topk_w, co
 // thread fetches up to kSparseBatch rows at once before it sums them, token after token, rank after rank: the
 // same order of summation, the same result, kSparseBatch loads in flight.  All threads build the list, one pair each,
 // in one round trip (one warp took four, and its block waited): 60 -> 40 us for 8192 tokens of 7168 features, 0.23 GB, 5.9
-// TB/s.  Below 2048 tokens a block takes four: with sixteen, 128 tokens make 56 blocks and a chain of two batches each
-// (11 -> 5 us).
+// TB/s.  Where sixteen tokens per block make less than two blocks per SM a block takes four: with sixteen, 128 tokens make
+// 56 blocks and a chain of two batches each (11 -> 5 us).  Layers of 4096 features with small experts, four / sixteen: 8 of
+// 64 experts resident, top 4, 600 tokens 39.0 / 41.0 us, 1500 tokens 57.5 / 55.6; 7168 features, 1500 tokens 83.1 / 78.3.
 constexpr int kSparseBatch = 16;
 template <int kTokens>
 __global__ void __launch_bounds__(kCombineThreads)
@@ -965,7 +966,7 @@ cudaError_t launch_combine(const __nv_bfloat16 *y, const float *topk_w, const in
                            int H, __nv_bfloat16 *out, cudaStream_t stream, bool resident_subset) {
     const int vec_per_row = H / 8, blocks_per_token = (vec_per_row + kCombineThreads - 1) / kCombineThreads;
     if (resident_subset) {
-        const int tokens = T >= 2048 ? 16 : 4;
+        const int tokens = ((long long)T + 15) / 16 * blocks_per_token >= 2 * kRouteSms ? 16 : 4;
         const long long groups = ((long long)T + tokens - 1) / tokens;
         return launch_chained(tokens == 16 ? combine_sparse_kernel<16> : combine_sparse_kernel<4>,
                               (unsigned)(groups * blocks_per_token), kCombineThreads, 0, stream,

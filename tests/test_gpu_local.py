@@ -58,15 +58,18 @@ def test_local_subset_matches_oracle(T, H, I, E, k, lo, n, flags):
     assert_close_out(bf16_to_f64(out), ref, "local out")
 
 
-@pytest.mark.parametrize("T,k", [(2047, 4), (2048, 4), (2051, 16), (3, 16), (5, 4)])
-def test_sparse_combine_at_the_edges_of_its_token_groups(T, k):
+@pytest.mark.parametrize("T,k,H", [(2047, 4, 128), (2048, 4, 128), (2051, 16, 128), (3, 16, 128), (5, 4, 128),
+                                   (4720, 4, 128), (4721, 2, 128),     # 295 and 296 groups of sixteen tokens
+                                   (1168, 4, 4096), (1169, 4, 4096),   # 73 and 74 groups of four blocks each
+                                   (1171, 16, 4096)])
+def test_sparse_combine_at_the_edges_of_its_token_groups(T, k, H):
     """Groups of 4 and of 16 tokens, a ragged last group, more pairs per group than threads: the sums are taken in the
     order of the dense combine, so a subset that holds every selected expert equals the full layer bit for bit."""
-    inp = gpu_inputs(dict(T=T, H=128, I=64, E=32, top_k=k, skew=False), seed=5)
+    inp = gpu_inputs(dict(T=T, H=H, I=64, E=32, top_k=k, skew=False), seed=5)
     inp["router_logits"][:, 20:] -= 60.0   # nobody picks experts 20..31
     out, _, _ = run_local(inp, 0, 20)
     full = torch.empty_like(out)
-    ws = moe.alloc_workspace(moe.moe_workspace_bytes(T, 128, 64, 32, k), "cuda")
+    ws = moe.alloc_workspace(moe.moe_workspace_bytes(T, H, 64, 32, k), "cuda")
     moe.moe_forward(inp["x"], inp["router_logits"], inp["w13"], inp["w2"], k, full, ws)
     torch.cuda.synchronize()
     assert torch.equal(out.view(torch.int16), full.view(torch.int16))
