@@ -6,6 +6,9 @@
 #include <math.h>
 
 namespace moe {
+namespace tc {
+int sm_count();  // (moe_tc_host.cu)
+}
 
 int check_device() {
     static int verdict[64];  // per device: 0 not asked yet, 1 compute capability 10.x, 2 anything else
@@ -94,6 +97,18 @@ int layer_token_tile_bound(int T, int H, int I, int E, int k, unsigned flags, bo
     return fp8w && bound > 192 ? 192 : bound;
 }
 
+// Whether the FP8-weight layer's down GEMM starts through the hand-over.  The counting costs a gate/up epilogue about a
+// microsecond per tile, a fence behind its stores, which a K loop of 16 slots (H = 2048) hides and a shorter one does not;
+// it saves the down GEMM's start and the gate/up GEMM's tail, some microseconds once.  So with short K loops it is taken
+// only where a CTA has few tiles: no more rounds of gate/up tiles than slots in each.  With / without: 16 experts, top 4,
+// H = 4096, I = 14336, 389 tokens 838 / 854 us; 256 experts, top 6, H = 256, I = 2048, 389 tokens 238 / 176 (211 before the
+// layer had a hand-over); 64 experts, top 6, H = 1024, I = 1536, 1575 tokens 193 / 183; 8 experts, top 2, H = 512, I = 1536,
+// 389 tokens 41.0 / 41.6.
+bool fp8w_hand_over(int T, int H, int I, int E, int k, int nt_max) {
+    const long long A = (long long)T * k, slots = H / 128, token_tiles = (A < E ? A : E) + A / nt_max;
+    return slots >= 16 || token_tiles * (I / 64) <= slots * tc::sm_count();
+}
+
 int forward_impl(const void *x, const float *logits, const void *w13, const void *w2, int T, int H, int I, int E, int k,
                  void *out, void *workspace, size_t workspace_bytes, cudaStream_t stream, unsigned flags,
                  void *const *stage_events = nullptr, int local_offset = 0, int n_local = -1,
@@ -166,7 +181,7 @@ int forward_impl(const void *x, const float *logits, const void *w13, const void
     // Hand-over: the down GEMM starts expert by expert as the gate/up GEMM finishes them (not with the opt-in
     // two-slab tiles, whose epilogue counts differently).
     const bool dense_tiles = (flags & MOE_FLAG_TWO_SLAB_GEMM) != 0;
-    if (!dense_tiles && !(flags & MOE_FLAG_VALIDATION_GEMM)) {
+    if (!dense_tiles && !(flags & MOE_FLAG_VALIDATION_GEMM) && (!fp8w || fp8w_hand_over(T, H, I, E, k, nt_max))) {
         g1.handover_role = 1;
         g2.handover_role = 2;
         g1.handover = g2.handover = status;

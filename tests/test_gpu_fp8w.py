@@ -70,6 +70,23 @@ def test_fp8w_long_rows_wrap_the_rings(T, H, I, E, k):
     assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k", [(40, 256, 1152, 16, 2),    # 18 slabs of 16 experts and more: two launches in sequence
+                                       (300, 896, 4096, 18, 2),   # 7 slots, more than seven rounds: the same
+                                       (24, 256, 256, 8, 2),      # one round: the down GEMM starts through the hand-over
+                                       (40, 2048, 256, 16, 2)])   # 16 slots: the same
+def test_fp8w_with_and_without_the_hand_over(T, H, I, E, k):
+    """Both ways from the gate/up GEMM to the down GEMM, and a second call in the same workspace after each."""
+    inp = make_fp8w_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=4, device="cuda")
+    out, _ = run_fp8w(inp)
+    assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
+    ws = moe.alloc_workspace(moe.moe_workspace_bytes(T, H, I, E, k), "cuda")
+    for _ in range(2):
+        again = torch.empty_like(out)
+        moe.moe_forward_fp8w(inp["x"], inp["router_logits"], inp["w13_q"], inp["w13_scale"], inp["w2_q"], inp["w2_scale"], k,
+                             again, ws)
+        assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
 def test_fp8w_with_unit_scales_equals_the_bf16_layer_bit_for_bit():
     """All E4M3 values are bf16 values, and a scale of 1 is exact in bf16: both paths see the same operands."""
     g = torch.Generator().manual_seed(0)
