@@ -321,8 +321,9 @@ __global__ void __launch_bounds__(kThreads) gqa_wait_timeout_selftest_kernel(int
 }
 
 __device__ __forceinline__ int cached_tokens(const Params &p, int b) {
-    const int pages = __ldg(&p.kv_indptr[b + 1]) - __ldg(&p.kv_indptr[b]);
-    return pages > 0 ? (pages - 1) * p.page_size + __ldg(&p.kv_last_page_len[b]) : 0;
+    const int first = __ldg(&p.kv_indptr[b]), behind = __ldg(&p.kv_indptr[b + 1]);
+    const int last = __ldg(&p.kv_last_page_len[b]);  // (all three in flight: one round trip)
+    return behind > first ? (behind - first - 1) * p.page_size + last : 0;
 }
 // out = 0, lse = -inf for the heads of one key-value head (all 128 compute threads call).
 __device__ __forceinline__ void write_empty(const Params &p, int b, int head0, int tid) {
@@ -674,28 +675,33 @@ gqa_row_decode_kernel(const Params p) {
 // resident blocks an equal piece of it: a few whole sequences and a part of one at either end, through ONE copy pipeline
 // that never drains between sequences; a block leaves at most two partial results.  It costs the counting and merging of
 // those parts at the end, when every block finishes at once, so the blocks of a batch that fits the machine once or twice
-// (kAdaptive) read all lengths first and take the form that balanced_is_faster says.  Batches of more blocks than that
-// balance themselves.
+// (kAdaptive) read all lengths first and take the form that balanced_is_faster says.  In the fixed form they then take the
+// i-th of the shares that have tokens, not the i-th of the grid: blocks that found their share empty only after reading all
+// lengths had already made the others share an SM (one sequence of 20 000 tokens, an empty one and a hint of 40 000:
+// 28.6 -> 26.7 us).  Batches of more blocks than that balance themselves.
 constexpr int kBalancedBlocks = 148 * 2;  // as many as are resident
 constexpr int kMinPiece = 4;              // chunks a balanced block takes at least
 constexpr int kSmemBytesTiled = kTiledStages * kTiledStageBytes + kMergeBytes + 1024;
 static_assert(kSmemBytesTiled + 1024 <= 113 * 1024, "two blocks per SM");
 static_assert(kMergeBytes <= kStages * kStageBytes, "the row kernel merges in its pipeline's memory");
 
-// Which form is faster, from measured sweeps (2 to 128 sequences of 2500 to 65 536 tokens, longest = 1, 2 and 8 times the
-// shortest).  Balanced: 5 ns per chunk of the batch, the memory's rate, and about 15 us.  Fixed shares in one wave: that
-// stream or the longest share alone (0.68 us per chunk), whichever is longer, 0.4 us per chunk that the longest share is
-// longer than the average one (the rest of the machine helps it with part of its bandwidth), and about 4 us.  Fixed
-// shares in two waves lost 5 to 35 us to the balanced form wherever the lengths differed and the longest sequence had 64
-// chunks or more, and were even with it or ahead elsewhere.  Fixed / balanced, us: 64 sequences of 1024..8192 tokens 120
-// / 103, equal 8192 164 / 179; 64 of 2048..16 384 239 / 205; 20 of 1000..8000 over 8 heads 106 / 81; 30 equal ones of 4000
-// over 8 heads 77 / 87.
+// Which form is faster, fitted to 500 measured batches (1 to 150 sequences of 128 to 65 536 tokens, equal and ragged, with
+// empty ones among them, length hints of 1 to 16 times the longest).  Balanced: 5 ns per chunk of the batch, the memory's
+// rate, and about 15 us.  Fixed shares in one wave: that stream, or the longest share alone (0.9 us per chunk), whichever is
+// longer; 0.15 us per chunk that the longest share is longer than the average one; about 4 us; and, where sequences are cut,
+// their merge, which costs the balanced form more the more parts they are cut into anyway.  Fixed shares in two waves lost 5
+// to 35 us to the balanced form wherever the lengths differed and the longest sequence had 64 chunks or more, and were even
+// with it or ahead elsewhere.  The form taken was 0.7 % slower than the better one on average over the 500 batches, and 2 %
+// over 400 others.
+// Fixed / balanced, us: 64 sequences of 1024..8192 tokens 120 / 105, equal 8192 164 / 179; 4 of 4096 over 8 heads with a
+// hint of 16 384 33 / 24; 7 of 20 000 beside an empty one, hint 40 000, 70 / 60; 30 equal ones of 4000 over 8 heads 77 / 87.
 __device__ __forceinline__ bool balanced_is_faster(long long total, int longest_share, int n_shares, int longest_sequence,
-                                                   int n_sequences) {
+                                                   int n_sequences, int most_parts) {
     if (n_shares > kBalancedBlocks)
         return longest_sequence >= 64 && (float)longest_sequence * (float)n_sequences > 1.15f * (float)total;
     const float stream = 0.005f * (float)total, average = (float)total / (float)n_shares, longest = (float)longest_share;
-    return fmaxf(stream, 0.68f * longest) + 0.4f * (longest - average) > stream + 11.f;
+    const float merge = most_parts > 1 ? 8.5f - 0.7f * (float)most_parts : 0.f;
+    return fmaxf(stream, 0.9f * longest) + 0.15f * (longest - average) + merge > stream + 11.f;
 }
 
 template <bool kAdaptive>
@@ -742,74 +748,83 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
                 if (parts_of > 1) longest = max(longest, split_chunks);
                 longest = max(longest, n - (parts_of - 1) * split_chunks);
             }
-        int incl = sum;
+        int incl = sum, shares_incl = shares;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += v;
+            const int v = __shfl_up_sync(0xffffffffu, incl, off), u = __shfl_up_sync(0xffffffffu, shares_incl, off);
+            if (lane >= off) { incl += v; shares_incl += u; }
         }
         longest = __reduce_max_sync(0xffffffffu, longest);
         sequence = __reduce_max_sync(0xffffffffu, sequence);
-        shares = __reduce_add_sync(0xffffffffu, shares);
         if (warp < kWarps && lane == 31) {
             warp_sum[warp] = incl;
             warp_longest[warp] = longest;
             warp_sequence[warp] = sequence;
-            warp_shares[warp] = shares;
+            warp_shares[warp] = shares_incl;
         }
         __syncthreads();
-        int before = 0, chunks = 0;
+        int before = incl - sum, chunks = 0, shares_before = shares_incl - shares;
         longest = sequence = shares = 0;
 #pragma unroll
         for (int i = 0; i < kWarps; ++i) {
-            if (i < warp) before += warp_sum[i];
+            if (i < warp) { before += warp_sum[i]; shares_before += warp_shares[i]; }
             chunks += warp_sum[i];
             longest = max(longest, warp_longest[i]);
             sequence = max(sequence, warp_sequence[i]);
             shares += warp_shares[i];
         }
         const long long total = (long long)chunks * p.Hkv;
-        balanced = total > 0 && balanced_is_faster(total, longest, shares * p.Hkv, sequence, p.B * p.Hkv);
+        balanced = total > 0 && balanced_is_faster(total, longest, shares * p.Hkv, sequence, p.B * p.Hkv,
+                                                   min(p.n_splits, (sequence + split_chunks - 1) / split_chunks));
+        if (tid < kThreads) range_start[tid] = balanced ? before : shares_before;
+        __syncthreads();
+        // items without tokens are dealt out to the blocks
+        if (tid < kThreads)
+            for (int i = blockIdx.x; i < p.B; i += gridDim.x)
+                if (cached_tokens(p, i) <= 0)
+                    for (int h = 0; h < p.Hkv; ++h) write_empty(p, i, h * p.group, tid);
+        // The blocks' work starts at a chunk of the line (balanced) or at a share; both lie item after item, head after head.
+        int n_blocks = shares * p.Hkv;
+        long long start = blockIdx.x;
         if (balanced) {
-            if (tid < kThreads) range_start[tid] = before + incl - sum;
-            __syncthreads();
-            // items without tokens are dealt out to the blocks
-            if (tid < kThreads)
-                for (int i = blockIdx.x; i < p.B; i += gridDim.x)
-                    if (cached_tokens(p, i) <= 0)
-                        for (int h = 0; h < p.Hkv; ++h) write_empty(p, i, h * p.group, tid);
             // no block takes less than kMinPiece chunks: short lines use fewer blocks
             const long long most = (total + kMinPiece - 1) / kMinPiece;
-            const int n_blocks = (int)(most < kBalancedBlocks ? most : kBalancedBlocks);
-            if ((int)blockIdx.x >= n_blocks) return;
+            n_blocks = (int)(most < kBalancedBlocks ? most : kBalancedBlocks);
+        }
+        if ((int)blockIdx.x >= n_blocks) return;
+        if (balanced) {
             w = divide(total * blockIdx.x, n_blocks);
             w_end = divide(total * (blockIdx.x + 1), n_blocks);
+            start = w;
             if (tid == 0) { line.total = total; line.begin = w; line.end = w_end; line.n_blocks = n_blocks; line.balanced = true; }
             if (blockIdx.x == 0 && tid == 0) p.status[3] = 1;  // (reporting: the batch was cut into equal pieces)
-            const int x = (int)divide(w, p.Hkv);
-            int r = 0;  // the last range that starts at or before chunk x of the items
-#pragma unroll
-            for (int step = kThreads / 2; step > 0; step >>= 1)
-                if (range_start[r + step] <= x) r += step;
-            int at = range_start[r];
-            b = r * per;
-            L = cached_tokens(p, b);
-            n_chunks = (L + kChunk - 1) / kChunk;
-            while (at + n_chunks <= x) {
-                at += n_chunks;
-                L = cached_tokens(p, ++b);
-                n_chunks = (L + kChunk - 1) / kChunk;
-            }
-            const int rest = (int)(w - (long long)at * p.Hkv);
-            kvh = rest / n_chunks;
-            c = rest - kvh * n_chunks;
         }
-    }
-    if (!balanced) {
+        const int x = (int)divide(start, p.Hkv);
+        int r = 0;  // the last range that starts at or before chunk or share x of the items
+#pragma unroll
+        for (int step = kThreads / 2; step > 0; step >>= 1)
+            if (range_start[r + step] <= x) r += step;
+        int at = range_start[r], units;  // `units`: the item's chunks or shares per head
+        b = r * per - 1;
+        do {
+            L = cached_tokens(p, ++b);
+            n_chunks = (L + kChunk - 1) / kChunk;
+            units = balanced ? n_chunks : min(p.n_splits, (n_chunks + split_chunks - 1) / split_chunks);
+            at += max(units, 0);
+        } while (at <= x);
+        at -= units;
+        const int rest = (int)(start - (long long)at * p.Hkv);
+        kvh = rest / units;
+        c = rest - kvh * units;
+        if (!balanced) {
+            c *= split_chunks;
+            w_end = (c + split_chunks >= units * split_chunks ? n_chunks : c + split_chunks) - c;  // the last split runs to the end
+            if (tid == 0) { line.n_blocks = units; line.balanced = false; }
+        }
+    } else {
         const int split = blockIdx.x % p.n_splits;
         kvh = (blockIdx.x / p.n_splits) % p.Hkv;
         b = blockIdx.x / p.n_splits / p.Hkv;
-        if (kAdaptive && b >= p.B) return;
         L = cached_tokens(p, b);
         n_chunks = (L + kChunk - 1) / kChunk;
         if (L <= 0) {
@@ -927,7 +942,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
             seg.n_parts = line.n_blocks;
             seg.first_slot = bh * p.n_splits;
             seg.second_slot = seg.first_slot + 1;
-            seg.slot = seg.first_slot + blockIdx.x % p.n_splits;
+            seg.slot = seg.first_slot + c / split_chunks;
             seg.slot_step = 1;
         }
         store_segment(p, seg, o_acc, m_run, l_run, merge, warp, lane);

@@ -124,6 +124,24 @@ def test_an_item_without_tokens_does_not_change_the_form(B, Hkv, n, max_kv_len):
         assert not ran_equal_pieces(inp, max_kv_len)
 
 
+@pytest.mark.parametrize("Hkv,lengths,max_kv_len", [
+    (1, [30000, 0, 0, 29000], 60000),                  # empty items between, half of the splits of the others empty
+    (4, [0, 20000], 40000),                            # the shares start behind an empty item
+    (4, [0, 0, 0, 700, 64, 0, 1, 0], 20000),           # one short share per sequence, far below the hint
+    (2, [2990 + i % 7 for i in range(131)] + [0] * 9, 3000),   # more items than the 128 ranges they are summed in
+    (4, [0] * 8, 20000),                               # nothing cached at all
+])
+def test_shares_of_a_batch_that_leaves_some_empty_match_oracle(Hkv, lengths, max_kv_len):
+    """The fixed form of a batch with empty items and with splits no sequence reaches: the blocks take the shares that
+    have tokens one after the other, whatever the hint, and write the results of empty items."""
+    B = len(lengths)
+    inp = make_gqa_inputs(dict(B=B, Hq=4 * Hkv, Hkv=Hkv, D=128, page_size=16, lengths=lengths), seed=B, device="cuda")
+    if not any(lengths):
+        inp["kv_indices"] = torch.zeros(1, dtype=torch.int32, device="cuda")   # (an empty tensor has no address)
+    check(inp, max_kv_len)
+    assert not ran_equal_pieces(inp, max_kv_len)
+
+
 def test_stages_refilled_behind_a_zeroed_tail_hold_the_next_sequence():
     """Equal pieces of many short sequences with ragged ends: nearly every stage whose last value rows were zeroed is
     filled again by the same block.  A zero that lands on the next sequence's values would change a result."""
