@@ -86,7 +86,8 @@ def test_decode_matches_oracle(B, Hq, Hkv, P, lengths):
     (24, 64, 8, 16, [8000, 0, 4100, 64], 65),     # one sequence in dozens of parts, empty items, pieces of whole sequences
     (24, 8, 8, 8, [0, 0, 8191], 1),               # groups of one head, the line starts behind empty items
     (140, 32, 2, 64, [6000, 2049, 0], 63),        # groups of 16 heads, more items than the 128 ranges they are summed in
-    (300, 2, 1, 32, [9000, 128], 0),              # nearly everything empty: fewer pieces than blocks
+    (300, 2, 1, 32, [9000, 128], 0),              # nearly everything empty: too many fixed shares for equal pieces
+    (250, 2, 1, 32, [9000, 128], 0),              # nearly everything empty: fewer pieces than blocks
 ])
 def test_equal_pieces_of_a_ragged_batch_match_oracle(B, Hq, Hkv, P, long, short):
     """Lengths ragged enough for the balanced form: sequences cut by the blocks' pieces at any chunk."""
@@ -95,8 +96,9 @@ def test_equal_pieces_of_a_ragged_batch_match_oracle(B, Hq, Hkv, P, long, short)
         lengths[(i * 7 + (0 if i % 2 else B - 1)) % B] = n
     inp = make_gqa_inputs(dict(B=B, Hq=Hq, Hkv=Hkv, D=128, page_size=P, lengths=lengths), seed=B, device="cuda")
     full = check(inp)
-    # a workspace that holds only as many partial results as fixed splits need, whatever the lengths: the same answer
-    check(inp, max_kv_len=64)
+    assert ran_equal_pieces(inp) == (B != 300)
+    check(inp, max_kv_len=64)   # a hint far below the lengths: one fixed share per sequence, whatever its length
+    assert not ran_equal_pieces(inp, max_kv_len=64)
     again, _ = run_gpu(inp)
     assert torch.equal(full.view(torch.int16), again.view(torch.int16))   # the merge order does not depend on arrival
 
@@ -148,9 +150,30 @@ def test_stages_refilled_behind_a_zeroed_tail_hold_the_next_sequence():
     lengths = [6100] + [64 * (i % 3 + 1) + (7 * i) % 63 + 1 for i in range(47)]
     inp = make_gqa_inputs(dict(B=48, Hq=32, Hkv=4, D=128, page_size=16, lengths=lengths), seed=1, device="cuda")
     first = check(inp)
+    assert ran_equal_pieces(inp)
     for _ in range(10):
         again, _ = run_gpu(inp)
         assert torch.equal(first.view(torch.int16), again.view(torch.int16))
+
+
+@pytest.mark.parametrize("B,Hkv,long,short", [(24, 8, 8000, 65), (64, 4, 8192, 1024), (250, 1, 9000, 0)])
+def test_a_workspace_of_the_fixed_splits_results_is_enough(B, Hkv, long, short):
+    """The documented size makes room for equal pieces; the size that holds one partial result per fixed split (as sized
+    before there were pieces) is accepted, keeps the fixed form and its bounds, and a byte less than that is refused."""
+    Hq = 2 * Hkv
+    inp = make_gqa_inputs(dict(B=B, Hq=Hq, Hkv=Hkv, D=128, page_size=16, lengths=[short] * (B - 1) + [long]), seed=B, device="cuda")
+    n_splits = -(-long // moe.gqa_decode_split_tokens(B, Hq, Hkv, 128, long))
+    up = lambda v: (v + 255) // 256 * 256
+    least = 512 + up(B * Hkv * 4) + up(B * Hkv * n_splits * 2 * 8) + up(B * Hkv * n_splits * 2 * 512)
+    assert least < moe.gqa_decode_workspace_bytes(B, Hq, Hkv, 128, long)
+    assert ran_equal_pieces(inp)
+    assert not ran_equal_pieces(inp, workspace_bytes=least)
+    out = torch.zeros((B, Hq, 128), dtype=torch.bfloat16, device="cuda")
+    ws = moe.alloc_workspace(least, "cuda")
+    assert moe.gqa_paged_decode(inp["q"], inp["k_cache"], inp["v_cache"], inp["kv_indptr"], inp["kv_indices"],
+                                inp["kv_last_page_len"], long, inp["sm_scale"], out, ws[:least - 1], check=False) == -5
+    torch.cuda.synchronize()
+    assert (out == 0).all()
 
 
 @pytest.mark.parametrize("P", [16, 12, 64, 128])
