@@ -705,7 +705,7 @@ def measure_gqa(ctx: Ctx, name: str) -> dict:
                             cached_tokens=sum(inp["kv_len"]), kv_len_min=min(inp["kv_len"]), kv_len_max=max_len,
                             split_tokens=moe.gqa_decode_split_tokens(B, Hq, Hkv, D, max_len),
                             l2="flushed between steps" if need_flush else "cache larger than L2, no flush"),
-                roofline=dict(bound="hbm", kernel="gqa_paged_decode_kernel", algorithmic_per_launch=kv_bytes, peak=peaks["hbm_gbs"],
+                roofline=dict(bound="hbm", kernel="gqa_tiled_decode_kernel", algorithmic_per_launch=kv_bytes, peak=peaks["hbm_gbs"],
                               frac=kv_bytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"], peak_source=f"of {peaks['source']}",
                               traffic=None, **hbm_fractions(kv_bytes, ms * 1e-3, peaks)),
                 clocks=clocks, cpu_baseline=cpu, dtype="bf16")

@@ -64,18 +64,18 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kStages = 2;         // one chunk in flight while the previous one is used ...
 constexpr int kBlocksPerSm = 3;    // ... in each of three blocks per SM (168 registers per thread, 69 KiB each)
 constexpr int kRowBytes = kD * 2;  // 256 bytes per token and head in the cache
-// Two layouts of a 64-token tile in shared memory, one per gather mode, inside the same 17 KiB:
+// Two layouts of a 64-token tile in shared memory, one per kernel:
 //   tiled: one block per TMA box, [64 / box_rows boxes][2 halves of the dims][box_rows rows][128 bytes], each half
-//          block in TMA's 128-byte swizzle (16 KiB);
-//   rows:  [64 rows][272 bytes], the 16 bytes of padding keeping ldmatrix free of bank conflicts.
+//          block in TMA's 128-byte swizzle: 16 KiB;
+//   rows:  [64 rows][272 bytes], the 16 bytes of padding keeping ldmatrix free of bank conflicts: 17 KiB.
 constexpr int kRowPitch = kRowBytes + 16;
-constexpr int kTileBytes = kChunk * kRowPitch;        // 17 KiB, a multiple of 1024 (the swizzle's alignment)
+constexpr int kTileBytes = kChunk * kRowPitch;
 constexpr int kStageBytes = 2 * kTileBytes;           // keys, then values: 34 KiB
-constexpr int kModelBlocksPerSm = 2;  // blocks per SM the split model counts with (the copy-warp variant's)
+constexpr int kModelBlocksPerSm = 2;  // blocks per SM the split model counts with (the tiled kernel's)
 constexpr int kSmemBytes = kStages * kStageBytes + 1024;  // (the base is rounded up to 1024 bytes)
 // The tiled gather: three stages in each of two blocks per SM, and the segment merge's buffer behind them.
 constexpr int kTiledStages = 3, kTiledTileBytes = kChunk * kRowBytes, kTiledStageBytes = 2 * kTiledTileBytes;
-static_assert(kTileBytes % 1024 == 0, "tiles must keep the swizzle's alignment");
+static_assert(kTiledTileBytes % 1024 == 0, "tiles must keep the swizzle's alignment");
 constexpr int kWaitLimit = 1 << 22;                   // polls of a stage's barrier before the block gives up
 constexpr int kMaxSplits = 128;
 constexpr float kLog2e = 1.4426950408889634f;

@@ -16,7 +16,8 @@ constexpr int kMaxExperts = 256;        // router keeps ceil(E/32) <= 8 logits p
 constexpr int kMaxTopK = 32;            // lane j of the token's warp owns rank j
 constexpr int kRouteTokensPerBlock = 32;  // tokens per router block = one histogram chunk
 constexpr int kStatusInts = 4;          // status word: {status, site, aux0, aux1}
-constexpr int kDoneCounterInt = 4;      // int index, in the status word's zeroed padding, of the fused router's block counter
+constexpr int kDoneCounterInt = 4;      // int index, in the status word's zeroed padding, of the count of finished blocks
+                                        // (of the fused router, or of the scan over the chunks)
 // A forward call's status region is larger and also holds the hand-over between its two GEMMs (all zeroed by the
 // memset that opens the call): a flag the gate/up GEMM raises once it has waited for its predecessors (the tile
 // schedule is then complete), and per expert a count of finished gate/up epilogue passes.  With them the down GEMM
@@ -181,7 +182,7 @@ bool grouped_gemm_tc_ring_applies(const GroupedGemmArgs &args);
 int launch_grouped_gemm_tc_ring(const GroupedGemmArgs &args, cudaStream_t stream);
 
 // The one-CTA kernel for FP8 (E4M3) block-scaled weights: args.w holds one code byte per weight and
-// args.w_scale one fp32 scale per 128 x 128 block; converter warps rebuild bf16 operand tiles in shared
+// args.w_scale one fp32 scale per 128 x 128 block; converter warps rebuild the bf16 weight operand in tensor
 // memory and the bf16 tensor-core path does the rest.  Needs K % 128 == 0.
 int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &args, cudaStream_t stream);
 

@@ -59,7 +59,7 @@ template <bool kScatter>
 __global__ void __launch_bounds__(256)
 mx_quantize_rows_kernel(const uint4 *__restrict__ x, const int *__restrict__ flat_to_sorted,
                         const int *__restrict__ topk_ids, const int *__restrict__ expert_offsets,
-                        const int *__restrict__ tile_rows, int local_offset, int n_local, int n_rows, int k, int vec_per_row,
+                        const int *__restrict__ tile_rows, int local_offset, int n_rows, int k, int vec_per_row,
                         int warps_per_row, uint2 *__restrict__ codes, uint8_t *__restrict__ scales, int n_atoms, int tile) {
     chain_release();
     chain_wait();
@@ -170,7 +170,7 @@ cudaError_t launch_mx_scatter_quantize(const __nv_bfloat16 *x, const int *flat_t
     const long long warps = (long long)T * wpr;
     return launch_chained(mx_quantize_rows_kernel<true>, (unsigned)((warps + 7) / 8), 256, 0, stream,
                           reinterpret_cast<const uint4 *>(x), flat_to_sorted, topk_ids, expert_offsets, tile_rows, local.offset,
-                          local.count, T, k, H / 8, wpr, reinterpret_cast<uint2 *>(xq), x_sf, n_atoms, tile);
+                          T, k, H / 8, wpr, reinterpret_cast<uint2 *>(xq), x_sf, n_atoms, tile);
 }
 
 cudaError_t launch_mx_quantize_rows(const __nv_bfloat16 *x, int R, int K, uint8_t *codes, uint8_t *scales,
@@ -178,7 +178,7 @@ cudaError_t launch_mx_quantize_rows(const __nv_bfloat16 *x, int R, int K, uint8_
     const int wpr = mx_quantize_warps_per_row(R, (K / 8 + 31) / 32);
     const long long warps = (long long)R * wpr;
     return launch_chained(mx_quantize_rows_kernel<false>, (unsigned)((warps + 7) / 8), 256, 0, stream,
-                          reinterpret_cast<const uint4 *>(x), nullptr, nullptr, nullptr, nullptr, 0, 0, R, 1, K / 8, wpr,
+                          reinterpret_cast<const uint4 *>(x), nullptr, nullptr, nullptr, nullptr, 0, R, 1, K / 8, wpr,
                           reinterpret_cast<uint2 *>(codes), scales, 0, 1);
 }
 
