@@ -8,8 +8,8 @@
 // by cutting the experts down to a few candidates and ranking those against each other (select_candidates), and the
 // sort-scatter is a counting sort made stable without ordered atomics:
 //   1. every router block histograms the assignments of its own 32 tokens (one "chunk");
-//   2. the [chunk, expert] histogram becomes start positions (scan over chunks, 32 experts per block); the block that
-//      finishes last scans over the experts and derives the GEMM token-tile schedule;
+//   2. the [chunk, expert] histogram becomes start positions (scan over chunks, by one block or by a block per 32
+//      experts); the one, or the last to finish, scans over the experts and derives the GEMM token-tile schedule;
 //   3. one warp per chunk walks its assignments in flat order, 32 at a time, ranking equal
 //      experts inside a group with match_any and carrying per-expert counters between groups.
 // Batches of up to 1024 tokens do all of it in one launch (route_fused_kernel).
