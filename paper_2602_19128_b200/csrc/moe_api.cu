@@ -190,10 +190,13 @@ int forward_impl(const void *x, const float *logits, const void *w13, const void
     if (fp8w) {
         g1.w_scale = w13_scale;
         g2.w_scale = w2_scale;
-        int st = launch_grouped_gemm_tc_fp8w(g1, stream);
+        auto run = [&](const GroupedGemmArgs &g) {
+            return grouped_gemm_tc_fp8w_pair_applies(g) ? launch_grouped_gemm_tc_fp8w_pair(g, stream) : launch_grouped_gemm_tc_fp8w(g, stream);
+        };
+        int st = run(g1);
         if (st != MOE_OK) return st;
         if (!mark(3)) return MOE_ERR_CUDA;
-        st = launch_grouped_gemm_tc_fp8w(g2, stream);
+        st = run(g2);
         if (st != MOE_OK) return st;
     } else if (flags & MOE_FLAG_VALIDATION_GEMM) {
         if (launch_grouped_gemm_validation(g1, stream) != cudaSuccess) return MOE_ERR_CUDA;

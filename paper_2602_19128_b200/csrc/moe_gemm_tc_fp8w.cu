@@ -27,19 +27,13 @@
 // scale * 2^120 per pair.  The scale is
 // rounded to bf16 once per slot and the product once per weight: at most 2^-8 relative on a weight, an
 // order of magnitude inside the layer's tolerance.  Scales must stay below 2^7 for scale * 2^120 to be finite.
-#include "moe_tc_common.cuh"
+#include "moe_fp8w_tc.cuh"
 
 namespace moe {
 namespace {
 
 using namespace tc;
-
-constexpr int kGroupWarps = 4;                     // converter warps per slot: one per quarter of tensor memory's lanes
-constexpr int kFirstConvWarp = 8;
-constexpr int kTokenWarp = 6;
-constexpr int kSlotK = 128;                        // K elements per ring slot: one scale block, two MMA K-chunks of 64
-constexpr int kSlotQBytes = kTileM * kSlotK;       // 16 KiB of codes
-constexpr int kConvCols = kSlotK / 2;              // tensor-memory columns of a converted slot (two bf16 per column)
+using namespace fp8w;
 
 // D[tmem] (+)= A[tmem] * B[smem]^T, bf16 inputs, fp32 accumulate, issued by one thread.
 __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
@@ -53,35 +47,6 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// 32 consecutive 32-bit columns of this thread's tensor-memory lane (tcgen05.wait::st completes it).
-__device__ __forceinline__ void tmem_store_32(uint32_t taddr, const uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-        ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
-          "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]),
-          "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]),
-          "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
-        : "memory");
-}
-
-// Two E4M3 codes (bytes `kSel` of a word) -> two bf16 values times the block scale.  The permute puts each code in the
-// low byte of a 16-bit lane under its replicated sign bit; shifted left by four, exponent and mantissa sit at the top of
-// bf16's exponent-low / mantissa-high positions, and the mask keeps them and the sign.  That bit pattern is a bf16
-// number equal to the code's value times 2^-120, for normal AND subnormal codes alike (E4M3's bias is 7, bf16's 127, and
-// a zero exponent field means "no hidden one" in both); one bf16x2 multiply by scale * 2^120 finishes it.
-template <uint32_t kSel>
-__device__ __forceinline__ uint32_t convert_two(uint32_t codes, __nv_bfloat162 scale2) {
-    uint32_t x;
-    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(x) : "r"(codes), "n"(kSel));
-    const uint32_t bits = (x << 4) & 0x87F087F0u;
-    __nv_bfloat162 v;
-    *reinterpret_cast<uint32_t *>(&v) = bits;
-    v = __hmul2(v, scale2);
-    return *reinterpret_cast<uint32_t *>(&v);
 }
 
 template <int NT_MAX, int STAGES_Q>

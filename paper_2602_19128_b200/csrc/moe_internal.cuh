@@ -185,6 +185,9 @@ int launch_grouped_gemm_tc_ring(const GroupedGemmArgs &args, cudaStream_t stream
 // args.w_scale one fp32 scale per 128 x 128 block; converter warps rebuild the bf16 weight operand in tensor
 // memory and the bf16 tensor-core path does the rest.  Needs K % 128 == 0.
 int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &args, cudaStream_t stream);
+// The same on CTA pairs: a 256 x N tile, each CTA converts its own 128 weight rows and stages half of the tokens.
+bool grouped_gemm_tc_fp8w_pair_applies(const GroupedGemmArgs &args);
+int launch_grouped_gemm_tc_fp8w_pair(const GroupedGemmArgs &args, cudaStream_t stream);
 
 // ---- MX FP8 (E4M3 codes, one E8M0 scale byte per 32 elements along K) ---------------------------------
 // The block-scaled MMA reads the scale bytes of its operands from tensor memory, where they arrive from

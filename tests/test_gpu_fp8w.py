@@ -70,6 +70,18 @@ def test_fp8w_long_rows_wrap_the_rings(T, H, I, E, k):
     assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k,skew", [(70, 1280, 1024, 2, 2, False),    # tiles of up to 128 rows, 10 and 8 slots of K
+                                            (75, 1024, 1408, 2, 2, False),    # 8 and 11
+                                            (190, 1280, 1152, 2, 2, False),   # 192, one tile per expert
+                                            (193, 1024, 1152, 2, 2, False),   # 192, two ragged tiles per expert
+                                            (300, 1024, 1024, 16, 4, True)])  # skewed: from many tiles per expert to none
+def test_fp8w_cta_pairs_for_both_gemms(T, H, I, E, k, skew):
+    """K loops of eight slots and more and whole pair tiles of features: both GEMMs run on CTA pairs."""
+    inp = make_fp8w_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=5, device="cuda")
+    out, _ = run_fp8w(inp)
+    assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
+
+
 @pytest.mark.parametrize("T,H,I,E,k", [(40, 256, 1152, 16, 2),    # 18 slabs of 16 experts and more: two launches in sequence
                                        (300, 896, 4096, 18, 2),   # 7 slots, more than seven rounds: the same
                                        (24, 256, 256, 8, 2),      # one round: the down GEMM starts through the hand-over
