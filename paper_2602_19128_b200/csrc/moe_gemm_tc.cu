@@ -88,6 +88,10 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    if (warp == 0 && lane == 0) {
+        prefetch_map(&maps.w);
+        prefetch_map(&maps.act[0]);
+    }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + L::kTmemSlot),
                      "r"(kTmemCols)
@@ -107,6 +111,13 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true, gate_up_done = false;
+        auto load_weights = [&](const Tile &t, int w_row, int kb, int slot) {  // by one thread
+            const uint32_t sa = base + L::kA + slot * kSlotABytes, full = bar_full + slot * 8;
+            if (SWIGLU)  // 64 features = groups 4f..4f+3 of 16, gate and up rows interleaved per group
+                tma_load_5d(sa, &maps.w, kb * kBlockK, 0, 0, t.f * 4, t.e, full);
+            else
+                tma_load_2d(sa, &maps.w, kb * kBlockK, w_row, full);
+        };
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
             if (tile >= total_tiles) break;
@@ -114,6 +125,18 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             const int n_mma = (t.n_valid + 15) & ~15;
             const int w_row = t.e * p.w_rows + t.f * kTileM;  // down projection: 128 rows of w2[e]
             const uint32_t tx_bytes = kSlotABytes + n_mma * kRowBytes;
+            // The first tile's weights do not wait for its token rows: the ring's slots are filled with them beforehand (a
+            // one-token Mixtral-shaped layer streams weights while the rows are scattered, and while the last gate/up tiles run).
+            int filled = 0;
+            if (round == 0 && p.handover_role != 0) {
+                filled = p.n_k_blocks < STAGES ? p.n_k_blocks : STAGES;
+                if (elect_one())
+                    for (int kb = 0; kb < filled; ++kb) {
+                        mbar_expect_tx(bar_full + kb * 8, tx_bytes);
+                        load_weights(t, w_row, kb, kb);
+                    }
+                __syncwarp();
+            }
             ok = handover_wait_expert(p.handover_role, p.handover, t.e, t.n_tok_tiles, p.handover_per_token_tile,
                                       p.tile_prefix[p.E], gate_up_done, abort_flag, p.status, lane);
             if (!ok) break;
@@ -121,18 +144,13 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
                 int slot = stage;
                 uint32_t ph = phase;
                 for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                    ok = mbar_wait(bar_empty + slot * 8, ph ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
-                    if (!ok) break;
-                    const uint32_t full = bar_full + slot * 8;
-                    mbar_expect_tx(full, tx_bytes);
-                    const uint32_t sa = base + L::kA + slot * kSlotABytes;
-                    const uint32_t sb = base + L::kB + slot * L::kSlotBBytes;
-                    const int k0 = kb * kBlockK;
-                    if (SWIGLU)  // 64 features = groups 4f..4f+3 of 16, gate and up rows interleaved per group
-                        tma_load_5d(sa, &maps.w, k0, 0, 0, t.f * 4, t.e, full);
-                    else
-                        tma_load_2d(sa, &maps.w, k0, w_row, full);
-                    tma_load_2d(sb, act_map<16>(maps, n_mma), k0, t.row0, full);
+                    if (kb >= filled) {
+                        ok = mbar_wait(bar_empty + slot * 8, ph ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                        if (!ok) break;
+                        mbar_expect_tx(bar_full + slot * 8, tx_bytes);
+                        load_weights(t, w_row, kb, slot);
+                    }
+                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), kb * kBlockK, t.row0, bar_full + slot * 8);
                     if (++slot == STAGES) { slot = 0; ph ^= 1u; }
                 }
             }

@@ -102,6 +102,10 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    if (warp == 0 && lane == 0) {
+        prefetch_map(&maps.w);
+        prefetch_map(&maps.act[0]);
+    }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + L::kTmemSlot),
                      "r"(kTmemCols)

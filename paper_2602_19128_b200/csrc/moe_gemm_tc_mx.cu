@@ -98,6 +98,10 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    if (warp == 0 && lane == 0) {
+        prefetch_map(&maps.w);
+        prefetch_map(&maps.act[0]);
+    }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(base + L::kTmemSlot),
                      "r"(kTmemColsMx)
@@ -117,6 +121,14 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true, gate_up_done = false;
+        auto load_weights = [&](const MxTile &t, int w_row, const uint8_t *w_sf, int kb, int slot) {  // by one thread
+            const uint32_t sa = base + L::kA + slot * kMxSlotABytes, full = bar_full + slot * 8;
+            if (SWIGLU)
+                tma_load_5d(sa, &maps.w, kb * kMxSlotK, 0, 0, t.f * 4, t.e, full);
+            else
+                tma_load_2d(sa, &maps.w, kb * kMxSlotK, w_row, full);
+            bulk_load(base + L::kSfA + slot * kMxSfAtomBytes, w_sf + (size_t)kb * kMxSfAtomBytes, kMxSfAtomBytes, full);
+        };
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
             if (tile >= total_tiles) break;
@@ -126,6 +138,16 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             const uint32_t tx_bytes = kMxSlotABytes + n_mma * kMxSlotK + kMxSfAtomBytes + kMxSfBBytes;
             const uint8_t *w_sf = p.w_sf + ((size_t)t.e * p.n_feature_tiles + t.f) * p.n_k_blocks * kMxSfAtomBytes;
             const uint8_t *a_sf = p.act_sf + (size_t)t.atom * kMxSfAtomBytes;
+            int filled = 0;  // the first tile's weights do not wait for its token rows (moe_gemm_tc.cu)
+            if (round == 0 && p.handover_role != 0) {
+                filled = p.n_k_blocks < STAGES ? p.n_k_blocks : STAGES;
+                if (elect_one())
+                    for (int kb = 0; kb < filled; ++kb) {
+                        mbar_expect_tx(bar_full + kb * 8, tx_bytes);
+                        load_weights(t, w_row, w_sf, kb, kb);
+                    }
+                __syncwarp();
+            }
             ok = handover_wait_expert(p.handover_role, p.handover, t.e, t.n_tok_tiles, p.handover_per_token_tile,
                                       p.tile_prefix[p.E], gate_up_done, abort_flag, p.status, lane);
             if (!ok) break;
@@ -133,19 +155,14 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
                 int slot = stage;
                 uint32_t ph = phase;
                 for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                    ok = mbar_wait(bar_empty + slot * 8, ph ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
-                    if (!ok) break;
                     const uint32_t full = bar_full + slot * 8;
-                    mbar_expect_tx(full, tx_bytes);
-                    const uint32_t sa = base + L::kA + slot * kMxSlotABytes;
-                    const uint32_t sb = base + L::kB + slot * L::kSlotBBytes;
-                    const int k0 = kb * kMxSlotK;
-                    if (SWIGLU)
-                        tma_load_5d(sa, &maps.w, k0, 0, 0, t.f * 4, t.e, full);
-                    else
-                        tma_load_2d(sa, &maps.w, k0, w_row, full);
-                    tma_load_2d(sb, act_map<16>(maps, n_mma), k0, t.row0, full);
-                    bulk_load(base + L::kSfA + slot * kMxSfAtomBytes, w_sf + (size_t)kb * kMxSfAtomBytes, kMxSfAtomBytes, full);
+                    if (kb >= filled) {
+                        ok = mbar_wait(bar_empty + slot * 8, ph ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                        if (!ok) break;
+                        mbar_expect_tx(full, tx_bytes);
+                        load_weights(t, w_row, w_sf, kb, slot);
+                    }
+                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), kb * kMxSlotK, t.row0, full);
                     bulk_load(base + L::kSfB + slot * kMxSfBBytes, a_sf + (size_t)kb * p.n_atoms * kMxSfAtomBytes,
                               kMxSfBBytes, full);
                     if (++slot == STAGES) { slot = 0; ph ^= 1u; }

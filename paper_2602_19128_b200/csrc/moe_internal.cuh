@@ -18,10 +18,10 @@ constexpr int kRouteTokensPerBlock = 32;  // tokens per router block = one histo
 constexpr int kStatusInts = 4;          // status word: {status, site, aux0, aux1}
 constexpr int kDoneCounterInt = 4;      // int index, in the status word's zeroed padding, of the count of finished blocks
                                         // (of the fused router, or of the scan over the chunks)
-// A forward call's status region is larger and also holds the hand-over between its two GEMMs (all zeroed by the
-// memset that opens the call): a flag the gate/up GEMM raises once it has waited for its predecessors (the tile
-// schedule is then complete), and per expert a count of finished gate/up epilogue passes.  With them the down GEMM
-// starts on the SMs the gate/up GEMM has already left, expert by expert, instead of waiting for its whole grid.
+// A forward call's status region is larger and also holds the hand-over to and between its two GEMMs (all zeroed when the
+// call opens, by a memset or by its one-block router): a flag the router raises once the tile schedule is complete, and per
+// expert a count of finished gate/up epilogue passes.  With them both GEMMs fetch weights as soon as there is a schedule, and
+// the down GEMM starts on the SMs the gate/up GEMM has already left, expert by expert, instead of waiting for its whole grid.
 constexpr int kStatusBytesRoute = 256;
 constexpr int kStatusBytesForward = 2048;
 constexpr int kHandoverFlagInt = 8;
@@ -54,7 +54,7 @@ int check_route_args(const float *logits, int T, int E, int k, const int32_t *id
 // (chain_wait) before it touches memory a predecessor writes.  A kernel's launch latency and prologue (barrier
 // set-up, tensor-memory allocation) then overlap the tail of the kernel before it.  Because EVERY block of
 // every kernel waits, completion is transitive: when a kernel's predecessor is complete, so is everything
-// earlier in the chain.  (The down GEMM of a hand-over pair starts on flags instead of this wait, so its blocks
+// earlier in the chain.  (The GEMMs of a hand-over pair start on flags instead of this wait, so their blocks
 // make the wait at their end, before teardown: gemm_chain_finish.)
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -156,8 +156,8 @@ struct GroupedGemmArgs {
     int *status;               // status word
     bool swiglu;
     const float *w_scale = nullptr;  // FP8-weight GEMM: w points at E4M3 codes, this at [E, w_rows/128, K/128] scales
-    // hand-over between the two GEMMs of a call: 0 none; 1 this GEMM raises the flag and counts finished tiles per
-    // expert; 2 this GEMM waits for the flag instead of the previous grid, and per tile for its expert's count
+    // hand-over between the two GEMMs of a call: 0 none; else this GEMM starts on the schedule's flag instead of the previous
+    // grid, and 1: counts finished tiles per expert; 2: waits per tile for its expert's count
     int handover_role = 0;
     int *handover = nullptr;            // the call's status region (flag and counters at the offsets above)
     int handover_per_token_tile = 0;    // role 2: counts that complete one token tile of an expert

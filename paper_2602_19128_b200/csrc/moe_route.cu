@@ -345,10 +345,10 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
 }
 
 // Routes tokens [t0, t1) of the block (warp w takes tokens t0 + w, t0 + w + n_warps, ...) and writes ids and weights;
-// hist, if given, collects the histogram over the resident experts (zeroed by the caller).
+// hist, if given, collects the histogram over the resident experts (zeroed by the caller); ids_here, if given, the ids.
 __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, int t0, int t1, int E, int k, int local_offset,
                                              int n_local, const RouterParams &rp, int *topk_ids, float *topk_w, Candidates *cand,
-                                             int *hist) {
+                                             int *hist, int *ids_here = nullptr) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     for (int t = t0 + warp; t < t1; t += n_warps) {
         int my_id;
@@ -360,10 +360,17 @@ __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, i
         if (lane < k) {
             topk_ids[(size_t)t * k + lane] = my_id;
             topk_w[(size_t)t * k + lane] = my_w;
+            if (ids_here) ids_here[(t - t0) * k + lane] = my_id;
             const int local = my_id - local_offset;  // only experts resident here are scheduled
             if (hist && local >= 0 && local < n_local) atomicAdd(&hist[local], 1);
         }
     }
+}
+
+// The tile schedule is in memory: a forward call's GEMMs, which may be resident already, start on it (gemm_chain_start).  By
+// one thread, behind a block barrier that follows the last write of the schedule.
+__device__ __forceinline__ void raise_schedule_flag(int *status) {
+    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(status + kHandoverFlagInt), "r"(1) : "memory");
 }
 
 template <int kThreads>
@@ -500,7 +507,7 @@ __host__ __device__ inline int scan_warps_per_group(int n_chunks, int groups) {
 }
 __global__ void __launch_bounds__(kScanThreads)
 route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_quantum, int *expert_offsets,
-                  int *tile_prefix, int *tile_order, int *tile_rows, int *totals, int *done_counter) {
+                  int *tile_prefix, int *tile_order, int *tile_rows, int *totals, int *status) {
     __shared__ int partial[kScanWarps][32], all_totals[kMaxExperts];
     __shared__ ScheduleShared sh;
     __shared__ int is_last;
@@ -559,7 +566,7 @@ route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_qu
     } else {
         __threadfence();
         __syncthreads();
-        if (threadIdx.x == 0) is_last = atomicAdd(done_counter, 1) == (int)gridDim.x - 1;
+        if (threadIdx.x == 0) is_last = atomicAdd(status + kDoneCounterInt, 1) == (int)gridDim.x - 1;
         __syncthreads();
         if (!is_last) return;
         __threadfence();
@@ -567,6 +574,8 @@ route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_qu
         __syncthreads();  // (the totals may sit where the schedule is written)
     }
     schedule_phase(count, E, nt_max, row_quantum, expert_offsets, tile_prefix, tile_order, tile_rows, sh);
+    __syncthreads();
+    if (threadIdx.x == 0) raise_schedule_flag(status);
 }
 
 // Stable scatter of 32 consecutive assignments by one warp: lane l holds assignment a (flat order) of local expert e;
@@ -643,27 +652,40 @@ route_scatter_kernel(const int *topk_ids, const int *chunk_starts, const int *ex
 constexpr int kFusedThreads = 1024;
 constexpr int kFusedMaxChunks = 32;  // of kRouteTokensPerBlock tokens
 constexpr int kFusedWarps = kFusedThreads / 32;
+constexpr int kFusedOneBlockTokens = 16;  // up to here one block, nothing to hand over
 constexpr int kFusedGroups = 8;  // groups of 32 assignments a warp keeps in registers between counting and walking
 
 __global__ void __launch_bounds__(kFusedThreads)
 route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int local_offset, int n_local, int nt_max,
                    int row_quantum, int tokens_per_block, const RouterParams rp, int *topk_ids, float *topk_w, int *expert_offsets,
-                   int *tile_prefix, int *tile_order, int *tile_rows, int *sorted_to_flat, int *flat_to_sorted, int *done_counter) {
+                   int *tile_prefix, int *tile_order, int *tile_rows, int *sorted_to_flat, int *flat_to_sorted, int *status,
+                   int status_ints) {
     __shared__ ScheduleShared sh;
     __shared__ union Scratch {
         Candidates cand[kFusedWarps];        // while routing
         int next[kFusedWarps][kMaxExperts];  // then: counts, start positions, cursors of each warp's span
     } u;
-    __shared__ int is_last;
+    __shared__ int is_last, ids_here[kFusedOneBlockTokens * kMaxTopK];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    chain_release();
-    chain_wait();
+    const bool one_block = gridDim.x == 1;  // every id is this block's own: it sorts from shared memory
+    if (status_ints > 0) {
+        // One block: it zeroes the call's status region itself, before any kernel that looks at it may start.
+        chain_wait();
+        for (int i = tid; i < status_ints; i += kFusedThreads) status[i] = 0;
+        __threadfence();
+        __syncthreads();
+        chain_release();
+    } else {
+        chain_release();
+        chain_wait();
+    }
     const int t0 = blockIdx.x * tokens_per_block;
-    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr);
-    if (gridDim.x > 1) {
+    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr,
+                 one_block ? ids_here : nullptr);
+    if (!one_block) {
         __threadfence();  // this block's ids and weights are visible before it is counted as done
         __syncthreads();
-        if (tid == 0) is_last = atomicAdd(done_counter, 1) == (int)gridDim.x - 1;
+        if (tid == 0) is_last = atomicAdd(status + kDoneCounterInt, 1) == (int)gridDim.x - 1;
         __syncthreads();
         if (!is_last) return;
         __threadfence();
@@ -678,7 +700,7 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
 #pragma unroll
     for (int g = 0; g < kFusedGroups; ++g) {
         const int a = a0 + g * 32 + lane;
-        ids[g] = a < a1 ? __ldcg(&topk_ids[a]) - local_offset : -1;
+        ids[g] = a < a1 ? (one_block ? ids_here[a] : __ldcg(&topk_ids[a])) - local_offset : -1;
     }
     int *next = u.next[warp];
     for (int e = lane; e < n_local; e += 32) next[e] = 0;
@@ -712,6 +734,7 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
     const int row_start = schedule_phase(tid < n_local ? count : 0, n_local, nt_max, row_quantum, expert_offsets, tile_prefix,
                                          tile_order, tile_rows, sh);
     __syncthreads();
+    if (tid == kFusedThreads - 1) raise_schedule_flag(status);  // (a thread of the warp that has the least to sort)
     if (tid < kMaxExperts) sh.counts[tid] = row_start;
     __syncthreads();
     if (pe < n_local) {
@@ -917,18 +940,24 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
                          float *topk_w, int *expert_offsets, int *sorted_to_flat, int *flat_to_sorted,
                          RouteScratch scratch, int *status, cudaStream_t stream, int row_quantum, RouterParams router,
                          size_t status_bytes) {
-    cudaError_t err = cudaMemsetAsync(status, 0, status_bytes, stream);  // the status word and what shares its region
-    if (err != cudaSuccess) return err;
     const int A = T * k;
     if (scratch.n_chunks <= kFusedMaxChunks) {
-        // Up to 16 tokens: one block, nothing to hand over.  Else at least four tokens per block, at most 64 blocks.
-        int per_block = T <= 16 ? 16 : (T + 63) / 64;
+        // Up to 16 tokens: one block.  Else at least four tokens per block, at most 64 blocks.
+        // The one block also zeroes the status region (with a memset in front of it the tiny layer takes 21.5 instead of 19.4 us); several cannot, since they count
+        // themselves in it.
+        int per_block = T <= kFusedOneBlockTokens ? kFusedOneBlockTokens : (T + 63) / 64;
         if (per_block < 4) per_block = 4;
+        if (T > kFusedOneBlockTokens) {
+            const cudaError_t err = cudaMemsetAsync(status, 0, status_bytes, stream);
+            if (err != cudaSuccess) return err;
+        }
         return launch_chained(route_fused_kernel, (T + per_block - 1) / per_block, kFusedThreads, 0, stream, logits, T, E, k,
                               local.offset, local.count, nt_max, row_quantum, per_block, router, topk_ids, topk_w, expert_offsets,
                               scratch.tile_prefix, scratch.tile_order, scratch.tile_rows, sorted_to_flat, flat_to_sorted,
-                              status + kDoneCounterInt);
+                              status, T <= kFusedOneBlockTokens ? (int)(status_bytes / sizeof(int)) : 0);
     }
+    cudaError_t err = cudaMemsetAsync(status, 0, status_bytes, stream);  // the status word and what shares its region
+    if (err != cudaSuccess) return err;
     const bool many = scratch.n_chunks > kRouteSms;
     err = launch_chained(many ? route_topk_kernel<kRouteThreadsManyChunks> : route_topk_kernel<kRouteThreads>, scratch.n_chunks,
                          many ? kRouteThreadsManyChunks : kRouteThreads, 0, stream, logits, T, E, k, local.offset, local.count,
@@ -939,7 +968,7 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
     const int scan_blocks = (scratch.n_chunks + warps_per_group - 1) / warps_per_group <= kScanBatch ? 1 : groups;
     err = launch_chained(route_scan_kernel, scan_blocks, kScanThreads, 0, stream, scratch.chunk_counts, scratch.n_chunks,
                          local.count, nt_max, row_quantum, expert_offsets, scratch.tile_prefix, scratch.tile_order,
-                         scratch.tile_rows, scratch.tile_rows, status + kDoneCounterInt);
+                         scratch.tile_rows, scratch.tile_rows, status);
     if (err != cudaSuccess) return err;
     return launch_chained(route_scatter_kernel, scratch.n_chunks, 32, 0, stream, topk_ids, scratch.chunk_counts,
                           expert_offsets, A, local.count, local.offset, k, sorted_to_flat, flat_to_sorted);

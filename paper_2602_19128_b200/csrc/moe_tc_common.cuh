@@ -148,6 +148,11 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+// A tensor map into the descriptor cache, ahead of the first copy that uses it.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap *map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+
 __device__ __forceinline__ void tcgen05_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tcgen05_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -253,27 +258,24 @@ __device__ __forceinline__ bool poll_at_least(const int *addr, int target, volat
         __nanosleep(200);
     }
 }
-// Start of a GEMM kernel's work, after its prologue.  Role 2 (down GEMM with hand-over) does not wait for the
-// whole gate/up grid: it waits until that grid has raised the flag, i.e. has itself waited for the router and the
-// gather, so the tile schedule is complete.  Every other kernel waits for its predecessors; role 1 then raises the flag.
+// Start of a GEMM kernel's work, after its prologue.  The two GEMMs of a hand-over pair (roles 1 and 2) do not wait for the
+// grids before them: they wait for the flag the router raises once the tile schedule is complete, and fetch weights from
+// then on; only their token side waits for more (handover_wait_expert).  Every other kernel waits for its predecessors.
 __device__ __forceinline__ bool gemm_chain_start(int role, int *handover, volatile int *abort_flag, int *status) {
-    if (role == 2) {
+    if (role != 0) {
         bool ok = true;
         if (threadIdx.x == 0) ok = poll_at_least(handover + kHandoverFlagInt, 1, abort_flag, status, kSiteHandoverFlag);
         __syncthreads();
         return !*abort_flag && ok;
     }
     chain_wait();
-    if (role == 1 && threadIdx.x == 0) {
-        asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(handover + kHandoverFlagInt), "r"(1) : "memory");
-    }
     return true;
 }
-// End of a GEMM kernel's work, before its teardown.  A role-2 grid never waited for the grid before it, only for that
-// grid's flag and counts; it waits here (the gate/up grid is finished or finishing by now, so this costs nothing), so
-// that "this grid is complete" again implies "everything before it in the stream is complete" for whatever follows.
+// End of a GEMM kernel's work, before its teardown.  A grid of a hand-over pair never waited for the grid before it, only
+// for flags and counts; it waits here (that grid is finished or finishing by now, so this costs nothing), so that "this grid
+// is complete" again implies "everything before it in the stream is complete" for whatever follows.
 __device__ __forceinline__ void gemm_chain_finish(int role) {
-    if (role == 2) chain_wait();
+    if (role != 0) chain_wait();
 }
 // Role 1, called by every epilogue warp after it has stored its part of a tile: the stores of all its lanes are
 // made visible, then the expert's count goes up by one.
@@ -286,15 +288,22 @@ __device__ __forceinline__ void handover_count_tile(int role, int *handover, int
         atomicAdd(handover + kReadyTotalInt, 1);
     }
 }
-// Role 2, called by the token-side producer warp before the first load of a tile: all gate/up tiles of the expert
-// must have been counted; then generic-proxy writes become visible to the TMA loads that follow.
-// Once the total over all experts has been seen complete (`all_done`, kept by the caller across tiles) nothing is
+// Called by the token-side producer warp before the first load of a tile.  Role 1: its token rows are complete with the grid
+// before this one.  Role 2: all gate/up tiles of the expert must have been counted; then generic-proxy writes become visible
+// to the TMA loads that follow.
+// Once everything has been seen complete (`all_done`, kept by the caller across tiles) nothing is
 // read any more: a load from global memory in front of every tile would starve the ring of a memory-bound GEMM.
 // (whole warp: lane 0 reads, every lane fences, the result is uniform)
 __device__ __forceinline__ bool handover_wait_expert(int role, int *handover, int expert, int n_tok_tiles, int per_token_tile,
                                                      int total_token_tiles, bool &all_done, volatile int *abort_flag,
                                                      int *status, int lane) {
-    if (role != 2 || all_done) return true;
+    if (role == 0 || all_done) return true;
+    if (role == 1) {
+        chain_wait();
+        all_done = true;
+        asm volatile("fence.proxy.async;" ::: "memory");
+        return true;
+    }
     bool ok = true, done = false;
     if (lane == 0) {
         int total;
