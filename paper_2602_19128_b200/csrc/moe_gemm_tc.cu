@@ -21,9 +21,13 @@
 //  * Warp 0 issues TMA loads into a STAGES-deep ring; warp 1 issues the MMAs and commits ring
 //    slots back; warps 2..5 drain the accumulator (double-buffered in TMEM, so the epilogue of
 //    one tile overlaps the MMAs of the next).
+//  * A down GEMM with fewer tiles than half of the SMs (a token or two on a few experts) has two CTAs of a cluster on each
+//    tile, half of its K range each (SplitK, moe_tc_pair.cuh): an SM takes in about 100 GB/s, so 32 or 64 of them do not
+//    reach the memory's rate.  One Mixtral-shaped token 134 -> 126 us, with MX weights 83.7 -> 79.8, with FP8 weights
+//    97.6 -> 86.4.
 //  * Every wait is bounded: if one expires the CTA records MOE_ERR_DEVICE_TIMEOUT and the site in
 //    the status word, every role stops, TMEM is released and the kernel returns.
-#include "moe_tc_common.cuh"
+#include "moe_tc_pair.cuh"
 
 namespace moe {
 namespace {
@@ -45,22 +49,25 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-template <int NT_MAX, int STAGES>
+template <int NT_MAX, int STAGES, bool SPLIT>
 struct SmemLayout {
     static constexpr int kSlotBBytes = NT_MAX * kRowBytes;
     static constexpr int kA = 0;
     static constexpr int kB = STAGES * kSlotABytes;
-    static constexpr int kBars = kB + STAGES * kSlotBBytes;  // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2]
-    static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
+    static constexpr int kSplit = kB + STAGES * kSlotBBytes;
+    // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], SplitK's full
+    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : 0);
+    static constexpr int kTmemSlot = kBars + (2 * STAGES + 5) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
     static constexpr int kDynamicBytes = kBytes + 1024;  // slack to align the base to 1024 bytes
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
-    using L = SmemLayout<NT_MAX, STAGES>;
+    using L = SmemLayout<NT_MAX, STAGES, SPLIT>;
+    static_assert(!(SPLIT && SWIGLU), "the gate/up epilogue pairs rows that a split would part");
     constexpr int kTmemCols = 2 * NT_MAX;
     static_assert(kTmemCols >= 32 && kTmemCols <= 512 && (kTmemCols & (kTmemCols - 1)) == 0,
                   "a tensor-memory allocation must be a power of two between 32 and 512 columns");
@@ -75,6 +82,20 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    SplitK<NT_MAX> split;
+    uint32_t peer_abort = 0;
+    if (SPLIT) {
+        split.rank = cluster_ctarank();
+        split.full = bar_acc_empty + 16;
+        split.buf = reinterpret_cast<float *>(base_ptr + L::kSplit);
+        split.peer_buf = map_to_cta(base + L::kSplit, split.rank ^ 1u);
+        split.peer_full = map_to_cta(split.full, split.rank ^ 1u);
+        peer_abort = map_to_cta(base + L::kAbort, split.rank ^ 1u);
+    }
+    auto wait = [&](uint32_t bar, uint32_t parity, int site) {
+        return SPLIT ? pair_wait(bar, parity, abort_flag, peer_abort, p.status, site + kSiteOffset)
+                     : mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
+    };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + s * 8, 1);
@@ -84,6 +105,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             mbar_init(bar_acc_full + a * 8, 1);
             mbar_init(bar_acc_empty + a * 8, kEpilogueWarps);
         }
+        if (SPLIT) mbar_init(split.full, kEpilogueWarps / 2);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -100,11 +122,17 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     }
     tcgen05_fence_before();
     __syncthreads();
+    if (SPLIT) cluster_sync_all();  // the peer's barriers exist before anything can signal them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // everything above overlapped the previous kernel; its results are read from here on
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
+    const int worker = SPLIT ? blockIdx.x >> 1 : blockIdx.x, n_workers = SPLIT ? gridDim.x >> 1 : gridDim.x;
+    // this CTA's slots of a tile
+    const int first_half = (p.n_k_blocks + 1) >> 1;
+    const int k_first = SPLIT && split.rank ? first_half : 0;
+    const int n_slots = !SPLIT ? p.n_k_blocks : split.rank ? p.n_k_blocks - first_half : first_half;
 
     if (warp == 0) {
         // ---------------- TMA producer: one elected thread issues a whole tile's copies ----------------
@@ -114,12 +142,12 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
         auto load_weights = [&](const Tile &t, int w_row, int kb, int slot) {  // by one thread
             const uint32_t sa = base + L::kA + slot * kSlotABytes, full = bar_full + slot * 8;
             if (SWIGLU)  // 64 features = groups 4f..4f+3 of 16, gate and up rows interleaved per group
-                tma_load_5d(sa, &maps.w, kb * kBlockK, 0, 0, t.f * 4, t.e, full);
+                tma_load_5d(sa, &maps.w, (k_first + kb) * kBlockK, 0, 0, t.f * 4, t.e, full);
             else
-                tma_load_2d(sa, &maps.w, kb * kBlockK, w_row, full);
+                tma_load_2d(sa, &maps.w, (k_first + kb) * kBlockK, w_row, full);
         };
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
+            const int tile = tile_of_round(round, worker, n_workers);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p);
             const int n_mma = (t.n_valid + 15) & ~15;
@@ -129,7 +157,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             // one-token Mixtral-shaped layer streams weights while the rows are scattered, and while the last gate/up tiles run).
             int filled = 0;
             if (round == 0 && p.handover_role != 0) {
-                filled = p.n_k_blocks < STAGES ? p.n_k_blocks : STAGES;
+                filled = n_slots < STAGES ? n_slots : STAGES;
                 if (elect_one())
                     for (int kb = 0; kb < filled; ++kb) {
                         mbar_expect_tx(bar_full + kb * 8, tx_bytes);
@@ -143,20 +171,21 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             if (elect_one()) {
                 int slot = stage;
                 uint32_t ph = phase;
-                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                for (int kb = 0; kb < n_slots; ++kb) {
                     if (kb >= filled) {
-                        ok = mbar_wait(bar_empty + slot * 8, ph ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                        ok = wait(bar_empty + slot * 8, ph ^ 1u, kSiteProducerEmpty);
                         if (!ok) break;
                         mbar_expect_tx(bar_full + slot * 8, tx_bytes);
                         load_weights(t, w_row, kb, slot);
                     }
-                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), kb * kBlockK, t.row0, bar_full + slot * 8);
+                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), (k_first + kb) * kBlockK, t.row0,
+                                bar_full + slot * 8);
                     if (++slot == STAGES) { slot = 0; ph ^= 1u; }
                 }
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
+            ring_advance<STAGES>(stage, phase, n_slots);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: one elected thread walks a whole tile's slots ----------------
@@ -166,19 +195,19 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
         uint32_t phase = 0, acc_phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
+            const int tile = tile_of_round(round, worker, n_workers);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p);
             const uint32_t idesc = instr_desc_bf16(kTileM, (t.n_valid + 15) & ~15);
-            ok = mbar_wait_warp(bar_acc_empty + acc * 8, acc_phase ^ 1u, abort_flag, p.status, kSiteMmaTmemEmpty + kSiteOffset);
+            ok = __all_sync(0xffffffffu, wait(bar_acc_empty + acc * 8, acc_phase ^ 1u, kSiteMmaTmemEmpty));
             if (!ok) break;
             tcgen05_fence_after();
             const uint32_t d_tmem = tmem_base + acc * NT_MAX;
             if (elect_one()) {
                 int s = stage;
                 uint32_t ph = phase;
-                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                    ok = mbar_wait(bar_full + s * 8, ph, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
+                for (int kb = 0; kb < n_slots; ++kb) {
+                    ok = wait(bar_full + s * 8, ph, kSiteMmaFull);
                     if (!ok) break;
                     tcgen05_fence_after();
                     const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + s * kSlotABytes);
@@ -193,7 +222,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
+            ring_advance<STAGES>(stage, phase, n_slots);
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -204,11 +233,15 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
         uint32_t acc_phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
+            const int tile = tile_of_round(round, worker, n_workers);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p);
             const int n_mma = (t.n_valid + 15) & ~15;
-            ok = mbar_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, p.status, kSiteEpilogueTmemFull + kSiteOffset);
+            ok = wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
+            if (SPLIT && ok && split.receives(q)) {  // the peer's sums
+                ok = wait(split.full, 0, kSiteEpilogueTmemFull);
+                fence_cluster();
+            }
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tcgen05_fence_after();
@@ -234,6 +267,13 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
                 for (int c0 = 0; c0 < n_mma; c0 += 16) {
                     float v[16];
                     tmem_load_16(taddr + c0, v);
+                    if (SPLIT) {
+                        if (!split.receives(q)) {
+                            split.send_16(q, c0, lane, v);
+                            continue;
+                        }
+                        split.add_16(q, c0, lane, v);
+                    }
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
                         if (c0 + i < t.n_valid) dst[(size_t)(c0 + i) * p.n_out] = __float2bfloat16_rn(v[i]);
@@ -242,6 +282,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty + acc * 8);
+            if (SPLIT && lane == 0 && !split.receives(q)) mbar_arrive_cluster(split.peer_full);
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -251,6 +292,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     gemm_chain_finish(p.handover_role);
     tcgen05_fence_before();
     __syncthreads();
+    if (SPLIT) cluster_sync_all();  // (the peer may still write here, or signal)
     if (*abort_flag) {
         // give copies that may still be in flight time to land before the CTA's memory is released
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
@@ -261,14 +303,15 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     }
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT = false>
 int launch_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
-    using L = SmemLayout<NT_MAX, STAGES>;
+    using L = SmemLayout<NT_MAX, STAGES, SPLIT>;
     static_assert(L::kDynamicBytes <= 232448, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_kernel<NT_MAX, STAGES, SWIGLU>;
+    auto kernel = grouped_gemm_tc_kernel<NT_MAX, STAGES, SWIGLU, SPLIT>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+    return launch_chained_clusters(kernel, SPLIT ? 2 : 1, grid, kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+               ? MOE_OK : MOE_ERR_CUDA;
 }
 
 template <bool SWIGLU>
@@ -331,6 +374,8 @@ int launch_grouped_gemm_tc(const GroupedGemmArgs &a, cudaStream_t stream) {
     const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
     const long long max_tiles = max_token_tiles * p.n_feature_tiles;
     const int sms = sm_count();
+    if (split_k_applies(a.swiglu, a.nt_max, max_tiles, p.n_k_blocks, kBlockK))
+        return launch_instance<32, 10, false, true>(maps, p, 2 * (int)max_tiles, stream);
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
     return a.swiglu ? dispatch<true>(a.nt_max, maps, p, grid, stream) : dispatch<false>(a.nt_max, maps, p, grid, stream);
 }

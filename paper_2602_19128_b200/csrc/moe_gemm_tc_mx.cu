@@ -23,6 +23,7 @@
 //    exchange with the neighbouring warp through shared memory, then each lane scales and encodes its
 //    values and the scale byte goes straight into the atom layout the down GEMM loads.
 #include "moe_mx_tc.cuh"
+#include "moe_tc_pair.cuh"
 
 namespace moe {
 namespace {
@@ -53,7 +54,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-template <int NT_MAX, int STAGES>
+template <int NT_MAX, int STAGES, bool SPLIT>
 struct MxSmem {
     static constexpr int kSlotBBytes = NT_MAX * kMxSlotK;
     static constexpr int kA = 0;
@@ -61,17 +62,20 @@ struct MxSmem {
     static constexpr int kSfA = kB + STAGES * kSlotBBytes;
     static constexpr int kSfB = kSfA + STAGES * kMxSfAtomBytes;
     static constexpr int kAmax = kSfB + STAGES * kMxSfBBytes;     // [2 buffers][4 warps][16 tokens] magnitudes
-    static constexpr int kBars = kAmax + 2 * 4 * 16 * 4;          // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2]
-    static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
+    static constexpr int kSplit = kAmax + 2 * 4 * 16 * 4;
+    // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], SplitK's full
+    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : 0);
+    static constexpr int kTmemSlot = kBars + (2 * STAGES + 5) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParams p) {
-    using L = MxSmem<NT_MAX, STAGES>;
+    using L = MxSmem<NT_MAX, STAGES, SPLIT>;
+    static_assert(!(SPLIT && SWIGLU), "the gate/up epilogue pairs rows that a split would part");
     static_assert(2 * NT_MAX + 32 <= kTmemColsMx, "accumulators and scale columns exceed tensor memory");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
     constexpr uint32_t kSfACol = 2 * NT_MAX, kSfBCol = 2 * NT_MAX + 16;
@@ -85,6 +89,20 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    SplitK<NT_MAX> split;
+    uint32_t peer_abort = 0;
+    if (SPLIT) {
+        split.rank = cluster_ctarank();
+        split.full = bar_acc_empty + 16;
+        split.buf = reinterpret_cast<float *>(base_ptr + L::kSplit);
+        split.peer_buf = map_to_cta(base + L::kSplit, split.rank ^ 1u);
+        split.peer_full = map_to_cta(split.full, split.rank ^ 1u);
+        peer_abort = map_to_cta(base + L::kAbort, split.rank ^ 1u);
+    }
+    auto wait = [&](uint32_t bar, uint32_t parity, int site) {
+        return SPLIT ? pair_wait(bar, parity, abort_flag, peer_abort, p.status, site + kSiteOffset)
+                     : mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
+    };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + s * 8, 1);
@@ -94,6 +112,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             mbar_init(bar_acc_full + a * 8, 1);
             mbar_init(bar_acc_empty + a * 8, kEpilogueWarps);
         }
+        if (SPLIT) mbar_init(split.full, kEpilogueWarps / 2);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -110,11 +129,17 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     }
     tcgen05_fence_before();
     __syncthreads();
+    if (SPLIT) cluster_sync_all();  // the peer's barriers exist before anything can signal them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // everything above overlapped the previous kernel; its results are read from here on
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
+    const int worker = SPLIT ? blockIdx.x >> 1 : blockIdx.x, n_workers = SPLIT ? gridDim.x >> 1 : gridDim.x;
+    // this CTA's slots of a tile
+    const int first_half = (p.n_k_blocks + 1) >> 1;
+    const int k_first = SPLIT && split.rank ? first_half : 0;
+    const int n_slots = !SPLIT ? p.n_k_blocks : split.rank ? p.n_k_blocks - first_half : first_half;
 
     if (warp == 0) {
         // ---------------- producer: codes by TMA, scale atoms by bulk copies ----------------
@@ -124,13 +149,13 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
         auto load_weights = [&](const MxTile &t, int w_row, const uint8_t *w_sf, int kb, int slot) {  // by one thread
             const uint32_t sa = base + L::kA + slot * kMxSlotABytes, full = bar_full + slot * 8;
             if (SWIGLU)
-                tma_load_5d(sa, &maps.w, kb * kMxSlotK, 0, 0, t.f * 4, t.e, full);
+                tma_load_5d(sa, &maps.w, (k_first + kb) * kMxSlotK, 0, 0, t.f * 4, t.e, full);
             else
-                tma_load_2d(sa, &maps.w, kb * kMxSlotK, w_row, full);
-            bulk_load(base + L::kSfA + slot * kMxSfAtomBytes, w_sf + (size_t)kb * kMxSfAtomBytes, kMxSfAtomBytes, full);
+                tma_load_2d(sa, &maps.w, (k_first + kb) * kMxSlotK, w_row, full);
+            bulk_load(base + L::kSfA + slot * kMxSfAtomBytes, w_sf + (size_t)(k_first + kb) * kMxSfAtomBytes, kMxSfAtomBytes, full);
         };
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
+            const int tile = tile_of_round(round, worker, n_workers);
             if (tile >= total_tiles) break;
             const MxTile t = decode_mx_tile(tile, p);
             const int n_mma = (t.n_valid + 15) & ~15;
@@ -140,7 +165,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             const uint8_t *a_sf = p.act_sf + (size_t)t.atom * kMxSfAtomBytes;
             int filled = 0;  // the first tile's weights do not wait for its token rows (moe_gemm_tc.cu)
             if (round == 0 && p.handover_role != 0) {
-                filled = p.n_k_blocks < STAGES ? p.n_k_blocks : STAGES;
+                filled = n_slots < STAGES ? n_slots : STAGES;
                 if (elect_one())
                     for (int kb = 0; kb < filled; ++kb) {
                         mbar_expect_tx(bar_full + kb * 8, tx_bytes);
@@ -154,23 +179,23 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             if (elect_one()) {
                 int slot = stage;
                 uint32_t ph = phase;
-                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
+                for (int kb = 0; kb < n_slots; ++kb) {
                     const uint32_t full = bar_full + slot * 8;
                     if (kb >= filled) {
-                        ok = mbar_wait(bar_empty + slot * 8, ph ^ 1u, abort_flag, p.status, kSiteProducerEmpty + kSiteOffset);
+                        ok = wait(bar_empty + slot * 8, ph ^ 1u, kSiteProducerEmpty);
                         if (!ok) break;
                         mbar_expect_tx(full, tx_bytes);
                         load_weights(t, w_row, w_sf, kb, slot);
                     }
-                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), kb * kMxSlotK, t.row0, full);
-                    bulk_load(base + L::kSfB + slot * kMxSfBBytes, a_sf + (size_t)kb * p.n_atoms * kMxSfAtomBytes,
+                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), (k_first + kb) * kMxSlotK, t.row0, full);
+                    bulk_load(base + L::kSfB + slot * kMxSfBBytes, a_sf + (size_t)(k_first + kb) * p.n_atoms * kMxSfAtomBytes,
                               kMxSfBBytes, full);
                     if (++slot == STAGES) { slot = 0; ph ^= 1u; }
                 }
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
+            ring_advance<STAGES>(stage, phase, n_slots);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: one elected thread walks a whole tile's slots ----------------
@@ -179,19 +204,19 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
         bool ok = true;
         const uint32_t sfa_tmem = tmem_base + kSfACol, sfb_tmem = tmem_base + kSfBCol;
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
+            const int tile = tile_of_round(round, worker, n_workers);
             if (tile >= total_tiles) break;
             const MxTile t = decode_mx_tile(tile, p);
             const int n_mma = (t.n_valid + 15) & ~15;
-            ok = mbar_wait_warp(bar_acc_empty + acc * 8, acc_phase ^ 1u, abort_flag, p.status, kSiteMmaTmemEmpty + kSiteOffset);
+            ok = __all_sync(0xffffffffu, wait(bar_acc_empty + acc * 8, acc_phase ^ 1u, kSiteMmaTmemEmpty));
             if (!ok) break;
             tcgen05_fence_after();
             const uint32_t d_tmem = tmem_base + acc * NT_MAX;
             if (elect_one()) {
                 int s = stage;
                 uint32_t ph = phase;
-                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
-                    ok = mbar_wait(bar_full + s * 8, ph, abort_flag, p.status, kSiteMmaFull + kSiteOffset);
+                for (int kb = 0; kb < n_slots; ++kb) {
+                    ok = wait(bar_full + s * 8, ph, kSiteMmaFull);
                     if (!ok) break;
                     tcgen05_fence_after();
                     tmem_copy_sf_atom(sfa_tmem, smem_desc_sf_atom(base + L::kSfA + s * kMxSfAtomBytes));
@@ -209,7 +234,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
+            ring_advance<STAGES>(stage, phase, n_slots);
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -221,13 +246,18 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
         uint32_t *amax_s = reinterpret_cast<uint32_t *>(base_ptr + L::kAmax);
         int buf = 0;  // exchange buffer, flipped every 16-token chunk (across tiles too): a warp may run one chunk ahead of its partner
         for (int round = 0;; ++round) {
-            const int tile = tile_of_round(round, blockIdx.x, gridDim.x);
+            const int tile = tile_of_round(round, worker, n_workers);
             if (tile >= total_tiles) break;
             const MxTile t = decode_mx_tile(tile, p);
             const int n_mma = (t.n_valid + 15) & ~15;
-            const bool ok = mbar_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, p.status, kSiteEpilogueTmemFull + kSiteOffset);
-            // the four warps synchronise inside the tile (SwiGLU), so they must agree on leaving
-            if (epilogue_any(!ok)) break;
+            bool ok = wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
+            if (SPLIT && ok && split.receives(q)) {  // the peer's sums
+                ok = wait(split.full, 0, kSiteEpilogueTmemFull);
+                fence_cluster();
+            }
+            // The four warps synchronise inside the tile (SwiGLU), so they must agree on leaving.  With a split they must not wait
+            // for one another here: two of them wait for the peer's other two.
+            if (SPLIT ? !__all_sync(0xffffffffu, ok) : epilogue_any(!ok)) break;
             tcgen05_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
             if (SWIGLU) {
@@ -241,6 +271,13 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
                 for (int c0 = 0; c0 < n_mma; c0 += 16) {
                     float v[16];
                     tmem_load_16(taddr + c0, v);
+                    if (SPLIT) {
+                        if (!split.receives(q)) {
+                            split.send_16(q, c0, lane, v);
+                            continue;
+                        }
+                        split.add_16(q, c0, lane, v);
+                    }
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
                         if (c0 + i < t.n_valid) dst[(size_t)(c0 + i) * p.n_out] = __float2bfloat16_rn(v[i]);
@@ -249,6 +286,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty + acc * 8);
+            if (SPLIT && lane == 0 && !split.receives(q)) mbar_arrive_cluster(split.peer_full);
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -258,6 +296,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     gemm_chain_finish(p.handover_role);
     tcgen05_fence_before();
     __syncthreads();
+    if (SPLIT) cluster_sync_all();  // (the peer may still write here, or signal)
     if (*abort_flag) {
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     }
@@ -267,14 +306,15 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     }
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT = false>
 int launch_instance(const TensorMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
-    using L = MxSmem<NT_MAX, STAGES>;
+    using L = MxSmem<NT_MAX, STAGES, SPLIT>;
     static_assert(L::kDynamicBytes <= 232448, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_mx_kernel<NT_MAX, STAGES, SWIGLU>;
+    auto kernel = grouped_gemm_tc_mx_kernel<NT_MAX, STAGES, SWIGLU, SPLIT>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+    return launch_chained_clusters(kernel, SPLIT ? 2 : 1, grid, kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+               ? MOE_OK : MOE_ERR_CUDA;
 }
 
 template <bool SWIGLU>
@@ -325,6 +365,8 @@ int launch_grouped_gemm_tc_mx(const MxGemmArgs &a, cudaStream_t stream) {
     const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
     const long long max_tiles = max_token_tiles * p.n_feature_tiles;
     const int sms = sm_count();
+    if (split_k_applies(a.swiglu, a.nt_max, max_tiles, p.n_k_blocks, kMxSlotK))  // (moe_gemm_tc.cu)
+        return launch_instance<32, 10, false, true>(maps, p, 2 * (int)max_tiles, stream);
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
     return a.swiglu ? dispatch<true>(a.nt_max, maps, p, grid, stream) : dispatch<false>(a.nt_max, maps, p, grid, stream);
 }

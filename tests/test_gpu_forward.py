@@ -59,6 +59,19 @@ def test_forward_matches_oracle(T, H, I, E, k, skew, flags):
     assert_close_out(bf16_to_f64(out), ref, "out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2112, 2, 2), (30, 384, 2304, 4, 2)])
+def test_few_down_tiles_split_along_k(T, H, I, E, k):
+    """Down GEMMs of a few tiles with a long K: two CTAs per tile, half of the K slots each (2112: 17 and 16 of them)."""
+    inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=0)
+    out, views, _ = run_forward(inp)
+    *_, h, y, ref = oracle_everything(to_host_case(inp))
+    assert_close_out(bf16_to_f64(views["h"]), h, "h")
+    assert_close_out(bf16_to_f64(views["y"]), y, "y")
+    assert_close_out(bf16_to_f64(out), ref, "out")
+    again, _, _ = run_forward(inp)
+    assert torch.equal(out, again)
+
+
 @pytest.mark.parametrize("T,H,I,E,k,skew", [(520, 256, 256, 4, 2, False), (900, 256, 128, 8, 2, True),
                                             (1200, 512, 384, 8, 2, False), (700, 256, 256, 2, 1, False)])
 def test_gather_in_load_matches_oracle(T, H, I, E, k, skew):

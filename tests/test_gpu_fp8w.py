@@ -82,6 +82,14 @@ def test_fp8w_cta_pairs_for_both_gemms(T, H, I, E, k, skew):
     assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
+def test_fp8w_few_down_tiles_split_along_k(T, H, I, E, k):
+    """Two CTAs per tile of the down GEMM, half of the K slots each (2176: 9 and 8 of them)."""
+    inp = make_fp8w_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=6, device="cuda")
+    out, _ = run_fp8w(inp)
+    assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
+
+
 @pytest.mark.parametrize("T,H,I,E,k", [(40, 256, 1152, 16, 2),    # 18 slabs of 16 experts and more: two launches in sequence
                                        (300, 896, 4096, 18, 2),   # 7 slots, more than seven rounds: the same
                                        (24, 256, 256, 8, 2),      # one round: the down GEMM starts through the hand-over

@@ -185,6 +185,14 @@ def test_mxfp8_forward_matches_oracle(T, H, I, E, k, skew):
     assert_close_out(bf16_to_f64(out), ref, "mxfp8 out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
+def test_mxfp8_few_down_tiles_split_along_k(T, H, I, E, k):
+    """Two CTAs per tile of the down GEMM, half of the K slots each (2176: 9 and 8 of them)."""
+    inp = make_mxfp8_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=2, device="cuda")
+    out, _ = run_mx(inp)
+    assert_close_out(bf16_to_f64(out), oracle_mx(inp), "mxfp8 out")
+
+
 @pytest.mark.parametrize("cfg,lo,n", [(dict(T=160, H=256, I=128, E=16, top_k=4, skew=False), 4, 8),
                                       # wide token tiles (bound 384) with resident experts in the middle of the range
                                       (dict(T=1200, H=256, I=128, E=8, top_k=2, skew=False), 2, 4),
