@@ -246,38 +246,21 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             if (!ok) break;
             tcgen05_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
-            if (SWIGLU) {
-                const int hi = lane >> 4;
-                __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + t.f * (kTileM / 2) + q * 16 + (lane & 15);
+            const int feat = SWIGLU ? t.f * (kTileM / 2) + q * 16 + (lane & 15) : t.f * kTileM + q * 32 + lane;
+            __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + feat;
+            if (SPLIT) {
                 for (int c0 = 0; c0 < n_mma; c0 += 16) {
                     float v[16];
                     tmem_load_16(taddr + c0, v);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float other = __shfl_xor_sync(0xffffffffu, hi ? v[i] : v[8 + i], 16);
-                        const float g = hi ? other : v[i];
-                        const float u = hi ? v[8 + i] : other;
-                        const int col = c0 + hi * 8 + i;
-                        if (col < t.n_valid)
-                            dst[(size_t)col * p.n_out] = __float2bfloat16_rn(swiglu(g, u));
+                    if (!split.receives(q)) {
+                        split.send_16(q, c0, lane, v);
+                    } else {
+                        split.add_16(q, c0, lane, v);
+                        store_column(v, t.n_valid - c0, dst + (size_t)c0 * p.n_out, (size_t)p.n_out);
                     }
                 }
             } else {
-                __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + t.f * kTileM + q * 32 + lane;
-                for (int c0 = 0; c0 < n_mma; c0 += 16) {
-                    float v[16];
-                    tmem_load_16(taddr + c0, v);
-                    if (SPLIT) {
-                        if (!split.receives(q)) {
-                            split.send_16(q, c0, lane, v);
-                            continue;
-                        }
-                        split.add_16(q, c0, lane, v);
-                    }
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (c0 + i < t.n_valid) dst[(size_t)(c0 + i) * p.n_out] = __float2bfloat16_rn(v[i]);
-                }
+                drain_accumulator<SWIGLU>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
             }
             tcgen05_fence_before();
             __syncwarp();

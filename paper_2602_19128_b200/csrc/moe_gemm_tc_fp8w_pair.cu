@@ -408,31 +408,8 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMaps maps, const 
             if (!ok) break;
             tcgen05_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
-            if (SWIGLU) {
-                const int hi = lane >> 4;
-                __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + feat0 + q * 16 + (lane & 15);
-                for (int c0 = 0; c0 < n_mma; c0 += 16) {
-                    float v[16];
-                    tmem_load_16(taddr + c0, v);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float other = __shfl_xor_sync(0xffffffffu, hi ? v[i] : v[8 + i], 16);
-                        const float g = hi ? other : v[i];
-                        const float u = hi ? v[8 + i] : other;
-                        const int col = c0 + hi * 8 + i;
-                        if (col < t.n_valid) dst[(size_t)col * p.n_out] = __float2bfloat16_rn(swiglu(g, u));
-                    }
-                }
-            } else {
-                __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + feat0 + q * 32 + lane;
-                for (int c0 = 0; c0 < n_mma; c0 += 16) {
-                    float v[16];
-                    tmem_load_16(taddr + c0, v);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (c0 + i < t.n_valid) dst[(size_t)(c0 + i) * p.n_out] = __float2bfloat16_rn(v[i]);
-                }
-            }
+            __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + feat0 + (SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane);
+            drain_accumulator<SWIGLU>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + acc * 8, 0));

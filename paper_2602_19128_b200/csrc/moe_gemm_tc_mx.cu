@@ -268,19 +268,19 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
                 drain_swiglu_mx(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, sf_dst, amax_s, buf, q, lane);
             } else {
                 __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.out) + (size_t)t.row0 * p.n_out + t.f * kTileM + q * 32 + lane;
-                for (int c0 = 0; c0 < n_mma; c0 += 16) {
-                    float v[16];
-                    tmem_load_16(taddr + c0, v);
-                    if (SPLIT) {
+                if (SPLIT) {
+                    for (int c0 = 0; c0 < n_mma; c0 += 16) {
+                        float v[16];
+                        tmem_load_16(taddr + c0, v);
                         if (!split.receives(q)) {
                             split.send_16(q, c0, lane, v);
-                            continue;
+                        } else {
+                            split.add_16(q, c0, lane, v);
+                            store_column(v, t.n_valid - c0, dst + (size_t)c0 * p.n_out, (size_t)p.n_out);
                         }
-                        split.add_16(q, c0, lane, v);
                     }
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (c0 + i < t.n_valid) dst[(size_t)(c0 + i) * p.n_out] = __float2bfloat16_rn(v[i]);
+                } else {
+                    drain_accumulator<false>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
                 }
             }
             tcgen05_fence_before();

@@ -310,7 +310,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
             // An even tile is drained from its highest 16 columns down, an odd tile from its lowest up: the columns the
             // next tile of this pair is waiting for go back first.  Accumulator column j is tile row j.
             const int n_groups = n_mma >> 4;
-            const int hi = lane >> 4, j16 = lane & 15;
+            const int j16 = lane & 15;
             uint8_t *dst_q = nullptr, *sf_dst = nullptr;
             __nv_bfloat16 *dst_rows = nullptr;
             if (SWIGLU) {
@@ -331,38 +331,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
                 if (lane == 0)
                     mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + ((parts.first_col + c0) / kChunkCols) * 8, 0));
                 if (SWIGLU) {
-                    // lanes 0..15 hold gate, lanes 16..31 up of the same 16 features; h is quantised in blocks of 32
-                    // features: this warp's 16 and its partner's (warps q and q ^ 1), maxima exchanged through amax_s
-                    float hv[8];
-                    uint32_t mag[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float other = __shfl_xor_sync(0xffffffffu, hi ? v[i] : v[8 + i], 16);
-                        const float gt = hi ? other : v[i];
-                        const float up = hi ? v[8 + i] : other;
-                        hv[i] = swiglu(gt, up);
-                        mag[i] = __float_as_uint(hv[i]) & 0x7FFFFFFFu;  // magnitudes compare as integers; NaN and inf on top
-                    }
-                    const uint32_t col_max = half_warp_max8(mag, j16);  // of column c0 + hi * 8 + j16 / 2, this warp's 16 features
-                    buf ^= 1;
-                    if ((j16 & 1) == 0) amax_s[(buf * 4 + q) * 16 + hi * 8 + (j16 >> 1)] = col_max;
-                    pair_sync(q >> 1);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const uint32_t block_mag = max(amax_s[(buf * 4 + q) * 16 + hi * 8 + i],
-                                                       amax_s[(buf * 4 + (q ^ 1)) * 16 + hi * 8 + i]);
-                        const uint32_t sb = mx_scale_byte(block_mag);
-                        const int col = c0 + hi * 8 + i;
-                        if (col < t.n_valid) {
-                            uint8_t code = 0x7F;
-                            if (sb != 255u)
-                                code = (uint8_t)__nv_cvt_float_to_fp8(hv[i] * __uint_as_float((254u - sb) << 23), __NV_SATFINITE,
-                                                                      __NV_E4M3);
-                            dst_q[(size_t)col * p.n_out] = code;
-                            if ((q & 1) == 0 && j16 == 0)  // row `col` of the tile: atom col / 128, atom row col % 128
-                                sf_dst[(size_t)(col >> 7) * kMxSfAtomBytes + mx_atom_byte(col & 127, 0)] = (uint8_t)sb;
-                        }
-                    }
+                    store_swiglu_mx_16(v, t.n_valid - c0, dst_q + (size_t)c0 * p.n_out, (size_t)p.n_out, sf_dst, c0, amax_s, buf, q, lane);
                 } else {
                     // Output rows are the token's: a lane holds one output feature of 16 tokens, and stored from here
                     // a warp instruction would write 32 x 2 bytes of one token -- measured, those stores took as long

@@ -56,37 +56,6 @@ struct PairSmem {
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
-// Drain one accumulator (this warp's 32 TMEM lanes x n_mma columns) to global memory.
-//   SWIGLU: lanes 0..15 hold gate, lanes 16..31 up of the same 16 features; dst points at this lane's
-//           feature in row 0 of the tile.  Plain: one output feature per lane.
-template <bool SWIGLU>
-__device__ __forceinline__ void drain_accumulator(uint32_t taddr, int n_mma, int n_valid, __nv_bfloat16 *dst,
-                                                  size_t row_stride, int lane) {
-    if (SWIGLU) {
-        const int hi = lane >> 4;
-        for (int c0 = 0; c0 < n_mma; c0 += 16) {
-            float v[16];
-            tmem_load_16(taddr + c0, v);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float other = __shfl_xor_sync(0xffffffffu, hi ? v[i] : v[8 + i], 16);
-                const float g = hi ? other : v[i];
-                const float u = hi ? v[8 + i] : other;
-                const int col = c0 + hi * 8 + i;
-                if (col < n_valid) dst[(size_t)col * row_stride] = __float2bfloat16_rn(swiglu(g, u));
-            }
-        }
-    } else {
-        for (int c0 = 0; c0 < n_mma; c0 += 16) {
-            float v[16];
-            tmem_load_16(taddr + c0, v);
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (c0 + i < n_valid) dst[(size_t)(c0 + i) * row_stride] = __float2bfloat16_rn(v[i]);
-        }
-    }
-}
-
 template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {

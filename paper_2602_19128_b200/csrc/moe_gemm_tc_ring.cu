@@ -335,19 +335,11 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
                 __syncwarp();
                 if (lane == 0)
                     mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + ((parts.first_col + tile_col) / kChunkCols) * 8, 0));
-                const bool all_valid = row_a + 8 <= t.n_valid && row_b + 8 <= t.n_valid;  // (uniform over the warp)
-                if (SWIGLU) {  // lanes 0..15 hold gate, lanes 16..31 up of the same 16 features
-                    const int hi = lane >> 4;
-                    const int row0 = hi ? row_b : row_a;  // this lane stores columns hi*8 .. hi*8+7 of the group
-                    __nv_bfloat16 *out_row = dst + (size_t)row0 * row_stride;
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const float other = __shfl_xor_sync(0xffffffffu, hi ? v[u] : v[8 + u], 16);
-                        const float gt = hi ? other : v[u];
-                        const float up = hi ? v[8 + u] : other;
-                        if (all_valid || row0 + u < t.n_valid) *out_row = __float2bfloat16_rn(swiglu(gt, up));
-                        out_row += row_stride;
-                    }
+                if (SWIGLU) {  // this lane stores columns hi*8 .. hi*8+7 of the group
+                    float hv[8];
+                    swiglu_16(v, lane, hv);
+                    const int row0 = (lane & 16) ? row_b : row_a;
+                    store_column(hv, t.n_valid - row0, dst + (size_t)row0 * row_stride, row_stride);
                 } else {
                     // A lane holds one output feature of 16 tokens; stored from here a warp instruction would write
                     // 32 x 2 bytes of one token.  The four warps transpose the group through shared memory instead and
