@@ -380,7 +380,7 @@ int launch_fp8_instance(const TensorMaps &maps, const KernelParams &p, int grid,
     auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES_Q, SWIGLU, SPLIT>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained_clusters(kernel, SPLIT ? 2 : 1, grid, L::kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+    return launch_clusters(kernel, true, SPLIT ? 2 : 1, grid, L::kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 

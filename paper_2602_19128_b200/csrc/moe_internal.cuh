@@ -60,28 +60,34 @@ int check_route_args(const float *logits, int T, int E, int k, const int32_t *id
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// (cluster > 1: in clusters of that many blocks, for kernels that do not carry __cluster_dims__)
+// (chained: as above; cluster > 1: in clusters of that many blocks, for kernels that do not carry __cluster_dims__)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_chained_clusters(void (*kernel)(KArgs...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                    Args &&...args) {
+cudaError_t launch_clusters(void (*kernel)(KArgs...), bool chained, int cluster, dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t stream, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = cluster;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    int n = 0;
+    if (chained) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster;
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
-    return launch_chained_clusters(kernel, 1, grid, block, smem, stream, static_cast<KArgs>(args)...);
+    return launch_clusters(kernel, true, 1, grid, block, smem, stream, static_cast<KArgs>(args)...);
 }
 #endif
 

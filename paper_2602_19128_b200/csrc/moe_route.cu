@@ -345,10 +345,11 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
 }
 
 // Routes tokens [t0, t1) of the block (warp w takes tokens t0 + w, t0 + w + n_warps, ...) and writes ids and weights;
-// hist, if given, collects the histogram over the resident experts (zeroed by the caller); ids_here, if given, the ids.
+// hist, if given, collects the histogram over the resident experts (zeroed by the caller); ids_smem, if not 0, is the address
+// (in the cluster's shared memory) of an array of all tokens' ids, which are left there too.
 __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, int t0, int t1, int E, int k, int local_offset,
                                              int n_local, const RouterParams &rp, int *topk_ids, float *topk_w, Candidates *cand,
-                                             int *hist, int *ids_here = nullptr) {
+                                             int *hist, uint32_t ids_smem = 0) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     for (int t = t0 + warp; t < t1; t += n_warps) {
         int my_id;
@@ -360,7 +361,8 @@ __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, i
         if (lane < k) {
             topk_ids[(size_t)t * k + lane] = my_id;
             topk_w[(size_t)t * k + lane] = my_w;
-            if (ids_here) ids_here[(t - t0) * k + lane] = my_id;
+            if (ids_smem)
+                asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(ids_smem + (uint32_t)(t * k + lane) * 4), "r"(my_id) : "memory");
             const int local = my_id - local_offset;  // only experts resident here are scheduled
             if (hist && local >= 0 && local < n_local) atomicAdd(&hist[local], 1);
         }
@@ -642,8 +644,8 @@ route_scatter_kernel(const int *topk_ids, const int *chunk_starts, const int *ex
 }
 
 // Small batches (at most 1024 tokens): everything in ONE launch.  The tokens are dealt out to up to 64 blocks (a token is a
-// chain of warp reductions: spread over the SMs, not queued on a few); the block that finishes last (a counter in the
-// status word's padding, zeroed by the caller's memset) sorts all assignments from their ids alone: warp w takes the
+// chain of warp reductions: spread over the SMs, not queued on a few); one block -- the first of a cluster, or the one that
+// finishes last (a counter in the status word's padding) -- sorts all assignments from their ids alone: warp w takes the
 // w-th span of the flat order, counts it, turns the counts into start positions and walks it as scatter_chunk does.
 // Which block is last does not affect any result.
 // Counts, starts and cursors stay in shared memory: through global memory each hand-over cost an L2 round trip, and with
@@ -652,7 +654,13 @@ route_scatter_kernel(const int *topk_ids, const int *chunk_starts, const int *ex
 constexpr int kFusedThreads = 1024;
 constexpr int kFusedMaxChunks = 32;  // of kRouteTokensPerBlock tokens
 constexpr int kFusedWarps = kFusedThreads / 32;
-constexpr int kFusedOneBlockTokens = 16;  // up to here one block, nothing to hand over
+// Two ways from the blocks to the one that sorts.  Up to 16 tokens: one block.  Up to 256 (and kFusedIds ids): the blocks are
+// a cluster of eight, which leave their ids in the first one's shared memory and meet at the cluster's barrier; that
+// block also zeroes the call's status region, so the call needs neither a memset in front nor an atomic count and a trip of
+// the ids through L2.  Beyond, eight SMs would have more than a token per warp, and up to 64 blocks count themselves.
+// Layers, 64 blocks / a cluster: 100 tokens of 8 experts of 256 x 512, top 2, 23.6 / 21.5 us; 64 tokens of 32 of 1024 x 1024,
+// top 4, 57.6 / 54.8; 64 tokens on 32 of 256 bf16 experts of 7168 x 2048, top 8, grouped router, 361.9 / 355.7.
+constexpr int kFusedOneBlockTokens = 16, kFusedClusterTokens = 256, kFusedCluster = 8, kFusedIds = 2048;
 constexpr int kFusedGroups = 8;  // groups of 32 assignments a warp keeps in registers between counting and walking
 
 __global__ void __launch_bounds__(kFusedThreads)
@@ -665,24 +673,40 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
         Candidates cand[kFusedWarps];        // while routing
         int next[kFusedWarps][kMaxExperts];  // then: counts, start positions, cursors of each warp's span
     } u;
-    __shared__ int is_last, ids_here[kFusedOneBlockTokens * kMaxTopK];
+    __shared__ int is_last, ids_here[kFusedIds];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool one_block = gridDim.x == 1;  // every id is this block's own: it sorts from shared memory
-    if (status_ints > 0) {
-        // One block: it zeroes the call's status region itself, before any kernel that looks at it may start.
+    const bool ids_local = status_ints > 0;  // one block or a cluster: the first block sorts from its shared memory
+    const bool cluster = ids_local && gridDim.x > 1;
+    if (cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (the blocks have started)
+    if (ids_local) {
+        // The first block zeroes the call's status region, before any kernel that looks at it may start.
         chain_wait();
-        for (int i = tid; i < status_ints; i += kFusedThreads) status[i] = 0;
-        __threadfence();
+        if (blockIdx.x == 0) {
+            for (int i = tid; i < status_ints; i += kFusedThreads) status[i] = 0;
+            __threadfence();
+        }
         __syncthreads();
         chain_release();
     } else {
         chain_release();
         chain_wait();
     }
+    uint32_t ids_smem = 0;
+    if (ids_local) {
+        ids_smem = (uint32_t)__cvta_generic_to_shared(ids_here);
+        if (cluster) {
+            asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(ids_smem));
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        }
+    }
     const int t0 = blockIdx.x * tokens_per_block;
-    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr,
-                 one_block ? ids_here : nullptr);
-    if (!one_block) {
+    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr, ids_smem);
+    if (cluster) {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        if (blockIdx.x != 0) return;
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else if (!ids_local) {
         __threadfence();  // this block's ids and weights are visible before it is counted as done
         __syncthreads();
         if (tid == 0) is_last = atomicAdd(status + kDoneCounterInt, 1) == (int)gridDim.x - 1;
@@ -700,7 +724,7 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
 #pragma unroll
     for (int g = 0; g < kFusedGroups; ++g) {
         const int a = a0 + g * 32 + lane;
-        ids[g] = a < a1 ? (one_block ? ids_here[a] : __ldcg(&topk_ids[a])) - local_offset : -1;
+        ids[g] = a < a1 ? (ids_local ? ids_here[a] : __ldcg(&topk_ids[a])) - local_offset : -1;
     }
     int *next = u.next[warp];
     for (int e = lane; e < n_local; e += 32) next[e] = 0;
@@ -942,19 +966,24 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
                          size_t status_bytes) {
     const int A = T * k;
     if (scratch.n_chunks <= kFusedMaxChunks) {
-        // Up to 16 tokens: one block.  Else at least four tokens per block, at most 64 blocks.
-        // The one block also zeroes the status region (with a memset in front of it the tiny layer takes 21.5 instead of 19.4 us); several cannot, since they count
-        // themselves in it.
-        int per_block = T <= kFusedOneBlockTokens ? kFusedOneBlockTokens : (T + 63) / 64;
-        if (per_block < 4) per_block = 4;
+        // One block, a cluster of eight, or up to 64 blocks of at least four tokens (the comment at kFusedOneBlockTokens).
+        const bool ids_local = T <= kFusedOneBlockTokens || (T <= kFusedClusterTokens && A <= kFusedIds);
+        int blocks = 1, per_block = T;
         if (T > kFusedOneBlockTokens) {
+            per_block = ids_local ? (T + kFusedCluster - 1) / kFusedCluster : (T + 63) / 64 < 4 ? 4 : (T + 63) / 64;
+            blocks = ids_local ? kFusedCluster : (T + per_block - 1) / per_block;
+        }
+        if (!ids_local) {
             const cudaError_t err = cudaMemsetAsync(status, 0, status_bytes, stream);
             if (err != cudaSuccess) return err;
         }
-        return launch_chained(route_fused_kernel, (T + per_block - 1) / per_block, kFusedThreads, 0, stream, logits, T, E, k,
-                              local.offset, local.count, nt_max, row_quantum, per_block, router, topk_ids, topk_w, expert_offsets,
-                              scratch.tile_prefix, scratch.tile_order, scratch.tile_rows, sorted_to_flat, flat_to_sorted,
-                              status, T <= kFusedOneBlockTokens ? (int)(status_bytes / sizeof(int)) : 0);
+        // (The cluster starts when everything before it is done.  Launched early, its blocks of 48 KB and 1024 threads held SMs
+        // while the last kernels of the call before were still at work: 64 tokens on 32 MX experts of 7168 x 2048 202.8 -> 214 us.)
+        const bool cluster = ids_local && blocks > 1;
+        return launch_clusters(route_fused_kernel, !cluster, cluster ? blocks : 1, blocks, kFusedThreads, 0, stream, logits, T, E, k,
+                               local.offset, local.count, nt_max, row_quantum, per_block, router, topk_ids, topk_w,
+                               expert_offsets, scratch.tile_prefix, scratch.tile_order, scratch.tile_rows, sorted_to_flat,
+                               flat_to_sorted, status, ids_local ? (int)(status_bytes / sizeof(int)) : 0);
     }
     cudaError_t err = cudaMemsetAsync(status, 0, status_bytes, stream);  // the status word and what shares its region
     if (err != cudaSuccess) return err;

@@ -62,6 +62,26 @@ def test_route_odd_shapes(T, E, k):
     check_against_oracle(torch.randn(T, E, generator=g), k)
 
 
+@pytest.mark.parametrize("T,E,k", [(16, 64, 32), (17, 64, 4), (65, 256, 31), (64, 256, 32), (255, 256, 8), (256, 256, 8),
+                                   (228, 97, 9), (257, 8, 2)])
+def test_route_one_block_cluster_and_many_blocks(T, E, k):
+    """The edges between the three forms of the small-batch router: 16 / 17 tokens, 256 / 257 tokens, 2048 / 2052 ids (a
+    cluster keeps at most 2048), blocks of the cluster without tokens (17), twice into the same workspace."""
+    g = torch.Generator().manual_seed(T + E)
+    logits = torch.randn(T, E, generator=g)
+    check_against_oracle(logits, k)
+    ws = moe.alloc_workspace(moe.moe_route_workspace_bytes(T, E, k), "cuda")
+    ws.fill_(0xFF)
+    out = [torch.empty(n, dtype=dt, device="cuda") for n, dt in ((T * k, torch.int32), (T * k, torch.float32), (E + 1, torch.int32),
+                                                                 (T * k, torch.int32), (T * k, torch.int32))]
+    first = None
+    for _ in range(2):
+        moe.moe_route(logits.cuda(), k, out[0].view(T, k), out[1].view(T, k), out[2], out[3], out[4], ws)
+        assert moe.moe_last_status(ws) == moe.MOE_OK
+        first = first or [o.clone() for o in out]
+    assert all(torch.equal(a, b) for a, b in zip(first, out))
+
+
 def test_route_constructed_ties():
     g = torch.Generator().manual_seed(5)
     T, E, k = 512, 64, 8
