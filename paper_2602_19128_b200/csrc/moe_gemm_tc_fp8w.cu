@@ -52,6 +52,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 
 template <int NT_MAX, int STAGES_Q, bool SPLIT>
 struct Fp8Smem {
+    static constexpr bool kStaged = NT_MAX > 32 && NT_MAX < 192;     // through shared memory (Stage), where there is room
     // converted slots in tensor memory (beside two accumulators), token tiles in shared memory, and converter groups
     static constexpr int kConv = NT_MAX > 128 ? 2 : NT_MAX > 64 ? 3 : 4;
     static constexpr int kThreads = (kFirstConvWarp + kConv * kGroupWarps) * 32;
@@ -60,7 +61,7 @@ struct Fp8Smem {
     static constexpr int kQ = kB + kConv * kSlotBBytes;           // STAGES_Q code tiles
     static constexpr int kSplit = kQ + STAGES_Q * kSlotQBytes;
     // q_full[SQ], q_empty[SQ], op_full[C], op_empty[C], acc_full[2], acc_empty[2], SplitK's full
-    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : 0);
+    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : kStaged ? kStageBytes : 0);
     static constexpr int kTmemSlot = kBars + (2 * STAGES_Q + 2 * kConv + 5) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
@@ -317,7 +318,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     } else if (warp < kTokenWarp) {
         // ---------------- epilogue: TMEM -> registers -> global ----------------
         const int q = warp & 3;
-        int acc = 0;
+        int acc = 0, flip = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
@@ -330,13 +331,14 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
                 ok = wait(split.full, 0, kSiteEpilogueTmemFull);
                 fence_cluster();
             }
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
+            if (L::kStaged ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
             tcgen05_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
-            const int feat = SWIGLU ? t.f * (kTileM / 2) + q * 16 + (lane & 15) : t.f * kTileM + q * 32 + lane;
-            __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + feat;
-            if (SPLIT) {
+            __nv_bfloat16 *rows = p.out + (size_t)t.row0 * p.n_out + t.f * (SWIGLU ? kTileM / 2 : kTileM);  // this tile's features
+            __nv_bfloat16 *dst = rows + (SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane);
+            if constexpr (L::kStaged) {
+                drain_staged<SWIGLU>(taddr, n_mma, t.n_valid, rows, (size_t)p.n_out, base_ptr + L::kSplit, flip, q, lane);
+            } else if constexpr (SPLIT) {
                 for (int c0 = 0; c0 < n_mma; c0 += 16) {
                     float v[16];
                     tmem_load_16(taddr + c0, v);

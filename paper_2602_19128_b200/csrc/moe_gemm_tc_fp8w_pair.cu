@@ -114,7 +114,8 @@ struct Fp8PairSmem {
     static constexpr int kSlotBBytes = NT_MAX * kRowBytes;  // this CTA's rows, two swizzled chunks (K 0..63 | 64..127)
     static constexpr int kB = 0;                                     // kStagesT token slots
     static constexpr int kQ = kB + kStagesT * kSlotBBytes;           // kStagesQ code tiles
-    static constexpr int kBars = kQ + kStagesQ * kSlotQBytes;
+    static constexpr int kStage = kQ + kStagesQ * kSlotQBytes;       // the epilogue's buffers
+    static constexpr int kBars = kStage + kStageBytes;
     static constexpr int kNumBars = 2 * kStagesQ + 2 * kStagesT + 4;
     static constexpr int kTmemSlot = kBars + kNumBars * 8;
     static constexpr int kAbort = kTmemSlot + 4;
@@ -395,7 +396,7 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMaps maps, const 
     } else if (warp < kTokenWarp) {
         // ---------------- epilogue (both CTAs): own 128 weight rows x all N tokens, TMEM -> registers -> global ----------------
         const int q = warp & 3;
-        int acc = 0;
+        int acc = 0, flip = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
@@ -404,12 +405,11 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMaps maps, const 
             const Tile t = decode_tile(tile, p, sched);
             const int n_mma = (t.n_valid + 15) & ~15;
             const int feat0 = (2 * t.f + (int)rank) * kFeatPerCta;
-            ok = __all_sync(0xffffffffu, wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull));
-            if (!ok) break;
+            ok = wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
+            if (epilogue_any(!ok)) break;  // the four warps meet inside the tile: they leave together
             tcgen05_fence_after();
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
-            __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + feat0 + (SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane);
-            drain_accumulator<SWIGLU>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
+            drain_staged<SWIGLU>(tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX, n_mma, t.n_valid,
+                                 p.out + (size_t)t.row0 * p.n_out + feat0, (size_t)p.n_out, base_ptr + L::kStage, flip, q, lane);
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + acc * 8, 0));

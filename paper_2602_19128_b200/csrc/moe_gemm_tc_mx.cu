@@ -56,15 +56,16 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 
 template <int NT_MAX, int STAGES, bool SPLIT>
 struct MxSmem {
+    static constexpr bool kStaged = NT_MAX > 32;  // stored through shared memory (as in moe_gemm_tc.cu)
     static constexpr int kSlotBBytes = NT_MAX * kMxSlotK;
     static constexpr int kA = 0;
     static constexpr int kB = STAGES * kMxSlotABytes;
     static constexpr int kSfA = kB + STAGES * kSlotBBytes;
     static constexpr int kSfB = kSfA + STAGES * kMxSfAtomBytes;
-    static constexpr int kAmax = kSfB + STAGES * kMxSfBBytes;     // [2 buffers][4 warps][16 tokens] magnitudes
-    static constexpr int kSplit = kAmax + 2 * 4 * 16 * 4;
+    static constexpr int kAmax = kSfB + STAGES * kMxSfBBytes;     // [2 buffers][4 warps][32 tokens] magnitudes
+    static constexpr int kSplit = kAmax + kAmaxBytes;
     // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], SplitK's full
-    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : 0);
+    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : kStaged ? kStageBytes : 0);
     static constexpr int kTmemSlot = kBars + (2 * STAGES + 5) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
@@ -265,10 +266,12 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
                 // scale bytes of h: features 64f + 16q.. lie in block 2f + q/2 = K-slot block/4 of the down GEMM
                 const int block = 2 * t.f + (q >> 1);
                 uint8_t *sf_dst = p.out_sf + ((size_t)(block >> 2) * p.n_atoms + t.atom) * kMxSfAtomBytes + (block & 3);
-                drain_swiglu_mx(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, sf_dst, amax_s, buf, q, lane);
+                drain_swiglu_mx<L::kStaged>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, sf_dst, amax_s, buf, base_ptr + L::kSplit, q, lane);
             } else {
                 __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.out) + (size_t)t.row0 * p.n_out + t.f * kTileM + q * 32 + lane;
-                if (SPLIT) {
+                if constexpr (L::kStaged) {
+                    drain_staged<false>(taddr, n_mma, t.n_valid, dst - (q * 32 + lane), (size_t)p.n_out, base_ptr + L::kSplit, buf, q, lane);
+                } else if constexpr (SPLIT) {
                     for (int c0 = 0; c0 < n_mma; c0 += 16) {
                         float v[16];
                         tmem_load_16(taddr + c0, v);

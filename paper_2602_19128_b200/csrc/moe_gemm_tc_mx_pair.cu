@@ -47,7 +47,7 @@ __device__ __forceinline__ void umma_mx_pair(uint32_t d_tmem, uint64_t a_desc, u
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem)
         : "memory");
 }
-template <int NT_MAX, int STAGES>
+template <int NT_MAX, int STAGES, int STAGE_BYTES>
 struct MxPairSmem {
     static constexpr int kAtomsB = (NT_MAX + 127) / 128;
     static constexpr int kSlotBBytes = (NT_MAX / 2) * kMxSlotK;
@@ -57,17 +57,18 @@ struct MxPairSmem {
     static constexpr int kSfA = kB + STAGES * kSlotBBytes;
     static constexpr int kSfB = kSfA + STAGES * kMxSfAtomBytes;
     static constexpr int kAmax = kSfB + STAGES * kSfBBytes;
-    static constexpr int kBars = kAmax + 2 * 4 * 16 * 4;  // full[S], empty[S], acc_full[2], acc_empty[2]
+    static constexpr int kStage = kAmax + kAmaxBytes;  // the epilogue's buffers
+    static constexpr int kBars = kStage + STAGE_BYTES;  // full[S], empty[S], acc_full[2], acc_empty[2]
     static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const MxParams p) {
-    using L = MxPairSmem<NT_MAX, STAGES>;
+    using L = MxPairSmem<NT_MAX, STAGES, !STAGED ? 0 : SWIGLU ? 2 * kMxStageBytes : Stage<false>::kBytes>;
     static_assert(2 * NT_MAX + 16 + 4 * L::kAtomsB <= kTmemColsMx, "accumulators and scale columns exceed tensor memory");
     static_assert(NT_MAX % 16 == 0 && (NT_MAX / 2) % 8 == 0, "token tile halves must be whole 8-row swizzle groups");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
@@ -252,14 +253,17 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
                 uint8_t *dst = static_cast<uint8_t *>(p.out) + (size_t)t.row0 * p.n_out + feat0 + q * 16 + (lane & 15);
                 const int block = (feat0 + q * 16) >> 5;  // 32-feature block = scale byte `block % 4` of K-slot `block / 4`
                 uint8_t *sf_dst = p.out_sf + ((size_t)(block >> 2) * p.n_atoms + t.atom) * kMxSfAtomBytes + (block & 3);
-                drain_swiglu_mx(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, sf_dst, amax_s, buf, q, lane);
+                drain_swiglu_mx<STAGED>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, sf_dst, amax_s, buf, base_ptr + L::kStage, q, lane);
             } else {
                 __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.out) + (size_t)t.row0 * p.n_out + feat0 + q * 32 + lane;
-                drain_accumulator<false>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
+                if constexpr (STAGED)
+                    drain_staged<false>(taddr, n_mma, t.n_valid, dst - (q * 32 + lane), (size_t)p.n_out, base_ptr + L::kStage, buf, q, lane);
+                else
+                    drain_accumulator<false>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
             }
             tcgen05_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(bar_acc_empty + acc * 8, 0));
+            if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + acc * 8, 0));
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -276,11 +280,11 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
     tmem_release_pair(tmem_base, kTmemColsMx, warp);
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
 int launch_pair_instance(const MxPairMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
-    using L = MxPairSmem<NT_MAX, STAGES>;
+    using L = MxPairSmem<NT_MAX, STAGES, !STAGED ? 0 : SWIGLU ? 2 * kMxStageBytes : Stage<false>::kBytes>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU>;
+    auto kernel = grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
@@ -335,13 +339,18 @@ int launch_grouped_gemm_tc_mx_pair(const MxGemmArgs &a, cudaStream_t stream) {
     const int n_pairs = (int)(max_tiles < pairs_on_device ? max_tiles : pairs_on_device);
     const int grid = 2 * (n_pairs > 0 ? n_pairs : 1);
     if (a.nt_max == 240)
-        return a.swiglu ? launch_pair_instance<240, 6, true>(maps, p, grid, stream)
-                        : launch_pair_instance<240, 6, false>(maps, p, grid, stream);
-    if (a.nt_max == 160)  // a smaller token slot buys two more ring slots: more weight bytes in flight per SM
-        return a.swiglu ? launch_pair_instance<160, 8, true>(maps, p, grid, stream)
-                        : launch_pair_instance<160, 8, false>(maps, p, grid, stream);
-    return a.swiglu ? launch_pair_instance<128, 8, true>(maps, p, grid, stream)
-                    : launch_pair_instance<128, 8, false>(maps, p, grid, stream);
+        return a.swiglu ? launch_pair_instance<240, 6, true, true>(maps, p, grid, stream)
+                        : launch_pair_instance<240, 6, false, true>(maps, p, grid, stream);
+    // A smaller token slot buys two more ring slots (more weight bytes in flight per SM), or one and the epilogue's buffers
+    // (kDirectFromK).
+    if (a.nt_max == 160 && a.K >= kDirectFromK)
+        return a.swiglu ? launch_pair_instance<160, 8, true, false>(maps, p, grid, stream)
+                        : launch_pair_instance<160, 8, false, false>(maps, p, grid, stream);
+    if (a.nt_max == 160)
+        return a.swiglu ? launch_pair_instance<160, 7, true, true>(maps, p, grid, stream)
+                        : launch_pair_instance<160, 7, false, true>(maps, p, grid, stream);
+    return a.swiglu ? launch_pair_instance<128, 8, true, true>(maps, p, grid, stream)
+                    : launch_pair_instance<128, 8, false, true>(maps, p, grid, stream);
 }
 
 }  // namespace moe

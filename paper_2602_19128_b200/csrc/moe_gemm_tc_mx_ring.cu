@@ -35,7 +35,6 @@ constexpr int kNumChunks = kAccCols / kChunkCols;  // 31
 constexpr int kAccFullBars = 32;     // tiles between the MMA warp and the epilogue: each holds at least one chunk
 constexpr int kTileQueue = 16;       // more entries than ring slots: the producer is at most STAGES tiles ahead
 constexpr uint32_t kSfACol = kAccCols, kSfBCol = kAccCols + 4;
-constexpr int kOutStageBytes = 16 * kTileM * 2;  // one 16-column group of a CTA's 128 output rows, token-major
 
 struct MxRingMaps {
     TensorMaps ops;            // weight codes, token codes (boxes of 8, 16, ..., 128 rows)
@@ -56,7 +55,7 @@ __device__ __forceinline__ void umma_mx_pair(uint32_t d_tmem, uint64_t a_desc, u
         : "memory");
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
 struct MxRingSmem {
     static constexpr int kAtomsB = (NT_MAX + 127) / 128;
     static constexpr int kSlotBBytes = (NT_MAX / 2) * kMxSlotK;
@@ -66,8 +65,9 @@ struct MxRingSmem {
     static constexpr int kSfA = kB + STAGES * kSlotBBytes;
     static constexpr int kSfB = kSfA + STAGES * kMxSfAtomBytes;
     static constexpr int kAmax = kSfB + STAGES * kSfBBytes;
-    static constexpr int kOutStage = kAmax + 2 * 4 * 16 * 4;  // down projection only: two [16 tokens][128 rows] bf16 tiles
-    static constexpr int kBars = kOutStage + (SWIGLU ? 0 : 2 * kOutStageBytes);  // full[S], empty[S], acc_full[32], acc_empty[32 (31 used)]
+    static constexpr int kOutStage = kAmax + kAmaxBytes;  // the epilogue's buffers
+    // full[S], empty[S], acc_full[32], acc_empty[32 (31 used)]
+    static constexpr int kBars = kOutStage + (!SWIGLU ? Stage<false>::kBytes : STAGED ? 2 * kMxStageBytes : 0);
     static constexpr int kQueue = kBars + (2 * STAGES + kAccFullBars + 32) * 8;
     static constexpr int kTmemSlot = kQueue + kTileQueue * 4;
     static constexpr int kAbort = kTmemSlot + 4;
@@ -94,10 +94,10 @@ __device__ __forceinline__ MxParts split_mx_tile(int seq, int n_cols) {
     return s;
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMxRingThreads, 1)
 grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const MxParams p) {
-    using L = MxRingSmem<NT_MAX, STAGES, SWIGLU>;
+    using L = MxRingSmem<NT_MAX, STAGES, SWIGLU, STAGED>;
     static_assert(NT_MAX % 16 == 0 && NT_MAX <= 384 && NT_MAX > 256, "token-tile bound of the wide-tile kernel");
     static_assert(L::kAtomsB == 3, "three token scale atoms next to the weight scales");
     static_assert(STAGES < kTileQueue, "the tile queue must outlast the ring");
@@ -320,37 +320,35 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
             } else {
                 dst_rows = static_cast<__nv_bfloat16 *>(p.out) + (size_t)t.row0 * p.n_out + feat0;
             }
-#pragma unroll 1
-            for (int g = 0; g < n_groups; ++g) {
-                const int c0 = ((seq & 1) ? g : n_groups - 1 - g) << 4;  // first column of the group = its first tile row
-                float v[16];
-                tmem_load_16(lane_base + parts.first_col + c0, v);
-                // the chunk goes back as soon as its columns have been read
+            auto hand_back = [&](int first_col, int n) {  // n chunks go back as soon as their columns have been read
                 tcgen05_fence_before();
                 __syncwarp();
-                if (lane == 0)
-                    mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + ((parts.first_col + c0) / kChunkCols) * 8, 0));
-                if (SWIGLU) {
-                    store_swiglu_mx_16(v, t.n_valid - c0, dst_q + (size_t)c0 * p.n_out, (size_t)p.n_out, sf_dst, c0, amax_s, buf, q, lane);
-                } else {
-                    // Output rows are the token's: a lane holds one output feature of 16 tokens, and stored from here
-                    // a warp instruction would write 32 x 2 bytes of one token -- measured, those stores took as long
-                    // as the MMAs of a tile.  The four warps transpose the group through shared memory instead and
-                    // each stores four whole 256-byte token rows, 16 bytes per lane.
-                    out_flip ^= 1;  // (across tiles too: two consecutive groups never share a buffer)
-                    uint8_t *stage_buf = base_ptr + L::kOutStage + out_flip * kOutStageBytes;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        reinterpret_cast<__nv_bfloat16 *>(stage_buf)[i * kTileM + q * 32 + lane] = __float2bfloat16_rn(v[i]);
-                    asm volatile("bar.sync 2, 128;" ::: "memory");  // (two buffers: the next group's writes cannot pass this)
-#pragma unroll
-                    for (int it = 0; it < 2; ++it) {
-                        const int r = q * 4 + it * 2 + (lane >> 4);  // token of the group
-                        const uint4 val = *reinterpret_cast<const uint4 *>(stage_buf + r * (kTileM * 2) + (lane & 15) * 16);
-                        if (c0 + r < t.n_valid)
-                            *reinterpret_cast<uint4 *>(dst_rows + (size_t)(c0 + r) * p.n_out + (lane & 15) * 8) = val;
-                    }
+                if (lane < n)
+                    mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + ((parts.first_col + first_col) / kChunkCols + lane) * 8, 0));
+            };
+#pragma unroll 1
+            for (int g = 0; g < n_groups; ++g) {
+                if (SWIGLU && g + 1 < n_groups) {  // two groups at a time, the lower one first
+                    const int c0 = ((seq & 1) ? g : n_groups - 2 - g) << 4;
+                    ++g;
+                    float v[2][16];
+                    tmem_load_2x16(lane_base + parts.first_col + c0, v);
+                    hand_back(c0, 2);
+                    store_swiglu_mx<2, STAGED>(v, t.n_valid - c0, dst_q + (size_t)c0 * p.n_out, (size_t)p.n_out, sf_dst, c0, amax_s, buf,
+                                               base_ptr + L::kOutStage, q, lane);
+                    continue;
                 }
+                const int c0 = ((seq & 1) ? g : n_groups - 1 - g) << 4;  // first column of the group = its first tile row
+                float v[1][16];
+                tmem_load_16(lane_base + parts.first_col + c0, v[0]);
+                hand_back(c0, 1);
+                if (SWIGLU)
+                    store_swiglu_mx<1, STAGED>(v, t.n_valid - c0, dst_q + (size_t)c0 * p.n_out, (size_t)p.n_out, sf_dst, c0, amax_s, buf,
+                                               base_ptr + L::kOutStage, q, lane);
+                else
+                    store_staged<false>(v, base_ptr + L::kOutStage, out_flip, [&](int token) -> __nv_bfloat16 * {
+                        return c0 + token < t.n_valid ? dst_rows + (size_t)(c0 + token) * p.n_out : nullptr;
+                    }, q, lane);
             }
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator has been handed back)
         }
@@ -367,11 +365,11 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
     tmem_release_pair(tmem_base, kTmemColsMx, warp);
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED = true>
 int launch_mx_ring_instance(const MxRingMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
-    using L = MxRingSmem<NT_MAX, STAGES, SWIGLU>;
+    using L = MxRingSmem<NT_MAX, STAGES, SWIGLU, STAGED>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU>;
+    auto kernel = grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kMxRingThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
@@ -425,8 +423,10 @@ int launch_grouped_gemm_tc_mx_ring(const MxGemmArgs &a, cudaStream_t stream) {
     const int pairs_on_device = sm_count() / 2;
     const int n_pairs = (int)(max_tiles < pairs_on_device ? max_tiles : pairs_on_device);
     const int grid = 2 * (n_pairs > 0 ? n_pairs : 1);
-    if (a.nt_max == 304)  // (the gate/up kernel has no output staging buffer: room for a sixth ring slot)
-        return a.swiglu ? launch_mx_ring_instance<304, 6, true>(maps, p, grid, stream)
+    // (a gate/up kernel that stores its codes directly has room for a sixth ring slot: kDirectFromK)
+    if (a.nt_max == 304 && a.swiglu && a.K >= kDirectFromK) return launch_mx_ring_instance<304, 6, true, false>(maps, p, grid, stream);
+    if (a.nt_max == 304)
+        return a.swiglu ? launch_mx_ring_instance<304, 5, true>(maps, p, grid, stream)
                         : launch_mx_ring_instance<304, 5, false>(maps, p, grid, stream);
     return a.swiglu ? launch_mx_ring_instance<384, 5, true>(maps, p, grid, stream)
                     : launch_mx_ring_instance<384, 5, false>(maps, p, grid, stream);

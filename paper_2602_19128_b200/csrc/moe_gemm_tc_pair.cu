@@ -43,23 +43,24 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc,
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-template <int NT_MAX, int STAGES, int SLABS>
+template <int NT_MAX, int STAGES, int SLABS, int STAGE_BYTES>
 struct PairSmem {
     static constexpr int kSlotABytesAll = SLABS * kSlotABytes;
     static constexpr int kSlotBBytes = (NT_MAX / 2) * kRowBytes;
     static constexpr int kA = 0;
     static constexpr int kB = STAGES * kSlotABytesAll;
-    static constexpr int kBars = kB + STAGES * kSlotBBytes;  // full[S], empty[S], acc_full[2], acc_empty[2]
+    static constexpr int kStage = kB + STAGES * kSlotBBytes;  // the epilogue's buffers
+    static constexpr int kBars = kStage + STAGE_BYTES;        // full[S], empty[S], acc_full[2], acc_empty[2]
     static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
-template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU>
+template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
-    using L = PairSmem<NT_MAX, STAGES, SLABS>;
+    using L = PairSmem<NT_MAX, STAGES, SLABS, STAGED ? kStageBytes : 0>;
     constexpr int kAccBufs = SLABS == 1 ? 2 : 1;          // accumulator sets in TMEM
     // accumulator columns (2 * NT_MAX either way), rounded up to the power of two an allocation must be
     constexpr int kAccCols = SLABS * kAccBufs * NT_MAX;
@@ -227,7 +228,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     } else {
         // ---------------- epilogue (both CTAs): own 128 weight rows per slab x all N tokens ----------------
         const int q = warp & 3;  // a warp may only read TMEM lanes 32*(warp%4) .. +31
-        int acc = 0;
+        int acc = 0, flip = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
@@ -236,20 +237,21 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             const Tile t = decode_tile(tile, p);
             const int n_mma = (t.n_valid + 15) & ~15;
             ok = pair_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, peer_abort, p.status, kSiteEpilogueTmemFull + kSiteOffset);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
+            if (STAGED ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
             tcgen05_fence_after();
-            const int lane_feat = SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane;
 #pragma unroll
             for (int s = 0; s < SLABS; ++s) {
                 const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (acc * SLABS + s) * NT_MAX;
-                __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + t.f * kFeatPerTile + s * kFeatPerSlab +
-                                     (int)rank * kFeatPerCta + lane_feat;
-                drain_accumulator<SWIGLU>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
+                __nv_bfloat16 *dst = p.out + (size_t)t.row0 * p.n_out + t.f * kFeatPerTile + s * kFeatPerSlab + (int)rank * kFeatPerCta;
+                if constexpr (STAGED)
+                    drain_staged<SWIGLU>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, base_ptr + L::kStage, flip, q, lane);
+                else
+                    drain_accumulator<SWIGLU>(taddr, n_mma, t.n_valid, dst + (SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane),
+                                              (size_t)p.n_out, lane);
             }
             tcgen05_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(bar_acc_empty + acc * 8, 0));
+            if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + acc * 8, 0));
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1u; }
         }
@@ -267,11 +269,11 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     tmem_release_pair(tmem_base, kTmemCols, warp);
 }
 
-template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU>
+template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED>
 int launch_pair_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
-    using L = PairSmem<NT_MAX, STAGES, SLABS>;
+    using L = PairSmem<NT_MAX, STAGES, SLABS, STAGED ? kStageBytes : 0>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU>;
+    auto kernel = grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
@@ -319,13 +321,17 @@ int launch_grouped_gemm_tc_pair(const GroupedGemmArgs &a, int slabs, cudaStream_
     const int n_pairs = (int)(max_tiles < pairs_on_device ? max_tiles : pairs_on_device);
     const int grid = 2 * (n_pairs > 0 ? n_pairs : 1);
     if (slabs == 2)
-        return a.swiglu ? launch_pair_instance<256, 4, 2, true>(maps, p, grid, stream)
-                        : launch_pair_instance<256, 4, 2, false>(maps, p, grid, stream);
+        return a.swiglu ? launch_pair_instance<256, 4, 2, true, false>(maps, p, grid, stream)
+                        : launch_pair_instance<256, 4, 2, false, false>(maps, p, grid, stream);
+    // 256-row tiles: seven slots leave no room for the epilogue's buffers (kDirectFromK).
+    if (a.nt_max == 256 && a.K >= kDirectFromK)
+        return a.swiglu ? launch_pair_instance<256, 7, 1, true, false>(maps, p, grid, stream)
+                        : launch_pair_instance<256, 7, 1, false, false>(maps, p, grid, stream);
     if (a.nt_max == 256)
-        return a.swiglu ? launch_pair_instance<256, 7, 1, true>(maps, p, grid, stream)
-                        : launch_pair_instance<256, 7, 1, false>(maps, p, grid, stream);
-    return a.swiglu ? launch_pair_instance<128, 9, 1, true>(maps, p, grid, stream)
-                    : launch_pair_instance<128, 9, 1, false>(maps, p, grid, stream);
+        return a.swiglu ? launch_pair_instance<256, 6, 1, true, true>(maps, p, grid, stream)
+                        : launch_pair_instance<256, 6, 1, false, true>(maps, p, grid, stream);
+    return a.swiglu ? launch_pair_instance<128, 9, 1, true, true>(maps, p, grid, stream)
+                    : launch_pair_instance<128, 9, 1, false, true>(maps, p, grid, stream);
 }
 
 }  // namespace moe

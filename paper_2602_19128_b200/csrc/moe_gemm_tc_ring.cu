@@ -42,7 +42,6 @@ constexpr int kNumChunks = 32;      // 512 columns of tensor memory
 constexpr int kAccFullBars = 32;    // tiles between the MMA warp and the epilogue: each holds at least one chunk
 constexpr int kTileQueue = 16;      // more entries than ring slots: the producer is at most STAGES tiles ahead
 constexpr int kRingActMaps = 24;    // act[i]: box of 8 * (i + 1) rows, up to 192 rows per CTA (N = 384)
-constexpr int kOutStageBytes = 16 * kTileM * 2;  // one 16-column group of a CTA's 128 output rows, token-major
 
 struct RingMaps {
     CUtensorMap w;
@@ -76,8 +75,8 @@ struct RingSmem {
     static constexpr int kSlotBBytes = (NT_MAX / 2) * kRowBytes;
     static constexpr int kA = 0;
     static constexpr int kB = STAGES * kSlotABytes;
-    static constexpr int kOutStage = kB + STAGES * kSlotBBytes;  // down projection: two [16 tokens][128 rows] bf16 tiles
-    static constexpr int kBars = kOutStage + 2 * kOutStageBytes;  // full[S], empty[S], acc_full[32], acc_empty[32]
+    static constexpr int kOutStage = kB + STAGES * kSlotBBytes;  // the epilogue's buffers (Stage)
+    static constexpr int kBars = kOutStage + kStageBytes;  // full[S], empty[S], acc_full[32], acc_empty[32]
     static constexpr int kQueue = kBars + (2 * STAGES + kAccFullBars + kNumChunks) * 8;
     static constexpr int kTmemSlot = kQueue + kTileQueue * 4;
     static constexpr int kAbort = kTmemSlot + 4;
@@ -308,57 +307,52 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
             const Parts parts = split_tile(seq, n_mma);
             ok = pair_wait(bar_acc_full + (seq & (kAccFullBars - 1)) * 8, (uint32_t)(seq / kAccFullBars) & 1u, abort_flag, peer_abort,
                            p.status, kSiteEpilogueTmemFull + kSiteOffset);
-            if (epilogue_any(!ok)) break;  // the four warps synchronise inside a down-projection tile: they leave together
+            if (epilogue_any(!ok)) break;  // the four warps synchronise inside the tile: they leave together
             tcgen05_fence_after();
-            const int lane_feat = SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane;
             __nv_bfloat16 *dst_rows = p.out + (size_t)t.row0 * p.n_out + t.f * kFeatPerTile + (int)rank * kFeatPerCta;
-            __nv_bfloat16 *dst = dst_rows + lane_feat;
             const size_t row_stride = (size_t)p.n_out;
             // An even tile is drained from its highest 16 columns down, an odd tile from its lowest up: the columns the
             // next tile of this pair is waiting for go back first.
             const int n_groups = n_mma >> 4;
-#pragma unroll 1
-            for (int g = 0; g < n_groups; ++g) {
-                const int tile_col = ((seq & 1) ? g : n_groups - 1 - g) << 4;        // first column of the group, within the tile
+            // Accumulator column j of a part is tile row  j < half ? row + j : N/2 + row + (j - half).  `half` is a
+            // multiple of 8, so a group's columns 0..7 are eight consecutive rows (from row_a on) and so are its columns
+            // 8..15 (from row_b on).
+            auto row_of = [&](int col) -> __nv_bfloat16 * {  // the row of a tile's column, or null past the last row
+                const int tile_col = col & ~15, r = col & 15;
                 const int part = tile_col >= parts.cols[0] ? 1 : 0;
                 const int c0 = tile_col - (part ? parts.cols[0] : 0);               // ... within its part
                 const int half = (part ? parts.cols[1] : parts.cols[0]) >> 1;
-                // Accumulator column j of a part is tile row  j < half ? row + j : N/2 + row + (j - half).  `half` is a
-                // multiple of 8, so the group's columns 0..7 are eight consecutive rows and so are its columns 8..15.
                 const int row_lo = part ? parts.row[1] : 0, row_hi = half_tile + row_lo - half;
                 const int row_a = c0 < half ? row_lo + c0 : row_hi + c0;
                 const int row_b = c0 + 8 < half ? row_lo + c0 + 8 : row_hi + c0 + 8;
-                float v[16];
-                tmem_load_16(lane_base + parts.first_col + tile_col, v);
-                // the chunk goes back as soon as its columns have been read
+                const int row = r < 8 ? row_a + r : row_b + r - 8;
+                return row < t.n_valid ? dst_rows + (size_t)row * row_stride : nullptr;
+            };
+            constexpr int kStep = Stage<SWIGLU>::kGroups;  // gate/up: two groups at a time, the lower one first
+#pragma unroll 1
+            for (int g = 0; g < n_groups; g += kStep) {
+                const int groups = g + kStep <= n_groups ? kStep : n_groups - g;
+                const int tile_col = ((seq & 1) ? g : n_groups - groups - g) << 4;  // the step's first column, within the tile
+                float v[kStep][16];
+                if constexpr (SWIGLU) {
+                    if (groups == 2) {
+                        tmem_load_2x16(lane_base + parts.first_col + tile_col, v);
+                    } else {
+                        tmem_load_16(lane_base + parts.first_col + tile_col, v[0]);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) v[1][i] = 0.f;
+                    }
+                } else {
+                    tmem_load_16(lane_base + parts.first_col + tile_col, v[0]);
+                }
+                // the chunks go back as soon as their columns have been read
                 tcgen05_fence_before();
                 __syncwarp();
-                if (lane == 0)
-                    mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + ((parts.first_col + tile_col) / kChunkCols) * 8, 0));
-                if (SWIGLU) {  // this lane stores columns hi*8 .. hi*8+7 of the group
-                    float hv[8];
-                    swiglu_16(v, lane, hv);
-                    const int row0 = (lane & 16) ? row_b : row_a;
-                    store_column(hv, t.n_valid - row0, dst + (size_t)row0 * row_stride, row_stride);
-                } else {
-                    // A lane holds one output feature of 16 tokens; stored from here a warp instruction would write
-                    // 32 x 2 bytes of one token.  The four warps transpose the group through shared memory instead and
-                    // each stores four whole 256-byte token rows, 16 bytes per lane.
-                    out_flip ^= 1;  // (across tiles too: two consecutive groups never share a buffer)
-                    uint8_t *stage_buf = base_ptr + L::kOutStage + out_flip * kOutStageBytes;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        reinterpret_cast<__nv_bfloat16 *>(stage_buf)[i * kTileM + q * 32 + lane] = __float2bfloat16_rn(v[i]);
-                    asm volatile("bar.sync 2, 128;" ::: "memory");  // (two buffers: the next group's writes cannot pass this)
-#pragma unroll
-                    for (int it = 0; it < 2; ++it) {
-                        const int r = q * 4 + it * 2 + (lane >> 4);          // column of the group
-                        const int row = r < 8 ? row_a + r : row_b + r - 8;   // ... and its tile row
-                        const uint4 val = *reinterpret_cast<const uint4 *>(stage_buf + r * (kTileM * 2) + (lane & 15) * 16);
-                        if (row < t.n_valid)
-                            *reinterpret_cast<uint4 *>(dst_rows + (size_t)row * row_stride + (lane & 15) * 8) = val;
-                    }
-                }
+                if (lane < groups)
+                    mbar_arrive_cluster_relaxed(map_to_cta(bar_acc_empty + ((parts.first_col + tile_col) / kChunkCols + lane) * 8, 0));
+                store_staged<SWIGLU>(v, base_ptr + L::kOutStage, out_flip, [&](int token) -> __nv_bfloat16 * {
+                    return (token >> 4) < groups ? row_of(tile_col + token) : nullptr;
+                }, q, lane);
             }
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator has been handed back)
         }

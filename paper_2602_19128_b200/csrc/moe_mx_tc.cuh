@@ -103,67 +103,102 @@ __device__ __forceinline__ uint32_t half_warp_max8(const uint32_t (&mag)[8], int
     return max(m1, __shfl_xor_sync(0xffffffffu, m1, 1));
 }
 
-// Gate/up epilogue of one warp for 16 accumulator columns: its 32 TMEM lanes hold, for 16 features, the gate rows (lanes
-// 0..15) and the up rows (lanes 16..31).  Computes h = SiLU(gate) * up, quantises it in blocks of 32 features (this warp's 16
-// and its partner warp's 16, warps q and q^1; their maxima are exchanged through shared memory), and stores the codes and the
-// scale bytes.  As in the bf16 epilogue (moe_tc_common.cuh) everything is computed before the first store, and whole groups
-// are stored without conditions.
-//   left     rows of the tile from the group's first column on
-//   dst      -> code of this lane's feature in the group's first row; row stride n_out bytes
-//   sf_dst   -> byte of the block's scale in row 0 of the tile's first atom (K-slot and block already applied); c0: the
-//               group's first row within the tile
-//   amax_s   [2][4][16] exchange buffer in shared memory; buf is flipped every group (across tiles too): a
-//            warp may run one group ahead of its partner
-__device__ __forceinline__ void store_swiglu_mx_16(const float (&v)[16], int left, uint8_t *dst, size_t n_out, uint8_t *sf_dst, int c0,
-                                                   uint32_t *amax_s, int &buf, int q, int lane) {
+// Gate/up epilogue of one warp for G groups of 16 accumulator columns: its 32 TMEM lanes hold, for 16 features, the gate rows
+// (lanes 0..15) and the up rows (lanes 16..31).  Computes h = SiLU(gate) * up, quantises it in blocks of 32 features (this
+// warp's 16 and its partner warp's 16, warps q and q^1; their maxima are exchanged through shared memory), and stores the
+// codes and the scale bytes.  As in the bf16 epilogue (moe_tc_common.cuh) everything is computed before the first store, and
+// whole groups are stored without conditions; two groups share one exchange.
+//   left     rows of the tile from the first group's first column on
+//   dst      -> code of this lane's feature in that first row; row stride n_out bytes
+//   sf_dst   -> byte of the block's scale in row 0 of the tile's first atom (K-slot and block already applied); c0: that
+//               first row within the tile
+//   amax_s   [2][4][32] exchange buffer in shared memory; buf is flipped every call (across tiles too): a
+//            warp may run one call ahead of its partner
+//   stage    STAGED: two buffers of kMxStageBytes through which the CTA's 64 features of a token are stored as one row
+//            (as in moe_tc_common.cuh, Stage; flipped with buf)
+constexpr int kAmaxBytes = 2 * 4 * 32 * 4;
+constexpr int kMxStagePitch = 80, kMxStageBytes = 32 * kMxStagePitch + 16;
+__device__ __forceinline__ int mx_stage_at(int token) { return token * kMxStagePitch + ((token >> 3) & 1) * 16; }
+template <int G, bool STAGED>
+__device__ __forceinline__ void store_swiglu_mx(const float (&v)[G][16], int left, uint8_t *dst, size_t n_out, uint8_t *sf_dst, int c0,
+                                                uint32_t *amax_s, int &buf, uint8_t *stage, int q, int lane) {
     const int hi = lane >> 4, j = lane & 15;
-    float hv[8];
-    swiglu_16(v, lane, hv);
-    uint32_t mag[8];
+    float hv[G][8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) mag[i] = __float_as_uint(hv[i]) & 0x7FFFFFFFu;  // magnitudes compare as integers; NaN and inf on top
-    const uint32_t col_max = half_warp_max8(mag, j);  // of column hi * 8 + j / 2 over this warp's 16 features
+    for (int g = 0; g < G; ++g) swiglu_16(v[g], lane, hv[g]);
     buf ^= 1;
-    if ((j & 1) == 0) amax_s[(buf * 4 + q) * 16 + hi * 8 + (j >> 1)] = col_max;
+    uint32_t *mine = &amax_s[(buf * 4 + q) * 32 + hi * 8];
+    const uint32_t *partner = &amax_s[(buf * 4 + (q ^ 1)) * 32 + hi * 8];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        uint32_t mag[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) mag[i] = __float_as_uint(hv[g][i]) & 0x7FFFFFFFu;  // magnitudes compare as integers; NaN and inf on top
+        const uint32_t col_max = half_warp_max8(mag, j);  // of column hi * 8 + j / 2 over this warp's 16 features
+        if ((j & 1) == 0) mine[g * 16 + (j >> 1)] = col_max;
+    }
     pair_sync(q >> 1);
-    const uint32_t *mine = &amax_s[(buf * 4 + q) * 16 + hi * 8], *partner = &amax_s[(buf * 4 + (q ^ 1)) * 16 + hi * 8];
-    uint32_t sb[8];
 #pragma unroll
-    for (int i = 0; i < 8; i += 4) {
-        const uint4 a = *reinterpret_cast<const uint4 *>(mine + i), b = *reinterpret_cast<const uint4 *>(partner + i);
-        sb[i] = mx_scale_byte(max(a.x, b.x));
-        sb[i + 1] = mx_scale_byte(max(a.y, b.y));
-        sb[i + 2] = mx_scale_byte(max(a.z, b.z));
-        sb[i + 3] = mx_scale_byte(max(a.w, b.w));
+    for (int g = 0; g < G; ++g) {
+        uint32_t sb[8];
+#pragma unroll
+        for (int i = 0; i < 8; i += 4) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(mine + g * 16 + i), b = *reinterpret_cast<const uint4 *>(partner + g * 16 + i);
+            sb[i] = mx_scale_byte(max(a.x, b.x));
+            sb[i + 1] = mx_scale_byte(max(a.y, b.y));
+            sb[i + 2] = mx_scale_byte(max(a.z, b.z));
+            sb[i + 3] = mx_scale_byte(max(a.w, b.w));
+        }
+        uint8_t code[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint8_t c = (uint8_t)__nv_cvt_float_to_fp8(hv[g][i] * __uint_as_float((254u - sb[i]) << 23), __NV_SATFINITE, __NV_E4M3);
+            code[i] = sb[i] == 255u ? (uint8_t)0x7F : c;
+        }
+        const int here = left - g * 16 - hi * 8;
+        if constexpr (STAGED) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) stage[buf * kMxStageBytes + mx_stage_at(g * 16 + hi * 8 + i) + q * 16 + j] = code[i];
+        } else {
+            uint8_t *row = dst + (size_t)(g * 16 + hi * 8) * n_out;
+            if (left >= (g + 1) * 16) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) row[(size_t)i * n_out] = code[i];
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (i < here) row[(size_t)i * n_out] = code[i];
+            }
+        }
+        if ((q & 1) == 0 && j < 8 && j < here) {  // lane j: the scale of column hi * 8 + j; row r of the tile: atom r / 128, atom row r % 128
+            const int r = c0 + g * 16 + hi * 8 + j;
+            sf_dst[(size_t)(r >> 7) * kMxSfAtomBytes + mx_atom_byte(r & 127, 0)] = (uint8_t)mx_scale_byte(max(mine[g * 16 + j], partner[g * 16 + j]));
+        }
     }
-    uint8_t code[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint8_t c = (uint8_t)__nv_cvt_float_to_fp8(hv[i] * __uint_as_float((254u - sb[i]) << 23), __NV_SATFINITE, __NV_E4M3);
-        code[i] = sb[i] == 255u ? (uint8_t)0x7F : c;
-    }
-    uint8_t *row = dst + (size_t)(hi * 8) * n_out;
-    const int here = left - hi * 8;
-    if (left >= 16) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) row[(size_t)i * n_out] = code[i];
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (i < here) row[(size_t)i * n_out] = code[i];
-    }
-    if ((q & 1) == 0 && j < 8 && j < here) {  // lane j: the scale of column hi * 8 + j; row r of the tile: atom r / 128, atom row r % 128
-        const int r = c0 + hi * 8 + j;
-        sf_dst[(size_t)(r >> 7) * kMxSfAtomBytes + mx_atom_byte(r & 127, 0)] = (uint8_t)mx_scale_byte(max(mine[j], partner[j]));
+    if constexpr (STAGED) {  // four lanes per token: warp q stores tokens 4 G q .. 4 G q + 4 G - 1
+        epilogue_sync();
+        const int token = q * (4 * G) + (lane >> 2);
+        if (lane < 16 * G && token < left) {
+            const uint4 val = *reinterpret_cast<const uint4 *>(stage + buf * kMxStageBytes + mx_stage_at(token) + (lane & 3) * 16);
+            // (dst is this lane's feature: back to the CTA's first)
+            *reinterpret_cast<uint4 *>(dst - (q * 16 + j) + (size_t)token * n_out + (lane & 3) * 16) = val;
+        }
     }
 }
 // ... and for a tile's n_mma columns, of which n_valid are rows of h (dst: this lane's feature in the first).
+template <bool STAGED>
 __device__ __forceinline__ void drain_swiglu_mx(uint32_t taddr, int n_mma, int n_valid, uint8_t *dst, size_t n_out,
-                                                uint8_t *sf_dst, uint32_t *amax_s, int &buf, int q, int lane) {
-    for (int c0 = 0; c0 < n_mma; c0 += 16) {
-        float v[16];
-        tmem_load_16(taddr + c0, v);
-        store_swiglu_mx_16(v, n_valid - c0, dst + (size_t)c0 * n_out, n_out, sf_dst, c0, amax_s, buf, q, lane);
+                                                uint8_t *sf_dst, uint32_t *amax_s, int &buf, uint8_t *stage, int q, int lane) {
+    int c0 = 0;
+    for (; c0 + 32 <= n_mma; c0 += 32) {
+        float v[2][16];
+        tmem_load_2x16(taddr + c0, v);
+        store_swiglu_mx<2, STAGED>(v, n_valid - c0, dst + (size_t)c0 * n_out, n_out, sf_dst, c0, amax_s, buf, stage, q, lane);
+    }
+    if (c0 < n_mma) {
+        float v[1][16];
+        tmem_load_16(taddr + c0, v[0]);
+        store_swiglu_mx<1, STAGED>(v, n_valid - c0, dst + (size_t)c0 * n_out, n_out, sf_dst, c0, amax_s, buf, stage, q, lane);
     }
 }
 

@@ -170,6 +170,23 @@ __device__ __forceinline__ void tmem_load_16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 32 of them, as two groups of 16.
+__device__ __forceinline__ void tmem_load_2x16(uint32_t taddr, float (&v)[2][16]) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i >> 4][i & 15] = __uint_as_float(r[i]);
+}
+
 // Shared-memory matrix descriptor for a K-major bf16 tile whose rows are 128 bytes with the 128-byte
 // swizzle TMA applies: start address, leading offset 1 (unused for swizzled K-major), stride between
 // 8-row groups 1024 bytes, descriptor version 1, layout type 2 (128-byte swizzle).
@@ -399,6 +416,87 @@ __device__ __forceinline__ void drain_accumulator(uint32_t taddr, int n_mma, int
         } else {
             store_column(v, n_valid - c0, dst + (size_t)c0 * stride, stride);
         }
+    }
+}
+
+// ---- the same through shared memory -------------------------------------------------------------------------------
+// Stored from its registers, a warp's 32 rows of the accumulator are 64 bytes (gate/up: 32) of each token's row, two bytes
+// per lane, and every such piece costs the load/store unit about 18 cycles beside the operand copies: 1200 cycles per group
+// of 16 columns, whatever was computed.  Here the four warps of a CTA transpose a step of columns through shared memory and
+// store whole rows, 16 bytes per lane: 128 features of the down projection are 256 bytes, 64 of h are 128.  Two buffers and
+// one barrier of the 128 threads per step: a step's writes cannot pass the barrier of the step before it.  4096 tokens of 32 experts
+// of 1024 x 1024, top 4: bf16 141.9 -> 139.1 us, MX 176.7 -> 167.2; 1024 tokens 75.8 -> 72.8 and 71.2 -> 68.9.
+// Where the buffers cost a ring slot, kernels with K of 4096 and more store directly: their slots hide the epilogue, and
+// want the depth (direct / staged: 512 Mixtral-shaped tokens 498 / 516 us, MX prefill on 32 of 256 experts of 7168 x 2048
+// 477 / 496; staged wins at K = 2048, 2000 tokens of 64 MX experts, top 4, 234 / 231, and below).
+constexpr int kDirectFromK = 4096;
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 4, 128;" ::: "memory"); }
+template <bool SWIGLU>
+struct Stage {
+    static constexpr int kGroups = SWIGLU ? 2 : 1;                 // of 16 tokens, per step
+    static constexpr int kRowBytes = SWIGLU ? kTileM : 2 * kTileM;  // a token's features of this CTA, bf16
+    // Byte `byte` of a token's row.  Gate/up: 16-byte pieces are swizzled, since the half-warps write eight rows apart.
+    __device__ static int at(int token, int byte) {
+        return token * kRowBytes + (SWIGLU ? byte ^ (((token & 7) ^ ((token >> 1) & 4)) << 4) : byte);
+    }
+    static constexpr int kBufferBytes = kGroups * 16 * kRowBytes;
+    static constexpr int kBytes = 2 * kBufferBytes;
+};
+constexpr int kStageBytes = Stage<true>::kBytes;
+static_assert(Stage<true>::kBytes == Stage<false>::kBytes, "either GEMM's buffers");
+// One step: kGroups x 16 columns of this warp's 32 rows.  row_of(token): where this CTA's features of the step's token go in
+// the result, or null if there is no such row.
+template <bool SWIGLU, typename RowOf>
+__device__ __forceinline__ void store_staged(const float (&v)[Stage<SWIGLU>::kGroups][16], uint8_t *stage, int &flip, RowOf row_of,
+                                             int q, int lane) {
+    using S = Stage<SWIGLU>;
+    flip ^= 1;
+    uint8_t *buf = stage + flip * S::kBufferBytes;
+    if constexpr (SWIGLU) {
+        float h[S::kGroups][8];
+#pragma unroll
+        for (int g = 0; g < S::kGroups; ++g) swiglu_16(v[g], lane, h[g]);
+#pragma unroll
+        for (int g = 0; g < S::kGroups; ++g)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<__nv_bfloat16 *>(buf + S::at(g * 16 + ((lane & 16) >> 1) + i, (q * 16 + (lane & 15)) * 2)) = __float2bfloat16_rn(h[g][i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            *reinterpret_cast<__nv_bfloat16 *>(buf + S::at(i, (q * 32 + lane) * 2)) = __float2bfloat16_rn(v[0][i]);
+    }
+    epilogue_sync();
+    constexpr int kLanes = S::kRowBytes / 16, kRows = 32 / kLanes;  // lanes per row, rows per warp instruction
+#pragma unroll
+    for (int it = 0; it < S::kGroups * 16 / 4 / kRows; ++it) {
+        const int token = q * (S::kGroups * 4) + it * kRows + lane / kLanes;
+        const uint4 val = *reinterpret_cast<const uint4 *>(buf + S::at(token, (lane % kLanes) * 16));
+        __nv_bfloat16 *row = row_of(token);
+        if (row) *reinterpret_cast<uint4 *>(row + (lane % kLanes) * 8) = val;
+    }
+}
+// A tile: n_mma columns from taddr on, n_valid of which are rows of the result (dst: this CTA's first feature in the first).
+template <bool SWIGLU>
+__device__ __forceinline__ void drain_staged(uint32_t taddr, int n_mma, int n_valid, __nv_bfloat16 *dst, size_t stride, uint8_t *stage,
+                                             int &flip, int q, int lane) {
+    constexpr int kStep = Stage<SWIGLU>::kGroups * 16;
+    for (int c0 = 0; c0 < n_mma; c0 += kStep) {
+        float v[Stage<SWIGLU>::kGroups][16];
+        if constexpr (SWIGLU) {
+            if (c0 + 32 <= n_mma) {
+                tmem_load_2x16(taddr + c0, v);
+            } else {
+                tmem_load_16(taddr + c0, v[0]);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[1][i] = 0.f;
+            }
+        } else {
+            tmem_load_16(taddr + c0, v[0]);
+        }
+        store_staged<SWIGLU>(v, stage, flip, [&](int token) -> __nv_bfloat16 * {
+            return c0 + token < n_valid ? dst + (size_t)(c0 + token) * stride : nullptr;
+        }, q, lane);
     }
 }
 
