@@ -27,7 +27,7 @@ namespace {
 using namespace tc;
 using namespace mxtc;
 
-constexpr int kPairThreads = 224;  // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA
+constexpr int kPairThreads = 256;  // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA, warp 7 tile decoder
 
 struct MxPairMaps {
     TensorMaps ops;            // weight codes, token codes (boxes of 8, 16, ..., 128 rows)
@@ -61,7 +61,8 @@ struct MxPairSmem {
     static constexpr int kBars = kStage + STAGE_BYTES;  // full[S], empty[S], acc_full[2], acc_empty[2]
     static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
-    static constexpr int kBytes = kAbort + 4;
+    static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
+    static constexpr int kBytes = kTiles + TileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
@@ -86,6 +87,9 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
+    const TileQueue tiles(base_ptr, base, L::kTiles);
+    auto decode = [&](int tile) { return decode_mx_tile(tile, p); };
+    auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + s * 8, 1);
@@ -95,6 +99,7 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
             mbar_init(bar_acc_full + a * 8, 1);
             mbar_init(bar_acc_empty + a * 8, 2 * kEpilogueWarps);
         }
+        tiles.init((rank == 0 ? 3 : 2) + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -130,7 +135,9 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const MxTile t = decode_mx_tile(tile, p);
+            MxTile t;
+            ok = tiles.take(t, round, lane, queue_wait);
+            if (!ok) break;
             const int n_mma = (t.n_valid + 15) & ~15, half = n_mma >> 1;
             const int cta_tile = 2 * t.f + (int)rank;  // this CTA's 128 weight rows
             const int w_sf_row = (t.e * w_tiles_per_expert + cta_tile) * p.n_k_blocks;
@@ -176,7 +183,7 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
     };
     if (warp == 0) {
         producer_loop(true, false);
-    } else if (warp == kPairThreads / 32 - 1) {
+    } else if (warp == 6) {
         producer_loop(false, true);
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader CTA only): one elected thread walks a whole tile's slots ----------------
@@ -188,7 +195,9 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
             for (int round = 0; ok; ++round) {
                 const int tile = tile_of_round(round, pair, n_pairs);
                 if (tile >= total_tiles) break;
-                const MxTile t = decode_mx_tile(tile, p);
+                MxTile t;
+                ok = tiles.take(t, round, lane, queue_wait);
+                if (!ok) break;
                 const int n_mma = (t.n_valid + 15) & ~15;
                 ok = __all_sync(0xffffffffu, pair_wait(bar_acc_empty + acc * 8, acc_phase ^ 1u, abort_flag, peer_abort,
                                                        p.status, kSiteMmaTmemEmpty + kSiteOffset));
@@ -231,7 +240,7 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
                 if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
         }
-    } else {
+    } else if (warp < 6) {
         // ---------------- epilogue (both CTAs): own 128 weight rows x all N tokens ----------------
         const int q = warp & 3;
         int acc = 0;
@@ -241,9 +250,10 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
         for (int round = 0;; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const MxTile t = decode_mx_tile(tile, p);
+            MxTile t;
+            const bool taken = tiles.take(t, round, lane, queue_wait);
             const int n_mma = (t.n_valid + 15) & ~15;
-            const bool ok = pair_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, peer_abort, p.status,
+            const bool ok = taken && pair_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, peer_abort, p.status,
                                       kSiteEpilogueTmemFull + kSiteOffset);
             if (epilogue_any(!ok)) break;  // the four warps synchronise inside the tile, so they leave together
             tcgen05_fence_after();
@@ -267,6 +277,9 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const Mx
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
+    } else if (warp == 7) {
+        // ---------------- decoder ----------------
+        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------

@@ -28,7 +28,7 @@ namespace {
 using namespace tc;
 using namespace mxtc;
 
-constexpr int kMxRingThreads = 224;  // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA
+constexpr int kMxRingThreads = 256;  // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA, warp 7 tile decoder
 constexpr int kChunkCols = 16;       // granularity of the accumulator ring: the MMA's N granularity
 constexpr int kAccCols = 496;        // accumulator columns; the scales take the last 16 of tensor memory
 constexpr int kNumChunks = kAccCols / kChunkCols;  // 31
@@ -71,7 +71,8 @@ struct MxRingSmem {
     static constexpr int kQueue = kBars + (2 * STAGES + kAccFullBars + 32) * 8;
     static constexpr int kTmemSlot = kQueue + kTileQueue * 4;
     static constexpr int kAbort = kTmemSlot + 4;
-    static constexpr int kBytes = kAbort + 4;
+    static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
+    static constexpr int kBytes = kTiles + TileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
@@ -116,6 +117,9 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
+    const TileQueue tiles(base_ptr, base, L::kTiles);
+    auto decode = [&](int tile) { return decode_mx_tile(tile, p); };
+    auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + s * 8, 1);
@@ -123,6 +127,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
         }
         for (int a = 0; a < kAccFullBars; ++a) mbar_init(bar_acc_full + a * 8, 1);
         for (int c = 0; c < kNumChunks; ++c) mbar_init(bar_acc_empty + c * 8, 2 * kEpilogueWarps);
+        tiles.init(2 + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -158,7 +163,9 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
         for (int round = 0; ok; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const MxTile t = decode_mx_tile(tile, p);
+            MxTile t;
+            ok = tiles.take(t, round, lane, queue_wait);
+            if (!ok) break;
             const int n_mma = (t.n_valid + 15) & ~15;
             const MxParts parts = split_mx_tile(seq, n_mma);
             const int cta_tile = 2 * t.f + (int)rank;  // this CTA's 128 weight rows
@@ -216,7 +223,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
     };
     if (warp == 0) {
         producer_loop(true, false);
-    } else if (warp == kMxRingThreads / 32 - 1) {
+    } else if (warp == 6) {
         producer_loop(false, true);
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader CTA only): one elected thread walks a whole tile's slots ----------------
@@ -290,7 +297,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
                 ok = __all_sync(0xffffffffu, mine);
             }
         }
-    } else {
+    } else if (warp < 6) {
         // ---------------- epilogue (both CTAs): own 128 weight rows x all N tokens ----------------
         const int q = warp & 3;  // a warp may only read TMEM lanes 32*(warp%4) .. +31
         const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
@@ -299,10 +306,11 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
         for (int round = 0;; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const MxTile t = decode_mx_tile(tile, p);
+            MxTile t;
+            const bool taken = tiles.take(t, round, lane, queue_wait);
             const int n_mma = (t.n_valid + 15) & ~15;
             const MxParts parts = split_mx_tile(seq, n_mma);
-            const bool ok = pair_wait(bar_acc_full + (seq & (kAccFullBars - 1)) * 8, (uint32_t)(seq / kAccFullBars) & 1u, abort_flag,
+            const bool ok = taken && pair_wait(bar_acc_full + (seq & (kAccFullBars - 1)) * 8, (uint32_t)(seq / kAccFullBars) & 1u, abort_flag,
                                       peer_abort, p.status, kSiteEpilogueTmemFull + kSiteOffset);
             if (epilogue_any(!ok)) break;  // the four warps synchronise inside the tile, so they leave together
             tcgen05_fence_after();
@@ -352,6 +360,9 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
             }
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator has been handed back)
         }
+    } else if (warp == 7) {
+        // ---------------- decoder ----------------
+        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------

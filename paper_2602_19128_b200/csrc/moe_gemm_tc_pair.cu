@@ -31,7 +31,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kPairThreads = 224;  // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA
+constexpr int kPairThreads = 256;  // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA, warp 7 tile decoder
 
 // D[tmem of both CTAs] (+)= A * B^T over the pair: M = 256 (128 rows per CTA), B halves from both CTAs.
 __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
@@ -53,7 +53,8 @@ struct PairSmem {
     static constexpr int kBars = kStage + STAGE_BYTES;        // full[S], empty[S], acc_full[2], acc_empty[2]
     static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
-    static constexpr int kBytes = kAbort + 4;
+    static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
+    static constexpr int kBytes = kTiles + TileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
@@ -84,6 +85,9 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
+    const TileQueue tiles(base_ptr, base, L::kTiles);
+    auto decode = [&](int tile) { return decode_tile(tile, p); };
+    auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + s * 8, 1);
@@ -93,6 +97,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             mbar_init(bar_acc_full + a * 8, 1);
             mbar_init(bar_acc_empty + a * 8, 2 * kEpilogueWarps);
         }
+        tiles.init((rank == 0 ? 3 : 2) + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -128,7 +133,9 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const Tile t = decode_tile(tile, p);
+            Tile t;
+            ok = tiles.take(t, round, lane, queue_wait);
+            if (!ok) break;
             const int n_mma = (t.n_valid + 15) & ~15, half = n_mma >> 1;  // each CTA stages half: a multiple of 8 rows
             const int feat0 = t.f * kFeatPerTile + (int)rank * kFeatPerCta;  // this CTA's part of slab 0
             if (load_act) {  // the token rows of a down GEMM are the gate/up GEMM's output for this expert
@@ -173,7 +180,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     };
     if (warp == 0) {
         producer_loop(true, false);
-    } else if (warp == kPairThreads / 32 - 1) {
+    } else if (warp == 6) {
         producer_loop(false, true);
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader CTA only): one elected thread walks a whole tile's slots ----------------
@@ -184,7 +191,9 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             for (int round = 0; ok; ++round) {
                 const int tile = tile_of_round(round, pair, n_pairs);
                 if (tile >= total_tiles) break;
-                const Tile t = decode_tile(tile, p);
+                Tile t;
+                ok = tiles.take(t, round, lane, queue_wait);
+                if (!ok) break;
                 const uint32_t idesc = instr_desc_bf16(2 * kTileM, (t.n_valid + 15) & ~15);
                 ok = __all_sync(0xffffffffu, pair_wait(bar_acc_empty + acc * 8, acc_phase ^ 1u, abort_flag, peer_abort,
                                                        p.status, kSiteMmaTmemEmpty + kSiteOffset));
@@ -225,7 +234,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
                 if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1u; }
             }
         }
-    } else {
+    } else if (warp < 6) {
         // ---------------- epilogue (both CTAs): own 128 weight rows per slab x all N tokens ----------------
         const int q = warp & 3;  // a warp may only read TMEM lanes 32*(warp%4) .. +31
         int acc = 0, flip = 0;
@@ -234,9 +243,10 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const Tile t = decode_tile(tile, p);
+            Tile t;
+            const bool taken = tiles.take(t, round, lane, queue_wait);
             const int n_mma = (t.n_valid + 15) & ~15;
-            ok = pair_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, peer_abort, p.status, kSiteEpilogueTmemFull + kSiteOffset);
+            ok = taken && pair_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, peer_abort, p.status, kSiteEpilogueTmemFull + kSiteOffset);
             if (STAGED ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
             tcgen05_fence_after();
 #pragma unroll
@@ -255,6 +265,9 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1u; }
         }
+    } else if (warp == 7) {
+        // ---------------- decoder ----------------
+        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------

@@ -36,7 +36,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kRingThreads = 224;   // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA
+constexpr int kRingThreads = 256;   // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA, warp 7 tile decoder
 constexpr int kChunkCols = 16;      // granularity of the accumulator ring: the MMA's N granularity
 constexpr int kNumChunks = 32;      // 512 columns of tensor memory
 constexpr int kAccFullBars = 32;    // tiles between the MMA warp and the epilogue: each holds at least one chunk
@@ -80,7 +80,8 @@ struct RingSmem {
     static constexpr int kQueue = kBars + (2 * STAGES + kAccFullBars + kNumChunks) * 8;
     static constexpr int kTmemSlot = kQueue + kTileQueue * 4;
     static constexpr int kAbort = kTmemSlot + 4;
-    static constexpr int kBytes = kAbort + 4;
+    static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
+    static constexpr int kBytes = kTiles + TileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
@@ -127,6 +128,9 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
+    const TileQueue tiles(base_ptr, base, L::kTiles);
+    auto decode = [&](int tile) { return decode_tile(tile, p); };
+    auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(bar_full + s * 8, 1);
@@ -134,6 +138,7 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
         }
         for (int a = 0; a < kAccFullBars; ++a) mbar_init(bar_acc_full + a * 8, 1);
         for (int c = 0; c < kNumChunks; ++c) mbar_init(bar_acc_empty + c * 8, 2 * kEpilogueWarps);
+        tiles.init(2 + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -167,7 +172,9 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
         for (int round = 0; ok; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const Tile t = decode_tile(tile, p);
+            Tile t;
+            ok = tiles.take(t, round, lane, queue_wait);
+            if (!ok) break;
             const int n_mma = (t.n_valid + 15) & ~15, half = n_mma >> 1;  // each CTA stages half: a multiple of 8 rows
             const int feat0 = t.f * kFeatPerTile + (int)rank * kFeatPerCta;
             if (load_act) {  // the token rows of a down GEMM are the gate/up GEMM's output for this expert
@@ -233,7 +240,7 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
     };
     if (warp == 0) {
         producer_loop(true, false);
-    } else if (warp == kRingThreads / 32 - 1) {
+    } else if (warp == 6) {
         producer_loop(false, true);
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader CTA only): the warp walks the ring, one elected lane issues ----------------
@@ -293,7 +300,7 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
                 ok = __all_sync(0xffffffffu, pair_wait(bar_acc_empty + lane * 8, ((chunk_phase >> lane) & 1u) ^ 1u, abort_flag,
                                                        peer_abort, p.status, kSiteMmaTmemEmpty + kSiteOffset));
         }
-    } else {
+    } else if (warp < 6) {
         // ---------------- epilogue (both CTAs): own 128 weight rows x all N tokens ----------------
         const int q = warp & 3;  // a warp may only read TMEM lanes 32*(warp%4) .. +31
         const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
@@ -302,10 +309,11 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
         for (int round = 0; ok; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
             if (tile >= total_tiles) break;
-            const Tile t = decode_tile(tile, p);
+            Tile t;
+            const bool taken = tiles.take(t, round, lane, queue_wait);
             const int n_mma = (t.n_valid + 15) & ~15, half_tile = n_mma >> 1;
             const Parts parts = split_tile(seq, n_mma);
-            ok = pair_wait(bar_acc_full + (seq & (kAccFullBars - 1)) * 8, (uint32_t)(seq / kAccFullBars) & 1u, abort_flag, peer_abort,
+            ok = taken && pair_wait(bar_acc_full + (seq & (kAccFullBars - 1)) * 8, (uint32_t)(seq / kAccFullBars) & 1u, abort_flag, peer_abort,
                            p.status, kSiteEpilogueTmemFull + kSiteOffset);
             if (epilogue_any(!ok)) break;  // the four warps synchronise inside the tile: they leave together
             tcgen05_fence_after();
@@ -356,6 +364,9 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
             }
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator has been handed back)
         }
+    } else if (warp == 7) {
+        // ---------------- decoder ----------------
+        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------

@@ -72,6 +72,21 @@ def test_few_down_tiles_split_along_k(T, H, I, E, k):
     assert torch.equal(out, again)
 
 
+@pytest.mark.parametrize("T,H,I,E,k,skew", [(64, 256, 2048, 64, 4, False),   # one CTA per tile, 32-row tiles, 14 tiles each
+                                            (150, 256, 2048, 32, 8, True),   # 64-row tiles, ragged
+                                            (300, 256, 2048, 16, 4, False),  # pairs, 128-row tiles
+                                            (900, 256, 2048, 8, 1, True),    # pairs, 256-row tiles
+                                            (400, 256, 2048, 8, 4, False)])  # wide tiles
+def test_many_short_tiles_per_cta(T, H, I, E, k, skew):
+    """Four slots of K per gate/up tile and many tiles per CTA: the queue of decoded tiles and the epilogue's buffers wrap."""
+    inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=1)
+    out, views, _ = run_forward(inp)
+    *_, h, y, ref = oracle_everything(to_host_case(inp))
+    assert_close_out(bf16_to_f64(views["h"]), h, "h")
+    assert_close_out(bf16_to_f64(views["y"]), y, "y")
+    assert_close_out(bf16_to_f64(out), ref, "out")
+
+
 @pytest.mark.parametrize("T,H,I,E,k,skew", [(520, 256, 256, 4, 2, False), (900, 256, 128, 8, 2, True),
                                             (1200, 512, 384, 8, 2, False), (700, 256, 256, 2, 1, False)])
 def test_gather_in_load_matches_oracle(T, H, I, E, k, skew):

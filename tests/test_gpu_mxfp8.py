@@ -185,6 +185,16 @@ def test_mxfp8_forward_matches_oracle(T, H, I, E, k, skew):
     assert_close_out(bf16_to_f64(out), ref, "mxfp8 out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k,skew", [(64, 256, 2048, 64, 4, False), (150, 256, 2048, 32, 8, True),   # one CTA per tile
+                                            (300, 256, 2048, 16, 4, False), (300, 256, 2048, 8, 4, False),  # pairs, 128 and 240 rows
+                                            (250, 256, 2048, 8, 4, False), (400, 256, 2048, 8, 4, False)])  # 160 rows, wide tiles
+def test_mxfp8_many_short_tiles_per_cta(T, H, I, E, k, skew):
+    """Two slots of K per gate/up tile and many tiles per CTA: the queue of decoded tiles and the epilogue's buffers wrap."""
+    inp = make_mxfp8_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=3, device="cuda")
+    out, _ = run_mx(inp)
+    assert_close_out(bf16_to_f64(out), oracle_mx(inp), "mxfp8 out")
+
+
 @pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
 def test_mxfp8_few_down_tiles_split_along_k(T, H, I, E, k):
     """Two CTAs per tile of the down GEMM, half of the K slots each (2176: 9 and 8 of them)."""
