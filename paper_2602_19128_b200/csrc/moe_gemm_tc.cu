@@ -21,13 +21,17 @@
 //  * Warp 0 issues TMA loads into a STAGES-deep ring; warp 1 issues the MMAs and commits ring
 //    slots back; warps 2..5 drain the accumulator (double-buffered in TMEM, so the epilogue of
 //    one tile overlaps the MMAs of the next).
-//  * A down GEMM with fewer tiles than half of the SMs (a token or two on a few experts) has two CTAs of a cluster on each
-//    tile, half of its K range each (SplitK, moe_tc_pair.cuh): an SM takes in about 100 GB/s, so 32 or 64 of them do not
-//    reach the memory's rate.  One Mixtral-shaped token 134 -> 126 us, with MX weights 83.7 -> 79.8, with FP8 weights
-//    97.6 -> 86.4.
+//  * A down GEMM with fewer tiles than half of the SMs (a token or two on a few experts) has two CTAs on each tile, 64 of its
+//    128 weight rows each (HALVES): an SM takes in about 100 GB/s, so 32 or 64 of them do not reach the memory's rate.  Every
+//    sum runs over K as it does with one CTA per tile, so the results are the same bit for bit.  The MMA has 64 rows (with
+//    128, half of them unused, its reads of shared memory took as long as the stream), token rows come in eights, and
+//    a slot holds four 64-wide K chunks, each operand one copy: with one chunk per slot the handling of a slot took as long
+//    as its 8 KiB.  One Mixtral-shaped token 134.1 -> 126.5 us (128 rows and one chunk 137.0, two chunks 131.6; 64 rows and
+//    two chunks 129.3, three 126.3), the same on one expert 90.8 -> 80.7, 16 tokens of 8 experts of 512 x 4096, top 2, 45.7 ->
+//    38.0, one token of 1024 x 2048 25.6 -> 23.1.
 //  * Every wait is bounded: if one expires the CTA records MOE_ERR_DEVICE_TIMEOUT and the site in
 //    the status word, every role stops, TMEM is released and the kernel returns.
-#include "moe_tc_pair.cuh"
+#include "moe_tc_common.cuh"
 
 namespace moe {
 namespace {
@@ -49,29 +53,36 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+constexpr int kHalfChunks = 4, kHalfStages = 4;  // HALVES: 64-wide K chunks per slot, slots
+
 // Tiles of more than 32 rows are stored through shared memory (Stage); a smaller tile is one or two groups of columns, whose
 // stores do not show.
-template <int NT_MAX, int STAGES, bool SPLIT>
+template <int NT_MAX, int STAGES, bool HALVES>
 struct SmemLayout {
     static constexpr bool kStaged = NT_MAX > 32;
-    static constexpr int kSlotBBytes = NT_MAX * kRowBytes;
+    static constexpr int kRows = HALVES ? kTileM / 2 : kTileM;    // weight rows of this CTA's part of a tile
+    static constexpr int kChunks = HALVES ? kHalfChunks : 1;  // 64-wide K chunks per slot: weights [chunk][rows], tokens [chunk][n_mma rows]
+    static constexpr int kSlotABytes = kChunks * kRows * kRowBytes;
+    static constexpr int kSlotBBytes = kChunks * NT_MAX * kRowBytes;
     static constexpr int kA = 0;
     static constexpr int kB = STAGES * kSlotABytes;
-    static constexpr int kSplit = kB + STAGES * kSlotBBytes;
-    // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], SplitK's full
-    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : kStaged ? kStageBytes : 0);
-    static constexpr int kTmemSlot = kBars + (2 * STAGES + 5) * 8;
+    static constexpr int kStage = kB + STAGES * kSlotBBytes;
+    // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2]
+    static constexpr int kBars = kStage + (kStaged ? kStageBytes : 0);
+    static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
     static constexpr int kBytes = kTiles + TileQueue::kBytes;
     static constexpr int kDynamicBytes = kBytes + 1024;  // slack to align the base to 1024 bytes
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT, bool QUEUED>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool HALVES, bool QUEUED>
 __global__ void __launch_bounds__(QUEUED ? kThreads + 32 : kThreads, 1)
 grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
-    using L = SmemLayout<NT_MAX, STAGES, SPLIT>;
-    static_assert(!(SPLIT && SWIGLU), "the gate/up epilogue pairs rows that a split would part");
+    using L = SmemLayout<NT_MAX, STAGES, HALVES>;
+    static_assert(!HALVES || (!SWIGLU && !L::kStaged), "the halves of a tile are stored row by row");
+    constexpr int kRows = L::kRows;
+    constexpr int kQuantum = HALVES ? 8 : 16;            // token rows come in multiples of it: the MMA's step in N for so many rows
     constexpr int kTmemCols = 2 * NT_MAX;
     static_assert(kTmemCols >= 32 && kTmemCols <= 512 && (kTmemCols & (kTmemCols - 1)) == 0,
                   "a tensor-memory allocation must be a power of two between 32 and 512 columns");
@@ -86,19 +97,8 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    SplitK<NT_MAX> split;
-    uint32_t peer_abort = 0;
-    if (SPLIT) {
-        split.rank = cluster_ctarank();
-        split.full = bar_acc_empty + 16;
-        split.buf = reinterpret_cast<float *>(base_ptr + L::kSplit);
-        split.peer_buf = map_to_cta(base + L::kSplit, split.rank ^ 1u);
-        split.peer_full = map_to_cta(split.full, split.rank ^ 1u);
-        peer_abort = map_to_cta(base + L::kAbort, split.rank ^ 1u);
-    }
     auto wait = [&](uint32_t bar, uint32_t parity, int site) {
-        return SPLIT ? pair_wait(bar, parity, abort_flag, peer_abort, p.status, site + kSiteOffset)
-                     : mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
+        return mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
     };
     const TileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_tile(tile, p); };
@@ -118,7 +118,6 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             mbar_init(bar_acc_full + a * 8, 1);
             mbar_init(bar_acc_empty + a * 8, kEpilogueWarps);
         }
-        if (SPLIT) mbar_init(split.full, kEpilogueWarps / 2);
         tiles.init(2 + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -136,17 +135,14 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     }
     tcgen05_fence_before();
     __syncthreads();
-    if (SPLIT) cluster_sync_all();  // the peer's barriers exist before anything can signal them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // everything above overlapped the previous kernel; its results are read from here on
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
-    const int worker = SPLIT ? blockIdx.x >> 1 : blockIdx.x, n_workers = SPLIT ? gridDim.x >> 1 : gridDim.x;
-    // this CTA's slots of a tile
-    const int first_half = (p.n_k_blocks + 1) >> 1;
-    const int k_first = SPLIT && split.rank ? first_half : 0;
-    const int n_slots = !SPLIT ? p.n_k_blocks : split.rank ? p.n_k_blocks - first_half : first_half;
+    const int worker = HALVES ? blockIdx.x >> 1 : blockIdx.x, n_workers = HALVES ? gridDim.x >> 1 : gridDim.x;
+    const int row_half = HALVES ? blockIdx.x & 1 : 0;  // which 64 of a tile's rows are this CTA's
+    const int n_slots = HALVES ? (p.n_k_blocks + L::kChunks - 1) / L::kChunks : p.n_k_blocks;
 
     if (warp == 0) {
         // ---------------- TMA producer: one elected thread issues a whole tile's copies ----------------
@@ -154,11 +150,11 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
         uint32_t phase = 0;
         bool ok = true, gate_up_done = false;
         auto load_weights = [&](const Tile &t, int w_row, int kb, int slot) {  // by one thread
-            const uint32_t sa = base + L::kA + slot * kSlotABytes, full = bar_full + slot * 8;
+            const uint32_t sa = base + L::kA + slot * L::kSlotABytes, full = bar_full + slot * 8;
             if (SWIGLU)  // 64 features = groups 4f..4f+3 of 16, gate and up rows interleaved per group
-                tma_load_5d(sa, &maps.w, (k_first + kb) * kBlockK, 0, 0, t.f * 4, t.e, full);
+                tma_load_5d(sa, &maps.w, kb * kBlockK, 0, 0, t.f * 4, t.e, full);
             else
-                tma_load_2d(sa, &maps.w, (k_first + kb) * kBlockK, w_row, full);
+                HALVES ? tma_load_3d(sa, &maps.w, 0, w_row, L::kChunks * kb, full) : tma_load_2d(sa, &maps.w, kb * kBlockK, w_row, full);
         };
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
@@ -166,9 +162,9 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
-            const int n_mma = (t.n_valid + 15) & ~15;
-            const int w_row = t.e * p.w_rows + t.f * kTileM;  // down projection: 128 rows of w2[e]
-            const uint32_t tx_bytes = kSlotABytes + n_mma * kRowBytes;
+            const int n_mma = (t.n_valid + kQuantum - 1) & -kQuantum;
+            const int w_row = t.e * p.w_rows + t.f * kTileM + row_half * kRows;  // down projection: 128 rows of w2[e], or 64
+            const uint32_t tx_bytes = L::kSlotABytes + L::kChunks * n_mma * kRowBytes;
             // The first tile's weights do not wait for its token rows: the ring's slots are filled with them beforehand (a
             // one-token Mixtral-shaped layer streams weights while the rows are scattered, and while the last gate/up tiles run).
             int filled = 0;
@@ -194,8 +190,10 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
                         mbar_expect_tx(bar_full + slot * 8, tx_bytes);
                         load_weights(t, w_row, kb, slot);
                     }
-                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), (k_first + kb) * kBlockK, t.row0,
-                                bar_full + slot * 8);
+                    if (HALVES)
+                        tma_load_3d(base + L::kB + slot * L::kSlotBBytes, act_map<kQuantum>(maps, n_mma), 0, t.row0, L::kChunks * kb, bar_full + slot * 8);
+                    else
+                        tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<kQuantum>(maps, n_mma), kb * kBlockK, t.row0, bar_full + slot * 8);
                     if (++slot == STAGES) { slot = 0; ph ^= 1u; }
                 }
             }
@@ -216,7 +214,8 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
-            const uint32_t idesc = instr_desc_bf16(kTileM, (t.n_valid + 15) & ~15);
+            const int n_mma = (t.n_valid + kQuantum - 1) & -kQuantum;
+            const uint32_t idesc = instr_desc_bf16(kRows, n_mma);
             ok = __all_sync(0xffffffffu, wait(bar_acc_empty + acc * 8, acc_phase ^ 1u, kSiteMmaTmemEmpty));
             if (!ok) break;
             tcgen05_fence_after();
@@ -228,11 +227,16 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
                     ok = wait(bar_full + s * 8, ph, kSiteMmaFull);
                     if (!ok) break;
                     tcgen05_fence_after();
-                    const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + s * kSlotABytes);
+                    const uint64_t a_desc = smem_desc_k_major_sw128(base + L::kA + s * L::kSlotABytes);
                     const uint64_t b_desc = smem_desc_k_major_sw128(base + L::kB + s * L::kSlotBBytes);
 #pragma unroll
-                    for (int kk = 0; kk < kBlockK / 16; ++kk)  // 16 K-elements = 32 bytes = 2 descriptor units
-                        umma_bf16(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, (kb | kk) != 0);
+                    for (int j = 0; j < L::kChunks; ++j) {
+                        if (j && L::kChunks * kb + j == p.n_k_blocks) break;  // (the last slot may have fewer)
+#pragma unroll
+                        for (int kk = 0; kk < kBlockK / 16; ++kk)  // 16 K-elements = 32 bytes = 2 descriptor units
+                            umma_bf16(d_tmem, a_desc + (uint32_t)(j * (kRows * kRowBytes >> 4)) + 2 * kk,
+                                      b_desc + (uint32_t)(j * (n_mma * kRowBytes >> 4)) + 2 * kk, idesc, (kb | j | kk) != 0);
+                    }
                     umma_commit(bar_empty + s * 8);
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
@@ -255,37 +259,23 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
             if (tile >= total_tiles) break;
             Tile t;
             const bool taken = next_tile(t, round, tile);
-            const int n_mma = (t.n_valid + 15) & ~15;
+            const int n_mma = (t.n_valid + kQuantum - 1) & -kQuantum;
             ok = taken && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
-            if (SPLIT && ok && split.receives(q)) {  // the peer's sums
-                ok = wait(split.full, 0, kSiteEpilogueTmemFull);
-                fence_cluster();
-            }
             if (L::kStaged ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
             tcgen05_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
-            __nv_bfloat16 *rows = p.out + (size_t)t.row0 * p.n_out + t.f * (SWIGLU ? kTileM / 2 : kTileM);  // this tile's features
-            __nv_bfloat16 *dst = rows + (SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane);
+            __nv_bfloat16 *rows = p.out + (size_t)t.row0 * p.n_out + t.f * (SWIGLU ? kTileM / 2 : kTileM) + row_half * kRows;  // this CTA's features
             if constexpr (L::kStaged) {
-                drain_staged<SWIGLU>(taddr, n_mma, t.n_valid, rows, (size_t)p.n_out, base_ptr + L::kSplit, flip, q, lane);
-            } else if constexpr (SPLIT) {
-                for (int c0 = 0; c0 < n_mma; c0 += 16) {
-                    float v[16];
-                    tmem_load_16(taddr + c0, v);
-                    if (!split.receives(q)) {
-                        split.send_16(q, c0, lane, v);
-                    } else {
-                        split.add_16(q, c0, lane, v);
-                        store_column(v, t.n_valid - c0, dst + (size_t)c0 * p.n_out, (size_t)p.n_out);
-                    }
-                }
+                drain_staged<SWIGLU>(taddr, n_mma, t.n_valid, rows, (size_t)p.n_out, base_ptr + L::kStage, flip, q, lane);
             } else {
-                drain_accumulator<SWIGLU>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
+                // (the accumulator of an MMA of 64 rows: row 16 q + j in lane 32 q + j, the other lanes unused)
+                constexpr int kWarpRows = kRows / 4;
+                drain_accumulator<SWIGLU>(taddr, n_mma, lane < kWarpRows ? t.n_valid : 0,
+                                          rows + (SWIGLU ? q * 16 + (lane & 15) : q * kWarpRows + lane % kWarpRows), (size_t)p.n_out, lane);
             }
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty + acc * 8);
-            if (SPLIT && lane == 0 && !split.receives(q)) mbar_arrive_cluster(split.peer_full);
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -298,7 +288,6 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     gemm_chain_finish(p.handover_role);
     tcgen05_fence_before();
     __syncthreads();
-    if (SPLIT) cluster_sync_all();  // (the peer may still write here, or signal)
     if (*abort_flag) {
         // give copies that may still be in flight time to land before the CTA's memory is released
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
@@ -309,14 +298,14 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     }
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT = false, bool QUEUED = false>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool HALVES = false, bool QUEUED = false>
 int launch_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
-    using L = SmemLayout<NT_MAX, STAGES, SPLIT>;
+    using L = SmemLayout<NT_MAX, STAGES, HALVES>;
     static_assert(L::kDynamicBytes <= 232448, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_kernel<NT_MAX, STAGES, SWIGLU, SPLIT, QUEUED>;
+    auto kernel = grouped_gemm_tc_kernel<NT_MAX, STAGES, SWIGLU, HALVES, QUEUED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_clusters(kernel, true, SPLIT ? 2 : 1, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
@@ -354,10 +343,21 @@ int launch_grouped_gemm_tc(const GroupedGemmArgs &a, cudaStream_t stream) {
     const int features_per_tile = a.swiglu ? kTileM / 2 : kTileM;
     if (a.n_out % features_per_tile != 0) return MOE_ERR_UNSUPPORTED;
 
+    // The tile count is only known on the device; this is its upper bound.
+    const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
+    const long long max_tiles = max_token_tiles * (a.n_out / features_per_tile);
+    const int sms = sm_count();
+    // Two CTAs per tile (HALVES): a down GEMM of small token tiles that leaves half of the SMs or more without a tile, with K long
+    // enough that a tile's stream of weights is what takes the time.  One CTA per tile / two: 1 token of 16 experts of 2048 x 2112,
+    // top 2, 29.8 / 26.9 us; of 8 of 7168 x 2048, top 1, 42.0 / 42.1; of 8 of 4096 x 1536, top 2, 33.9 / 35.1; 16 tokens of 8 of
+    // 1024 x 512, top 2, 22.4 / 23.6.
+    const bool halves = !a.swiglu && a.nt_max == 32 && 2 * max_tiles <= sms && a.K >= 2048;
+
     TensorMaps maps;
-    const bool ok_w = a.swiglu ? encode_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
+    const bool ok_w = halves ? encode_map_chunks(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K, kTileM / 2, kHalfChunks)
+                    : a.swiglu ? encode_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
                                : encode_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_act_maps(maps.act, a.act, a.A, a.K, 16)) return MOE_ERR_CUDA;
+    if (!ok_w || !(halves ? encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 8, kHalfChunks) : encode_act_maps(maps.act, a.act, a.A, a.K, 16))) return MOE_ERR_CUDA;
 
     KernelParams p;
     p.out = a.out;
@@ -376,12 +376,8 @@ int launch_grouped_gemm_tc(const GroupedGemmArgs &a, cudaStream_t stream) {
     p.handover_per_token_tile = a.handover_per_token_tile;
     p.n_feature_tiles = a.n_out / features_per_tile;
 
-    // The tile count is only known on the device; this is its upper bound.
-    const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
-    const long long max_tiles = max_token_tiles * p.n_feature_tiles;
-    const int sms = sm_count();
-    if (split_k_applies(a.swiglu, a.nt_max, max_tiles, p.n_k_blocks, kBlockK))
-        return launch_instance<32, 10, false, true>(maps, p, 2 * (int)max_tiles, stream);
+    if (halves)
+        return launch_instance<32, kHalfStages, false, true>(maps, p, 2 * (int)max_tiles, stream);
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
     // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots do not hide the walk:
     // 16 tokens of 32 bf16 experts of 1024 x 1024, top 4, 50.7 -> 48.9 us; with longer K or one tile per CTA the queue costs

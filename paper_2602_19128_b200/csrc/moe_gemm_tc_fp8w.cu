@@ -28,7 +28,6 @@
 // rounded to bf16 once per slot and the product once per weight: at most 2^-8 relative on a weight, an
 // order of magnitude inside the layer's tolerance.  Scales must stay below 2^7 for scale * 2^120 to be finite.
 #include "moe_fp8w_tc.cuh"
-#include "moe_tc_pair.cuh"
 
 namespace moe {
 namespace {
@@ -50,7 +49,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-template <int NT_MAX, int STAGES_Q, bool SPLIT>
+template <int NT_MAX, int STAGES_Q>
 struct Fp8Smem {
     static constexpr bool kStaged = NT_MAX > 32 && NT_MAX < 192;     // through shared memory (Stage), where there is room
     // converted slots in tensor memory (beside two accumulators), token tiles in shared memory, and converter groups
@@ -59,20 +58,19 @@ struct Fp8Smem {
     static constexpr int kSlotBBytes = 2 * NT_MAX * kRowBytes;       // two swizzled token tiles (K 0..63 | 64..127)
     static constexpr int kB = 0;                                     // kConv token-tile pairs
     static constexpr int kQ = kB + kConv * kSlotBBytes;           // STAGES_Q code tiles
-    static constexpr int kSplit = kQ + STAGES_Q * kSlotQBytes;
-    // q_full[SQ], q_empty[SQ], op_full[C], op_empty[C], acc_full[2], acc_empty[2], SplitK's full
-    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : kStaged ? kStageBytes : 0);
-    static constexpr int kTmemSlot = kBars + (2 * STAGES_Q + 2 * kConv + 5) * 8;
+    static constexpr int kStage = kQ + STAGES_Q * kSlotQBytes;
+    // q_full[SQ], q_empty[SQ], op_full[C], op_empty[C], acc_full[2], acc_empty[2]
+    static constexpr int kBars = kStage + (kStaged ? kStageBytes : 0);
+    static constexpr int kTmemSlot = kBars + (2 * STAGES_Q + 2 * kConv + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kBytes = kAbort + 4;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
 
-template <int NT_MAX, int STAGES_Q, bool SWIGLU, bool SPLIT>
-__global__ void __launch_bounds__((Fp8Smem<NT_MAX, STAGES_Q, SPLIT>::kThreads), 1)
+template <int NT_MAX, int STAGES_Q, bool SWIGLU>
+__global__ void __launch_bounds__((Fp8Smem<NT_MAX, STAGES_Q>::kThreads), 1)
 grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
-    using L = Fp8Smem<NT_MAX, STAGES_Q, SPLIT>;
-    static_assert(!(SPLIT && SWIGLU), "the gate/up epilogue pairs rows that a split would part");
+    using L = Fp8Smem<NT_MAX, STAGES_Q>;
     constexpr int kConv = L::kConv;
     constexpr int kColsUsed = 2 * NT_MAX + kConv * kConvCols;
     constexpr int kTmemCols = kColsUsed <= 256 ? 256 : 512;  // (a power of two)
@@ -89,19 +87,8 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    SplitK<NT_MAX> split;
-    uint32_t peer_abort = 0;
-    if (SPLIT) {
-        split.rank = cluster_ctarank();
-        split.full = bar_acc_empty + 16;
-        split.buf = reinterpret_cast<float *>(base_ptr + L::kSplit);
-        split.peer_buf = map_to_cta(base + L::kSplit, split.rank ^ 1u);
-        split.peer_full = map_to_cta(split.full, split.rank ^ 1u);
-        peer_abort = map_to_cta(base + L::kAbort, split.rank ^ 1u);
-    }
     auto wait = [&](uint32_t bar, uint32_t parity, int site) {
-        return SPLIT ? pair_wait(bar, parity, abort_flag, peer_abort, p.status, site + kSiteOffset)
-                     : mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
+        return mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
     };
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES_Q; ++s) {
@@ -116,7 +103,6 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             mbar_init(bar_acc_full + a * 8, 1);
             mbar_init(bar_acc_empty + a * 8, kEpilogueWarps);
         }
-        if (SPLIT) mbar_init(split.full, kEpilogueWarps / 2);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -133,17 +119,12 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     }
     tcgen05_fence_before();
     __syncthreads();
-    if (SPLIT) cluster_sync_all();  // the peer's barriers exist before anything can signal them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // everything above overlapped the previous kernel; its results are read from here on
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
-    const int worker = SPLIT ? blockIdx.x >> 1 : blockIdx.x, n_workers = SPLIT ? gridDim.x >> 1 : gridDim.x;
-    // this CTA's slots of a tile
-    const int first_half = (p.n_k_blocks + 1) >> 1;
-    const int k_first = SPLIT && split.rank ? first_half : 0;
-    const int n_slots = !SPLIT ? p.n_k_blocks : split.rank ? p.n_k_blocks - first_half : first_half;
+    const int worker = blockIdx.x, n_workers = gridDim.x;
 
     if (warp == 0) {
         // ---------------- weight TMA ----------------
@@ -155,14 +136,14 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p);
             const int w_row = t.e * p.w_rows + t.f * kTileM;
-            for (int kb = 0; kb < n_slots; ++kb) {
+            for (int kb = 0; kb < p.n_k_blocks; ++kb) {
                 ok = __all_sync(0xffffffffu, wait(bar_q_empty + stage * 8, phase ^ 1u, kSiteProducerEmpty));
                 if (!ok) break;
                 if (elect_one()) {
                     const uint32_t full = bar_q_full + stage * 8;
                     mbar_expect_tx(full, kSlotQBytes);
                     const uint32_t sq = base + L::kQ + stage * kSlotQBytes;
-                    const int k0 = (k_first + kb) * kSlotK;
+                    const int k0 = kb * kSlotK;
                     if (SWIGLU)
                         tma_load_5d(sq, &maps.w, k0, 0, 0, t.f * 4, t.e, full);
                     else
@@ -185,14 +166,14 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             ok = handover_wait_expert(p.handover_role, p.handover, t.e, t.n_tok_tiles, p.handover_per_token_tile,
                                       p.tile_prefix[p.E], gate_up_done, abort_flag, p.status, lane);
             if (!ok) break;
-            for (int kb = 0; kb < n_slots; ++kb) {
+            for (int kb = 0; kb < p.n_k_blocks; ++kb) {
                 ok = __all_sync(0xffffffffu, wait(bar_op_empty + stage * 8, phase ^ 1u, kSiteProducerEmpty));
                 if (!ok) break;
                 if (elect_one()) {
                     const uint32_t full = bar_op_full + stage * 8;
                     mbar_expect_tx(full, 2 * n_mma * kRowBytes);
                     // one copy: rows x (two 64-wide K chunks), each chunk landing as its own swizzled tile of n_mma rows
-                    tma_load_3d(base + L::kB + stage * L::kSlotBBytes, act_map<16>(maps, n_mma), 0, t.row0, 2 * (k_first + kb), full);
+                    tma_load_3d(base + L::kB + stage * L::kSlotBBytes, act_map<16>(maps, n_mma), 0, t.row0, 2 * kb, full);
                 }
                 __syncwarp();
                 if (++stage == kConv) { stage = 0; phase ^= 1u; }
@@ -219,7 +200,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             if (elect_one()) {
                 int o = op;
                 uint32_t ph = op_phase;
-                for (int kb = 0; kb < n_slots; ++kb) {
+                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
                     ok = wait(bar_op_full + o * 8, ph, kSiteMmaFull);
                     if (!ok) break;
                     tcgen05_fence_after();
@@ -238,7 +219,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            ring_advance<kConv>(op, op_phase, n_slots);
+            ring_advance<kConv>(op, op_phase, p.n_k_blocks);
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -267,13 +248,13 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             // tile's single block (down)
             const int row_blocks = p.w_rows >> 7;
             const int block = !SWIGLU ? t.f : ((row & 16) ? (p.n_out + t.f * 64) >> 7 : (t.f * 64) >> 7);
-            const float *scale = p.w_scale + ((size_t)t.e * row_blocks + block) * p.n_k_blocks + k_first;
+            const float *scale = p.w_scale + ((size_t)t.e * row_blocks + block) * p.n_k_blocks;
             int kb = (group - turn + kConv) % kConv;  // first slot of this tile that is this group's
-            turn = (turn + n_slots) % kConv;
-            float next = kb < n_slots ? __ldg(scale + kb) : 0.f;
-            for (; kb < n_slots; kb += kConv) {
+            turn = (turn + p.n_k_blocks) % kConv;
+            float next = kb < p.n_k_blocks ? __ldg(scale + kb) : 0.f;
+            for (; kb < p.n_k_blocks; kb += kConv) {
                 const __nv_bfloat162 s2 = __float2bfloat162_rn(next * 1329227995784915872903807060280344576.0f);  // 2^120
-                if (kb + kConv < n_slots) next = __ldg(scale + kb + kConv);  // off the critical path
+                if (kb + kConv < p.n_k_blocks) next = __ldg(scale + kb + kConv);  // off the critical path
                 ok = __all_sync(0xffffffffu, wait(bar_q_full + stage * 8, phase, kSiteMmaFull));
                 if (!ok) break;
                 const uint8_t *src = my_row + stage * kSlotQBytes;
@@ -327,35 +308,19 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
             const Tile t = decode_tile(tile, p);
             const int n_mma = (t.n_valid + 15) & ~15;
             ok = wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
-            if (SPLIT && ok && split.receives(q)) {  // the peer's sums
-                ok = wait(split.full, 0, kSiteEpilogueTmemFull);
-                fence_cluster();
-            }
             if (L::kStaged ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
             tcgen05_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
             __nv_bfloat16 *rows = p.out + (size_t)t.row0 * p.n_out + t.f * (SWIGLU ? kTileM / 2 : kTileM);  // this tile's features
             __nv_bfloat16 *dst = rows + (SWIGLU ? q * 16 + (lane & 15) : q * 32 + lane);
             if constexpr (L::kStaged) {
-                drain_staged<SWIGLU>(taddr, n_mma, t.n_valid, rows, (size_t)p.n_out, base_ptr + L::kSplit, flip, q, lane);
-            } else if constexpr (SPLIT) {
-                for (int c0 = 0; c0 < n_mma; c0 += 16) {
-                    float v[16];
-                    tmem_load_16(taddr + c0, v);
-                    if (!split.receives(q)) {
-                        split.send_16(q, c0, lane, v);
-                    } else {
-                        split.add_16(q, c0, lane, v);
-                        store_column(v, t.n_valid - c0, dst + (size_t)c0 * p.n_out, (size_t)p.n_out);
-                    }
-                }
+                drain_staged<SWIGLU>(taddr, n_mma, t.n_valid, rows, (size_t)p.n_out, base_ptr + L::kStage, flip, q, lane);
             } else {
                 drain_accumulator<SWIGLU>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
             }
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty + acc * 8);
-            if (SPLIT && lane == 0 && !split.receives(q)) mbar_arrive_cluster(split.peer_full);
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -365,7 +330,6 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     gemm_chain_finish(p.handover_role);
     tcgen05_fence_before();
     __syncthreads();
-    if (SPLIT) cluster_sync_all();  // (the peer may still write here, or signal)
     if (*abort_flag) {
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     }
@@ -375,14 +339,14 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     }
 }
 
-template <int NT_MAX, int STAGES_Q, bool SWIGLU, bool SPLIT = false>
+template <int NT_MAX, int STAGES_Q, bool SWIGLU>
 int launch_fp8_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
-    using L = Fp8Smem<NT_MAX, STAGES_Q, SPLIT>;
+    using L = Fp8Smem<NT_MAX, STAGES_Q>;
     static_assert(L::kDynamicBytes <= 232448, "rings do not fit in shared memory");
-    auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES_Q, SWIGLU, SPLIT>;
+    auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES_Q, SWIGLU>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_clusters(kernel, true, SPLIT ? 2 : 1, grid, L::kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+    return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
@@ -404,10 +368,15 @@ int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &a, cudaStream_t stream) {
     const int features_per_tile = a.swiglu ? kTileM / 2 : kTileM;
     if (a.n_out % 128 != 0) return MOE_ERR_UNSUPPORTED;  // gate and up halves must both start on a scale block
 
+    // The tile count is only known on the device; this is its upper bound.
+    const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
+    const long long max_tiles = max_token_tiles * (a.n_out / features_per_tile);
+    const int sms = sm_count();
+
     TensorMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
                                : encode_mx_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_act_maps_k128(maps.act, a.act, a.A, a.K, 16)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 16, 2)) return MOE_ERR_CUDA;
 
     KernelParams p;
     p.out = a.out;
@@ -426,11 +395,6 @@ int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &a, cudaStream_t stream) {
     p.handover = a.handover;
     p.handover_per_token_tile = a.handover_per_token_tile;
 
-    const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
-    const long long max_tiles = max_token_tiles * p.n_feature_tiles;
-    const int sms = sm_count();
-    if (split_k_applies(a.swiglu, a.nt_max, max_tiles, p.n_k_blocks, kSlotK))  // (moe_gemm_tc.cu; eight slots and the buffer)
-        return launch_fp8_instance<32, 8, false, true>(maps, p, 2 * (int)max_tiles, stream);
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
     return a.swiglu ? dispatch_fp8<true>(a.nt_max, maps, p, grid, stream) : dispatch_fp8<false>(a.nt_max, maps, p, grid, stream);
 }

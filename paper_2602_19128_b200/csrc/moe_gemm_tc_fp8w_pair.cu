@@ -459,7 +459,7 @@ int launch_grouped_gemm_tc_fp8w_pair(const GroupedGemmArgs &a, cudaStream_t stre
     TensorMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
                                : encode_mx_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_act_maps_k128(maps.act, a.act, a.A, a.K, 8)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 8, 2)) return MOE_ERR_CUDA;
 
     KernelParams p;
     p.out = a.out;

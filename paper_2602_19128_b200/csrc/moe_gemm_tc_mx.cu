@@ -23,7 +23,6 @@
 //    exchange with the neighbouring warp through shared memory, then each lane scales and encodes its
 //    values and the scale byte goes straight into the atom layout the down GEMM loads.
 #include "moe_mx_tc.cuh"
-#include "moe_tc_pair.cuh"
 
 namespace moe {
 namespace {
@@ -54,7 +53,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-template <int NT_MAX, int STAGES, bool SPLIT>
+template <int NT_MAX, int STAGES>
 struct MxSmem {
     static constexpr bool kStaged = NT_MAX > 32;  // stored through shared memory (as in moe_gemm_tc.cu)
     static constexpr int kSlotBBytes = NT_MAX * kMxSlotK;
@@ -63,21 +62,20 @@ struct MxSmem {
     static constexpr int kSfA = kB + STAGES * kSlotBBytes;
     static constexpr int kSfB = kSfA + STAGES * kMxSfAtomBytes;
     static constexpr int kAmax = kSfB + STAGES * kMxSfBBytes;     // [2 buffers][4 warps][32 tokens] magnitudes
-    static constexpr int kSplit = kAmax + kAmaxBytes;
-    // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], SplitK's full
-    static constexpr int kBars = kSplit + (SPLIT ? SplitK<NT_MAX>::kFloats * 4 : kStaged ? kStageBytes : 0);
-    static constexpr int kTmemSlot = kBars + (2 * STAGES + 5) * 8;
+    static constexpr int kStage = kAmax + kAmaxBytes;
+    // full[STAGES], empty[STAGES], acc_full[2], acc_empty[2]
+    static constexpr int kBars = kStage + (kStaged ? kStageBytes : 0);
+    static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
     static constexpr int kBytes = kTiles + TileQueue::kBytes;
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT, bool QUEUED>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool QUEUED>
 __global__ void __launch_bounds__(QUEUED ? kThreads + 32 : kThreads, 1)
 grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParams p) {
-    using L = MxSmem<NT_MAX, STAGES, SPLIT>;
-    static_assert(!(SPLIT && SWIGLU), "the gate/up epilogue pairs rows that a split would part");
+    using L = MxSmem<NT_MAX, STAGES>;
     static_assert(2 * NT_MAX + 32 <= kTmemColsMx, "accumulators and scale columns exceed tensor memory");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
     constexpr uint32_t kSfACol = 2 * NT_MAX, kSfBCol = 2 * NT_MAX + 16;
@@ -91,19 +89,8 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    SplitK<NT_MAX> split;
-    uint32_t peer_abort = 0;
-    if (SPLIT) {
-        split.rank = cluster_ctarank();
-        split.full = bar_acc_empty + 16;
-        split.buf = reinterpret_cast<float *>(base_ptr + L::kSplit);
-        split.peer_buf = map_to_cta(base + L::kSplit, split.rank ^ 1u);
-        split.peer_full = map_to_cta(split.full, split.rank ^ 1u);
-        peer_abort = map_to_cta(base + L::kAbort, split.rank ^ 1u);
-    }
     auto wait = [&](uint32_t bar, uint32_t parity, int site) {
-        return SPLIT ? pair_wait(bar, parity, abort_flag, peer_abort, p.status, site + kSiteOffset)
-                     : mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
+        return mbar_wait(bar, parity, abort_flag, p.status, site + kSiteOffset);
     };
     const TileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_mx_tile(tile, p); };
@@ -123,7 +110,6 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             mbar_init(bar_acc_full + a * 8, 1);
             mbar_init(bar_acc_empty + a * 8, kEpilogueWarps);
         }
-        if (SPLIT) mbar_init(split.full, kEpilogueWarps / 2);
         tiles.init(2 + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -141,17 +127,12 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     }
     tcgen05_fence_before();
     __syncthreads();
-    if (SPLIT) cluster_sync_all();  // the peer's barriers exist before anything can signal them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     // everything above overlapped the previous kernel; its results are read from here on
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
-    const int worker = SPLIT ? blockIdx.x >> 1 : blockIdx.x, n_workers = SPLIT ? gridDim.x >> 1 : gridDim.x;
-    // this CTA's slots of a tile
-    const int first_half = (p.n_k_blocks + 1) >> 1;
-    const int k_first = SPLIT && split.rank ? first_half : 0;
-    const int n_slots = !SPLIT ? p.n_k_blocks : split.rank ? p.n_k_blocks - first_half : first_half;
+    const int worker = blockIdx.x, n_workers = gridDim.x;
 
     if (warp == 0) {
         // ---------------- producer: codes by TMA, scale atoms by bulk copies ----------------
@@ -161,10 +142,10 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
         auto load_weights = [&](const MxTile &t, int w_row, const uint8_t *w_sf, int kb, int slot) {  // by one thread
             const uint32_t sa = base + L::kA + slot * kMxSlotABytes, full = bar_full + slot * 8;
             if (SWIGLU)
-                tma_load_5d(sa, &maps.w, (k_first + kb) * kMxSlotK, 0, 0, t.f * 4, t.e, full);
+                tma_load_5d(sa, &maps.w, kb * kMxSlotK, 0, 0, t.f * 4, t.e, full);
             else
-                tma_load_2d(sa, &maps.w, (k_first + kb) * kMxSlotK, w_row, full);
-            bulk_load(base + L::kSfA + slot * kMxSfAtomBytes, w_sf + (size_t)(k_first + kb) * kMxSfAtomBytes, kMxSfAtomBytes, full);
+                tma_load_2d(sa, &maps.w, kb * kMxSlotK, w_row, full);
+            bulk_load(base + L::kSfA + slot * kMxSfAtomBytes, w_sf + (size_t)kb * kMxSfAtomBytes, kMxSfAtomBytes, full);
         };
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
@@ -179,7 +160,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             const uint8_t *a_sf = p.act_sf + (size_t)t.atom * kMxSfAtomBytes;
             int filled = 0;  // the first tile's weights do not wait for its token rows (moe_gemm_tc.cu)
             if (round == 0 && p.handover_role != 0) {
-                filled = n_slots < STAGES ? n_slots : STAGES;
+                filled = p.n_k_blocks < STAGES ? p.n_k_blocks : STAGES;
                 if (elect_one())
                     for (int kb = 0; kb < filled; ++kb) {
                         mbar_expect_tx(bar_full + kb * 8, tx_bytes);
@@ -193,7 +174,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             if (elect_one()) {
                 int slot = stage;
                 uint32_t ph = phase;
-                for (int kb = 0; kb < n_slots; ++kb) {
+                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
                     const uint32_t full = bar_full + slot * 8;
                     if (kb >= filled) {
                         ok = wait(bar_empty + slot * 8, ph ^ 1u, kSiteProducerEmpty);
@@ -201,15 +182,15 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
                         mbar_expect_tx(full, tx_bytes);
                         load_weights(t, w_row, w_sf, kb, slot);
                     }
-                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), (k_first + kb) * kMxSlotK, t.row0, full);
-                    bulk_load(base + L::kSfB + slot * kMxSfBBytes, a_sf + (size_t)(k_first + kb) * p.n_atoms * kMxSfAtomBytes,
+                    tma_load_2d(base + L::kB + slot * L::kSlotBBytes, act_map<16>(maps, n_mma), kb * kMxSlotK, t.row0, full);
+                    bulk_load(base + L::kSfB + slot * kMxSfBBytes, a_sf + (size_t)kb * p.n_atoms * kMxSfAtomBytes,
                               kMxSfBBytes, full);
                     if (++slot == STAGES) { slot = 0; ph ^= 1u; }
                 }
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            ring_advance<STAGES>(stage, phase, n_slots);
+            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: one elected thread walks a whole tile's slots ----------------
@@ -231,7 +212,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             if (elect_one()) {
                 int s = stage;
                 uint32_t ph = phase;
-                for (int kb = 0; kb < n_slots; ++kb) {
+                for (int kb = 0; kb < p.n_k_blocks; ++kb) {
                     ok = wait(bar_full + s * 8, ph, kSiteMmaFull);
                     if (!ok) break;
                     tcgen05_fence_after();
@@ -250,7 +231,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             }
             __syncwarp();
             ok = __all_sync(0xffffffffu, ok);
-            ring_advance<STAGES>(stage, phase, n_slots);
+            ring_advance<STAGES>(stage, phase, p.n_k_blocks);
             if (!ok) break;
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -268,13 +249,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             const bool taken = next_tile(t, round, tile);
             const int n_mma = (t.n_valid + 15) & ~15;
             bool ok = taken && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
-            if (SPLIT && ok && split.receives(q)) {  // the peer's sums
-                ok = wait(split.full, 0, kSiteEpilogueTmemFull);
-                fence_cluster();
-            }
-            // The four warps synchronise inside the tile (SwiGLU), so they must agree on leaving.  With a split they must not wait
-            // for one another here: two of them wait for the peer's other two.
-            if (SPLIT ? !__all_sync(0xffffffffu, ok) : epilogue_any(!ok)) break;
+            if (epilogue_any(!ok)) break;  // the four warps synchronise inside the tile (SwiGLU): they leave together
             tcgen05_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX;
             if (SWIGLU) {
@@ -282,22 +257,11 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
                 // scale bytes of h: features 64f + 16q.. lie in block 2f + q/2 = K-slot block/4 of the down GEMM
                 const int block = 2 * t.f + (q >> 1);
                 uint8_t *sf_dst = p.out_sf + ((size_t)(block >> 2) * p.n_atoms + t.atom) * kMxSfAtomBytes + (block & 3);
-                drain_swiglu_mx<L::kStaged>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, sf_dst, amax_s, buf, base_ptr + L::kSplit, q, lane);
+                drain_swiglu_mx<L::kStaged>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, sf_dst, amax_s, buf, base_ptr + L::kStage, q, lane);
             } else {
                 __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.out) + (size_t)t.row0 * p.n_out + t.f * kTileM + q * 32 + lane;
                 if constexpr (L::kStaged) {
-                    drain_staged<false>(taddr, n_mma, t.n_valid, dst - (q * 32 + lane), (size_t)p.n_out, base_ptr + L::kSplit, buf, q, lane);
-                } else if constexpr (SPLIT) {
-                    for (int c0 = 0; c0 < n_mma; c0 += 16) {
-                        float v[16];
-                        tmem_load_16(taddr + c0, v);
-                        if (!split.receives(q)) {
-                            split.send_16(q, c0, lane, v);
-                        } else {
-                            split.add_16(q, c0, lane, v);
-                            store_column(v, t.n_valid - c0, dst + (size_t)c0 * p.n_out, (size_t)p.n_out);
-                        }
-                    }
+                    drain_staged<false>(taddr, n_mma, t.n_valid, dst - (q * 32 + lane), (size_t)p.n_out, base_ptr + L::kStage, buf, q, lane);
                 } else {
                     drain_accumulator<false>(taddr, n_mma, t.n_valid, dst, (size_t)p.n_out, lane);
                 }
@@ -305,7 +269,6 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_acc_empty + acc * 8);
-            if (SPLIT && lane == 0 && !split.receives(q)) mbar_arrive_cluster(split.peer_full);
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -318,7 +281,6 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     gemm_chain_finish(p.handover_role);
     tcgen05_fence_before();
     __syncthreads();
-    if (SPLIT) cluster_sync_all();  // (the peer may still write here, or signal)
     if (*abort_flag) {
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     }
@@ -328,23 +290,23 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     }
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool SPLIT = false, bool QUEUED = false>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool QUEUED>
 int launch_instance(const TensorMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
-    using L = MxSmem<NT_MAX, STAGES, SPLIT>;
+    using L = MxSmem<NT_MAX, STAGES>;
     static_assert(L::kDynamicBytes <= 232448, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_mx_kernel<NT_MAX, STAGES, SWIGLU, SPLIT, QUEUED>;
+    auto kernel = grouped_gemm_tc_mx_kernel<NT_MAX, STAGES, SWIGLU, QUEUED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_clusters(kernel, true, SPLIT ? 2 : 1, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
 template <bool SWIGLU, bool QUEUED>
 int dispatch(int nt_max, const TensorMaps &maps, const MxParams &p, int grid, cudaStream_t s) {
     switch (nt_max) {
-        case 32: return launch_instance<32, 10, SWIGLU, false, QUEUED>(maps, p, grid, s);
-        case 64: return launch_instance<64, 8, SWIGLU, false, QUEUED>(maps, p, grid, s);
-        case 128: return launch_instance<128, 6, SWIGLU, false, QUEUED>(maps, p, grid, s);
+        case 32: return launch_instance<32, 10, SWIGLU, QUEUED>(maps, p, grid, s);
+        case 64: return launch_instance<64, 8, SWIGLU, QUEUED>(maps, p, grid, s);
+        case 128: return launch_instance<128, 6, SWIGLU, QUEUED>(maps, p, grid, s);
         default: return MOE_ERR_UNSUPPORTED;
     }
 }
@@ -356,6 +318,11 @@ int launch_grouped_gemm_tc_mx(const MxGemmArgs &a, cudaStream_t stream) {
     const int features_per_tile = a.swiglu ? kTileM / 2 : kTileM;
     if (a.n_out % features_per_tile != 0) return MOE_ERR_UNSUPPORTED;
     if (a.swiglu && a.n_out % 128 != 0) return MOE_ERR_UNSUPPORTED;  // h is the next GEMM's K
+
+    // The tile count is only known on the device; this is its upper bound.
+    const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
+    const long long max_tiles = max_token_tiles * (a.n_out / features_per_tile);
+    const int sms = sm_count();
 
     TensorMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.w, a.w_q, a.E, a.n_out, a.K)
@@ -384,11 +351,6 @@ int launch_grouped_gemm_tc_mx(const MxGemmArgs &a, cudaStream_t stream) {
     p.handover = a.handover;
     p.handover_per_token_tile = a.handover_per_token_tile;
 
-    const long long max_token_tiles = (long long)(a.A < a.E ? a.A : a.E) + a.A / a.nt_max;
-    const long long max_tiles = max_token_tiles * p.n_feature_tiles;
-    const int sms = sm_count();
-    if (split_k_applies(a.swiglu, a.nt_max, max_tiles, p.n_k_blocks, kMxSlotK))  // (moe_gemm_tc.cu)
-        return launch_instance<32, 10, false, true>(maps, p, 2 * (int)max_tiles, stream);
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
     // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots do not hide the walk:
     // 16 tokens of 32 bf16 experts of 1024 x 1024, top 4, 50.7 -> 48.9 us; with longer K or one tile per CTA the queue costs

@@ -555,20 +555,15 @@ __device__ __forceinline__ void drain_staged(uint32_t taddr, int n_mma, int n_va
 
 // ---- host side ----------------------------------------------------------------------------------
 bool encode_weight_map_2d(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K);
+bool encode_map_chunks(CUtensorMap *map, const void *base, uint64_t rows, uint64_t K, int box_rows, int chunks);
 bool encode_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int I, int H);
-bool encode_act_maps_k128(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum);
+bool encode_act_maps_chunks(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int chunks);
 bool encode_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int count = kNumActMaps);
 bool encode_row_map(CUtensorMap *map, const void *act, uint64_t rows, uint64_t K);
 bool encode_mx_weight_map_2d(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K);
 bool encode_mx_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int I, int H);
 bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum);
 int sm_count();
-// Whether a one-CTA GEMM's tiles are split in two along K (SplitK): a down GEMM of small token tiles whose tiles number at
-// most half of the SMs, so that a cluster of two has a tile to itself, with K long enough (two rings of slots) for the
-// exchange not to show.
-inline bool split_k_applies(bool swiglu, int nt_max, long long max_tiles, int n_k_blocks, int block_k) {
-    return !swiglu && nt_max == 32 && 2 * max_tiles <= sm_count() && (long long)n_k_blocks * block_k >= 2048;
-}
 bool set_max_dynamic_smem_once(const void *kernel, int bytes);
 
 }  // namespace tc

@@ -174,15 +174,17 @@ bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint6
     return true;
 }
 
-// Activation maps whose box spans 128 K-elements: the tensor [rows, K] viewed as [K/64][rows][64], box
-// {64, q*(i+1), 2}, so one copy delivers two consecutive 128-byte-swizzled tiles (K 0..63, then 64..127).
-bool encode_act_maps_k128(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum) {
-    for (int i = 0; i < kNumActMaps; ++i) {
-        const cuuint64_t dims[3] = {(cuuint64_t)kBlockK, rows, K / kBlockK};
-        const cuuint64_t strides[2] = {K * 2, (cuuint64_t)kBlockK * 2};
-        const cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)row_quantum * (cuuint32_t)(i + 1), 2};
-        if (!encode(&maps[i], act, 3, dims, strides, box)) return false;
-    }
+// Maps whose box spans several 64-wide K chunks: the bf16 tensor [rows, K] viewed as [K/64][rows][64], box
+// {64, box_rows, chunks}, so one copy delivers consecutive 128-byte-swizzled tiles (zeros for chunks past the end).
+bool encode_map_chunks(CUtensorMap *map, const void *base, uint64_t rows, uint64_t K, int box_rows, int chunks) {
+    const cuuint64_t dims[3] = {(cuuint64_t)kBlockK, rows, K / kBlockK};
+    const cuuint64_t strides[2] = {K * 2, (cuuint64_t)kBlockK * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)box_rows, (cuuint32_t)chunks};
+    return encode(map, base, 3, dims, strides, box);
+}
+bool encode_act_maps_chunks(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int chunks) {
+    for (int i = 0; i < kNumActMaps; ++i)
+        if (!encode_map_chunks(&maps[i], act, rows, K, row_quantum * (i + 1), chunks)) return false;
     return true;
 }
 

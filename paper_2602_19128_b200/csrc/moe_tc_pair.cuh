@@ -83,32 +83,5 @@ __device__ __forceinline__ bool pair_wait(uint32_t bar, uint32_t parity, volatil
     return ok;
 }
 
-// ---- a tile's K range split over a cluster of two one-CTA workers -----------------------------------------------
-// Each CTA multiplies its half of the K range into its own accumulator [128 rows, N]; CTA r finishes rows 64 r .. 64 r + 63.
-// Epilogue warps come in two kinds: those whose 32 rows the peer finishes hand their sums over through its shared memory,
-// the others wait for the peer's and add them.  The sum of two numbers does not depend on the order: results are the same
-// whichever CTA is first.  A cluster has ONE tile in a launch (split_k_applies), so the buffer is written once.
-//   buf   [2 warps][NT_MAX columns][32 lanes] floats in each CTA, written by the peer
-//   full  one arrival per sending warp of the peer
-template <int NT_MAX>
-struct SplitK {
-    static constexpr int kFloats = 2 * NT_MAX * 32;
-    uint32_t full, peer_full;  // this CTA's barrier, the peer's
-    float *buf;
-    uint32_t peer_buf, rank;
-    __device__ __forceinline__ bool receives(int q) const { return (uint32_t)(q >> 1) == rank; }
-    __device__ __forceinline__ static int at(int q, int col, int lane) { return ((q & 1) * NT_MAX + col) * 32 + lane; }
-    __device__ __forceinline__ void send_16(int q, int c0, int lane, const float (&v)[16]) const {
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_buf + (uint32_t)at(q, c0 + i, lane) * 4), "f"(v[i]) : "memory");
-    }
-    __device__ __forceinline__ void add_16(int q, int c0, int lane, float (&v)[16]) const {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] += buf[at(q, c0 + i, lane)];
-    }
-};
-__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
-
 }  // namespace tc
 }  // namespace moe

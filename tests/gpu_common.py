@@ -139,3 +139,12 @@ def assert_routing_exact(views: dict, ids, w, off, s2f, f2s):
 
 def gpu_inputs(cfg, seed=0):
     return make_inputs(cfg, seed=seed, device="cuda")
+
+
+def widen_hidden(x, to, w13, w2):
+    """x [T,H] and the weights w13 [E,2I,H], w2 [E,H,I] (values or codes) of a layer whose hidden dimension is `to` >= H:
+    zeros behind x and w13, w2's rows repeated."""
+    H = x.shape[1]
+    pad = lambda t: torch.nn.functional.pad(t, (0, to - H))
+    rows = torch.arange(to, device=w2.device) % H
+    return dict(x=pad(x), w13=pad(w13), w2=w2[:, rows].contiguous())

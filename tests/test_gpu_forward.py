@@ -6,7 +6,7 @@ import torch
 import paper_2602_19128_b200 as moe
 from oracle import moe_oracle
 from tests.gpu_common import (assert_close_out, assert_routing_exact, bf16_to_f64, gpu_inputs, run_forward,
-                              to_host_case)
+                              to_host_case, widen_hidden)
 
 pytestmark = pytest.mark.gpu
 
@@ -60,8 +60,8 @@ def test_forward_matches_oracle(T, H, I, E, k, skew, flags):
 
 
 @pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2112, 2, 2), (30, 384, 2304, 4, 2)])
-def test_few_down_tiles_split_along_k(T, H, I, E, k):
-    """Down GEMMs of a few tiles with a long K: two CTAs per tile, half of the K slots each (2112: 17 and 16 of them)."""
+def test_few_down_tiles_with_two_ctas_each(T, H, I, E, k):
+    """Down GEMMs of a few tiles with a long K (2112: 33 slots): two CTAs per tile, half of its rows each."""
     inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=0)
     out, views, _ = run_forward(inp)
     *_, h, y, ref = oracle_everything(to_host_case(inp))
@@ -70,6 +70,20 @@ def test_few_down_tiles_split_along_k(T, H, I, E, k):
     assert_close_out(bf16_to_f64(out), ref, "out")
     again, _, _ = run_forward(inp)
     assert torch.equal(out, again)
+
+
+@pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2112, 2, 2), (30, 384, 2304, 4, 2)])
+def test_few_down_tiles_have_the_bits_of_many(T, H, I, E, k):
+    """A token's result does not depend on how many tiles the call has: the same layer with the hidden dimension padded
+    (zeros in x and w13, further rows in w2: above half of the SMs, one CTA per tile) has the same h, and the same y
+    and out in the features both have."""
+    inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=0)
+    wide = dict(inp, **widen_hidden(inp["x"], w13=inp["w13"], w2=inp["w2"], to=5120))
+    out, views, _ = run_forward(inp)
+    out_wide, views_wide, _ = run_forward(wide)
+    assert torch.equal(views["h"].view(torch.int16), views_wide["h"].view(torch.int16))
+    assert torch.equal(views["y"].view(torch.int16), views_wide["y"][:, :H].view(torch.int16))
+    assert torch.equal(out.view(torch.int16), out_wide[:, :H].view(torch.int16))
 
 
 @pytest.mark.parametrize("T,H,I,E,k,skew", [(64, 256, 2048, 64, 4, False),   # one CTA per tile, 32-row tiles, 14 tiles each

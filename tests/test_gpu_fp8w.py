@@ -8,7 +8,7 @@ from oracle import moe_oracle
 from paper_2602_19128_b200.inputs import bf16_bits
 from tests.weight_quantizers import make_fp8w_inputs
 from tests.gpu_common import (Guarded, assert_close_out, assert_routing_exact, bf16_to_f64, check_guards, guarded_out,
-                              layer_regions)
+                              layer_regions, widen_hidden)
 
 pytestmark = pytest.mark.gpu
 
@@ -83,11 +83,19 @@ def test_fp8w_cta_pairs_for_both_gemms(T, H, I, E, k, skew):
 
 
 @pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
-def test_fp8w_few_down_tiles_split_along_k(T, H, I, E, k):
-    """Two CTAs per tile of the down GEMM, half of the K slots each (2176: 9 and 8 of them)."""
+def test_fp8w_few_down_tiles_with_two_ctas_each(T, H, I, E, k):
+    """Two CTAs per tile of the down GEMM, half of its rows each (2176: 17 slots); the same bits as with one CTA per tile,
+    which the layer has with its hidden dimension padded (tests/test_gpu_forward.py)."""
     inp = make_fp8w_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=6, device="cuda")
     out, _ = run_fp8w(inp)
     assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
+    to = 5120
+    w = widen_hidden(inp["x"], w13=inp["w13_q"], w2=inp["w2_q"], to=to)
+    blocks = torch.arange(to // 128, device="cuda") % (H // 128)
+    wide = dict(inp, x=w["x"], w13_q=w["w13"], w2_q=w["w2"], w2_scale=inp["w2_scale"][:, blocks].contiguous(),
+                w13_scale=torch.nn.functional.pad(inp["w13_scale"], (0, (to - H) // 128), value=1.0))
+    out_wide, _ = run_fp8w(wide)
+    assert torch.equal(out.view(torch.int16), out_wide[:, :H].view(torch.int16))
 
 
 @pytest.mark.parametrize("T,H,I,E,k", [(40, 256, 1152, 16, 2),    # 18 slabs of 16 experts and more: two launches in sequence

@@ -10,7 +10,7 @@ from oracle import moe_oracle
 from paper_2602_19128_b200.inputs import bf16_bits
 from tests.weight_quantizers import make_mxfp8_inputs
 from tests.gpu_common import (Guarded, assert_close_out, assert_routing_exact, bf16_to_f64, check_guards, guarded_out,
-                              mx_regions)
+                              mx_regions, widen_hidden)
 
 pytestmark = pytest.mark.gpu
 
@@ -196,11 +196,19 @@ def test_mxfp8_many_short_tiles_per_cta(T, H, I, E, k, skew):
 
 
 @pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
-def test_mxfp8_few_down_tiles_split_along_k(T, H, I, E, k):
-    """Two CTAs per tile of the down GEMM, half of the K slots each (2176: 9 and 8 of them)."""
+def test_mxfp8_few_down_tiles_with_two_ctas_each(T, H, I, E, k):
+    """Two CTAs per tile of the down GEMM, half of its rows each (2176: 17 slots); the same bits as with one CTA per tile,
+    which the layer has with its hidden dimension padded (tests/test_gpu_forward.py)."""
     inp = make_mxfp8_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=2, device="cuda")
     out, _ = run_mx(inp)
     assert_close_out(bf16_to_f64(out), oracle_mx(inp), "mxfp8 out")
+    to = 5120
+    w = widen_hidden(inp["x"], w13=inp["w13_q"], w2=inp["w2_q"], to=to)
+    rows = torch.arange(to, device="cuda") % H
+    wide = dict(inp, x=w["x"], w13_q=w["w13"], w2_q=w["w2"], w2_s=inp["w2_s"][:, rows].contiguous(),
+                w13_s=torch.nn.functional.pad(inp["w13_s"], (0, (to - H) // 32)))
+    out_wide, _ = run_mx(wide)
+    assert torch.equal(out.view(torch.int16), out_wide[:, :H].view(torch.int16))
 
 
 @pytest.mark.parametrize("cfg,lo,n", [(dict(T=160, H=256, I=128, E=16, top_k=4, skew=False), 4, 8),
