@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <unordered_map>
 
 namespace moe {
 namespace tc {
@@ -206,21 +207,19 @@ bool encode_scale_atoms(CUtensorMap *map, const void *atoms, uint64_t n_atoms, u
 }
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel and device instead of once per launch (it is a
-// driver call on the host path of every forward call otherwise).  A small table under the cache's mutex.
+// driver call on the host path of every forward call otherwise).  One entry for every kernel there is, each a mask of
+// devices; under a mutex of its own, which nothing holds across a driver call except the first launch of a kernel.
 bool set_max_dynamic_smem_once(const void *kernel, int bytes) {
-    struct Entry { const void *kernel; unsigned long long devices; };
-    static Entry table[64];
-    static int used = 0;
+    static std::mutex mutex;
+    static std::unordered_map<const void *, unsigned long long> devices;  // (a few dozen kernels)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-    std::lock_guard<std::mutex> lock(g_cache_mutex);
-    Entry *e = nullptr;
-    for (int i = 0; i < used; ++i)
-        if (table[i].kernel == kernel) { e = &table[i]; break; }
-    if (e && ((e->devices >> dev) & 1ull)) return true;
+    std::lock_guard<std::mutex> lock(mutex);
+    unsigned long long *done = nullptr;
+    try { done = &devices[kernel]; } catch (...) {}  // (no host memory for an entry: set again at the next launch)
+    if (done && ((*done >> dev) & 1ull)) return true;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
-    if (!e && used < 64) { e = &table[used++]; e->kernel = kernel; e->devices = 0; }
-    if (e) e->devices |= 1ull << dev;
+    if (done) *done |= 1ull << dev;
     return true;
 }
 

@@ -168,3 +168,43 @@ def test_product_sources_never_reach_the_oracle():
         if f.suffix in (".py", ".c", ".h"):
             text = f.read_text()
             assert "csrc" not in text and "binding" not in text and "libmoe_b200" not in text, f
+
+
+_ATTRIBUTE_HARNESS = r"""
+#include <cuda_runtime.h>
+#include <thread>
+#include <vector>
+static int device = 0, calls = 0;
+static cudaError_t current_device(int *d) { *d = device; return cudaSuccess; }
+static cudaError_t count_call(const void *, cudaFuncAttribute, int) { ++calls; return cudaSuccess; }
+#define cudaGetDevice current_device
+#define cudaFuncSetAttribute count_call
+#include "moe_tc_host.cu"
+static bool set_all() {
+    bool ok = true;
+    for (size_t k = 1; k <= 300; ++k) ok = moe::tc::set_max_dynamic_smem_once(reinterpret_cast<const void *>(k * 16), 1024) && ok;
+    return ok;
+}
+int main() {
+    if (!set_all() || calls != 300) return 1;                       // every kernel once ...
+    std::vector<std::thread> threads;
+    for (int i = 0; i < 4; ++i) threads.emplace_back([] { for (int r = 0; r < 20; ++r) set_all(); });
+    for (auto &t : threads) t.join();
+    if (calls != 300) return 2;                                     // ... however often and from wherever it is launched
+    device = 3;
+    if (!set_all() || !set_all() || calls != 600) return 3;         // and once more on another device
+    return 0;
+}
+"""
+
+
+def test_the_shared_memory_attribute_is_set_once_per_kernel_and_device(tmp_path):
+    """The driver call in front of a launch is made once, for any number of kernels (the library has more than 64): the
+    host helper compiled with the two runtime calls replaced by counters."""
+    from paper_2602_19128_b200.build import CSRC, _nvcc
+    src, exe = tmp_path / "attribute.cu", tmp_path / "attribute"
+    src.write_text(_ATTRIBUTE_HARNESS)
+    r = subprocess.run([_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-cudart", "static",
+                        "-I", str(ROOT / "include"), "-I", str(CSRC), str(src), "-o", str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    assert subprocess.run([str(exe)], timeout=60).returncode == 0
