@@ -700,7 +700,7 @@ def measure_gqa(ctx: Ctx, name: str) -> dict:
         cpu = dict(value=B / wall, unit="decode tokens/s", cores=o.num_threads, kind="oracle",
                    sample=f"the whole batch of '{name}' once, double-precision oracle, {wall:.2f} s wall")
     return dict(metric="gqa_paged_decode_tokens_per_s", value=ctx.world * B / (ms * 1e-3), unit="decode tokens/s",
-                ms_per_step=ms, steps=steps, gpu_launches=steps,  # (the decode kernel; the one that zeroes its counters is not counted)
+                ms_per_step=ms, steps=steps, gpu_launches=steps,
                 config=dict(workload=name, **{k_: cfg[k_] for k_ in ("B", "Hq", "Hkv", "D", "page_size")},
                             cached_tokens=sum(inp["kv_len"]), kv_len_min=min(inp["kv_len"]), kv_len_max=max_len,
                             split_tokens=moe.gqa_decode_split_tokens(B, Hq, Hkv, D, max_len),

@@ -65,9 +65,8 @@ MOE_API size_t gqa_decode_workspace_bytes(int B, int Hq, int Hkv, int D, int max
  * Pointers of q, the caches and out must be 16-byte aligned, the int arrays and lse 4-byte aligned.
  * B == 0 succeeds without a launch.  Page numbers and lengths are NOT validated (they live on the device); page
  * numbers outside [0, num_pages) are outside the contract.  num_pages * page_size must be below 2^31
- * (MOE_ERR_UNSUPPORTED).  Enqueues one kernel, or two where sequences are split (the first
- * zeroes the words they are counted in); returns MOE_ERR_CUDA when a tensor map cannot be encoded
- * or the launch fails. */
+ * (MOE_ERR_UNSUPPORTED).  Enqueues one kernel, behind a memset where sequences may be split; returns
+ * MOE_ERR_CUDA when a tensor map cannot be encoded or the launch fails. */
 MOE_API int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, const int32_t *kv_indptr,
                              const int32_t *kv_indices, const int32_t *kv_last_page_len, int B, int Hq, int Hkv, int D,
                              int page_size, int num_pages, int max_kv_len, float sm_scale, void *out, float *lse,

@@ -85,34 +85,24 @@ struct Params {
     const int *kv_indptr, *kv_indices, *kv_last_page_len;
     __nv_bfloat16 *out;
     float *lse;
-    int *status;       // the workspace's status word, zeroed before the launch
-    int *counters;     // [B * Hkv], zeroed before the launch
+    int *status;       // the workspace's status word, zeroed before the launch (or by its first block: own_status)
+    int *counters;     // [B * Hkv], zeroed before the launch (not with own_status: nothing is counted)
     float *part_ml;    // [slots, group, 2]  (max in the base-2 domain, sum); at least B * Hkv * n_splits slots
     float *part_o;     // [slots, group, D]  unnormalised
     int B, Hq, Hkv, group, page_size, split_tokens, n_splits;
     int box_rows;      // tiled gather: token rows one TMA box brings (min(page_size, 64))
-    int own_status;    // no zeroing kernel ran: the first block zeroes the status word
+    int own_status;    // no memset in front: the first block zeroes the status word
     float scale_log2;  // sm_scale * log2(e)
 };
 
 // ---- the launches of a call --------------------------------------------------------------------------------------
-// Where parts of sequences may have to be counted, a small kernel zeroes the status word and the counters; the decode kernel
-// is launched with programmatic stream serialisation, so its blocks start as soon as that kernel has (which starts after
-// everything before it in the stream) and stream the cache meanwhile.  Only what the zeroed words are used for -- the status
-// word, the counting of parts -- waits for it, as does every block before it leaves, so that what follows in the stream
-// follows both.  Behind a memset node the decode kernel's launch was serialised: 1 sequence of 65 536 tokens 36.8 -> 36.0 us,
-// 8 of 1000..8000 24.6 -> 23.6.  Where no sequence is split there is nothing to count, and the decode kernel's first block
-// zeroes the status word (Params::own_status): one launch: 1
-// sequence of 100 tokens 9.1 -> 8.0 us, 32 of 100..500 12.3 -> 10.5, 256 of 256..2048 105.3 -> 102.8.  A wait gives up after 4 million polls, long
-// after that block has started.
-__device__ __forceinline__ void zeroed_words_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-constexpr int kZeroThreads = 256;
-__global__ void __launch_bounds__(kZeroThreads) gqa_zero_kernel(uint4 *words, int n) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int i = blockIdx.x * kZeroThreads + threadIdx.x;
-    if (i < n) words[i] = make_uint4(0, 0, 0, 0);
-}
+// Where parts of sequences may have to be counted, a memset in front of the kernel zeroes the status word and the counters.
+// Where no sequence is split there is nothing to count, and the kernel's first block zeroes the status word
+// (Params::own_status): one launch.  In a loop / on the first pass over new inputs: 1 sequence of 100 tokens 8.5 -> 7.6 us / 25.7 ->
+// 21.7, 256 of 256..2048 105.5 -> 102.8 / 138 -> 133.  A wait gives up after 4 million polls, long after that block has started.
+// (A small kernel that zeroed the words beside a decode kernel launched with programmatic serialisation made loops 0.7 to 2
+// us shorter, but first passes 2.3 longer, memset / small kernel: 1 sequence of 65 536 tokens 36.9 / 36.2 and 58.3 / 61.3, 1 of
+// 4000 14.3 / 13.2 and 32.4 / 34.8, 16 of 8000 51.1 / 50.2 and 73.7 / 75.6.)
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -175,7 +165,6 @@ __device__ __forceinline__ bool bounded_wait(uint32_t bar, uint32_t parity, int 
         if (*gave_up) return false;
     }
     *gave_up = 1;
-    zeroed_words_wait();
     if (atomicCAS(status, 0, (int)MOE_ERR_DEVICE_TIMEOUT) == 0) { status[1] = 12; status[2] = blockIdx.x; }
     return false;
 }
@@ -563,7 +552,6 @@ struct BlockParts {
     int is_last[2];
 };
 __device__ __forceinline__ void count_and_merge(const Params &p, BlockParts &s, float *merge, volatile int *gave_up, int tid) {
-    zeroed_words_wait();
     sync_compute();  // the parts are stored ...
     if (s.part[0].n_parts <= 1 && s.part[1].n_parts <= 1) return;
     if (tid < 2) {
@@ -596,14 +584,10 @@ gqa_row_decode_kernel(const Params p) {
 
     if (L <= 0) {  // nothing cached: out = 0, lse = -inf (written by the first split's block)
         if (split == 0) write_empty(p, b, head0, tid);
-        zeroed_words_wait();
         return;
     }
     const int n_active = min(p.n_splits, (L + p.split_tokens - 1) / p.split_tokens);
-    if (split >= n_active) {
-        zeroed_words_wait();
-        return;
-    }
+    if (split >= n_active) return;
     const int begin = split * p.split_tokens;
     const int end = split == n_active - 1 ? L : begin + p.split_tokens;  // the last active split runs to the end
     const int n_chunks = (end - begin + kChunk - 1) / kChunk;
@@ -675,7 +659,6 @@ gqa_row_decode_kernel(const Params p) {
     // A block that gave up waits (bounded) for its copies in flight, then leaves without a result: the status word says so.
     if (!ok) {
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
-        zeroed_words_wait();
         return;
     }
     __syncthreads();  // all copies were waited for: the pipeline's shared memory becomes the merge buffer
@@ -829,15 +812,13 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
             const long long most = (total + kMinPiece - 1) / kMinPiece;
             n_blocks = (int)(most < kBalancedBlocks ? most : kBalancedBlocks);
         }
-        if ((int)blockIdx.x >= n_blocks) {
-            zeroed_words_wait();
-            return;
-        }
+        if ((int)blockIdx.x >= n_blocks) return;
         if (balanced) {
             w = divide(total * blockIdx.x, n_blocks);
             w_end = divide(total * (blockIdx.x + 1), n_blocks);
             start = w;
             if (tid == 0) { line.total = total; line.begin = w; line.end = w_end; line.n_blocks = n_blocks; line.balanced = true; }
+            if (blockIdx.x == 0 && tid == 0) p.status[3] = 1;  // (reporting: the batch was cut into equal pieces)
         }
         const int x = (int)divide(start, p.Hkv);
         int r = 0;  // the last range that starts at or before chunk or share x of the items
@@ -869,14 +850,10 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         n_chunks = (L + kChunk - 1) / kChunk;
         if (L <= 0) {
             if (split == 0 && tid < kThreads) write_empty(p, b, kvh * p.group, tid);
-            zeroed_words_wait();
             return;
         }
         const int n_parts = min(p.n_splits, (n_chunks + split_chunks - 1) / split_chunks);
-        if (split >= n_parts) {
-            zeroed_words_wait();
-            return;
-        }
+        if (split >= n_parts) return;
         c = split * split_chunks;
         w_end = (split == n_parts - 1 ? n_chunks : c + split_chunks) - c;  // the last split runs to the end
         if (tid == 0) { line.n_blocks = n_parts; line.balanced = false; }
@@ -933,7 +910,6 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
             }
             if (++stage == kTiledStages) { stage = 0; parity ^= 1u; }
         }
-        zeroed_words_wait();
         return;
     }
 
@@ -996,7 +972,6 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         if (left > 0) next_sequence();
     }
     count_and_merge(p, parts, merge, &gave_up, tid);
-    if (kAdaptive && balanced && blockIdx.x == 0 && tid == 0) p.status[3] = 1;  // (reporting: the batch was cut into equal pieces)
     // A block that gave up waits (bounded) for its copies in flight before it leaves.
     if (!ok)
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
@@ -1157,25 +1132,11 @@ int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, co
     if (tiled && (!moe::tc::encode_kv_cache_map(&k_map, k_cache, (uint64_t)num_pages, (uint32_t)page_size, (uint32_t)Hkv, (uint32_t)p.box_rows) ||
                   !moe::tc::encode_kv_cache_map(&v_map, v_cache, (uint64_t)num_pages, (uint32_t)page_size, (uint32_t)Hkv, (uint32_t)p.box_rows)))
         return MOE_ERR_CUDA;
-    // (whole 16-byte words: what follows the counters up to the next multiple of 256 bytes is nobody's)
-    const int zero_words = (int)((256 + bh * sizeof(int) + 15) / 16);
     auto launch = [&](auto kernel, dim3 grid, int threads, int smem_bytes, const auto &...args) {
         if (!moe::tc::set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), smem_bytes)) return MOE_ERR_CUDA;
-        if (!p.own_status) {
-            gqa_zero_kernel<<<(zero_words + kZeroThreads - 1) / kZeroThreads, kZeroThreads, 0, st>>>(reinterpret_cast<uint4 *>(p.status), zero_words);
-            if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
-        }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid;
-        cfg.blockDim = threads;
-        cfg.dynamicSmemBytes = smem_bytes;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = p.own_status ? 0 : 1;
-        return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+        if (!p.own_status && cudaMemsetAsync(p.status, 0, 256 + bh * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
+        kernel<<<grid, threads, smem_bytes, st>>>(args...);
+        return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
     };
     const unsigned shares = (unsigned)(bh * p.n_splits);
     // Two slots per balanced block: where the workspace has them, and the fixed shares fill the machine at most twice.

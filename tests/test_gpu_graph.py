@@ -1,10 +1,10 @@
-"""The layer captured into a CUDA graph: the library never synchronises, allocates or reads device memory on the
+"""The layer and the decode step captured into a CUDA graph: the library never synchronises, allocates or reads device memory on the
 host, so its launch sequence can be recorded once and replayed; a replay on new inputs must equal a plain call."""
 import pytest
 import torch
 
 import paper_2602_19128_b200 as moe
-from paper_2602_19128_b200.inputs import make_inputs
+from paper_2602_19128_b200.inputs import make_gqa_inputs, make_inputs
 from tests.weight_quantizers import make_mxfp8_inputs
 
 pytestmark = pytest.mark.gpu
@@ -64,6 +64,63 @@ def test_mxfp8_layer_replays_from_a_graph():
     moe.moe_forward_mxfp8(b["x"], b["router_logits"], a["w13_q"], sf13, a["w2_q"], sf2, k, ref, ws2)
     torch.cuda.synchronize()
     assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
+
+
+def _graph_nodes(graph):
+    """How many kernel and memset nodes a captured graph has."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.12")
+    n = ctypes.c_size_t(0)
+    assert rt.cudaGraphGetNodes(ctypes.c_void_p(graph), None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert rt.cudaGraphGetNodes(ctypes.c_void_p(graph), nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for node in nodes:
+        kind = ctypes.c_int(-1)
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    return kinds.count(0), kinds.count(2)
+
+
+@pytest.mark.parametrize("page_size,lengths,memsets", [
+    (16, [20000, 9000], 1),                           # fixed splits, counted
+    (16, [8000, 3000] + [70] * 22, 1),                # equal pieces
+    (12, [20000, 9000], 1),                           # the row gather, counted
+    (16, [100 + 37 * i for i in range(40)], 0),       # nothing split
+    (12, [100 + 37 * i for i in range(40)], 0),
+])
+def test_decode_attention_is_one_kernel_and_replays_from_a_graph(page_size, lengths, memsets):
+    """The call's launches, and a replay on a new query and shorter sequences against a plain call.  (A second kernel in
+    front costs a first pass over new inputs more than a memset does.)"""
+    cfg = dict(B=len(lengths), Hq=32, Hkv=4, D=128, page_size=page_size, lengths=lengths)
+    a, b = make_gqa_inputs(cfg, seed=1, device="cuda"), make_gqa_inputs(cfg, seed=2, device="cuda")
+    n = max(lengths)
+    ws = moe.alloc_workspace(moe.gqa_decode_workspace_bytes(len(lengths), 32, 4, 128, n), "cuda")
+    ws.fill_(0xFF)
+    out, lse = torch.empty_like(a["q"]), torch.empty((len(lengths), 32), dtype=torch.float32, device="cuda")
+    def call(o, l, w, stream=None):
+        moe.gqa_paged_decode(a["q"], a["k_cache"], a["v_cache"], a["kv_indptr"], a["kv_indices"], a["kv_last_page_len"], n,
+                             a["sm_scale"], o, w, lse=l, stream=stream)
+    call(out, lse, ws)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    s = torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        call(out, lse, ws, torch.cuda.current_stream())
+    assert _graph_nodes(g.raw_cuda_graph()) == (1, memsets)
+    g.instantiate()
+    first = a["q"].clone()
+    for q, last in ((b["q"], 1), (first, page_size), (b["q"], 1)):
+        a["q"].copy_(q)
+        a["kv_last_page_len"].fill_(last)
+        ws.fill_(0xFF)
+        g.replay()
+        torch.cuda.synchronize()
+        assert moe.moe_last_status(ws) == moe.MOE_OK
+        ref, ref_lse = torch.empty_like(out), torch.empty_like(lse)
+        call(ref, ref_lse, moe.alloc_workspace(ws.numel(), "cuda"))
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int16), ref.view(torch.int16)) and torch.equal(lse, ref_lse)
 
 
 def test_two_streams_with_their_own_workspaces_do_not_interfere():
