@@ -345,11 +345,11 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
 }
 
 // Routes tokens [t0, t1) of the block (warp w takes tokens t0 + w, t0 + w + n_warps, ...) and writes ids and weights;
-// hist, if given, collects the histogram over the resident experts (zeroed by the caller); ids_smem, if not 0, is the address
-// (in the cluster's shared memory) of an array of all tokens' ids, which are left there too.
+// hist, if given, collects the histogram over the resident experts (zeroed by the caller); with ids_local all tokens' ids are
+// left in the array at address ids_smem of the cluster's shared memory too (any value is an address, 0 among them).
 __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, int t0, int t1, int E, int k, int local_offset,
                                              int n_local, const RouterParams &rp, int *topk_ids, float *topk_w, Candidates *cand,
-                                             int *hist, uint32_t ids_smem = 0) {
+                                             int *hist, bool ids_local = false, uint32_t ids_smem = 0) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     for (int t = t0 + warp; t < t1; t += n_warps) {
         int my_id;
@@ -361,7 +361,7 @@ __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, i
         if (lane < k) {
             topk_ids[(size_t)t * k + lane] = my_id;
             topk_w[(size_t)t * k + lane] = my_w;
-            if (ids_smem)
+            if (ids_local)
                 asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(ids_smem + (uint32_t)(t * k + lane) * 4), "r"(my_id) : "memory");
             const int local = my_id - local_offset;  // only experts resident here are scheduled
             if (hist && local >= 0 && local < n_local) atomicAdd(&hist[local], 1);
@@ -700,7 +700,7 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
         }
     }
     const int t0 = blockIdx.x * tokens_per_block;
-    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr, ids_smem);
+    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr, ids_local, ids_smem);
     if (cluster) {
         __syncwarp();
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
