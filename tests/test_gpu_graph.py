@@ -24,7 +24,10 @@ def _capture(call):
 
 
 @pytest.mark.parametrize("cfg", [dict(T=16, H=256, I=512, E=8, top_k=2, skew=False),
-                                 dict(T=1500, H=256, I=128, E=32, top_k=4, skew=True)])  # fused and three-kernel router
+                                 dict(T=64, H=256, I=512, E=8, top_k=2, skew=False),    # routers: one block, a cluster,
+                                 dict(T=700, H=256, I=256, E=16, top_k=4, skew=True),   # many blocks,
+                                 dict(T=1500, H=256, I=128, E=32, top_k=4, skew=True),  # three kernels;
+                                 dict(T=1, H=512, I=2048, E=4, top_k=2, skew=False)])   # two CTAs per tile of the down GEMM
 def test_bf16_layer_replays_from_a_graph(cfg):
     a, b = make_inputs(cfg, seed=1, device="cuda"), make_inputs(cfg, seed=2, device="cuda")
     T, H, I, E, k = cfg["T"], cfg["H"], cfg["I"], cfg["E"], cfg["top_k"]
@@ -180,6 +183,65 @@ def test_alternating_problems_on_one_workspace_stay_bit_identical():
     assert moe.moe_last_status(ws) == moe.MOE_OK
     for out, r in zip(outs, refs):
         assert torch.equal(out.view(torch.int16), r.view(torch.int16))
+
+
+def test_alternating_forms_of_the_router_and_the_down_gemm_on_one_workspace():
+    """One-block, cluster, many-block and three-kernel routers zero the status region in different places (a memset, or their
+    own first block) and a call's GEMMs start on a flag there: queued behind one another in every order on one workspace,
+    each call has the bits of a lone one."""
+    cfgs = [dict(T=1, H=512, I=2048, E=4, top_k=2, skew=False), dict(T=64, H=256, I=512, E=8, top_k=2, skew=False),
+            dict(T=16, H=256, I=512, E=8, top_k=2, skew=False), dict(T=300, H=256, I=128, E=16, top_k=8, skew=True),
+            dict(T=1100, H=128, I=64, E=16, top_k=2, skew=False)]
+    inps = [make_inputs(c, seed=80 + i, device="cuda") for i, c in enumerate(cfgs)]
+    need = max(moe.moe_workspace_bytes(c["T"], c["H"], c["I"], c["E"], c["top_k"]) for c in cfgs)
+    def call(i, out, ws):
+        moe.moe_forward(inps[i]["x"], inps[i]["router_logits"], inps[i]["w13"], inps[i]["w2"], cfgs[i]["top_k"], out, ws)
+    refs = [torch.empty_like(inp["x"]) for inp in inps]
+    for i, ref in enumerate(refs):
+        call(i, ref, moe.alloc_workspace(need, "cuda"))
+    torch.cuda.synchronize()
+    ws = moe.alloc_workspace(need, "cuda")
+    ws.fill_(0xFF)
+    order = [i for a in range(5) for b in range(5) for i in (a, b)] * 8
+    outs = [torch.empty_like(refs[i]) for i in order]
+    for i, out in zip(order, outs):
+        call(i, out, ws)
+    torch.cuda.synchronize()
+    assert moe.moe_last_status(ws) == moe.MOE_OK
+    for i, out in zip(order, outs):
+        assert torch.equal(out.view(torch.int16), refs[i].view(torch.int16)), cfgs[i]
+
+
+def test_alternating_forms_of_the_decode_call_on_one_workspace():
+    """A call that splits nothing zeroes the status word itself and leaves the counters as they are; one that splits has a
+    memset in front.  Queued behind one another in every order on one workspace, each has the bits of a lone call."""
+    shapes = [[100 + 37 * i for i in range(40)],       # nothing split
+              [20000, 9000],                           # fixed splits
+              [8000, 3000] + [70] * 22,                # equal pieces
+              [5, 0, 64]]                              # an empty item, nothing split
+    inps = [make_gqa_inputs(dict(B=len(n), Hq=32, Hkv=4, D=128, page_size=p, lengths=n), seed=90, device="cuda")
+            for n in shapes for p in (16, 12)]
+    need = max(moe.gqa_decode_workspace_bytes(i["B"], 32, 4, 128, max(i["kv_len"])) for i in inps)
+    def call(i, out, lse, ws):
+        moe.gqa_paged_decode(i["q"], i["k_cache"], i["v_cache"], i["kv_indptr"], i["kv_indices"], i["kv_last_page_len"],
+                             max(i["kv_len"]), i["sm_scale"], out, ws, lse=lse)
+    def results():
+        return [(torch.empty_like(i["q"]), torch.empty((i["B"], 32), dtype=torch.float32, device="cuda")) for i in inps]
+    refs = results()
+    for i, r in zip(inps, refs):
+        call(i, *r, moe.alloc_workspace(need, "cuda"))
+        torch.cuda.synchronize()
+    ws = moe.alloc_workspace(need, "cuda")
+    ws.fill_(0xFF)
+    n = len(inps)
+    order = [i for a in range(n) for b in range(n) for i in (a, b)]
+    outs = [results()[i] for i in order]
+    for i, o in zip(order, outs):
+        call(inps[i], *o, ws)
+    torch.cuda.synchronize()
+    assert moe.moe_last_status(ws) == moe.MOE_OK
+    for i, (out, lse) in zip(order, outs):
+        assert torch.equal(out.view(torch.int16), refs[i][0].view(torch.int16)) and torch.equal(lse, refs[i][1])
 
 
 def test_an_expired_device_wait_is_reported_and_leaves_the_device_usable():
@@ -359,5 +421,67 @@ def test_many_overlapping_mxfp8_calls_on_two_streams_complete():
     T, H, I, E, k = 2048, 512, 256, 64, 8
     assert moe.moe_mxfp8_workspace_layout(T, H, I, E, k).tile_rows == 304
     src = _OVERLAP_MX.format(root=str(Path(__file__).resolve().parent.parent), T=T, H=H, I=I, E=E, k=k, groups=100)
+    r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, timeout=240)
+    assert r.returncode == 0 and "overlap ok" in r.stdout, r.stderr[-2000:]
+
+
+_OVERLAP_PAIR = r"""
+import sys, torch
+sys.path.insert(0, {root!r})
+import paper_2602_19128_b200 as moe
+from paper_2602_19128_b200.inputs import make_gqa_inputs, make_inputs
+from tests.weight_quantizers import make_fp8w_inputs
+def layer(T, H, I, E, k, fp8=False):
+    cfg = dict(T=T, H=H, I=I, E=E, top_k=k, skew=False)
+    inp = (make_fp8w_inputs if fp8 else make_inputs)(cfg, seed=72, device="cuda")
+    def call(o, w, stream=None):
+        if fp8:
+            moe.moe_forward_fp8w(inp["x"], inp["router_logits"], inp["w13_q"], inp["w13_scale"], inp["w2_q"], inp["w2_scale"],
+                                 k, o, w, stream=stream)
+        else:
+            moe.moe_forward(inp["x"], inp["router_logits"], inp["w13"], inp["w2"], k, o, w, stream=stream)
+    return call, lambda: torch.empty_like(inp["x"]), lambda: moe.alloc_workspace(moe.moe_workspace_bytes(T, H, I, E, k), "cuda")
+def decode(lengths):
+    B, n = len(lengths), max(lengths)
+    inp = make_gqa_inputs(dict(B=B, Hq=32, Hkv=4, D=128, page_size=16, lengths=lengths), seed=73, device="cuda")
+    def call(o, w, stream=None):
+        moe.gqa_paged_decode(inp["q"], inp["k_cache"], inp["v_cache"], inp["kv_indptr"], inp["kv_indices"],
+                             inp["kv_last_page_len"], n, inp["sm_scale"], o, w, stream=stream)
+    return call, lambda: torch.empty_like(inp["q"]), lambda: moe.alloc_workspace(moe.gqa_decode_workspace_bytes(B, 32, 4, 128, n), "cuda")
+lanes = []
+for call, out, ws in ({first}, {second}):
+    ref = out()
+    call(ref, ws())
+    torch.cuda.synchronize()
+    lanes.append((call, out(), ws(), ref, torch.cuda.Stream()))
+torch.cuda.synchronize()
+for it in range({groups}):
+    for i in range(10):
+        for call, out, ws, ref, stream in lanes:
+            call(out, ws, stream)
+    torch.cuda.synchronize()
+for call, out, ws, ref, stream in lanes:
+    assert moe.moe_last_status(ws, stream=stream) == 0
+    assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
+print("overlap ok")
+"""
+
+_FP8_PAIRS = "layer(600, 1024, 1024, 8, 2, True)"       # CTA pairs for both GEMMs, many-block router
+_CLUSTER = "layer(64, 256, 512, 8, 2)"                  # cluster router
+_ONE_TOKEN = "layer(1, 512, 2048, 4, 2)"                # one-block router, two CTAs per tile of the down GEMM
+_PIECES = "decode([8000, 3000] + [70] * 22)"            # equal pieces
+_UNSPLIT = "decode([100 + 37 * i for i in range(40)])"  # its own status word
+
+
+@pytest.mark.parametrize("first,second", [(_FP8_PAIRS, _FP8_PAIRS), (_FP8_PAIRS, _CLUSTER), (_CLUSTER, _CLUSTER),
+                                          (_ONE_TOKEN, _FP8_PAIRS), (_PIECES, _UNSPLIT), (_PIECES, _CLUSTER)],
+                         ids=["fp8w_pairs", "fp8w_pairs_and_cluster", "cluster", "one_token_and_fp8w_pairs", "decode", "decode_and_cluster"])
+def test_overlapping_calls_of_two_kinds_on_two_streams_complete(first, second):
+    """The stress of the tests above for the other launch forms, and for two different ones at a time: a child process
+    with a time limit, every result with the bits of a lone call."""
+    import subprocess
+    import sys
+    from pathlib import Path
+    src = _OVERLAP_PAIR.format(root=str(Path(__file__).resolve().parent.parent), first=first, second=second, groups=150)
     r = subprocess.run([sys.executable, "-c", src], capture_output=True, text=True, timeout=240)
     assert r.returncode == 0 and "overlap ok" in r.stdout, r.stderr[-2000:]
