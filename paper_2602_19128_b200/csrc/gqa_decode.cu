@@ -737,10 +737,6 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
     const uint32_t smem_base = smem_u32(smem), full_base = smem_u32(full_bar), empty_base = smem_u32(empty_bar);
     const int sh = 31 - __clz(p.box_rows);  // log2 of the rows of a box
     if (!kAdaptive) zero_own_status(p, blockIdx.x == 0, tid);
-    if (tid == kThreads) {  // the descriptors on their way while the block finds its work
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&k_map) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&v_map) : "memory");
-    }
     if (tid == 0) {
         for (int s = 0; s < kTiledStages; ++s) {
             mbar_init(full_base + s * 8, 32);       // the copy warp's lanes
