@@ -97,13 +97,13 @@ int layer_token_tile_bound(int T, int H, int I, int E, int k, unsigned flags, bo
     return fp8w && bound > 192 ? 192 : bound;
 }
 
-// Whether the FP8-weight layer's down GEMM starts through the hand-over.  The counting costs a gate/up epilogue about a
-// microsecond per tile, a fence behind its stores, which a K loop of 16 slots (H = 2048) hides and a shorter one does not;
-// it saves the down GEMM's start and the gate/up GEMM's tail, some microseconds once.  So with short K loops it is taken
-// only where a CTA has few tiles: no more rounds of gate/up tiles than slots in each.  With / without: 16 experts, top 4,
-// H = 4096, I = 14336, 389 tokens 838 / 854 us; 256 experts, top 6, H = 256, I = 2048, 389 tokens 238 / 176 (211 before the
-// layer had a hand-over); 64 experts, top 6, H = 1024, I = 1536, 1575 tokens 193 / 183; 8 experts, top 2, H = 512, I = 1536,
-// 389 tokens 41.0 / 41.6.
+// Whether the FP8-weight layer's GEMMs start through the hand-over.  The counting costs a gate/up epilogue a fence behind the
+// stores of every tile; it saves both GEMMs' starts and the gate/up GEMM's tail, some microseconds once.  With many short
+// tiles per CTA the fences are the larger part, so with K loops below 16 slots (H = 2048) it is taken only where a CTA has
+// few tiles: no more rounds of gate/up tiles than slots in each.  With / without: 256 experts, top 6, H = 256, I = 2048, 389
+// tokens 223 / 165 us; 64 experts, top 6, H = 1024, I = 1536, 1575 tokens 137 / 131; 64 tokens of 32, top 4, 1024 x 1024 47.5 /
+// 49.1; 8 experts, top 2, H = 512, I = 1536, 389 tokens 37.3 / 37.9; from 16 slots on it is 2 % either way: 32 experts, top 4, 2048 x
+// 2048, 700 tokens 126.7 / 126.3; 16, top 4, 4096 x 14336, 389 tokens 724 / 710; 256, top 8, 7168 x 2048, 16 tokens 751 / 766.
 bool fp8w_hand_over(int T, int H, int I, int E, int k, int nt_max) {
     const long long A = (long long)T * k, slots = H / 128, token_tiles = (A < E ? A : E) + A / nt_max;
     return slots >= 16 || token_tiles * (I / 64) <= slots * tc::sm_count();

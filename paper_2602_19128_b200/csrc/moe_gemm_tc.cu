@@ -87,7 +87,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     static_assert(kTmemCols >= 32 && kTmemCols <= 512 && (kTmemCols & (kTmemCols - 1)) == 0,
                   "a tensor-memory allocation must be a power of two between 32 and 512 columns");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;  // the down GEMM reports sites 5..8
-    chain_release();  // the next kernel of the forward call may be scheduled; it waits for this grid to finish
+    chain_release();  // the next kernel of the forward call may be scheduled; it waits for what it needs of this grid
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -137,7 +137,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelPara
     __syncthreads();
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    // everything above overlapped the previous kernel; its results are read from here on
+    // everything above overlapped the kernels in front; from here on there is a schedule (the token side waits for more)
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
     const int worker = HALVES ? blockIdx.x >> 1 : blockIdx.x, n_workers = HALVES ? gridDim.x >> 1 : gridDim.x;
@@ -379,9 +379,9 @@ int launch_grouped_gemm_tc(const GroupedGemmArgs &a, cudaStream_t stream) {
     if (halves)
         return launch_instance<32, kHalfStages, false, true>(maps, p, 2 * (int)max_tiles, stream);
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
-    // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots do not hide the walk:
-    // 16 tokens of 32 bf16 experts of 1024 x 1024, top 4, 50.7 -> 48.9 us; with longer K or one tile per CTA the queue costs
-    // (100 tokens of 128 experts of 4096 x 1536, top 8, 720 -> 731, the tiny layer 19.2 -> 19.7).
+    // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots do not hide the walk.  Without / with: 16 tokens of
+    // 32 experts of 1024 x 1024, top 4, 51.5 / 50.4 us; 64 of 2048 x 2048 140.4 / 140.8; 100 tokens of 128 of 4096 x 1536, top 8,
+    // 722 / 731; one tile per CTA, the tiny layer 19.2 / 19.7.
     const bool queued = max_tiles > sms && a.K <= 1024;
     if (queued) return a.swiglu ? dispatch<true, true>(a.nt_max, maps, p, grid, stream) : dispatch<false, true>(a.nt_max, maps, p, grid, stream);
     return a.swiglu ? dispatch<true, false>(a.nt_max, maps, p, grid, stream) : dispatch<false, false>(a.nt_max, maps, p, grid, stream);

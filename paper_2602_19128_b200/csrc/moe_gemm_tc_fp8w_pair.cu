@@ -11,8 +11,8 @@
 // What bounded the one-CTA kernel at 64 rows per tile and more: a slot of 96 rows takes in 16 KiB of codes and 24 KiB of
 // tokens, 640 cycles at 64 bytes per cycle, and three token slots, tied to the three converted ones, do not cover the
 // microsecond a token slot takes to arrive from L2: 1030 cycles per slot.  A pair's CTA takes in half of the tokens and keeps
-// six token slots, two per converted one.  333 Mixtral-shaped tokens 359 -> 324 us, 2000 tokens 1390 -> 1231 us, 4096 tokens
-// of 128 experts of 4096 x 1536 1624 -> 1508 us.  What bounds it now: a slot takes 620 to 750 cycles, and the MMA thread
+// six token slots, two per converted one.  333 Mixtral-shaped tokens 338 -> 311 us, 2000 tokens 1380 -> 1186 us, 4096 tokens
+// of 128 experts of 4096 x 1536 1559 -> 1330 us.  What bounds it now: a slot takes 620 to 750 cycles, and the MMA thread
 // never waits for an operand there, so it is the eight MMAs (about 77 cycles each at N = 96); the converters' ALU and FMA
 // pipes are half busy beside them.
 //
@@ -55,7 +55,8 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 // front of every tile of every role, and the converters and the MMA warp run only two or three slots ahead of one another:
 // they stood still for it.  So the CTA copies the schedule once, in one round trip, and walks its copy (200-300 cycles):
 // 333-token Mixtral-shaped layer 342 -> 324 us, 4096 tokens of 128 experts 1531 -> 1493 us.  (The other GEMMs, whose
-// producers run a ring of six slots or more ahead, gained nothing from the same copy and lost up to 1 %.)
+// producers run a ring of six slots or more ahead, lost up to 1 % by the same copy; their short tiles are decoded ahead by a warp
+// of its own, TileQueue.)
 constexpr int kScheduleInts = 3 * kMaxExperts + 2;
 struct Schedule {
     const int *prefix, *offsets;  // [E+1] token tiles before a schedule position; first row of an expert
@@ -134,7 +135,7 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMaps maps, const 
     static_assert(kColsUsed <= 512 && kConv * kConvCols <= 256, "accumulators and converted slots exceed tensor memory");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
     constexpr int kFeatPerCta = SWIGLU ? kTileM / 2 : kTileM;
-    chain_release();  // the next kernel of the forward call may be scheduled; it waits for this grid to finish
+    chain_release();  // the next kernel of the forward call may be scheduled; it waits for what it needs of this grid
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -182,7 +183,7 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMaps maps, const 
     cluster_sync_all();  // the peer's barriers exist before anything can signal them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    // everything above overlapped the previous kernel; its results are read from here on
+    // everything above overlapped the kernels in front; from here on there is a schedule (the token side waits for more)
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const Schedule sched = stage_schedule(p, reinterpret_cast<int *>(base_ptr + L::kSchedule), started);
     const int total_tiles = sched.total_token_tiles * p.n_feature_tiles;
@@ -442,10 +443,11 @@ int launch_fp8w_pair_instance(const TensorMaps &maps, const KernelParams &p, int
 }  // namespace
 
 // Tiles of more than 64 rows, in K loops of eight slots or more (shorter ones do not hide what a pair's barriers cost), whose
-// features fill whole pair tiles.  One CTA per tile / pairs: 2000 tokens of 8 experts of 4096 x 14336, top 2, 1421 / 1270 us;
-// 1024 of 64 experts of 7168 x 2048, top 8, 994 / 862; 1500 of 128 of 4096 x 1536, top 8, 775 / 703; 1200 of 20 of 2048 x
-// 1024, top 2, 89.4 / 89.3; 700 of 4 of 384 x 512, top 2, 40.0 / 42.0; 8192 of 8 of 256 x 512, top 2, 101.5 / 103.3; tiles of
-// up to 64 rows, 150 of 8 of 4096 x 14336, top 2, 278 / 292.
+// features fill whole pair tiles.  One CTA per tile / pairs: 2000 tokens of 8 experts of 4096 x 14336, top 2, 1380 / 1186 us;
+// 1024 of 64 of 7168 x 2048, top 8, 971 / 817; 1500 of 128 of 4096 x 1536, top 8, 742 / 641; 1200 of 20 of 2048 x 1024, top 2,
+// 83.1 / 78.8; 2000 of 16 of 1280 x 1280, top 2, 85.0 / 84.7; at eight slots 4096 of 32 of 1024 x 1024, top 4, 157 / 144, but calls of
+// few tiles lose, 2000 of 16, top 2, 70.1 / 72.2; below, 2000 of 16 of 768 x 768, top 2, 55.5 / 57.4 and 8192 of 8 of 256 x 512, top 2,
+// 68.8 / 71.4.  (Tiles of up to 64 rows, with an earlier epilogue: 150 of 8 of 4096 x 14336, top 2, 278 / 292.)
 bool grouped_gemm_tc_fp8w_pair_applies(const GroupedGemmArgs &a) {
     return (a.nt_max == 128 || a.nt_max == 192) && a.K >= 8 * kSlotK && a.n_out % (a.swiglu ? kTileM : 2 * kTileM) == 0;
 }

@@ -79,7 +79,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     static_assert(2 * NT_MAX + 32 <= kTmemColsMx, "accumulators and scale columns exceed tensor memory");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
     constexpr uint32_t kSfACol = 2 * NT_MAX, kSfBCol = 2 * NT_MAX + 16;
-    chain_release();  // the next kernel of the forward call may be scheduled; it waits for this grid to finish
+    chain_release();  // the next kernel of the forward call may be scheduled; it waits for what it needs of this grid
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -129,7 +129,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
     __syncthreads();
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    // everything above overlapped the previous kernel; its results are read from here on
+    // everything above overlapped the kernels in front; from here on there is a schedule (the token side waits for more)
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
     const int worker = blockIdx.x, n_workers = gridDim.x;
@@ -241,7 +241,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParam
         int acc = 0;
         uint32_t acc_phase = 0;
         uint32_t *amax_s = reinterpret_cast<uint32_t *>(base_ptr + L::kAmax);
-        int buf = 0;  // exchange buffer, flipped every 16-token chunk (across tiles too): a warp may run one chunk ahead of its partner
+        int buf = 0;  // exchange buffer, flipped every step (across tiles too): a warp may run one step ahead of its partner
         for (int round = 0;; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
             if (tile >= total_tiles) break;
@@ -352,9 +352,9 @@ int launch_grouped_gemm_tc_mx(const MxGemmArgs &a, cudaStream_t stream) {
     p.handover_per_token_tile = a.handover_per_token_tile;
 
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
-    // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots do not hide the walk:
-    // 16 tokens of 32 bf16 experts of 1024 x 1024, top 4, 50.7 -> 48.9 us; with longer K or one tile per CTA the queue costs
-    // (100 tokens of 128 experts of 4096 x 1536, top 8, 720 -> 731, the tiny layer 19.2 -> 19.7).
+    // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots (of 128 here) do not hide the walk.  Without / with:
+    // 16 tokens of 128 experts of 512 x 512, top 8, 44.4 / 39.1 us; 64 of 32 of 1024 x 1024, top 4, 45.2 / 43.1; of 2048 x 2048 88.9 /
+    // 88.1; 100 tokens of 128 of 4096 x 1536, top 8, 393.7 / 397.0.
     const bool queued = max_tiles > sms && a.K <= 1024;
     if (queued) return a.swiglu ? dispatch<true, true>(a.nt_max, maps, p, grid, stream) : dispatch<false, true>(a.nt_max, maps, p, grid, stream);
     return a.swiglu ? dispatch<true, false>(a.nt_max, maps, p, grid, stream) : dispatch<false, false>(a.nt_max, maps, p, grid, stream);

@@ -73,7 +73,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     constexpr int kFeatPerCta = SWIGLU ? kTileM / 2 : kTileM;
     constexpr int kFeatPerSlab = 2 * kFeatPerCta;
     constexpr int kFeatPerTile = SLABS * kFeatPerSlab;
-    chain_release();  // the next kernel of the forward call may be scheduled; it waits for this grid to finish
+    chain_release();  // the next kernel of the forward call may be scheduled; it waits for what it needs of this grid
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -117,7 +117,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const Kerne
     cluster_sync_all();  // the peer's barriers exist before anything can signal them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    // everything above overlapped the previous kernel; its results are read from here on
+    // everything above overlapped the kernels in front; from here on there is a schedule (the token side waits for more)
     const bool started = gemm_chain_start(p.handover_role, p.handover, abort_flag, p.status);
     const int total_tiles = started ? p.tile_prefix[p.E] * p.n_feature_tiles : 0;
     const int n_pairs = gridDim.x >> 1, pair = blockIdx.x >> 1;

@@ -19,7 +19,7 @@ constexpr int kStatusInts = 4;          // status word: {status, site, aux0, aux
 constexpr int kDoneCounterInt = 4;      // int index, in the status word's zeroed padding, of the count of finished blocks
                                         // (of the fused router, or of the scan over the chunks)
 // A forward call's status region is larger and also holds the hand-over to and between its two GEMMs (all zeroed when the
-// call opens, by a memset or by its one-block router): a flag the router raises once the tile schedule is complete, and per
+// call opens, by a memset or by a one-block or cluster router): a flag the router raises once the tile schedule is complete, and per
 // expert a count of finished gate/up epilogue passes.  With them both GEMMs fetch weights as soon as there is a schedule, and
 // the down GEMM starts on the SMs the gate/up GEMM has already left, expert by expert, instead of waiting for its whole grid.
 constexpr int kStatusBytesRoute = 256;

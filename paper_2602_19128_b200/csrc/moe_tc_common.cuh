@@ -122,12 +122,6 @@ __device__ __forceinline__ void ring_advance(int &stage, uint32_t &phase, int n)
     phase ^= (uint32_t)(uses / kStages) & 1u;
     stage = uses % kStages;
 }
-// Bounded wait by a whole warp; the result is made uniform.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status,
-                                               int site) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, site));
-}
-
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
