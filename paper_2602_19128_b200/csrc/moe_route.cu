@@ -344,12 +344,13 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
     my_w = __fmul_rn(__fdiv_rn(my_s, denom), rp.scale);
 }
 
+constexpr uint32_t kNoIds = 0xFFFFFFFFu;
 // Routes tokens [t0, t1) of the block (warp w takes tokens t0 + w, t0 + w + n_warps, ...) and writes ids and weights;
-// hist, if given, collects the histogram over the resident experts (zeroed by the caller); with ids_local all tokens' ids are
-// left in the array at address ids_smem of the cluster's shared memory too (any value is an address, 0 among them).
+// hist, if given, collects the histogram over the resident experts (zeroed by the caller); all tokens' ids are left in the array
+// at address ids_smem of the cluster's shared memory too, if there is one (0 would be an address; kNoIds, misaligned, is none).
 __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, int t0, int t1, int E, int k, int local_offset,
                                              int n_local, const RouterParams &rp, int *topk_ids, float *topk_w, Candidates *cand,
-                                             int *hist, bool ids_local = false, uint32_t ids_smem = 0) {
+                                             int *hist, uint32_t ids_smem = kNoIds) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     for (int t = t0 + warp; t < t1; t += n_warps) {
         int my_id;
@@ -361,7 +362,7 @@ __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, i
         if (lane < k) {
             topk_ids[(size_t)t * k + lane] = my_id;
             topk_w[(size_t)t * k + lane] = my_w;
-            if (ids_local)
+            if (ids_smem != kNoIds)
                 asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(ids_smem + (uint32_t)(t * k + lane) * 4), "r"(my_id) : "memory");
             const int local = my_id - local_offset;  // only experts resident here are scheduled
             if (hist && local >= 0 && local < n_local) atomicAdd(&hist[local], 1);
@@ -371,6 +372,11 @@ __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, i
 
 // The tile schedule is in memory: a forward call's GEMMs, which may be resident already, start on it (gemm_chain_start).  By
 // one thread, behind a block barrier that follows the last write of the schedule.
+// A kernel in front of the call may have written the weights through the generic proxy, and no wait for a grid stands between it
+// and the GEMMs' first TMA copies of them, only this flag: the thread that will raise it links the two by a proxy fence
+// (fence_weights), behind its own wait for what is in front and far ahead of the flag, where it costs nothing (in front of the
+// copies it cost 0.15 us of the tiny layer's 19.6).  The token side has a fence of its own (handover_wait_expert).
+__device__ __forceinline__ void fence_weights() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void raise_schedule_flag(int *status) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(status + kHandoverFlagInt), "r"(1) : "memory");
 }
@@ -519,6 +525,7 @@ route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_qu
     const int e = group < groups ? ((one_block ? group : (int)blockIdx.x) * 32 + lane) : E;  // (warps left over: no expert)
     chain_release();
     chain_wait();
+    if (threadIdx.x == 0) fence_weights();
     const int per = (n_chunks + warps_per_group - 1) / warps_per_group;
     const int b_begin = min(n_chunks, share * per), b_end = min(n_chunks, b_begin + per);
     const bool one_batch = per <= kScanBatch;  // then the counts stay in registers between the passes
@@ -691,7 +698,8 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
         chain_release();
         chain_wait();
     }
-    uint32_t ids_smem = 0;
+    if (tid == kFusedThreads - 1) fence_weights();
+    uint32_t ids_smem = kNoIds;
     if (ids_local) {
         ids_smem = (uint32_t)__cvta_generic_to_shared(ids_here);
         if (cluster) {
@@ -700,7 +708,7 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
         }
     }
     const int t0 = blockIdx.x * tokens_per_block;
-    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr, ids_local, ids_smem);
+    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr, ids_smem);
     if (cluster) {
         __syncwarp();
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

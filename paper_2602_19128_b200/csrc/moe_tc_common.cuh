@@ -337,9 +337,6 @@ __device__ __forceinline__ bool gemm_chain_start(int role, int *handover, volati
         bool ok = true;
         if (threadIdx.x == 0) ok = poll_at_least(handover + kHandoverFlagInt, 1, abort_flag, status, kSiteHandoverFlag);
         __syncthreads();
-        // A kernel in front of the call may have written the weights through the generic proxy, and no wait for a grid stands
-        // between it and the first copies of warp 0, only the flag.  (The token side has its fence in handover_wait_expert.)
-        if (threadIdx.x < 32) asm volatile("fence.proxy.async.global;" ::: "memory");
         return !*abort_flag && ok;
     }
     chain_wait();
