@@ -13,8 +13,8 @@
 // microsecond a token slot takes to arrive from L2: 1030 cycles per slot.  A pair's CTA takes in half of the tokens and keeps
 // six token slots, two per converted one.  333 Mixtral-shaped tokens 338 -> 311 us, 2000 tokens 1380 -> 1186 us, 4096 tokens
 // of 128 experts of 4096 x 1536 1559 -> 1330 us.  What bounds it now: a slot takes 620 to 750 cycles, and the MMA thread
-// never waits for an operand there, so it is the eight MMAs (about 77 cycles each at N = 96, where the shape asks for 48: why is not established); the converters' ALU and FMA
-// pipes are half busy beside them.
+// never waits for an operand there, so it is the eight MMAs (about 77 cycles each at N = 96, where the shape asks for 48: why
+// is not established); the converters' ALU and FMA pipes are half busy beside them.
 //
 // Pair protocol (rank 0 = leader), as in the bf16 pair kernel (moe_gemm_tc_pair.cu):
 //   q_full, q_empty      each CTA's own weight ring, between its weight producer and its converters
