@@ -30,7 +30,6 @@ constexpr unsigned kFullMask = 0xffffffffu;
 // Router and sort of 64 experts, top 2, a warp per token / two tokens: 4096 tokens 16.4 / 16.4 us, 1025 14.4 / 15.4; 8192
 // 19.5 / 18.4.
 constexpr int kRouteThreads = 1024, kRouteThreadsManyChunks = 512, kRouteSms = 148;
-constexpr int kLogitsPerLane = kMaxExperts / 32;
 
 // Order-preserving map from float to unsigned: a > b  <=>  ordered_key(a) > ordered_key(b) (for non-NaN values;
 // -0 is first folded into +0 so that the two compare equal, as the floats do).
@@ -40,17 +39,18 @@ __device__ __forceinline__ unsigned ordered_key(float f) {
 }
 
 // k rounds of a warp arg-max under the strict order (larger key first, ties to the lower expert index).  Expert
-// e = 32 i + lane has key[i] in its lane; entries with e >= E must hold key 0 and are never selected while a real
+// e = 32 i + lane has key[i] in its lane (kRegs = ceil(E / 32), rounded up to 1, 4 or 8); entries with e >= E must hold key 0 and are never selected while a real
 // candidate is left.  Each round: every lane finds its best remaining entry, one warp reduction gives the largest
 // key, a second one the lowest expert index among the lanes that hold it.  Lane j < k returns rank j's expert.
-__device__ __forceinline__ int select_top_k(const unsigned (&key)[kLogitsPerLane], int E, int k, int lane) {
+template <int kRegs>
+__device__ __forceinline__ int select_top_k(const unsigned (&key)[kRegs], int E, int k, int lane) {
     unsigned taken = 0;
     int my_id = 0;
     for (int j = 0; j < k; ++j) {
         unsigned best = 0;
         int best_e = INT_MAX;  // no candidate
 #pragma unroll
-        for (int i = 0; i < kLogitsPerLane; ++i) {
+        for (int i = 0; i < kRegs; ++i) {
             const int e = i * 32 + lane;
             const bool free_slot = e < E && !((taken >> i) & 1u);
             if (free_slot && (best_e == INT_MAX || key[i] > best)) { best = key[i]; best_e = e; }
@@ -79,14 +79,15 @@ struct Candidates {
 // of k short reductions instead of k long ones (8192 tokens: router and sort 43 -> 25 us, grouped 56 -> 33 us).
 // k = 1 is a single arg-max (route_topk_kernel, 1500 tokens of 32 experts: 5.8 -> 5.1 us).
 // Lane j < k returns rank j's expert with its key and score.
-__device__ __forceinline__ void select_candidates(const unsigned (&key)[kLogitsPerLane], const float (&score)[kLogitsPerLane], int E,
+template <int kRegs>
+__device__ __forceinline__ void select_candidates(const unsigned (&key)[kRegs], const float (&score)[kRegs], int E,
                                                   int k, int lane, Candidates *c, int &my_id, unsigned &my_key, float &my_score) {
     if (k == 1) {  // one arg-max
         unsigned best = key[0];
         int e = lane;
         float v = score[0];
 #pragma unroll
-        for (int i = 1; i < kLogitsPerLane; ++i)
+        for (int i = 1; i < kRegs; ++i)
             if (key[i] > best) { best = key[i]; e = i * 32 + lane; v = score[i]; }
         my_key = __reduce_max_sync(kFullMask, lane < E ? best : 0u);
         my_id = (int)__reduce_min_sync(kFullMask, lane < E && best == my_key ? (unsigned)e : (unsigned)INT_MAX);
@@ -102,7 +103,7 @@ __device__ __forceinline__ void select_candidates(const unsigned (&key)[kLogitsP
     } else {
         unsigned m = key[0];
 #pragma unroll
-        for (int i = 1; i < kLogitsPerLane; ++i) m = max(m, key[i]);
+        for (int i = 1; i < kRegs; ++i) m = max(m, key[i]);
         unsigned bound = 0;
         for (int j = 0; j < k; ++j) {
             bound = __reduce_max_sync(kFullMask, m);
@@ -110,7 +111,7 @@ __device__ __forceinline__ void select_candidates(const unsigned (&key)[kLogitsP
         }
         n = 0;
 #pragma unroll
-        for (int i = 0; i < kLogitsPerLane; ++i) {
+        for (int i = 0; i < kRegs; ++i) {
             const bool in = key[i] >= bound;  // (a bound of 0 takes all 256 slots: the fallback)
             const unsigned mask = __ballot_sync(kFullMask, in);
             const int at = n + __popc(mask & ((1u << lane) - 1u));
@@ -123,7 +124,7 @@ __device__ __forceinline__ void select_candidates(const unsigned (&key)[kLogitsP
             my_key = 0;
             my_score = 0.f;
 #pragma unroll
-            for (int i = 0; i < kLogitsPerLane; ++i) {  // expert my_id lives in lane my_id % 32, register my_id / 32
+            for (int i = 0; i < kRegs; ++i) {  // expert my_id lives in lane my_id % 32, register my_id / 32
                 const unsigned got_key = __shfl_sync(kFullMask, key[i], my_id & 31);
                 const float got_score = __shfl_sync(kFullMask, score[i], my_id & 31);
                 if ((my_id >> 5) == i) { my_key = got_key; my_score = got_score; }
@@ -151,12 +152,13 @@ __device__ __forceinline__ void select_candidates(const unsigned (&key)[kLogitsP
 // renormalised softmax weights.  Softmax's normaliser cancels in the renormalisation, so only the k selected
 // logits are exponentiated: w_j = exp(l_j - l_0) / sum_j' exp(l_j' - l_0), the sum in rank order.
 // Lane j < k returns rank j's expert and weight.
+template <int kRegs>
 __device__ __forceinline__ void route_one_token(const float *__restrict__ row, int E, int k, int lane, Candidates *cand, int &my_id,
                                                 float &my_w) {
-    float v[kLogitsPerLane];
-    unsigned key[kLogitsPerLane];
+    float v[kRegs];
+    unsigned key[kRegs];
 #pragma unroll
-    for (int i = 0; i < kLogitsPerLane; ++i) {
+    for (int i = 0; i < kRegs; ++i) {
         const int e = i * 32 + lane;
         v[i] = e < E ? row[e] : 0.f;
         key[i] = e < E ? ordered_key(v[i]) : 0u;
@@ -204,12 +206,13 @@ __device__ __forceinline__ void top2_merge(float &t1, float &t2, float o1, float
 // One token by one warp.  Expert e = 32 i + lane lives in register i of its lane; a group is G = E / n_group
 // consecutive experts, G a power of two: either a segment of G lanes within one register index (G <= 32) or all
 // lanes of G / 32 consecutive register indices.
+template <int kRegs>
 __device__ __forceinline__ void route_one_token_grouped(const float *__restrict__ row, int E, int k, int lane,
                                                         const RouterParams &rp, Candidates *cand, int &my_id, float &my_w) {
     const int G = E / rp.n_group;
-    float s[kLogitsPerLane], c[kLogitsPerLane];
+    float s[kRegs], c[kRegs];
 #pragma unroll
-    for (int i = 0; i < kLogitsPerLane; ++i) {
+    for (int i = 0; i < kRegs; ++i) {
         const int e = i * 32 + lane;
         s[i] = e < E ? sigmoid_fixed(row[e]) : 0.f;
         c[i] = e < E ? (rp.bias ? __fadd_rn(s[i], rp.bias[e]) : s[i]) : -INFINITY;
@@ -222,8 +225,9 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
         const bool b16 = (lane & 16) != 0, b8 = (lane & 8) != 0, b4 = (lane & 4) != 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {  // (a single score has no second: -inf)
-            const float o1 = __shfl_xor_sync(kFullMask, b16 ? c[i] : c[4 + i], 16);
-            a1[i] = b16 ? c[4 + i] : c[i];
+            const float lo = i < kRegs ? c[i % kRegs] : -INFINITY, hi = 4 + i < kRegs ? c[(4 + i) % kRegs] : -INFINITY;
+            const float o1 = __shfl_xor_sync(kFullMask, b16 ? lo : hi, 16);
+            a1[i] = b16 ? hi : lo;
             a2[i] = -INFINITY;
             top2_merge(a1[i], a2[i], o1, -INFINITY);
         }
@@ -256,24 +260,24 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
         }
         const unsigned eligible = __ballot_sync(kFullMask, gid < rp.n_group && rank < rp.topk_group);  // group g: bit 4 g
 #pragma unroll
-        for (int i = 0; i < kLogitsPerLane; ++i)
+        for (int i = 0; i < kRegs; ++i)
             if (!((eligible >> (4 * i)) & 1u)) c[i] = -INFINITY;
     } else {
         // the two largest biased scores of every group
-        float t1[kLogitsPerLane], t2[kLogitsPerLane];
+        float t1[kRegs], t2[kRegs];
 #pragma unroll
-        for (int i = 0; i < kLogitsPerLane; ++i) {
+        for (int i = 0; i < kRegs; ++i) {
             t1[i] = c[i];
             t2[i] = -INFINITY;
         }
         if (G > 32) {  // registers of the same group first
             const int m = G >> 5;
 #pragma unroll
-            for (int i = 0; i < kLogitsPerLane; ++i) {
+            for (int i = 0; i < kRegs; ++i) {
                 const int first = i & ~(m - 1);
                 float a1 = -INFINITY, a2 = -INFINITY;
 #pragma unroll
-                for (int j = 0; j < kLogitsPerLane; ++j)
+                for (int j = 0; j < kRegs; ++j)
                     if (j >= first && j < first + m) top2_merge(a1, a2, c[j], -INFINITY);
                 t1[i] = a1;
                 t2[i] = a2;
@@ -281,21 +285,21 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
         }
         for (int off = (G < 32 ? G : 32) >> 1; off > 0; off >>= 1) {
 #pragma unroll
-            for (int i = 0; i < kLogitsPerLane; ++i) {
+            for (int i = 0; i < kRegs; ++i) {
                 const float o1 = __shfl_xor_sync(kFullMask, t1[i], off), o2 = __shfl_xor_sync(kFullMask, t2[i], off);
                 top2_merge(t1[i], t2[i], o1, o2);
             }
         }
-        float gs[kLogitsPerLane];  // score of the group that holds this register's expert
+        float gs[kRegs];  // score of the group that holds this register's expert
 #pragma unroll
-        for (int i = 0; i < kLogitsPerLane; ++i) gs[i] = G >= 2 ? __fadd_rn(t1[i], t2[i]) : t1[i];
+        for (int i = 0; i < kRegs; ++i) gs[i] = G >= 2 ? __fadd_rn(t1[i], t2[i]) : t1[i];
         // a group is eligible if fewer than topk_group groups rank before it (ties to the lower group index)
         if (rp.n_group <= 32) {
             // lane g fetches group g's score from the lane and register that hold the group's first expert ...
             const int first = lane < rp.n_group ? lane * G : 0;
             float mine = 0.f;
 #pragma unroll
-            for (int i = 0; i < kLogitsPerLane; ++i) {
+            for (int i = 0; i < kRegs; ++i) {
                 const float got = __shfl_sync(kFullMask, gs[i], first & 31);
                 if ((first >> 5) == i) mine = got;
             }
@@ -307,34 +311,34 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
             }
             const unsigned eligible = __ballot_sync(kFullMask, lane < rp.n_group && rank < rp.topk_group);
 #pragma unroll
-            for (int i = 0; i < kLogitsPerLane; ++i)
+            for (int i = 0; i < kRegs; ++i)
                 if (!((eligible >> ((i * 32 + lane) / G)) & 1u)) c[i] = -INFINITY;
         } else {  // more groups than lanes (groups of at most 4 experts): every register ranks its own group
-            int rank[kLogitsPerLane];
+            int rank[kRegs];
 #pragma unroll
-            for (int i = 0; i < kLogitsPerLane; ++i) rank[i] = 0;
+            for (int i = 0; i < kRegs; ++i) rank[i] = 0;
             for (int g = 0; g < rp.n_group; ++g) {
                 const int e0 = g * G, ip = e0 >> 5;
                 float pick = gs[0];
 #pragma unroll
-                for (int i = 1; i < kLogitsPerLane; ++i) pick = ip == i ? gs[i] : pick;
+                for (int i = 1; i < kRegs; ++i) pick = ip == i ? gs[i] : pick;
                 const float val = __shfl_sync(kFullMask, pick, e0 & 31);
 #pragma unroll
-                for (int i = 0; i < kLogitsPerLane; ++i) {
+                for (int i = 0; i < kRegs; ++i) {
                     const int gid = (i * 32 + lane) / G;
                     rank[i] += (val > gs[i] || (val == gs[i] && g < gid)) ? 1 : 0;
                 }
             }
 #pragma unroll
-            for (int i = 0; i < kLogitsPerLane; ++i)
+            for (int i = 0; i < kRegs; ++i)
                 if (rank[i] >= rp.topk_group) c[i] = -INFINITY;
         }
     }
 
     // top-k of the eligible biased scores; the weight uses the unbiased score of the selected expert
-    unsigned key[kLogitsPerLane];
+    unsigned key[kRegs];
 #pragma unroll
-    for (int i = 0; i < kLogitsPerLane; ++i) key[i] = i * 32 + lane < E ? ordered_key(c[i]) : 0u;
+    for (int i = 0; i < kRegs; ++i) key[i] = i * 32 + lane < E ? ordered_key(c[i]) : 0u;
     unsigned my_key;
     float my_s;
     select_candidates(key, s, E, k, lane, cand, my_id, my_key, my_s);
@@ -346,24 +350,26 @@ __device__ __forceinline__ void route_one_token_grouped(const float *__restrict_
 
 constexpr uint32_t kNoIds = 0xFFFFFFFFu;
 // Routes tokens [t0, t1) of the block (warp w takes tokens t0 + w, t0 + w + n_warps, ...) and writes ids and weights;
-// hist, if given, collects the histogram over the resident experts (zeroed by the caller); all tokens' ids are left in the array
-// at address ids_smem of the cluster's shared memory too, if there is one (0 would be an address; kNoIds, misaligned, is none).
+// hist, if given, collects the histogram over the resident experts (zeroed by the caller); all tokens' ids are left, a byte each,
+// in the array at address ids_smem of the cluster's shared memory too, if there is one (0 would be an address; kNoIds is none).
+template <int kRegs>
 __device__ __forceinline__ void route_tokens(const float *__restrict__ logits, int t0, int t1, int E, int k, int local_offset,
                                              int n_local, const RouterParams &rp, int *topk_ids, float *topk_w, Candidates *cand,
                                              int *hist, uint32_t ids_smem = kNoIds) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+#pragma unroll 1
     for (int t = t0 + warp; t < t1; t += n_warps) {
         int my_id;
         float my_w;
         if (rp.grouped)
-            route_one_token_grouped(logits + (size_t)t * E, E, k, lane, rp, &cand[warp], my_id, my_w);
+            route_one_token_grouped<kRegs>(logits + (size_t)t * E, E, k, lane, rp, &cand[warp], my_id, my_w);
         else
-            route_one_token(logits + (size_t)t * E, E, k, lane, &cand[warp], my_id, my_w);
+            route_one_token<kRegs>(logits + (size_t)t * E, E, k, lane, &cand[warp], my_id, my_w);
         if (lane < k) {
             topk_ids[(size_t)t * k + lane] = my_id;
             topk_w[(size_t)t * k + lane] = my_w;
             if (ids_smem != kNoIds)
-                asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(ids_smem + (uint32_t)(t * k + lane) * 4), "r"(my_id) : "memory");
+                asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(ids_smem + (uint32_t)(t * k + lane)), "r"(my_id) : "memory");
             const int local = my_id - local_offset;  // only experts resident here are scheduled
             if (hist && local >= 0 && local < n_local) atomicAdd(&hist[local], 1);
         }
@@ -381,7 +387,7 @@ __device__ __forceinline__ void raise_schedule_flag(int *status) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(status + kHandoverFlagInt), "r"(1) : "memory");
 }
 
-template <int kThreads>
+template <int kThreads, int kRegs>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 route_topk_kernel(const float *__restrict__ logits, int T, int E, int k, int local_offset, int n_local,
                   const RouterParams rp, int *__restrict__ topk_ids, float *__restrict__ topk_w,
@@ -393,109 +399,125 @@ route_topk_kernel(const float *__restrict__ logits, int T, int E, int k, int loc
     __syncthreads();
     chain_wait();
     const int t0 = blockIdx.x * kRouteTokensPerBlock;
-    route_tokens(logits, t0, min(T, t0 + kRouteTokensPerBlock), E, k, local_offset, n_local, rp, topk_ids, topk_w, cand, hist);
+    route_tokens<kRegs>(logits, t0, min(T, t0 + kRouteTokensPerBlock), E, k, local_offset, n_local, rp, topk_ids, topk_w, cand, hist);
     __syncthreads();
     for (int e = threadIdx.x; e < n_local; e += kThreads) chunk_counts[(size_t)blockIdx.x * n_local + e] = hist[e];
 }
 
-// Exclusive scan over threads 0..255 of the block (wider blocks may call it; their other threads pass 0
-// and ignore the result); returns the exclusive prefix, total in *total.
-__device__ __forceinline__ int block_exclusive_scan_256(int value, int *warp_sums, int *total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = value;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int n = __shfl_up_sync(kFullMask, incl, off);
-        if (lane >= off) incl += n;
-    }
-    if (lane == 31 && warp < 8) warp_sums[warp] = incl;
-    __syncthreads();
-    int base = 0, sum = 0;
-#pragma unroll
-    for (int wi = 0; wi < 8; ++wi) {
-        const int ws = warp_sums[wi];
-        if (wi < warp) base += ws;
-        sum += ws;
-    }
-    __syncthreads();
-    *total = sum;
-    return base + incl - value;
-}
-
 constexpr int kScanThreads = 1024;
 
+// Inclusive prefix sum over the lanes of a warp.
+__device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int n = __shfl_up_sync(kFullMask, v, off);
+        if (lane >= off) v += n;
+    }
+    return v;
+}
+
 // Schedule phase, run by one block of 1024 threads: exclusive scan over the experts' row counts and the token-tile
-// schedule.  `count` is expert threadIdx.x's rows in threads 0..E-1 and 0 in the others; returns the first row of
-// expert threadIdx.x (threads 0..255).
-struct ScheduleShared {
-    int warp_sums[8];
-    __align__(16) int counts[kMaxExperts];
-    int tiles_at[kMaxExperts], part_sums[kScanThreads];
+// schedule.  `count` is expert threadIdx.x's rows in threads 0..E-1 and 0 in the others; `started(row)` is called by
+// thread e < E with expert e's first row, and what it writes is visible to the block on return.  The schedule's flag is
+// raised (by the first thread of the last warp) as soon as the schedule is in memory.
+// This is a chain of short steps, between the router's last id and everything else of the call: two block barriers, the
+// first scan and the ranking side by side, the second scan by one warp, beside whatever the caller does next.  (With a
+// barrier per step -- twelve -- and a thousand threads counting spans of a few ids, the tiny layer's 32 ids took 3.9 us
+// from the last id to the flag; now 2.5.)  Every instruction runs once or a few times per call, so what is not a loop costs its
+// fetch more than its issue: loops are unrolled only where loads have to overlap.
+// The schedule's row quantum with ceil(2^32 / q): the rows of a tile (384 at most) are rounded up without a division.
+struct RowQuantum {
+    int q;
+    unsigned inverse;
+    explicit RowQuantum(int quantum) : q(quantum), inverse((unsigned)(((1ull << 32) + quantum - 1) / quantum)) {}
 };
-__device__ __forceinline__ int schedule_phase(int count, int E, int nt_max, int row_quantum, int *expert_offsets, int *tile_prefix,
-                                              int *tile_order, int *tile_rows, ScheduleShared &sh) {
-    const int e = threadIdx.x;
-    const bool lane_of_scan = e < kMaxExperts;
-    int *counts = sh.counts, *tiles_at = sh.tiles_at, *part_sums = sh.part_sums, *warp_sums = sh.warp_sums;
-    if (lane_of_scan) {
-        counts[e] = e < E ? count : -1;
-        tiles_at[e] = 0;
-    }
-    // token tiles of this expert: one tile if it fits under nt_max; otherwise as few as fit under min(nt_max, 256) --
-    // a wide bound (320 / 384) exists to keep an expert in ONE pass over its weights, and consecutive tiles wider than
-    // half of tensor memory cannot overlap their epilogues, so experts that need several tiles get 256-row ones --
-    // evenly sized, rounded up to the row quantum
-    // (16 rows, the MMA's N granularity; the MX path with a bound of up to 256 passes its tile size, so that every tile
-    // is exactly that many rows)
-    int n_tiles = 0, rows = 0;
-    if (count > 0) {
-        const int multi = nt_max > 256 ? 256 : nt_max;
-        n_tiles = count <= nt_max ? 1 : (count + multi - 1) / multi;
-        rows = (((count + n_tiles - 1) / n_tiles) + row_quantum - 1) / row_quantum * row_quantum;
-    }
-    int total_rows, total_tiles;
-    const int row_start = block_exclusive_scan_256(count, warp_sums, &total_rows);  // (syncs: counts[] is visible)
-    // Schedule order: experts with more rows first (ties to the lower index), so that tiles of similar
-    // cost are adjacent and the GEMMs' static tile assignment stays balanced; the small tiles come last.
-    // (all-pairs ranking, E^2 comparisons: every part of the block takes a share of the opponents)
-    {
-        const int pe = threadIdx.x % kMaxExperts, part = threadIdx.x / kMaxExperts, n_parts = blockDim.x / kMaxExperts;
-        part_sums[threadIdx.x] = 0;
-        if (pe < E) {
-            const int mine = counts[pe];
-            // (four opponents per load; counts past E are -1 and never rank before a real one)
-            const int per = ((E + n_parts - 1) / n_parts + 3) & ~3, o_end = min(kMaxExperts, (part + 1) * per);
-            int before = 0;
-#pragma unroll 4
-            for (int o = part * per; o < o_end; o += 4) {
-                const int4 c = *reinterpret_cast<const int4 *>(&counts[o]);
-                before += (c.x > mine || (c.x == mine && o < pe)) ? 1 : 0;
-                before += (c.y > mine || (c.y == mine && o + 1 < pe)) ? 1 : 0;
-                before += (c.z > mine || (c.z == mine && o + 2 < pe)) ? 1 : 0;
-                before += (c.w > mine || (c.w == mine && o + 3 < pe)) ? 1 : 0;
-            }
-            part_sums[threadIdx.x] = before;
+struct ScheduleShared {
+    int warp_sums[kMaxExperts / 32];
+    __align__(16) unsigned keys[kMaxExperts];
+    __align__(16) int tiles_at[kMaxExperts];
+    int tiles[kMaxExperts];
+};
+template <typename Started>
+__device__ __forceinline__ void schedule_phase(int count, int E, int nt_max, RowQuantum row_quantum, int *expert_offsets, int *tile_prefix,
+                                               int *tile_order, int *tile_rows, int *status, ScheduleShared &sh, Started started) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int incl = 0;
+    if (tid < kMaxExperts) {
+        // More rows first, ties to the lower index: one unsigned number per expert (past 2^24 rows the order is the index's).
+        sh.keys[tid] = ((unsigned)min(count, 0xFFFFFF) << 8) | (unsigned)(kMaxExperts - 1 - tid);
+        incl = warp_inclusive_scan(count, lane);
+        if (lane == 31) sh.warp_sums[warp] = incl;
+        // token tiles of this expert: one tile if it fits under nt_max; otherwise as few as fit under min(nt_max, 256) --
+        // a wide bound (320 / 384) exists to keep an expert in ONE pass over its weights, and consecutive tiles wider than
+        // half of tensor memory cannot overlap their epilogues, so experts that need several tiles get 256-row ones --
+        // evenly sized, rounded up to the row quantum
+        // (16 rows, the MMA's N granularity; the MX path with a bound of up to 256 passes its tile size, so that every tile
+        // is exactly that many rows)
+        int n_tiles = 0, rows = 0;
+        if (count > 0) {
+            const int multi = nt_max > 256 ? 256 : nt_max;
+            n_tiles = count <= nt_max ? 1 : (count + multi - 1) / multi;
+            const int per_tile = n_tiles == 1 ? count : (count + n_tiles - 1) / n_tiles;
+            rows = (int)__umulhi((unsigned)(per_tile + row_quantum.q - 1), row_quantum.inverse) * row_quantum.q;
         }
-        __syncthreads();
-        if (e < E) {
-            int pos = 0;
-            for (int p = 0; p < n_parts; ++p) pos += part_sums[p * kMaxExperts + e];
-            tiles_at[pos] = n_tiles;
-            tile_order[pos] = e;
-        }
+        sh.tiles[tid] = n_tiles;
+        if (tid < E) tile_rows[tid] = rows; else sh.tiles_at[tid] = 0;
     }
     __syncthreads();
-    const int tile_start = block_exclusive_scan_256(lane_of_scan ? tiles_at[e] : 0, warp_sums, &total_tiles);
-    if (e < E) {
-        expert_offsets[e] = row_start;
-        tile_prefix[e] = tile_start;  // indexed by schedule position
-        tile_rows[e] = rows;
+    // Schedule order: experts with more rows first (ties to the lower index), so that tiles of similar cost are adjacent and
+    // the GEMMs' static tile assignment stays balanced; the small tiles come last.  All-pairs ranking, E^2 comparisons: four
+    // neighbouring threads share an expert's opponents, four per load.
+    {
+        const int e = tid >> 2, part = tid & 3;
+        int before = 0;
+        if (e < E) {
+            const unsigned mine = sh.keys[e];
+#pragma unroll 2
+            for (int o = part * 4; o < E; o += 16) {  // (keys past E rank behind every real one)
+                const uint4 c = *reinterpret_cast<const uint4 *>(&sh.keys[o]);
+                before += (c.x > mine) + (c.y > mine) + (c.z > mine) + (c.w > mine);
+            }
+        }
+        before += __shfl_xor_sync(kFullMask, before, 1);
+        before += __shfl_xor_sync(kFullMask, before, 2);
+        if (e < E && part == 0) {
+            sh.tiles_at[before] = sh.tiles[e];
+            tile_order[before] = e;
+        }
     }
-    if (e == 0) {
-        expert_offsets[E] = total_rows;
-        tile_prefix[E] = total_tiles;
+    if (tid < kMaxExperts) {
+        int base = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < kMaxExperts / 32; ++w) {
+            const int v = sh.warp_sums[w];
+            if (w < warp) base += v;
+            total += v;
+        }
+        if (tid < E) {
+            const int row = base + incl - count;
+            expert_offsets[tid] = row;
+            started(row);
+        }
+        if (tid == 0) expert_offsets[E] = total;
     }
-    return row_start;
+    __syncthreads();
+    if (warp == kScanThreads / 32 - 1) {  // tile counts in schedule order -> first tile of each position
+        int v[8], sum = 0;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            *reinterpret_cast<int4 *>(&v[4 * i]) = *reinterpret_cast<const int4 *>(&sh.tiles_at[lane * 8 + 4 * i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sum += v[i];
+        int at = warp_inclusive_scan(sum, lane) - sum;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (lane * 8 + i <= E) tile_prefix[lane * 8 + i] = at;
+            at += v[i];
+        }
+        if (E == kMaxExperts && lane == 31) tile_prefix[E] = at;
+        __syncwarp();
+        if (lane == 0) raise_schedule_flag(status);
+    }
 }
 
 // Scan over the chunks, in groups of 32 experts: a warp takes a contiguous share of the chunks for one group, lane l its
@@ -514,7 +536,7 @@ __host__ __device__ inline int scan_warps_per_group(int n_chunks, int groups) {
     return useful < most ? useful : most;
 }
 __global__ void __launch_bounds__(kScanThreads)
-route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_quantum, int *expert_offsets,
+route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, RowQuantum row_quantum, int *expert_offsets,
                   int *tile_prefix, int *tile_order, int *tile_rows, int *totals, int *status) {
     __shared__ int partial[kScanWarps][32], all_totals[kMaxExperts];
     __shared__ ScheduleShared sh;
@@ -525,7 +547,7 @@ route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_qu
     const int e = group < groups ? ((one_block ? group : (int)blockIdx.x) * 32 + lane) : E;  // (warps left over: no expert)
     chain_release();
     chain_wait();
-    if (threadIdx.x == 0) fence_weights();
+    if (threadIdx.x == kScanThreads - 32) fence_weights();  // (the thread that raises the schedule's flag)
     const int per = (n_chunks + warps_per_group - 1) / warps_per_group;
     const int b_begin = min(n_chunks, share * per), b_end = min(n_chunks, b_begin + per);
     const bool one_batch = per <= kScanBatch;  // then the counts stay in registers between the passes
@@ -582,9 +604,7 @@ route_scan_kernel(int *chunk_counts, int n_chunks, int E, int nt_max, int row_qu
         if ((int)threadIdx.x < E) count = __ldcg(&totals[threadIdx.x]);
         __syncthreads();  // (the totals may sit where the schedule is written)
     }
-    schedule_phase(count, E, nt_max, row_quantum, expert_offsets, tile_prefix, tile_order, tile_rows, sh);
-    __syncthreads();
-    if (threadIdx.x == 0) raise_schedule_flag(status);
+    schedule_phase(count, E, nt_max, row_quantum, expert_offsets, tile_prefix, tile_order, tile_rows, status, sh, [](int) {});
 }
 
 // Stable scatter of 32 consecutive assignments by one warp: lane l holds assignment a (flat order) of local expert e;
@@ -667,38 +687,50 @@ constexpr int kFusedWarps = kFusedThreads / 32;
 // the ids through L2.  Beyond, eight SMs would have more than a token per warp, and up to 64 blocks count themselves.
 // Layers, 64 blocks / a cluster: 100 tokens of 8 experts of 256 x 512, top 2, 23.6 / 21.5 us; 64 tokens of 32 of 1024 x 1024,
 // top 4, 57.6 / 54.8; 64 tokens on 32 of 256 bf16 experts of 7168 x 2048, top 8, grouped router, 361.9 / 355.7.
-constexpr int kFusedOneBlockTokens = 16, kFusedClusterTokens = 256, kFusedCluster = 8, kFusedIds = 2048;
-constexpr int kFusedGroups = 8;  // groups of 32 assignments a warp keeps in registers between counting and walking
+constexpr int kFusedOneBlockTokens = 16, kFusedClusterTokens = 256, kFusedCluster = 8, kFusedClusterIds = 2048;
+constexpr int kFusedIds = 8192;  // ids the sorting block holds in shared memory, a byte each; further ones are read where they lie
+// Spans of the flat order, one per sorting warp: at least four groups of 32 each, since every further span is one more count
+// per expert to add up.
+constexpr int kFusedSpanGroups = 4;
+inline int fused_spans(int A) {
+    const int useful = (A + 32 * kFusedSpanGroups - 1) / (32 * kFusedSpanGroups);
+    return useful < kFusedWarps ? useful : kFusedWarps;
+}
 
+template <int kRegs>
 __global__ void __launch_bounds__(kFusedThreads)
 route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int local_offset, int n_local, int nt_max,
-                   int row_quantum, int tokens_per_block, const RouterParams rp, int *topk_ids, float *topk_w, int *expert_offsets,
-                   int *tile_prefix, int *tile_order, int *tile_rows, int *sorted_to_flat, int *flat_to_sorted, int *status,
-                   int status_ints) {
+                   RowQuantum row_quantum, int tokens_per_block, int spans, int span, const RouterParams rp, int *topk_ids, float *topk_w,
+                   int *expert_offsets, int *tile_prefix, int *tile_order, int *tile_rows, int *sorted_to_flat, int *flat_to_sorted,
+                   int *status, int status_ints) {
     __shared__ ScheduleShared sh;
     __shared__ union Scratch {
         Candidates cand[kFusedWarps];        // while routing
         int next[kFusedWarps][kMaxExperts];  // then: counts, start positions, cursors of each warp's span
     } u;
-    __shared__ int is_last, ids_here[kFusedIds];
+    __shared__ int is_last;
+    __shared__ __align__(16) unsigned char ids_here[kFusedIds];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool ids_local = status_ints > 0;  // one block or a cluster: the first block sorts from its shared memory
     const bool cluster = ids_local && gridDim.x > 1;
     if (cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // (the blocks have started)
     if (ids_local) {
-        // The first block zeroes the call's status region, before any kernel that looks at it may start.
+        // The first block's last warp zeroes the call's status region, before any kernel that looks at it may start; the
+        // others go on (a block that waited for the zeroes routed its tokens half a microsecond later).
         chain_wait();
-        if (blockIdx.x == 0) {
-            for (int i = tid; i < status_ints; i += kFusedThreads) status[i] = 0;
-            __threadfence();
+        if (warp == kFusedWarps - 1) {
+            if (blockIdx.x == 0) {
+                for (int i = lane; i < status_ints / 4; i += 32) reinterpret_cast<int4 *>(status)[i] = make_int4(0, 0, 0, 0);
+                __threadfence();
+                __syncwarp();
+            }
+            if (lane == 0) chain_release();
         }
-        __syncthreads();
-        chain_release();
     } else {
         chain_release();
         chain_wait();
     }
-    if (tid == kFusedThreads - 1) fence_weights();
+    if (tid == kFusedThreads - 32) fence_weights();  // (the thread that raises the schedule's flag)
     uint32_t ids_smem = kNoIds;
     if (ids_local) {
         ids_smem = (uint32_t)__cvta_generic_to_shared(ids_here);
@@ -708,7 +740,7 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
         }
     }
     const int t0 = blockIdx.x * tokens_per_block;
-    route_tokens(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr, ids_smem);
+    route_tokens<kRegs>(logits, t0, min(T, t0 + tokens_per_block), E, k, local_offset, n_local, rp, topk_ids, topk_w, u.cand, nullptr, ids_smem);
     if (cluster) {
         __syncwarp();
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -724,69 +756,47 @@ route_fused_kernel(const float *__restrict__ logits, int T, int E, int k, int lo
     } else {
         __syncthreads();
     }
-    // this warp's span of the assignments: whole groups of 32
     const int A = T * k;
-    const int span = ((A + 32 * kFusedWarps - 1) / (32 * kFusedWarps)) * 32;
+    if (!ids_local) {  // this block's copy of all ids, in one round trip
+        const int n = min(A, kFusedIds);
+#pragma unroll 4
+        for (int a = tid; a < n; a += kFusedThreads) ids_here[a] = (unsigned char)__ldcg(&topk_ids[a]);
+        __syncthreads();
+    }
+    auto id_of = [&](int a) { return (a < kFusedIds ? (int)ids_here[a] : __ldcg(&topk_ids[a])) - local_offset; };
+    // this warp's span of the assignments: whole groups of 32 (the first `spans` warps have one)
     const int a0 = min(A, warp * span), a1 = min(A, a0 + span);
-    int ids[kFusedGroups];
-#pragma unroll
-    for (int g = 0; g < kFusedGroups; ++g) {
-        const int a = a0 + g * 32 + lane;
-        ids[g] = a < a1 ? (ids_local ? ids_here[a] : __ldcg(&topk_ids[a])) - local_offset : -1;
-    }
     int *next = u.next[warp];
-    for (int e = lane; e < n_local; e += 32) next[e] = 0;
-    __syncwarp();
-#pragma unroll
-    for (int g = 0; g < kFusedGroups; ++g)
-        if (ids[g] >= 0 && ids[g] < n_local) atomicAdd(&next[ids[g]], 1);
-    for (int a = a0 + kFusedGroups * 32 + lane; a < a1; a += 32) {
-        const int e = __ldcg(&topk_ids[a]) - local_offset;
-        if (e >= 0 && e < n_local) atomicAdd(&next[e], 1);
-    }
-    __syncthreads();
-    // counts -> rows of earlier spans, four parts of eight spans per expert
-    constexpr int kParts = kFusedThreads / kMaxExperts, kSpansPerPart = kFusedWarps / kParts;
-    const int pe = tid % kMaxExperts, part = tid / kMaxExperts;
-    int c[kSpansPerPart], sum = 0, count = 0, run = 0;
-#pragma unroll
-    for (int i = 0; i < kSpansPerPart; ++i) {
-        c[i] = pe < n_local ? u.next[part * kSpansPerPart + i][pe] : 0;
-        sum += c[i];
-    }
-    sh.part_sums[tid] = sum;
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kParts; ++q) {
-        const int v = sh.part_sums[q * kMaxExperts + pe];
-        if (q < part) run += v;
-        count += v;
-    }
-    __syncthreads();  // (part_sums is used again)
-    const int row_start = schedule_phase(tid < n_local ? count : 0, n_local, nt_max, row_quantum, expert_offsets, tile_prefix,
-                                         tile_order, tile_rows, sh);
-    __syncthreads();
-    if (tid == kFusedThreads - 1) raise_schedule_flag(status);  // (a thread of the warp that has the least to sort)
-    if (tid < kMaxExperts) sh.counts[tid] = row_start;
-    __syncthreads();
-    if (pe < n_local) {
-        run += sh.counts[pe];
-#pragma unroll
-        for (int i = 0; i < kSpansPerPart; ++i) {
-            u.next[part * kSpansPerPart + i][pe] = run;
-            run += c[i];
+    if (warp < spans) {
+#pragma unroll 1
+        for (int e = lane; e < n_local; e += 32) next[e] = 0;
+        __syncwarp();
+#pragma unroll 1
+        for (int a = a0 + lane; a < a1; a += 32) {
+            const int e = id_of(a);
+            if (e >= 0 && e < n_local) atomicAdd(&next[e], 1);
         }
     }
     __syncthreads();
-#pragma unroll
-    for (int g = 0; g < kFusedGroups; ++g) {
-        const int a = a0 + g * 32 + lane;
-        if (a0 + g * 32 >= a1) break;  // uniform over the warp
-        scatter_group(ids[g], a, a < a1, n_local, next, sorted_to_flat, flat_to_sorted, lane);
+    int count = 0;  // rows of expert tid
+    if (tid < n_local) {
+#pragma unroll 4
+        for (int w = 0; w < spans; ++w) count += u.next[w][tid];
     }
-    for (int base = a0 + kFusedGroups * 32; base < a1; base += 32) {
+    schedule_phase(count, n_local, nt_max, row_quantum, expert_offsets, tile_prefix, tile_order, tile_rows, status, sh, [&](int row) {
+        // counts -> first positions of expert tid in the spans
+#pragma unroll 4
+        for (int w = 0; w < spans; ++w) {
+            const int c = u.next[w][tid];
+            u.next[w][tid] = row;
+            row += c;
+        }
+    });
+    if (warp >= spans) return;
+#pragma unroll 1
+    for (int base = a0; base < a1; base += 32) {
         const int a = base + lane;
-        scatter_group(a < a1 ? __ldcg(&topk_ids[a]) - local_offset : -1, a, a < a1, n_local, next, sorted_to_flat, flat_to_sorted, lane);
+        scatter_group(a < a1 ? id_of(a) : -1, a, a < a1, n_local, next, sorted_to_flat, flat_to_sorted, lane);
     }
 }
 
@@ -975,7 +985,7 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
     const int A = T * k;
     if (scratch.n_chunks <= kFusedMaxChunks) {
         // One block, a cluster of eight, or up to 64 blocks of at least four tokens (the comment at kFusedOneBlockTokens).
-        const bool ids_local = T <= kFusedOneBlockTokens || (T <= kFusedClusterTokens && A <= kFusedIds);
+        const bool ids_local = T <= kFusedOneBlockTokens || (T <= kFusedClusterTokens && A <= kFusedClusterIds);
         int blocks = 1, per_block = T;
         if (T > kFusedOneBlockTokens) {
             per_block = ids_local ? (T + kFusedCluster - 1) / kFusedCluster : (T + 63) / 64 < 4 ? 4 : (T + 63) / 64;
@@ -988,15 +998,21 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
         // (The cluster starts when everything before it is done.  Launched early, its blocks of 48 KB and 1024 threads held SMs
         // while the last kernels of the call before were still at work: 64 tokens on 32 MX experts of 7168 x 2048 202.8 -> 214 us.)
         const bool cluster = ids_local && blocks > 1;
-        return launch_clusters(route_fused_kernel, !cluster, cluster ? blocks : 1, blocks, kFusedThreads, 0, stream, logits, T, E, k,
-                               local.offset, local.count, nt_max, row_quantum, per_block, router, topk_ids, topk_w,
+        const int spans = fused_spans(A), span = ((A + 32 * spans - 1) / (32 * spans)) * 32;
+        auto kernel = E <= 32 ? route_fused_kernel<1> : E <= 128 ? route_fused_kernel<4> : route_fused_kernel<8>;
+        return launch_clusters(kernel, !cluster, cluster ? blocks : 1, blocks, kFusedThreads, 0, stream, logits, T, E, k,
+                               local.offset, local.count, nt_max, RowQuantum(row_quantum), per_block, spans, span, router, topk_ids, topk_w,
                                expert_offsets, scratch.tile_prefix, scratch.tile_order, scratch.tile_rows, sorted_to_flat,
                                flat_to_sorted, status, ids_local ? (int)(status_bytes / sizeof(int)) : 0);
     }
     cudaError_t err = cudaMemsetAsync(status, 0, status_bytes, stream);  // the status word and what shares its region
     if (err != cudaSuccess) return err;
     const bool many = scratch.n_chunks > kRouteSms;
-    err = launch_chained(many ? route_topk_kernel<kRouteThreadsManyChunks> : route_topk_kernel<kRouteThreads>, scratch.n_chunks,
+    auto topk_kernel = many ? (E <= 32 ? route_topk_kernel<kRouteThreadsManyChunks, 1>
+                               : E <= 128 ? route_topk_kernel<kRouteThreadsManyChunks, 4> : route_topk_kernel<kRouteThreadsManyChunks, 8>)
+                            : (E <= 32 ? route_topk_kernel<kRouteThreads, 1>
+                               : E <= 128 ? route_topk_kernel<kRouteThreads, 4> : route_topk_kernel<kRouteThreads, 8>);
+    err = launch_chained(topk_kernel, scratch.n_chunks,
                          many ? kRouteThreadsManyChunks : kRouteThreads, 0, stream, logits, T, E, k, local.offset, local.count,
                          router, topk_ids, topk_w, scratch.chunk_counts);
     if (err != cudaSuccess) return err;
@@ -1004,7 +1020,7 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
     const int groups = (local.count + 31) / 32, warps_per_group = scan_warps_per_group(scratch.n_chunks, groups);
     const int scan_blocks = (scratch.n_chunks + warps_per_group - 1) / warps_per_group <= kScanBatch ? 1 : groups;
     err = launch_chained(route_scan_kernel, scan_blocks, kScanThreads, 0, stream, scratch.chunk_counts, scratch.n_chunks,
-                         local.count, nt_max, row_quantum, expert_offsets, scratch.tile_prefix, scratch.tile_order,
+                         local.count, nt_max, RowQuantum(row_quantum), expert_offsets, scratch.tile_prefix, scratch.tile_order,
                          scratch.tile_rows, scratch.tile_rows, status);
     if (err != cudaSuccess) return err;
     return launch_chained(route_scatter_kernel, scratch.n_chunks, 32, 0, stream, topk_ids, scratch.chunk_counts,
