@@ -74,15 +74,17 @@ struct SmemLayout {
     static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
     static constexpr int kBytes = kTiles + TileQueue::kBytes;
     static constexpr int kDynamicBytes = kBytes + 1024;  // slack to align the base to 1024 bytes
+    static constexpr int kQuantum = HALVES ? 8 : 16;     // token rows come in multiples of it: the MMA's step in N for so many rows
+    using Maps = TensorMapsOf<NT_MAX / kQuantum>;
 };
 
 template <int NT_MAX, int STAGES, bool SWIGLU, bool HALVES, bool QUEUED>
 __global__ void __launch_bounds__(QUEUED ? kThreads + 32 : kThreads, 1)
-grouped_gemm_tc_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
+grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGES, HALVES>::Maps maps, const KernelParams p) {
     using L = SmemLayout<NT_MAX, STAGES, HALVES>;
     static_assert(!HALVES || (!SWIGLU && !L::kStaged), "the halves of a tile are stored row by row");
     constexpr int kRows = L::kRows;
-    constexpr int kQuantum = HALVES ? 8 : 16;            // token rows come in multiples of it: the MMA's step in N for so many rows
+    constexpr int kQuantum = L::kQuantum;
     constexpr int kTmemCols = 2 * NT_MAX;
     static_assert(kTmemCols >= 32 && kTmemCols <= 512 && (kTmemCols & (kTmemCols - 1)) == 0,
                   "a tensor-memory allocation must be a power of two between 32 and 512 columns");
@@ -305,7 +307,7 @@ int launch_instance(const TensorMaps &maps, const KernelParams &p, int grid, cud
     auto kernel = grouped_gemm_tc_kernel<NT_MAX, STAGES, SWIGLU, HALVES, QUEUED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, typename L::Maps(maps), p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
@@ -339,7 +341,7 @@ cudaError_t launch_wait_timeout_selftest(int *status, cudaStream_t stream) {
 }
 
 int launch_grouped_gemm_tc(const GroupedGemmArgs &a, cudaStream_t stream) {
-    if (a.K % kBlockK != 0 || a.A <= 0) return MOE_ERR_UNSUPPORTED;
+    if (a.K % kBlockK != 0 || a.A <= 0 || a.nt_max > 256) return MOE_ERR_UNSUPPORTED;
     const int features_per_tile = a.swiglu ? kTileM / 2 : kTileM;
     if (a.n_out % features_per_tile != 0) return MOE_ERR_UNSUPPORTED;
 
@@ -357,7 +359,8 @@ int launch_grouped_gemm_tc(const GroupedGemmArgs &a, cudaStream_t stream) {
     const bool ok_w = halves ? encode_map_chunks(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K, kTileM / 2, kHalfChunks)
                     : a.swiglu ? encode_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
                                : encode_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !(halves ? encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 8, kHalfChunks) : encode_act_maps(maps.act, a.act, a.A, a.K, 16))) return MOE_ERR_CUDA;
+    if (!ok_w || !(halves ? encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 8, kHalfChunks, a.nt_max / 8)
+                        : encode_act_maps(maps.act, a.act, a.A, a.K, 16, a.nt_max / 16))) return MOE_ERR_CUDA;
 
     KernelParams p;
     p.out = a.out;

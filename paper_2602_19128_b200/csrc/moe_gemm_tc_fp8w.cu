@@ -69,7 +69,7 @@ struct Fp8Smem {
 
 template <int NT_MAX, int STAGES_Q, bool SWIGLU>
 __global__ void __launch_bounds__((Fp8Smem<NT_MAX, STAGES_Q>::kThreads), 1)
-grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
+grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const KernelParams p) {
     using L = Fp8Smem<NT_MAX, STAGES_Q>;
     constexpr int kConv = L::kConv;
     constexpr int kColsUsed = 2 * NT_MAX + kConv * kConvCols;
@@ -346,7 +346,7 @@ int launch_fp8_instance(const TensorMaps &maps, const KernelParams &p, int grid,
     auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES_Q, SWIGLU>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+    return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
@@ -365,6 +365,7 @@ int dispatch_fp8(int nt_max, const TensorMaps &maps, const KernelParams &p, int 
 
 int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &a, cudaStream_t stream) {
     if (a.K % 128 != 0 || a.A <= 0 || !a.w_scale || a.w_rows % 128 != 0) return MOE_ERR_UNSUPPORTED;
+    if (a.nt_max > 192) return MOE_ERR_UNSUPPORTED;
     const int features_per_tile = a.swiglu ? kTileM / 2 : kTileM;
     if (a.n_out % 128 != 0) return MOE_ERR_UNSUPPORTED;  // gate and up halves must both start on a scale block
 
@@ -376,7 +377,7 @@ int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &a, cudaStream_t stream) {
     TensorMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
                                : encode_mx_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 16, 2)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 16, 2, a.nt_max / 16)) return MOE_ERR_CUDA;
 
     KernelParams p;
     p.out = a.out;

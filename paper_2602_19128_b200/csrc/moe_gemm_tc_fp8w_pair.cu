@@ -127,7 +127,7 @@ struct Fp8PairSmem {
 
 template <int NT_MAX, bool SWIGLU>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((Fp8PairSmem<NT_MAX>::kThreads), 1)
-grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
+grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const KernelParams p) {
     using L = Fp8PairSmem<NT_MAX>;
     constexpr int kConv = L::kConv, kStagesQ = L::kStagesQ, kStagesT = L::kStagesT;
     constexpr int kColsUsed = 2 * NT_MAX + kConv * kConvCols;
@@ -437,7 +437,7 @@ int launch_fp8w_pair_instance(const TensorMaps &maps, const KernelParams &p, int
     auto kernel = grouped_gemm_tc_fp8w_pair_kernel<NT_MAX, SWIGLU>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+    return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }
 
 }  // namespace
@@ -461,7 +461,7 @@ int launch_grouped_gemm_tc_fp8w_pair(const GroupedGemmArgs &a, cudaStream_t stre
     TensorMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
                                : encode_mx_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 8, 2)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_act_maps_chunks(maps.act, a.act, a.A, a.K, 8, 2, a.nt_max / 16)) return MOE_ERR_CUDA;
 
     KernelParams p;
     p.out = a.out;

@@ -74,7 +74,7 @@ struct MxSmem {
 
 template <int NT_MAX, int STAGES, bool SWIGLU, bool QUEUED>
 __global__ void __launch_bounds__(QUEUED ? kThreads + 32 : kThreads, 1)
-grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMaps maps, const MxParams p) {
+grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const MxParams p) {
     using L = MxSmem<NT_MAX, STAGES>;
     static_assert(2 * NT_MAX + 32 <= kTmemColsMx, "accumulators and scale columns exceed tensor memory");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
@@ -297,7 +297,7 @@ int launch_instance(const TensorMaps &maps, const MxParams &p, int grid, cudaStr
     auto kernel = grouped_gemm_tc_mx_kernel<NT_MAX, STAGES, SWIGLU, QUEUED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess
+    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
@@ -327,7 +327,7 @@ int launch_grouped_gemm_tc_mx(const MxGemmArgs &a, cudaStream_t stream) {
     TensorMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.w, a.w_q, a.E, a.n_out, a.K)
                                : encode_mx_weight_map_2d(&maps.w, a.w_q, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_mx_act_maps(maps.act, a.act_q, a.A, a.K, 16)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_mx_act_maps(maps.act, a.act_q, a.A, a.K, 16, a.nt_max / 16)) return MOE_ERR_CUDA;
 
     MxParams p;
     p.out = a.out;

@@ -29,10 +29,12 @@ using namespace mxtc;
 
 constexpr int kPairThreads = 256;  // warp 0 weight TMA, warp 1 MMA, warps 2..5 epilogue, warp 6 token TMA, warp 7 tile decoder
 
-struct MxPairMaps {
-    TensorMaps ops;            // weight codes, token codes (boxes of 8, 16, ..., 128 rows)
+template <int kMaps>
+struct MxPairMapsOf {
+    TensorMapsOf<kMaps> ops;   // weight codes, token codes (boxes of 8, 16, ..., 8 kMaps rows)
     CUtensorMap w_sf, act_sf;  // scale atoms
 };
+using MxPairMaps = MxPairMapsOf<kNumActMaps>;  // on the host, while it is filled
 
 // In both CTAs of the pair: one scale atom from that CTA's shared memory to its tensor memory.
 __device__ __forceinline__ void tmem_copy_sf_atom_pair(uint32_t taddr, uint64_t desc) {
@@ -68,7 +70,7 @@ struct MxPairSmem {
 
 template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
-grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMaps maps, const MxParams p) {
+grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16> maps, const MxParams p) {
     using L = MxPairSmem<NT_MAX, STAGES, !STAGED ? 0 : SWIGLU ? 2 * kMxStageBytes : Stage<false>::kBytes>;
     static_assert(2 * NT_MAX + 16 + 4 * L::kAtomsB <= kTmemColsMx, "accumulators and scale columns exceed tensor memory");
     static_assert(NT_MAX % 16 == 0 && (NT_MAX / 2) % 8 == 0, "token tile halves must be whole 8-row swizzle groups");
@@ -297,10 +299,11 @@ template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
 int launch_pair_instance(const MxPairMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
     using L = MxPairSmem<NT_MAX, STAGES, !STAGED ? 0 : SWIGLU ? 2 * kMxStageBytes : Stage<false>::kBytes>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
+    const MxPairMapsOf<NT_MAX / 16> own = {TensorMapsOf<NT_MAX / 16>(maps.ops), maps.w_sf, maps.act_sf};
     auto kernel = grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+    return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, own, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }
 
 }  // namespace
@@ -317,7 +320,7 @@ int launch_grouped_gemm_tc_mx_pair(const MxGemmArgs &a, cudaStream_t stream) {
     MxPairMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.ops.w, a.w_q, a.E, a.n_out, a.K)
                                : encode_mx_weight_map_2d(&maps.ops.w, a.w_q, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_mx_act_maps(maps.ops.act, a.act_q, a.A, a.K, 8)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_mx_act_maps(maps.ops.act, a.act_q, a.A, a.K, 8, a.nt_max / 16)) return MOE_ERR_CUDA;
     const uint64_t w_atoms = (uint64_t)a.E * (a.n_out / cta_feat) * (a.K / kMxSlotK);
     const uint64_t act_atoms = (uint64_t)(a.K / kMxSlotK) * a.n_atoms;
     if (!encode_mx_scale_map(&maps.w_sf, a.w_sf, w_atoms, 1) ||

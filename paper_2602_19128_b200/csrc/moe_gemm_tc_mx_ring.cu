@@ -400,7 +400,7 @@ int launch_grouped_gemm_tc_mx_ring(const MxGemmArgs &a, cudaStream_t stream) {
     MxRingMaps maps;
     const bool ok_w = a.swiglu ? encode_mx_weight_map_gate_up(&maps.ops.w, a.w_q, a.E, a.n_out, a.K)
                                : encode_mx_weight_map_2d(&maps.ops.w, a.w_q, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_mx_act_maps(maps.ops.act, a.act_q, a.A, a.K, 8)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_mx_act_maps(maps.ops.act, a.act_q, a.A, a.K, 8, kNumActMaps)) return MOE_ERR_CUDA;
     const uint64_t w_atoms = (uint64_t)a.E * (a.n_out / cta_feat) * (a.K / kMxSlotK);
     const uint64_t act_atoms = (uint64_t)(a.K / kMxSlotK) * a.n_atoms;
     if (!encode_mx_scale_map(&maps.w_sf, a.w_sf, w_atoms, 1) ||

@@ -60,7 +60,7 @@ struct PairSmem {
 
 template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
-grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMaps maps, const KernelParams p) {
+grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const KernelParams p) {
     using L = PairSmem<NT_MAX, STAGES, SLABS, STAGED ? kStageBytes : 0>;
     constexpr int kAccBufs = SLABS == 1 ? 2 : 1;          // accumulator sets in TMEM
     // accumulator columns (2 * NT_MAX either way), rounded up to the power of two an allocation must be
@@ -289,7 +289,7 @@ int launch_pair_instance(const TensorMaps &maps, const KernelParams &p, int grid
     auto kernel = grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+    return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }
 
 int features_per_pair_tile(const GroupedGemmArgs &a, int slabs) { return slabs * (a.swiglu ? kTileM : 2 * kTileM); }
@@ -309,7 +309,7 @@ int launch_grouped_gemm_tc_pair(const GroupedGemmArgs &a, int slabs, cudaStream_
     TensorMaps maps;
     const bool ok_w = a.swiglu ? encode_weight_map_gate_up(&maps.w, a.w, a.E, a.n_out, a.K)
                                : encode_weight_map_2d(&maps.w, a.w, (uint64_t)a.E * a.w_rows, a.K);
-    if (!ok_w || !encode_act_maps(maps.act, a.act, a.A, a.K, 8)) return MOE_ERR_CUDA;
+    if (!ok_w || !encode_act_maps(maps.act, a.act, a.A, a.K, 8, a.nt_max / 16)) return MOE_ERR_CUDA;
 
     KernelParams p;
     p.out = a.out;

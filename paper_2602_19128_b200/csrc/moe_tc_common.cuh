@@ -21,10 +21,21 @@ constexpr int kNumActMaps = 16;                    // activation boxes of q, 2q,
 // Tensor maps of one grouped GEMM.  `w` is either a 2-D map over [E*w_rows, K] with a 128-row box
 // (down projection) or a 5-D map over w13 viewed as [E][I/16][gate|up][16][H] whose
 // {64,16,2,4,1} box delivers 64 features as 4 x (16 gate rows, 16 up rows) in one copy.
-struct TensorMaps {
+// act[i]: box of q * (i + 1) rows, so any token tile is ONE copy.  A kernel's parameters carry the boxes its tiles can have and
+// no more (kMaps): a map is 128 bytes that the host looks up and copies and the launch carries, and sixteen where two are used
+// made the tiny layer's call 18.6 us of host time, now 16.3 (in a loop 18.6 us per call, now 17.0).
+template <int kMaps>
+struct TensorMapsOf {
     CUtensorMap w;
-    CUtensorMap act[kNumActMaps];  // act[i]: box of q * (i + 1) rows, so any token tile is ONE copy
+    CUtensorMap act[kMaps];
+    TensorMapsOf() {}
+    template <int kMore>
+    explicit TensorMapsOf(const TensorMapsOf<kMore> &m) : w(m.w) {
+        static_assert(kMore >= kMaps, "the first of more");
+        for (int i = 0; i < kMaps; ++i) act[i] = m.act[i];
+    }
 };
+using TensorMaps = TensorMapsOf<kNumActMaps>;  // on the host, while it is filled
 
 struct KernelParams {
     __nv_bfloat16 *out;
@@ -216,8 +227,8 @@ __device__ __forceinline__ bool epilogue_any(bool flag) {
         : "memory");
     return r != 0;
 }
-template <int kQuantum>
-__device__ __forceinline__ const CUtensorMap *act_map(const TensorMaps &maps, int n_rows) {
+template <int kQuantum, int kMaps>
+__device__ __forceinline__ const CUtensorMap *act_map(const TensorMapsOf<kMaps> &maps, int n_rows) {
     return &maps.act[n_rows / kQuantum - 1];
 }
 
@@ -551,12 +562,12 @@ __device__ __forceinline__ void drain_staged(uint32_t taddr, int n_mma, int n_va
 bool encode_weight_map_2d(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K);
 bool encode_map_chunks(CUtensorMap *map, const void *base, uint64_t rows, uint64_t K, int box_rows, int chunks);
 bool encode_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int I, int H);
-bool encode_act_maps_chunks(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int chunks);
-bool encode_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int count = kNumActMaps);
+bool encode_act_maps_chunks(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int chunks, int count);
+bool encode_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int count);
 bool encode_row_map(CUtensorMap *map, const void *act, uint64_t rows, uint64_t K);
 bool encode_mx_weight_map_2d(CUtensorMap *map, const void *w, uint64_t rows, uint64_t K);
 bool encode_mx_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int I, int H);
-bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum);
+bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int count);
 int sm_count();
 bool set_max_dynamic_smem_once(const void *kernel, int bytes);
 

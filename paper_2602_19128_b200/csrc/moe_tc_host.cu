@@ -30,7 +30,7 @@ EncodeTiledFn get_encode_fn() {
 }
 
 // ---- tensor-map cache ------------------------------------------------------------------------------------
-// A forward call needs 34 tensor maps (one weight map and sixteen activation maps per GEMM); encoding them through
+// A forward call needs 6 to 50 tensor maps (a weight map and up to 24 activation maps per GEMM); encoding them through
 // the driver costs more host time than everything else in a call.  An encoded map is a pure function of the
 // arguments of the encode call (address, element type, rank, extents, strides, box, swizzle): it does not depend on
 // the memory's contents, so an entry can never go stale -- a buffer freed and allocated again at the same address
@@ -165,8 +165,8 @@ bool encode_mx_weight_map_gate_up(CUtensorMap *map, const void *w13, int E, int 
     return encode(map, w13, 5, dims, strides, box, Operand::kCodes);
 }
 
-bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum) {
-    for (int i = 0; i < kNumActMaps; ++i) {
+bool encode_mx_act_maps(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int count) {
+    for (int i = 0; i < count; ++i) {
         const cuuint64_t dims[2] = {K, rows};
         const cuuint64_t strides[1] = {K};
         const cuuint32_t box[2] = {128, (cuuint32_t)row_quantum * (cuuint32_t)(i + 1)};
@@ -183,8 +183,8 @@ bool encode_map_chunks(CUtensorMap *map, const void *base, uint64_t rows, uint64
     const cuuint32_t box[3] = {(cuuint32_t)kBlockK, (cuuint32_t)box_rows, (cuuint32_t)chunks};
     return encode(map, base, 3, dims, strides, box);
 }
-bool encode_act_maps_chunks(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int chunks) {
-    for (int i = 0; i < kNumActMaps; ++i)
+bool encode_act_maps_chunks(CUtensorMap *maps, const void *act, uint64_t rows, uint64_t K, int row_quantum, int chunks, int count) {
+    for (int i = 0; i < count; ++i)
         if (!encode_map_chunks(&maps[i], act, rows, K, row_quantum * (i + 1), chunks)) return false;
     return true;
 }
