@@ -115,6 +115,17 @@ def test_fp8w_with_and_without_the_hand_over(T, H, I, E, k):
         assert torch.equal(out.view(torch.int16), again.view(torch.int16))
 
 
+@pytest.mark.parametrize("T,H,I,E,k,skew", [(64, 256, 2048, 64, 4, False),   # 32-row tiles, 14 per CTA, two slots each
+                                            (150, 256, 2048, 32, 8, True),   # 64 rows, ragged
+                                            (300, 128, 2048, 16, 4, False),  # 128 rows, one slot
+                                            (900, 384, 2048, 8, 1, True)])   # 192 rows, three slots
+def test_fp8w_many_short_tiles_per_cta(T, H, I, E, k, skew):
+    """More tiles per CTA than the queue of decoded tiles holds, with fewer slots of K than there are operand buffers."""
+    inp = make_fp8w_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=7, device="cuda")
+    out, _ = run_fp8w(inp)
+    assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
+
+
 def test_fp8w_with_unit_scales_equals_the_bf16_layer_bit_for_bit():
     """All E4M3 values are bf16 values, and a scale of 1 is exact in bf16: both paths see the same operands."""
     g = torch.Generator().manual_seed(0)
