@@ -16,7 +16,7 @@
 //    epilogue warp finds gate and up of the same 16 features in its own 32 TMEM lanes and
 //    pairs them with one shuffle; SiLU(gate)*up is applied before anything is stored.
 //  * One CTA per SM walks tiles  tile = blockIdx.x + i*gridDim.x  of a device-built schedule
-//    (no host round trip, no atomics).  Tiles of the same expert and weight slab are adjacent in
+//    (no host round trip; long tiles are drawn from a counter, TileQueue).  Tiles of the same expert and weight slab are adjacent in
 //    that order, so they run at the same time on neighbouring SMs and share the slab in L2.
 //  * Warp 0 issues TMA loads into a STAGES-deep ring; warp 1 issues the MMAs and commits ring
 //    slots back; warps 2..5 drain the accumulator (double-buffered in TMEM, so the epilogue of
@@ -78,8 +78,8 @@ struct SmemLayout {
     using Maps = TensorMapsOf<NT_MAX / kQuantum>;
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool HALVES, bool QUEUED>
-__global__ void __launch_bounds__(QUEUED ? kThreads + 32 : kThreads, 1)
+template <int NT_MAX, int STAGES, bool SWIGLU, bool HALVES, int QUEUE>
+__global__ void __launch_bounds__(QUEUE != kNoQueue ? kThreads + 32 : kThreads, 1)
 grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGES, HALVES>::Maps maps, const KernelParams p) {
     using L = SmemLayout<NT_MAX, STAGES, HALVES>;
     static_assert(!HALVES || (!SWIGLU && !L::kStaged), "the halves of a tile are stored row by row");
@@ -105,9 +105,9 @@ grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGE
     const TileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_tile(tile, p); };
     auto queue_wait = [&](uint32_t bar, uint32_t parity) { return wait(bar, parity, kSiteProducerEmpty); };
-    // the n-th tile, from the decoder warp or decoded here
+    // the n-th tile, from the decoder warp or decoded here; false at the end of the work
     auto next_tile = [&](Tile &t, int n, int tile) {
-        if constexpr (QUEUED) return tiles.take(t, n, lane, queue_wait);
+        if constexpr (QUEUE != kNoQueue) return tiles.take(t, n, lane, queue_wait) && (QUEUE != kOnDemand || t.e >= 0);
         t = decode(tile);
         return true;
     };
@@ -160,7 +160,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGE
         };
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -212,7 +212,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGE
         bool ok = true;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -258,9 +258,10 @@ grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGE
         bool ok = true;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             const bool taken = next_tile(t, round, tile);
+            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
             const int n_mma = (t.n_valid + kQuantum - 1) & -kQuantum;
             ok = taken && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
             if (L::kStaged ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
@@ -281,9 +282,15 @@ grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGE
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-    } else if (QUEUED && warp == 6) {
+    } else if (QUEUE != kNoQueue && warp == 6) {
         // ---------------- decoder ----------------
-        tiles.fill(worker, n_workers, total_tiles, lane, decode, queue_wait);
+        const auto tile_at = decode;
+        if constexpr (QUEUE == kOnDemand)
+            tiles.fill_on_demand<Tile>(worker, n_workers, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, tile_at, queue_wait);
+        else if constexpr (QUEUE == kBatchedQueue)
+            tiles.fill_batched<Tile>(worker, n_workers, total_tiles, lane, tile_at, queue_wait);
+        else
+            tiles.fill(worker, n_workers, total_tiles, lane, tile_at, queue_wait);
     }
 
     // ---------------- teardown ----------------
@@ -300,24 +307,39 @@ grouped_gemm_tc_kernel(const __grid_constant__ typename SmemLayout<NT_MAX, STAGE
     }
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool HALVES = false, bool QUEUED = false>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool HALVES = false, int QUEUE = kNoQueue>
 int launch_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = SmemLayout<NT_MAX, STAGES, HALVES>;
     static_assert(L::kDynamicBytes <= 232448, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_kernel<NT_MAX, STAGES, SWIGLU, HALVES, QUEUED>;
+    auto kernel = grouped_gemm_tc_kernel<NT_MAX, STAGES, SWIGLU, HALVES, QUEUE>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, typename L::Maps(maps), p) == cudaSuccess
+    return launch_chained(kernel, grid, QUEUE != kNoQueue ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, typename L::Maps(maps), p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
-template <bool SWIGLU, bool QUEUED>
-int dispatch(int nt_max, const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t s) {
+// How a CTA comes by its tiles.  Where it has more than one: on demand if they are long enough (tiles_on_demand), else decoded ahead
+// (kStaticQueue) if a tile's slots do not hide the walk.
+// Without a queue / on demand: one token of 128 experts of 4096 x 1536, top 8, 71.9 / 64.3 us; 100 tokens 707 / 697; 64 of 64 of
+// 1536 x 1536, top 4, 153.9 / 146.6; 128 of 256 of 7168 x 2048, top 8, 3147 / 3047; Mixtral-shaped, one token, 122.0 / 120.1.
+// Without / decoded ahead: 16 tokens of 32 experts of 1024 x 1024, top 4, 51.5 / 50.4; on demand there 45.8 against 45.6 decoded ahead,
+// 64 tokens 53.2 / 52.6.  One tile per CTA, the tiny layer: 19.2 without, 19.7 with.
+template <int NT_MAX, int STAGES, bool SWIGLU>
+int launch_queue(const TensorMaps &maps, const KernelParams &p, int grid, int tiles_per_cta, cudaStream_t s) {
+    if (tiles_per_cta <= 1) return launch_instance<NT_MAX, STAGES, SWIGLU>(maps, p, grid, s);
+    if (tiles_on_demand(p.n_k_blocks, STAGES)) return launch_instance<NT_MAX, STAGES, SWIGLU, false, kOnDemand>(maps, p, grid, s);
+    if (p.n_k_blocks * kBlockK > 1024) return launch_instance<NT_MAX, STAGES, SWIGLU>(maps, p, grid, s);
+    return static_queue(p.n_k_blocks, tiles_per_cta >= 8) == kBatchedQueue
+               ? launch_instance<NT_MAX, STAGES, SWIGLU, false, kBatchedQueue>(maps, p, grid, s)
+               : launch_instance<NT_MAX, STAGES, SWIGLU, false, kStaticQueue>(maps, p, grid, s);
+}
+template <bool SWIGLU>
+int dispatch(int nt_max, const TensorMaps &maps, const KernelParams &p, int grid, int tiles_per_cta, cudaStream_t s) {
     switch (nt_max) {
-        case 32: return launch_instance<32, 10, SWIGLU, false, QUEUED>(maps, p, grid, s);
-        case 64: return launch_instance<64, 8, SWIGLU, false, QUEUED>(maps, p, grid, s);
-        case 128: return launch_instance<128, 6, SWIGLU, false, QUEUED>(maps, p, grid, s);
-        case 256: return launch_instance<256, 4, SWIGLU, false, QUEUED>(maps, p, grid, s);
+        case 32: return launch_queue<32, 10, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 64: return launch_queue<64, 8, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 128: return launch_queue<128, 6, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 256: return launch_queue<256, 4, SWIGLU>(maps, p, grid, tiles_per_cta, s);
         default: return MOE_ERR_UNSUPPORTED;
     }
 }
@@ -382,12 +404,8 @@ int launch_grouped_gemm_tc(const GroupedGemmArgs &a, cudaStream_t stream) {
     if (halves)
         return launch_instance<32, kHalfStages, false, true>(maps, p, 2 * (int)max_tiles, stream);
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
-    // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots do not hide the walk.  Without / with: 16 tokens of
-    // 32 experts of 1024 x 1024, top 4, 51.5 / 50.4 us; 64 of 2048 x 2048 140.4 / 140.8; 100 tokens of 128 of 4096 x 1536, top 8,
-    // 722 / 731; one tile per CTA, the tiny layer 19.2 / 19.7.
-    const bool queued = max_tiles > sms && a.K <= 1024;
-    if (queued) return a.swiglu ? dispatch<true, true>(a.nt_max, maps, p, grid, stream) : dispatch<false, true>(a.nt_max, maps, p, grid, stream);
-    return a.swiglu ? dispatch<true, false>(a.nt_max, maps, p, grid, stream) : dispatch<false, false>(a.nt_max, maps, p, grid, stream);
+    const int tiles_per_cta = (int)((max_tiles + sms - 1) / sms);
+    return a.swiglu ? dispatch<true>(a.nt_max, maps, p, grid, tiles_per_cta, stream) : dispatch<false>(a.nt_max, maps, p, grid, tiles_per_cta, stream);
 }
 
 }  // namespace moe

@@ -13,7 +13,7 @@
 //                codes into bf16 * block scale and stores them to tensor memory, the MMA's A operand
 //   warp 1       MMA: A from tensor memory, B straight from the token slot
 //   warps 2..5   epilogue (SwiGLU or plain, two accumulators)
-//   warp 7       decodes tiles ahead (QUEUED)
+//   warp 7       decodes tiles ahead (QUEUE)
 //
 // What bounds it and why A sits in tensor memory: with A rebuilt in shared memory a slot of 96 token rows moved 144 KiB
 // through shared memory (codes in, codes out, 32 KiB of bf16 in and out again, tokens in and out), 1150 cycles at 128
@@ -69,7 +69,7 @@ struct Fp8Smem {
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
 
-template <int NT_MAX, int STAGES_Q, bool SWIGLU, bool QUEUED>
+template <int NT_MAX, int STAGES_Q, bool SWIGLU, int QUEUE>
 __global__ void __launch_bounds__((Fp8Smem<NT_MAX, STAGES_Q>::kThreads), 1)
 grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const KernelParams p) {
     using L = Fp8Smem<NT_MAX, STAGES_Q>;
@@ -94,9 +94,9 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
     };
     const TileQueue tiles(base_ptr, base, L::kTiles);
     auto queue_wait = [&](uint32_t bar, uint32_t parity) { return wait(bar, parity, kSiteProducerEmpty); };
-    // the n-th tile, from the decoder warp or decoded here
+    // the n-th tile, from the decoder warp or decoded here; false at the end of the work
     auto next_tile = [&](Tile &t, int n, int tile) {
-        if constexpr (QUEUED) return tiles.take(t, n, lane, queue_wait);
+        if constexpr (QUEUE != kNoQueue) return tiles.take(t, n, lane, queue_wait) && (QUEUE != kOnDemand || t.e >= 0);
         t = decode_tile(tile, p);
         return true;
     };
@@ -144,7 +144,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         bool ok = true;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -173,7 +173,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         bool ok = true, gate_up_done = false;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -205,7 +205,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         const uint64_t b_desc0 = smem_desc_k_major_sw128(base + L::kB);
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -259,7 +259,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         bool ok = true;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -323,9 +323,10 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         bool ok = true;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             const bool taken = next_tile(t, round, tile);
+            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
             const int n_mma = (t.n_valid + 15) & ~15;
             ok = taken && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
             if (L::kStaged ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
@@ -344,9 +345,15 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-    } else if (QUEUED && warp == 7) {
+    } else if (QUEUE != kNoQueue && warp == 7) {
         // ---------------- decoder ----------------
-        tiles.fill(worker, n_workers, total_tiles, lane, [&](int tile) { return decode_tile(tile, p); }, queue_wait);
+        const auto tile_at = [&](int tile) { return decode_tile(tile, p); };
+        if constexpr (QUEUE == kOnDemand)
+            tiles.fill_on_demand<Tile>(worker, n_workers, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, tile_at, queue_wait);
+        else if constexpr (QUEUE == kBatchedQueue)
+            tiles.fill_batched<Tile>(worker, n_workers, total_tiles, lane, tile_at, queue_wait);
+        else
+            tiles.fill(worker, n_workers, total_tiles, lane, tile_at, queue_wait);
     }
 
     // ---------------- teardown ----------------
@@ -362,24 +369,38 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
     }
 }
 
-template <int NT_MAX, int STAGES_Q, bool SWIGLU, bool QUEUED>
+template <int NT_MAX, int STAGES_Q, bool SWIGLU, int QUEUE>
 int launch_fp8_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = Fp8Smem<NT_MAX, STAGES_Q>;
     static_assert(L::kDynamicBytes <= 232448, "rings do not fit in shared memory");
-    auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES_Q, SWIGLU, QUEUED>;
+    auto kernel = grouped_gemm_tc_fp8w_kernel<NT_MAX, STAGES_Q, SWIGLU, QUEUE>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
-template <bool SWIGLU, bool QUEUED>
-int dispatch_fp8(int nt_max, const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t s) {
+// How a CTA comes by its tiles, where it has more than one: decoded ahead (TileQueue), since the converters and the MMA run two to four
+// slots ahead of one another and stood still for every walk, and on demand if they are long enough.  Without / decoded ahead:
+// 389 tokens of 256 experts of 256 x 2048, top 6, 162.3 / 137.9 us (walks batched 133.0); 77 of 128 of 1536 x 2432, top 1, 153.6 / 141.1; 16
+// of 256 of 7168 x 2048, top 8, 757 / 722; 1968 of 60 of 4608 x 4736, top 1, 768 / 746; one tile per CTA, 100 tokens of 8 of 256 x 512,
+// top 2, 19.1 / 19.3.  Decoded ahead / on demand: one token of 128 experts of 4096 x 1536, top 8, 57.1 / 52.5; Mixtral-shaped, 32 tokens,
+// 243.5 / 239.4, one 93.3 / 91.0.
+template <int NT_MAX, int STAGES_Q, bool SWIGLU>
+int launch_fp8_queue(const TensorMaps &maps, const KernelParams &p, int grid, int tiles_per_cta, cudaStream_t s) {
+    if (tiles_per_cta <= 1) return launch_fp8_instance<NT_MAX, STAGES_Q, SWIGLU, kNoQueue>(maps, p, grid, s);
+    if (tiles_on_demand(p.n_k_blocks, STAGES_Q)) return launch_fp8_instance<NT_MAX, STAGES_Q, SWIGLU, kOnDemand>(maps, p, grid, s);
+    return static_queue(p.n_k_blocks, tiles_per_cta >= 8) == kBatchedQueue
+               ? launch_fp8_instance<NT_MAX, STAGES_Q, SWIGLU, kBatchedQueue>(maps, p, grid, s)
+               : launch_fp8_instance<NT_MAX, STAGES_Q, SWIGLU, kStaticQueue>(maps, p, grid, s);
+}
+template <bool SWIGLU>
+int dispatch_fp8(int nt_max, const TensorMaps &maps, const KernelParams &p, int grid, int tiles_per_cta, cudaStream_t s) {
     switch (nt_max) {
-        case 32: return launch_fp8_instance<32, 12, SWIGLU, QUEUED>(maps, p, grid, s);
-        case 64: return launch_fp8_instance<64, 8, SWIGLU, QUEUED>(maps, p, grid, s);
-        case 128: return launch_fp8_instance<128, 6, SWIGLU, QUEUED>(maps, p, grid, s);
-        case 192: return launch_fp8_instance<192, 8, SWIGLU, QUEUED>(maps, p, grid, s);
+        case 32: return launch_fp8_queue<32, 12, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 64: return launch_fp8_queue<64, 8, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 128: return launch_fp8_queue<128, 6, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 192: return launch_fp8_queue<192, 8, SWIGLU>(maps, p, grid, tiles_per_cta, s);
         default: return MOE_ERR_UNSUPPORTED;
     }
 }
@@ -420,13 +441,8 @@ int launch_grouped_gemm_tc_fp8w(const GroupedGemmArgs &a, cudaStream_t stream) {
     p.handover_per_token_tile = a.handover_per_token_tile;
 
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
-    // Tiles decoded ahead (TileQueue) where a CTA has more than one: the converters and the MMA run two to four slots ahead of one
-    // another, and stood still for every walk.  Without / with: 389 tokens of 256 experts of 256 x 2048, top 6, 162.3 / 137.9 us; 77
-    // of 128 of 1536 x 2432, top 1, 153.6 / 141.1; 16 of 256 of 7168 x 2048, top 8, 757 / 722; 1968 of 60 of 4608 x 4736, top 1, 768 /
-    // 746; one tile per CTA, 100 tokens of 8 of 256 x 512, top 2, 19.1 / 19.3.
-    if (max_tiles > sms)
-        return a.swiglu ? dispatch_fp8<true, true>(a.nt_max, maps, p, grid, stream) : dispatch_fp8<false, true>(a.nt_max, maps, p, grid, stream);
-    return a.swiglu ? dispatch_fp8<true, false>(a.nt_max, maps, p, grid, stream) : dispatch_fp8<false, false>(a.nt_max, maps, p, grid, stream);
+    const int tiles_per_cta = (int)((max_tiles + sms - 1) / sms);
+    return a.swiglu ? dispatch_fp8<true>(a.nt_max, maps, p, grid, tiles_per_cta, stream) : dispatch_fp8<false>(a.nt_max, maps, p, grid, tiles_per_cta, stream);
 }
 
 }  // namespace moe

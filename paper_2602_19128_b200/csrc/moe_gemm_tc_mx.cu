@@ -72,8 +72,8 @@ struct MxSmem {
     static constexpr int kDynamicBytes = kBytes + 1024;
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool QUEUED>
-__global__ void __launch_bounds__(QUEUED ? kThreads + 32 : kThreads, 1)
+template <int NT_MAX, int STAGES, bool SWIGLU, int QUEUE>
+__global__ void __launch_bounds__(QUEUE != kNoQueue ? kThreads + 32 : kThreads, 1)
 grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const MxParams p) {
     using L = MxSmem<NT_MAX, STAGES>;
     static_assert(2 * NT_MAX + 32 <= kTmemColsMx, "accumulators and scale columns exceed tensor memory");
@@ -95,9 +95,9 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps
     const TileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_mx_tile(tile, p); };
     auto queue_wait = [&](uint32_t bar, uint32_t parity) { return wait(bar, parity, kSiteProducerEmpty); };
-    // the n-th tile, from the decoder warp or decoded here
+    // the n-th tile, from the decoder warp or decoded here; false at the end of the work
     auto next_tile = [&](MxTile &t, int n, int tile) {
-        if constexpr (QUEUED) return tiles.take(t, n, lane, queue_wait);
+        if constexpr (QUEUE != kNoQueue) return tiles.take(t, n, lane, queue_wait) && (QUEUE != kOnDemand || t.e >= 0);
         t = decode(tile);
         return true;
     };
@@ -149,7 +149,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps
         };
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -200,7 +200,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps
         const uint32_t sfa_tmem = tmem_base + kSfACol, sfb_tmem = tmem_base + kSfBCol;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
             ok = next_tile(t, round, tile);
             if (!ok) break;
@@ -244,9 +244,10 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps
         int buf = 0;  // exchange buffer, flipped every step (across tiles too): a warp may run one step ahead of its partner
         for (int round = 0;; ++round) {
             const int tile = tile_of_round(round, worker, n_workers);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
             const bool taken = next_tile(t, round, tile);
+            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
             const int n_mma = (t.n_valid + 15) & ~15;
             bool ok = taken && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
             if (epilogue_any(!ok)) break;  // the four warps synchronise inside the tile (SwiGLU): they leave together
@@ -272,9 +273,15 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-    } else if (QUEUED && warp == 6) {
+    } else if (QUEUE != kNoQueue && warp == 6) {
         // ---------------- decoder ----------------
-        tiles.fill(worker, n_workers, total_tiles, lane, decode, queue_wait);
+        const auto tile_at = decode;
+        if constexpr (QUEUE == kOnDemand)
+            tiles.fill_on_demand<MxTile>(worker, n_workers, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, tile_at, queue_wait);
+        else if constexpr (QUEUE == kBatchedQueue)
+            tiles.fill_batched<MxTile>(worker, n_workers, total_tiles, lane, tile_at, queue_wait);
+        else
+            tiles.fill(worker, n_workers, total_tiles, lane, tile_at, queue_wait);
     }
 
     // ---------------- teardown ----------------
@@ -290,23 +297,36 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps
     }
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool QUEUED>
+template <int NT_MAX, int STAGES, bool SWIGLU, int QUEUE>
 int launch_instance(const TensorMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
     using L = MxSmem<NT_MAX, STAGES>;
     static_assert(L::kDynamicBytes <= 232448, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_mx_kernel<NT_MAX, STAGES, SWIGLU, QUEUED>;
+    auto kernel = grouped_gemm_tc_mx_kernel<NT_MAX, STAGES, SWIGLU, QUEUE>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
-    return launch_chained(kernel, grid, QUEUED ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess
+    return launch_chained(kernel, grid, QUEUE != kNoQueue ? kThreads + 32 : kThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess
                ? MOE_OK : MOE_ERR_CUDA;
 }
 
-template <bool SWIGLU, bool QUEUED>
-int dispatch(int nt_max, const TensorMaps &maps, const MxParams &p, int grid, cudaStream_t s) {
+// How a CTA comes by its tiles (as launch_queue in moe_gemm_tc.cu; slots are of 128 here).  Without a queue / on demand: 100 tokens of
+// 128 experts of 4096 x 1536, top 8, 384.3 / 374.8 us; 273 of 256 of 7168 x 2048, top 8, 1698 / 1645; 40 of 160 of 768 x 3328, top 4,
+// 159.9 / 158.1; 128 on 32 of 256 of 7168 x 2048 224.5 / 218.6; 64 of 32 of 2048 x 2048, top 4, 86.6 / 86.3.  Without / decoded ahead: 16
+// tokens of 128 experts of 512 x 512, top 8, 44.4 / 39.1; 64 of 32 of 1024 x 1024, top 4, 45.2 / 43.1.
+template <int NT_MAX, int STAGES, bool SWIGLU>
+int launch_queue(const TensorMaps &maps, const MxParams &p, int grid, int tiles_per_cta, cudaStream_t s) {
+    if (tiles_per_cta <= 1) return launch_instance<NT_MAX, STAGES, SWIGLU, kNoQueue>(maps, p, grid, s);
+    if (tiles_on_demand(p.n_k_blocks, STAGES)) return launch_instance<NT_MAX, STAGES, SWIGLU, kOnDemand>(maps, p, grid, s);
+    if (p.n_k_blocks * kMxSlotK > 1024) return launch_instance<NT_MAX, STAGES, SWIGLU, kNoQueue>(maps, p, grid, s);
+    return static_queue(p.n_k_blocks, tiles_per_cta >= 8) == kBatchedQueue
+               ? launch_instance<NT_MAX, STAGES, SWIGLU, kBatchedQueue>(maps, p, grid, s)
+               : launch_instance<NT_MAX, STAGES, SWIGLU, kStaticQueue>(maps, p, grid, s);
+}
+template <bool SWIGLU>
+int dispatch(int nt_max, const TensorMaps &maps, const MxParams &p, int grid, int tiles_per_cta, cudaStream_t s) {
     switch (nt_max) {
-        case 32: return launch_instance<32, 10, SWIGLU, QUEUED>(maps, p, grid, s);
-        case 64: return launch_instance<64, 8, SWIGLU, QUEUED>(maps, p, grid, s);
-        case 128: return launch_instance<128, 6, SWIGLU, QUEUED>(maps, p, grid, s);
+        case 32: return launch_queue<32, 10, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 64: return launch_queue<64, 8, SWIGLU>(maps, p, grid, tiles_per_cta, s);
+        case 128: return launch_queue<128, 6, SWIGLU>(maps, p, grid, tiles_per_cta, s);
         default: return MOE_ERR_UNSUPPORTED;
     }
 }
@@ -352,12 +372,8 @@ int launch_grouped_gemm_tc_mx(const MxGemmArgs &a, cudaStream_t stream) {
     p.handover_per_token_tile = a.handover_per_token_tile;
 
     const int grid = (int)(max_tiles < sms ? max_tiles : sms);
-    // Tiles decoded ahead (TileQueue) where a CTA has several and a tile's slots (of 128 here) do not hide the walk.  Without / with:
-    // 16 tokens of 128 experts of 512 x 512, top 8, 44.4 / 39.1 us; 64 of 32 of 1024 x 1024, top 4, 45.2 / 43.1; of 2048 x 2048 88.9 /
-    // 88.1; 100 tokens of 128 of 4096 x 1536, top 8, 393.7 / 397.0.
-    const bool queued = max_tiles > sms && a.K <= 1024;
-    if (queued) return a.swiglu ? dispatch<true, true>(a.nt_max, maps, p, grid, stream) : dispatch<false, true>(a.nt_max, maps, p, grid, stream);
-    return a.swiglu ? dispatch<true, false>(a.nt_max, maps, p, grid, stream) : dispatch<false, false>(a.nt_max, maps, p, grid, stream);
+    const int tiles_per_cta = (int)((max_tiles + sms - 1) / sms);
+    return a.swiglu ? dispatch<true>(a.nt_max, maps, p, grid, tiles_per_cta, stream) : dispatch<false>(a.nt_max, maps, p, grid, tiles_per_cta, stream);
 }
 
 }  // namespace moe

@@ -25,6 +25,7 @@ constexpr int kDoneCounterInt = 4;      // int index, in the status word's zeroe
 constexpr int kStatusBytesRoute = 256;
 constexpr int kStatusBytesForward = 2048;
 constexpr int kHandoverFlagInt = 8;
+constexpr int kTileCounterInt = 10;      // two: tiles of the gate/up and the down GEMM handed out on demand
 constexpr int kReadyTotalInt = 9;       // all experts' counts together
 constexpr int kClockProbeInt = 32;      // 2 x 4 int64 (bytes 128..191): the GEMMs' clock probes (moe_tc_common.cuh)
 constexpr int kReadyCounterInt = 64;    // [kMaxExperts] ints from here

@@ -272,6 +272,13 @@ __device__ __forceinline__ int tile_of_round(int round, int worker, int n_worker
 // few ahead, and the others take them from a small queue.  4096 tokens of 32 experts of 1024 x
 // 1024, top 4: bf16 139.1 -> 134, MX 167.2 -> 155; 256 of them 60.3 -> 58.8 and 51.9 -> 48.9.
 //   kDepth entries of eight words, then full[kDepth] (the decoder's arrival) and empty[kDepth] (one per taking warp)
+// Tiles are handed out on demand where a tile is at least two rings of slots: with a static assignment the CTAs of the down GEMM
+// of 128 DeepSeek-V3-shaped tokens ended between 2993 and 3177 us of the call, whatever ran slower waited for by everything
+// behind it.  Where tiles are shorter the next one is wanted before it could be drawn (200 tokens of 32 experts of 1024 x 1024, top 4,
+// sixteen slots: 53.8 decoded ahead, 54.8 us on demand).
+enum { kNoQueue = 0, kStaticQueue = 1, kBatchedQueue = 2, kOnDemand = 3 };
+inline bool tiles_on_demand(int slots_per_tile, int ring) { return slots_per_tile >= 2 * ring && slots_per_tile >= 20; }
+inline int static_queue(int slots_per_tile, bool many) { return slots_per_tile <= 4 && many ? kBatchedQueue : kStaticQueue; }
 struct TileQueue {
     static constexpr int kDepth = 4, kBytes = kDepth * 32 + 2 * kDepth * 8;
     int *entries;
@@ -297,23 +304,73 @@ struct TileQueue {
         if (lane == 0) mbar_arrive(empty + i * 8);
         return ok;
     }
-    // The decoder warp: all tiles of this worker.
+    template <typename T>
+    __device__ __forceinline__ void publish(const T &t, int n, int lane) const {
+        static_assert(sizeof(T) <= 32, "an entry");
+        const int i = n & (kDepth - 1);
+        if (lane == 0) {
+            const int *w = reinterpret_cast<const int *>(&t);
+            volatile int *e = entries + i * 8;
+#pragma unroll
+            for (int k = 0; k < (int)(sizeof(T) / 4); ++k) e[k] = w[k];
+            mbar_arrive(full + i * 8);
+        }
+        __syncwarp();
+    }
+    // The decoder warp, static assignment: all tiles of this worker, up to kDepth ahead.
     template <typename Decode, typename Wait>
     __device__ __forceinline__ void fill(int worker, int n_workers, int total_tiles, int lane, Decode decode, Wait wait) const {
         for (int n = 0;; ++n) {
-            const int tile = tile_of_round(n, worker, n_workers), i = n & (kDepth - 1);
+            const int tile = tile_of_round(n, worker, n_workers);
             if (tile >= total_tiles) break;
             const auto t = decode(tile);
-            static_assert(sizeof(t) <= 32, "an entry");
-            if (!__all_sync(0xffffffffu, wait(empty + i * 8, ((n / kDepth) & 1) ^ 1))) break;
-            if (lane == 0) {
-                const int *w = reinterpret_cast<const int *>(&t);
-                volatile int *e = entries + i * 8;
+            if (!__all_sync(0xffffffffu, wait(empty + (n & (kDepth - 1)) * 8, ((n / kDepth) & 1) ^ 1))) break;
+            publish(t, n, lane);
+        }
+    }
+    // The same for tiles of very few slots, which one walk after the other holds up: after the first, 32 tiles at a time are
+    // decoded, one per lane.
+    template <typename T, typename Decode, typename Wait>
+    __device__ __forceinline__ void fill_batched(int worker, int n_workers, int total_tiles, int lane, Decode decode, Wait wait) const {
+        T batch;
+        for (int n = 0;; ++n) {
+            if (tile_of_round(n, worker, n_workers) >= total_tiles) break;
+            T t;
+            if (n == 0) {
+                t = decode(worker);
+            } else {
+                if ((n & 31) == 1) {
+                    const int tile = tile_of_round(n + lane, worker, n_workers);
+                    if (tile < total_tiles) batch = decode(tile);
+                    __syncwarp();
+                }
+                int *w = reinterpret_cast<int *>(&t);
+                const int *mine = reinterpret_cast<const int *>(&batch);
 #pragma unroll
-                for (int k = 0; k < (int)(sizeof(t) / 4); ++k) e[k] = w[k];
-                mbar_arrive(full + i * 8);
+                for (int k = 0; k < (int)(sizeof(T) / 4); ++k) w[k] = __shfl_sync(0xffffffffu, mine[k], (n - 1) & 31);
             }
-            __syncwarp();
+            if (!__all_sync(0xffffffffu, wait(empty + (n & (kDepth - 1)) * 8, ((n / kDepth) & 1) ^ 1))) break;
+            publish(t, n, lane);
+        }
+    }
+    // The decoder warp, tiles on demand: the worker's own number first, then whatever the call's counter says; the next one is drawn
+    // when the last role (the epilogue) has begun with the one before it.  An entry whose expert is -1 ends the work.
+    template <typename T, typename Decode, typename Wait>
+    __device__ __forceinline__ void fill_on_demand(int worker, int n_workers, int total_tiles, int *counter, int lane, Decode decode,
+                                                   Wait wait) const {
+        for (int n = 0;; ++n) {
+            int tile = worker;
+            if (n > 0) {
+                const int m = n - 1;
+                if (!__all_sync(0xffffffffu, wait(empty + (m & (kDepth - 1)) * 8, (m / kDepth) & 1))) break;
+                if (lane == 0) tile = n_workers + atomicAdd(counter, 1);
+                tile = __shfl_sync(0xffffffffu, tile, 0);
+            }
+            T t;
+            t.e = -1;
+            if (tile < total_tiles) t = decode(tile);
+            publish(t, n, lane);
+            if (t.e < 0) break;
         }
     }
 };

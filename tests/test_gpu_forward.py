@@ -101,6 +101,23 @@ def test_many_short_tiles_per_cta(T, H, I, E, k, skew):
     assert_close_out(bf16_to_f64(out), ref, "out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k,skew", [(40, 1280, 1344, 16, 2, False),   # 32-row tiles, 20 and 21 slots of K
+                                            (150, 1408, 1280, 16, 4, True),   # 64 rows, ragged
+                                            (32, 1280, 1280, 32, 8, True)])   # some experts without tokens
+def test_tiles_on_demand(T, H, I, E, k, skew):
+    """Long tiles and more than one per CTA in both GEMMs: handed out by a counter that every call starts anew."""
+    inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=2)
+    out, views, ws = run_forward(inp)
+    *_, h, y, ref = oracle_everything(to_host_case(inp))
+    assert_close_out(bf16_to_f64(views["h"]), h, "h")
+    assert_close_out(bf16_to_f64(views["y"]), y, "y")
+    assert_close_out(bf16_to_f64(out), ref, "out")
+    for _ in range(3):
+        again = torch.empty_like(out)
+        moe.moe_forward(inp["x"], inp["router_logits"], inp["w13"], inp["w2"], k, again, ws)
+        assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
 @pytest.mark.parametrize("T,H,I,E,k,skew", [(520, 256, 256, 4, 2, False), (900, 256, 128, 8, 2, True),
                                             (1200, 512, 384, 8, 2, False), (700, 256, 256, 2, 1, False)])
 def test_gather_in_load_matches_oracle(T, H, I, E, k, skew):

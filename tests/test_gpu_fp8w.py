@@ -126,6 +126,17 @@ def test_fp8w_many_short_tiles_per_cta(T, H, I, E, k, skew):
     assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k,skew", [(24, 3072, 3200, 8, 2, False),    # 32-row tiles, 24 and 25 slots of K
+                                            (60, 2560, 2688, 8, 4, True)])    # 64 rows, 20 and 21 slots
+def test_fp8w_tiles_on_demand(T, H, I, E, k, skew):
+    """Long tiles and more than one per CTA in both GEMMs."""
+    inp = make_fp8w_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=8, device="cuda")
+    out, _ = run_fp8w(inp)
+    assert_close_out(bf16_to_f64(out), oracle_out(inp), "fp8w out")
+    again, _ = run_fp8w(inp)
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
 def test_fp8w_with_unit_scales_equals_the_bf16_layer_bit_for_bit():
     """All E4M3 values are bf16 values, and a scale of 1 is exact in bf16: both paths see the same operands."""
     g = torch.Generator().manual_seed(0)

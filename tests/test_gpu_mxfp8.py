@@ -195,6 +195,16 @@ def test_mxfp8_many_short_tiles_per_cta(T, H, I, E, k, skew):
     assert_close_out(bf16_to_f64(out), oracle_mx(inp), "mxfp8 out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k,skew", [(24, 2560, 2688, 8, 2, False), (60, 2688, 2560, 8, 4, True)])  # 32 and 64 rows
+def test_mxfp8_tiles_on_demand(T, H, I, E, k, skew):
+    """20 and 21 slots of K and more than one tile per CTA in both GEMMs."""
+    inp = make_mxfp8_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=3, device="cuda")
+    out, _ = run_mx(inp)
+    assert_close_out(bf16_to_f64(out), oracle_mx(inp), "mxfp8 out")
+    again, _ = run_mx(inp)
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
 @pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
 def test_mxfp8_few_down_tiles_with_two_ctas_each(T, H, I, E, k):
     """Two CTAs per tile of the down GEMM, half of its rows each (2176: 17 slots); the same bits as with one CTA per tile,
