@@ -325,8 +325,7 @@ grouped_gemm_tc_fp8w_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
             const int tile = tile_of_round(round, worker, n_workers);
             if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
-            const bool taken = next_tile(t, round, tile);
-            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
+            const bool taken = next_tile(t, round, tile);  // (at the end of the work the four warps leave as if they gave up: together)
             const int n_mma = (t.n_valid + 15) & ~15;
             ok = taken && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
             if (L::kStaged ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)

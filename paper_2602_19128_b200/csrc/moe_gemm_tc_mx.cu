@@ -246,8 +246,7 @@ grouped_gemm_tc_mx_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps
             const int tile = tile_of_round(round, worker, n_workers);
             if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
-            const bool taken = next_tile(t, round, tile);
-            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
+            const bool taken = next_tile(t, round, tile);  // (at the end of the work the four warps leave as if they gave up: together)
             const int n_mma = (t.n_valid + 15) & ~15;
             bool ok = taken && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
             if (epilogue_any(!ok)) break;  // the four warps synchronise inside the tile (SwiGLU): they leave together

@@ -64,11 +64,11 @@ struct MxPairSmem {
     static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
-    static constexpr int kBytes = kTiles + TileQueue::kBytes;
+    static constexpr int kBytes = kTiles + PairTileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED, int QUEUE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16> maps, const MxParams p) {
     using L = MxPairSmem<NT_MAX, STAGES, !STAGED ? 0 : SWIGLU ? 2 * kMxStageBytes : Stage<false>::kBytes>;
@@ -89,7 +89,7 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16>
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
-    const TileQueue tiles(base_ptr, base, L::kTiles);
+    const PairTileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_mx_tile(tile, p); };
     auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
@@ -136,10 +136,11 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16>
         bool ok = true, gate_up_done = false;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
             ok = tiles.take(t, round, lane, queue_wait);
             if (!ok) break;
+            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
             const int n_mma = (t.n_valid + 15) & ~15, half = n_mma >> 1;
             const int cta_tile = 2 * t.f + (int)rank;  // this CTA's 128 weight rows
             const int w_sf_row = (t.e * w_tiles_per_expert + cta_tile) * p.n_k_blocks;
@@ -196,10 +197,11 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16>
             const uint32_t sfa_tmem = tmem_base + kSfACol, sfb_tmem = tmem_base + kSfBCol;
             for (int round = 0; ok; ++round) {
                 const int tile = tile_of_round(round, pair, n_pairs);
-                if (tile >= total_tiles) break;
+                if (QUEUE != kOnDemand && tile >= total_tiles) break;
                 MxTile t;
                 ok = tiles.take(t, round, lane, queue_wait);
                 if (!ok) break;
+                if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
                 const int n_mma = (t.n_valid + 15) & ~15;
                 ok = __all_sync(0xffffffffu, pair_wait(bar_acc_empty + acc * 8, acc_phase ^ 1u, abort_flag, peer_abort,
                                                        p.status, kSiteMmaTmemEmpty + kSiteOffset));
@@ -251,9 +253,9 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16>
         int buf = 0;
         for (int round = 0;; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
-            const bool taken = tiles.take(t, round, lane, queue_wait);
+            const bool taken = tiles.take(t, round, lane, queue_wait) && (QUEUE != kOnDemand || t.e >= 0);
             const int n_mma = (t.n_valid + 15) & ~15;
             const bool ok = taken && pair_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, peer_abort, p.status,
                                       kSiteEpilogueTmemFull + kSiteOffset);
@@ -281,7 +283,13 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16>
         }
     } else if (warp == 7) {
         // ---------------- decoder ----------------
-        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
+        if constexpr (QUEUE == kOnDemand)
+            tiles.fill_pair_on_demand<MxTile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+                                          [&](uint32_t bar, uint32_t parity) {
+                return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
+            });
+        else
+            tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------
@@ -300,7 +308,8 @@ int launch_pair_instance(const MxPairMaps &maps, const MxParams &p, int grid, cu
     using L = MxPairSmem<NT_MAX, STAGES, !STAGED ? 0 : SWIGLU ? 2 * kMxStageBytes : Stage<false>::kBytes>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
     const MxPairMapsOf<NT_MAX / 16> own = {TensorMapsOf<NT_MAX / 16>(maps.ops), maps.w_sf, maps.act_sf};
-    auto kernel = grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED>;
+    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
+    auto kernel = on_demand ? grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kOnDemand> : grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, own, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;

@@ -33,7 +33,6 @@ constexpr int kChunkCols = 16;       // granularity of the accumulator ring: the
 constexpr int kAccCols = 496;        // accumulator columns; the scales take the last 16 of tensor memory
 constexpr int kNumChunks = kAccCols / kChunkCols;  // 31
 constexpr int kAccFullBars = 32;     // tiles between the MMA warp and the epilogue: each holds at least one chunk
-constexpr int kTileQueue = 16;       // more entries than ring slots: the producer is at most STAGES tiles ahead
 constexpr uint32_t kSfACol = kAccCols, kSfBCol = kAccCols + 4;
 
 struct MxRingMaps {
@@ -68,11 +67,10 @@ struct MxRingSmem {
     static constexpr int kOutStage = kAmax + kAmaxBytes;  // the epilogue's buffers
     // full[S], empty[S], acc_full[32], acc_empty[32 (31 used)]
     static constexpr int kBars = kOutStage + (!SWIGLU ? Stage<false>::kBytes : STAGED ? 2 * kMxStageBytes : 0);
-    static constexpr int kQueue = kBars + (2 * STAGES + kAccFullBars + 32) * 8;
-    static constexpr int kTmemSlot = kQueue + kTileQueue * 4;
+    static constexpr int kTmemSlot = kBars + (2 * STAGES + kAccFullBars + 32) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
-    static constexpr int kBytes = kTiles + TileQueue::kBytes;
+    static constexpr int kBytes = kTiles + PairTileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
@@ -95,13 +93,12 @@ __device__ __forceinline__ MxParts split_mx_tile(int seq, int n_cols) {
     return s;
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED>
+template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED, int QUEUE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMxRingThreads, 1)
 grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const MxParams p) {
     using L = MxRingSmem<NT_MAX, STAGES, SWIGLU, STAGED>;
     static_assert(NT_MAX % 16 == 0 && NT_MAX <= 384 && NT_MAX > 256, "token-tile bound of the wide-tile kernel");
     static_assert(L::kAtomsB == 3, "three token scale atoms next to the weight scales");
-    static_assert(STAGES < kTileQueue, "the tile queue must outlast the ring");
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;
     constexpr int kFeatPerCta = SWIGLU ? kTileM / 2 : kTileM;  // h features resp. output rows per CTA of a pair tile
     chain_release();  // the next kernel of the forward call may be scheduled; it waits for what it needs of this grid
@@ -110,14 +107,13 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
     const uint32_t bar_full = base + L::kBars, bar_empty = bar_full + STAGES * 8;
     const uint32_t bar_acc_full = bar_empty + STAGES * 8, bar_acc_empty = bar_acc_full + kAccFullBars * 8;
-    volatile int *queue = reinterpret_cast<volatile int *>(base_ptr + L::kQueue);
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(base_ptr + L::kTmemSlot);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
-    const TileQueue tiles(base_ptr, base, L::kTiles);
+    const PairTileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_mx_tile(tile, p); };
     auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
@@ -127,7 +123,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
         }
         for (int a = 0; a < kAccFullBars; ++a) mbar_init(bar_acc_full + a * 8, 1);
         for (int c = 0; c < kNumChunks; ++c) mbar_init(bar_acc_empty + c * 8, 2 * kEpilogueWarps);
-        tiles.init(2 + kEpilogueWarps);
+        tiles.init((rank == 0 ? 3 : 2) + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -162,10 +158,11 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
         bool ok = true, gate_up_done = false;
         for (int round = 0; ok; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
             ok = tiles.take(t, round, lane, queue_wait);
             if (!ok) break;
+            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
             const int n_mma = (t.n_valid + 15) & ~15;
             const MxParts parts = split_mx_tile(seq, n_mma);
             const int cta_tile = 2 * t.f + (int)rank;  // this CTA's 128 weight rows
@@ -184,8 +181,6 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
                     const int k0 = kb * kMxSlotK;
                     if (load_w) {
                         if (rank == 0) {
-                            // the MMA warp learns the tile's width from here, after this slot's barrier
-                            if (kb == 0) queue[seq & (kTileQueue - 1)] = n_mma;
                             mbar_expect_tx(bar_full + stage * 8,
                                            2 * (kMxSlotABytes + kMxSfAtomBytes + L::kSfBBytes) + n_mma * kMxSlotK);
                         }
@@ -234,12 +229,16 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
             const uint32_t sfa_tmem = tmem_base + kSfACol, sfb_tmem = tmem_base + kSfBCol;
             for (int round = 0; ok; ++round, ++seq) {
                 const int tile = tile_of_round(round, pair, n_pairs);
-                if (tile >= total_tiles) break;
+                if (QUEUE != kOnDemand && tile >= total_tiles) break;
+                MxTile t;
+                ok = tiles.take(t, round, lane, queue_wait);
+                if (!ok) break;
+                if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
                 ok = __all_sync(0xffffffffu, pair_wait(bar_full + stage * 8, phase, abort_flag, peer_abort, p.status,
                                                        kSiteMmaFull + kSiteOffset));
                 if (!ok) break;
-                // the tile's width, then its chunks of the accumulator ring, each free of its last occupant
-                const int n_mma = queue[seq & (kTileQueue - 1)];
+                // the tile's chunks of the accumulator ring, each free of its last occupant
+                const int n_mma = (t.n_valid + 15) & ~15;
                 const int n_chunks = n_mma / kChunkCols;
                 const MxParts parts = split_mx_tile(seq, n_mma);
                 {   // lane c waits for the tile's c-th chunk (a tile has at most 24)
@@ -305,9 +304,9 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
         int buf = 0, seq = 0, out_flip = 0;
         for (int round = 0;; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             MxTile t;
-            const bool taken = tiles.take(t, round, lane, queue_wait);
+            const bool taken = tiles.take(t, round, lane, queue_wait) && (QUEUE != kOnDemand || t.e >= 0);
             const int n_mma = (t.n_valid + 15) & ~15;
             const MxParts parts = split_mx_tile(seq, n_mma);
             const bool ok = taken && pair_wait(bar_acc_full + (seq & (kAccFullBars - 1)) * 8, (uint32_t)(seq / kAccFullBars) & 1u, abort_flag,
@@ -362,7 +361,13 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
         }
     } else if (warp == 7) {
         // ---------------- decoder ----------------
-        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
+        if constexpr (QUEUE == kOnDemand)
+            tiles.fill_pair_on_demand<MxTile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+                                          [&](uint32_t bar, uint32_t parity) {
+                return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
+            });
+        else
+            tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------
@@ -380,7 +385,8 @@ template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED = true>
 int launch_mx_ring_instance(const MxRingMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
     using L = MxRingSmem<NT_MAX, STAGES, SWIGLU, STAGED>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED>;
+    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
+    auto kernel = on_demand ? grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kOnDemand> : grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kMxRingThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;

@@ -54,11 +54,11 @@ struct PairSmem {
     static constexpr int kTmemSlot = kBars + (2 * STAGES + 4) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
-    static constexpr int kBytes = kTiles + TileQueue::kBytes;
+    static constexpr int kBytes = kTiles + PairTileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
-template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED>
+template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED, int QUEUE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const KernelParams p) {
     using L = PairSmem<NT_MAX, STAGES, SLABS, STAGED ? kStageBytes : 0>;
@@ -85,7 +85,7 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
-    const TileQueue tiles(base_ptr, base, L::kTiles);
+    const PairTileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_tile(tile, p); };
     auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
@@ -132,10 +132,11 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         bool ok = true, gate_up_done = false;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = tiles.take(t, round, lane, queue_wait);
             if (!ok) break;
+            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
             const int n_mma = (t.n_valid + 15) & ~15, half = n_mma >> 1;  // each CTA stages half: a multiple of 8 rows
             const int feat0 = t.f * kFeatPerTile + (int)rank * kFeatPerCta;  // this CTA's part of slab 0
             if (load_act) {  // the token rows of a down GEMM are the gate/up GEMM's output for this expert
@@ -190,10 +191,11 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
             bool ok = true;
             for (int round = 0; ok; ++round) {
                 const int tile = tile_of_round(round, pair, n_pairs);
-                if (tile >= total_tiles) break;
+                if (QUEUE != kOnDemand && tile >= total_tiles) break;
                 Tile t;
                 ok = tiles.take(t, round, lane, queue_wait);
                 if (!ok) break;
+                if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
                 const uint32_t idesc = instr_desc_bf16(2 * kTileM, (t.n_valid + 15) & ~15);
                 ok = __all_sync(0xffffffffu, pair_wait(bar_acc_empty + acc * 8, acc_phase ^ 1u, abort_flag, peer_abort,
                                                        p.status, kSiteMmaTmemEmpty + kSiteOffset));
@@ -242,9 +244,9 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         bool ok = true;
         for (int round = 0; ok; ++round) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
-            const bool taken = tiles.take(t, round, lane, queue_wait);
+            const bool taken = tiles.take(t, round, lane, queue_wait) && (QUEUE != kOnDemand || t.e >= 0);
             const int n_mma = (t.n_valid + 15) & ~15;
             ok = taken && pair_wait(bar_acc_full + acc * 8, acc_phase, abort_flag, peer_abort, p.status, kSiteEpilogueTmemFull + kSiteOffset);
             if (STAGED ? epilogue_any(!ok) : !__all_sync(0xffffffffu, ok)) break;  // (the four warps meet inside a staged tile)
@@ -267,7 +269,13 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
         }
     } else if (warp == 7) {
         // ---------------- decoder ----------------
-        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
+        if constexpr (QUEUE == kOnDemand)
+            tiles.fill_pair_on_demand<Tile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+                                          [&](uint32_t bar, uint32_t parity) {
+                return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
+            });
+        else
+            tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------
@@ -286,7 +294,8 @@ template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED>
 int launch_pair_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = PairSmem<NT_MAX, STAGES, SLABS, STAGED ? kStageBytes : 0>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED>;
+    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
+    auto kernel = on_demand ? grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kOnDemand> : grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;

@@ -40,7 +40,6 @@ constexpr int kRingThreads = 256;   // warp 0 weight TMA, warp 1 MMA, warps 2..5
 constexpr int kChunkCols = 16;      // granularity of the accumulator ring: the MMA's N granularity
 constexpr int kNumChunks = 32;      // 512 columns of tensor memory
 constexpr int kAccFullBars = 32;    // tiles between the MMA warp and the epilogue: each holds at least one chunk
-constexpr int kTileQueue = 16;      // more entries than ring slots: the producer is at most STAGES tiles ahead
 constexpr int kRingActMaps = 24;    // act[i]: box of 8 * (i + 1) rows, up to 192 rows per CTA (N = 384)
 
 struct RingMaps {
@@ -77,11 +76,10 @@ struct RingSmem {
     static constexpr int kB = STAGES * kSlotABytes;
     static constexpr int kOutStage = kB + STAGES * kSlotBBytes;  // the epilogue's buffers (Stage)
     static constexpr int kBars = kOutStage + kStageBytes;  // full[S], empty[S], acc_full[32], acc_empty[32]
-    static constexpr int kQueue = kBars + (2 * STAGES + kAccFullBars + kNumChunks) * 8;
-    static constexpr int kTmemSlot = kQueue + kTileQueue * 4;
+    static constexpr int kTmemSlot = kBars + (2 * STAGES + kAccFullBars + kNumChunks) * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kTiles = (kAbort + 4 + 15) / 16 * 16;  // TileQueue
-    static constexpr int kBytes = kTiles + TileQueue::kBytes;
+    static constexpr int kBytes = kTiles + PairTileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
@@ -105,12 +103,11 @@ __device__ __forceinline__ Parts split_tile(int seq, int n_cols) {
     return s;
 }
 
-template <int NT_MAX, int STAGES, bool SWIGLU>
+template <int NT_MAX, int STAGES, bool SWIGLU, int QUEUE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kRingThreads, 1)
 grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelParams p) {
     using L = RingSmem<NT_MAX, STAGES>;
     static_assert(NT_MAX % 16 == 0 && NT_MAX <= 16 * kRingActMaps && NT_MAX <= 384, "token-tile bound");
-    static_assert(STAGES < kTileQueue, "the tile queue must outlast the ring");
     constexpr int kTmemCols = kNumChunks * kChunkCols;   // all of tensor memory (a power of two)
     constexpr int kSiteOffset = SWIGLU ? 0 : 4;          // the down GEMM reports sites 5..8
     constexpr int kFeatPerCta = SWIGLU ? kTileM / 2 : kTileM;
@@ -121,14 +118,13 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
     const uint32_t bar_full = base + L::kBars, bar_empty = bar_full + STAGES * 8;
     const uint32_t bar_acc_full = bar_empty + STAGES * 8, bar_acc_empty = bar_acc_full + kAccFullBars * 8;
-    volatile int *queue = reinterpret_cast<volatile int *>(base_ptr + L::kQueue);
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(base_ptr + L::kTmemSlot);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(base_ptr + L::kAbort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t peer_abort = map_to_cta(base + L::kAbort, rank ^ 1u);
-    const TileQueue tiles(base_ptr, base, L::kTiles);
+    const PairTileQueue tiles(base_ptr, base, L::kTiles);
     auto decode = [&](int tile) { return decode_tile(tile, p); };
     auto queue_wait = [&](uint32_t bar, uint32_t parity) { return pair_wait(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset); };
     if (threadIdx.x == 0) {
@@ -138,7 +134,7 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
         }
         for (int a = 0; a < kAccFullBars; ++a) mbar_init(bar_acc_full + a * 8, 1);
         for (int c = 0; c < kNumChunks; ++c) mbar_init(bar_acc_empty + c * 8, 2 * kEpilogueWarps);
-        tiles.init(2 + kEpilogueWarps);
+        tiles.init((rank == 0 ? 3 : 2) + kEpilogueWarps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -171,10 +167,11 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
         bool ok = true, gate_up_done = false;
         for (int round = 0; ok; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
             ok = tiles.take(t, round, lane, queue_wait);
             if (!ok) break;
+            if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
             const int n_mma = (t.n_valid + 15) & ~15, half = n_mma >> 1;  // each CTA stages half: a multiple of 8 rows
             const int feat0 = t.f * kFeatPerTile + (int)rank * kFeatPerCta;
             if (load_act) {  // the token rows of a down GEMM are the gate/up GEMM's output for this expert
@@ -212,8 +209,6 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
                     const int k0 = kb * kBlockK;
                     if (load_w) {
                         if (rank == 0) {
-                            // the MMA warp learns the tile's width from here, after this slot's barrier
-                            if (kb == 0) queue[seq & (kTileQueue - 1)] = n_mma;
                             mbar_expect_tx(bar_full + stage * 8, 2 * kSlotABytes + n_mma * kRowBytes);
                         }
                         const uint32_t sa = base + L::kA + stage * kSlotABytes;
@@ -250,7 +245,11 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
             bool ok = true;
             for (int round = 0; ok; ++round, ++seq) {
                 const int tile = tile_of_round(round, pair, n_pairs);
-                if (tile >= total_tiles) break;
+                if (QUEUE != kOnDemand && tile >= total_tiles) break;
+                Tile t;
+                ok = tiles.take(t, round, lane, queue_wait);
+                if (!ok) break;
+                if (QUEUE == kOnDemand && t.e < 0) break;  // (no more tiles)
                 Parts parts;
                 parts.n = 0;
                 for (int kb = 0; kb < p.n_k_blocks; ++kb) {
@@ -258,8 +257,8 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
                                                            kSiteMmaFull + kSiteOffset));
                     if (!ok) break;
                     if (kb == 0) {
-                        // the tile's width, then its chunks of the accumulator ring, each free of its last occupant
-                        const int n_mma = queue[seq & (kTileQueue - 1)];
+                        // the tile's chunks of the accumulator ring, each free of its last occupant
+                        const int n_mma = (t.n_valid + 15) & ~15;
                         const int n_chunks = n_mma / kChunkCols;
                         parts = split_tile(seq, n_mma);
                         {   // lane c waits for the tile's c-th chunk
@@ -308,9 +307,9 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
         bool ok = true;
         for (int round = 0; ok; ++round, ++seq) {
             const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
             Tile t;
-            const bool taken = tiles.take(t, round, lane, queue_wait);
+            const bool taken = tiles.take(t, round, lane, queue_wait) && (QUEUE != kOnDemand || t.e >= 0);
             const int n_mma = (t.n_valid + 15) & ~15, half_tile = n_mma >> 1;
             const Parts parts = split_tile(seq, n_mma);
             ok = taken && pair_wait(bar_acc_full + (seq & (kAccFullBars - 1)) * 8, (uint32_t)(seq / kAccFullBars) & 1u, abort_flag, peer_abort,
@@ -366,7 +365,13 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
         }
     } else if (warp == 7) {
         // ---------------- decoder ----------------
-        tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
+        if constexpr (QUEUE == kOnDemand)
+            tiles.fill_pair_on_demand<Tile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+                                          [&](uint32_t bar, uint32_t parity) {
+                return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
+            });
+        else
+            tiles.fill(pair, n_pairs, total_tiles, lane, decode, queue_wait);
     }
 
     // ---------------- teardown ----------------
@@ -385,7 +390,8 @@ template <int NT_MAX, int STAGES, bool SWIGLU>
 int launch_ring_instance(const RingMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = RingSmem<NT_MAX, STAGES>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    auto kernel = grouped_gemm_tc_ring_kernel<NT_MAX, STAGES, SWIGLU>;
+    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
+    auto kernel = on_demand ? grouped_gemm_tc_ring_kernel<NT_MAX, STAGES, SWIGLU, kOnDemand> : grouped_gemm_tc_ring_kernel<NT_MAX, STAGES, SWIGLU, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kRingThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;

@@ -83,5 +83,101 @@ __device__ __forceinline__ bool pair_wait(uint32_t bar, uint32_t parity, volatil
     return ok;
 }
 
+// The same, acquiring at cluster scope: for a barrier behind which the peer has written this CTA's shared memory.
+__device__ __forceinline__ bool pair_wait_acquire(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t peer_abort,
+                                                  int *status, int site) {
+    const long long start = clock64();
+    while (true) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity), "r"(kWaitSuspendNs)
+            : "memory");
+        if (done) return true;
+        bool expired = *abort_flag != 0;
+        if (!expired && clock64() - start > kWaitLimitCycles) {
+            *abort_flag = 1;
+            expired = true;
+            if (atomicCAS(status, 0, (int)MOE_ERR_DEVICE_TIMEOUT) == 0) {
+                status[1] = site;
+                status[2] = blockIdx.x;
+            }
+        }
+        if (expired) {
+            store_cluster_u32(peer_abort, 1u);
+            return false;
+        }
+    }
+}
+
+// Which pair GEMMs draw their tiles: those with K loops of 80 slots and more, whose tiles are so long that the static assignment's
+// rounds show (512 Mixtral-shaped tokens: 128 tiles of the down GEMM on 74 pairs, which began up to 30 us apart).  Static / on demand,
+// medians of alternating runs: that call 534 / 519 us, 1024 MX tokens of the same shape 436 / 409, MX prefill on 32 of 256 experts
+// 495 / 475..520 / 518.  With shorter loops the next tile is wanted before the epilogue, which is then most of a tile behind, lets it be
+// drawn: at 32 slots 4096 MX tokens of 128 experts of 4096 x 1536, top 8, 860 / 884 us, skewed 731 / 775; 2000 tokens of 64 of 2048 x
+// 2048, top 4, 346 / 353.  (Drawn two ahead those are level, but 512 Mixtral-shaped tokens take 575.)
+inline bool pair_tiles_on_demand(int slots_per_tile) { return slots_per_tile >= 80; }
+
+// Tiles on demand for a CTA pair: the leader's decoder draws them and passes each on to the peer's decoder through one entry in the
+// peer's shared memory; both publish them in their own CTA's queue.
+//   behind the queue: the inbox entry of eight words, inbox_full (in the peer: the leader's arrival), inbox_empty (in the leader: the
+//   peer's)
+struct PairTileQueue : TileQueue {
+    static constexpr int kBytes = TileQueue::kBytes + 32 + 16;
+    int *inbox;
+    uint32_t inbox_addr, inbox_full, inbox_empty;
+    __device__ __forceinline__ PairTileQueue(uint8_t *base_ptr, uint32_t base, int offset)
+        : TileQueue(base_ptr, base, offset), inbox(reinterpret_cast<int *>(base_ptr + offset + TileQueue::kBytes)),
+          inbox_addr(base + offset + TileQueue::kBytes), inbox_full(inbox_addr + 32), inbox_empty(inbox_addr + 40) {}
+    __device__ __forceinline__ void init(int takers) const {  // by one thread
+        TileQueue::init(takers);
+        mbar_init(inbox_full, 1);
+        mbar_init(inbox_empty, 1);
+    }
+    // wait / wait_acquire(bar, parity): bounded waits, the second acquiring at cluster scope.
+    template <typename T, typename Decode, typename Wait, typename WaitAcquire>
+    __device__ __forceinline__ void fill_pair_on_demand(uint32_t rank, int pair, int n_pairs, int total_tiles, int *counter, int lane,
+                                                        Decode decode, Wait wait, WaitAcquire wait_acquire) const {
+        constexpr int kWords = (int)(sizeof(T) / 4);
+        for (int n = 0;; ++n) {
+            T t;
+            int *w = reinterpret_cast<int *>(&t);
+            if (rank == 0) {
+                int tile = pair;
+                if (n > 0) {
+                    const int m = n - 1;
+                    if (!__all_sync(0xffffffffu, wait(empty + (m & (kDepth - 1)) * 8, (m / kDepth) & 1))) break;
+                    if (lane == 0) tile = n_pairs + atomicAdd(counter, 1);
+                    tile = __shfl_sync(0xffffffffu, tile, 0);
+                }
+                t.e = -1;
+                if (tile < total_tiles) t = decode(tile);
+                publish(t, n, lane);
+                if (n > 0 && !__all_sync(0xffffffffu, wait(inbox_empty, (n - 1) & 1))) break;
+                if (lane == 0) {
+                    const uint32_t dst = map_to_cta(inbox_addr, 1);
+#pragma unroll
+                    for (int k = 0; k < kWords; ++k) store_cluster_u32(dst + 4 * k, (uint32_t)w[k]);
+                    mbar_arrive_cluster(map_to_cta(inbox_full, 1));
+                }
+                __syncwarp();
+            } else {
+                if (!__all_sync(0xffffffffu, wait_acquire(inbox_full, n & 1))) break;
+                const volatile int *in = inbox;
+#pragma unroll
+                for (int k = 0; k < kWords; ++k) w[k] = in[k];
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_to_cta(inbox_empty, 0));
+                if (!__all_sync(0xffffffffu, wait(empty + (n & (kDepth - 1)) * 8, ((n / kDepth) & 1) ^ 1))) break;
+                publish(t, n, lane);
+            }
+            if (t.e < 0) break;
+        }
+    }
+};
+
 }  // namespace tc
 }  // namespace moe

@@ -103,7 +103,8 @@ def test_many_short_tiles_per_cta(T, H, I, E, k, skew):
 
 @pytest.mark.parametrize("T,H,I,E,k,skew", [(40, 1280, 1344, 16, 2, False),   # 32-row tiles, 20 and 21 slots of K
                                             (150, 1408, 1280, 16, 4, True),   # 64 rows, ragged
-                                            (32, 1280, 1280, 32, 8, True)])   # some experts without tokens
+                                            (32, 1280, 1280, 32, 8, True),    # some experts without tokens
+                                            (66, 5120, 5120, 2, 2, False)])   # CTA pairs, 80 slots, 80 tiles on 74 pairs
 def test_tiles_on_demand(T, H, I, E, k, skew):
     """Long tiles and more than one per CTA in both GEMMs: handed out by a counter that every call starts anew."""
     inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=2)

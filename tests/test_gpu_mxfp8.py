@@ -205,6 +205,19 @@ def test_mxfp8_tiles_on_demand(T, H, I, E, k, skew):
     assert torch.equal(out.view(torch.int16), again.view(torch.int16))
 
 
+@pytest.mark.parametrize("T", [100, 520])  # 128-row tiles and wide ones, 80 slots of K, 80 tiles of the gate/up GEMM on 74 pairs
+def test_mxfp8_pair_tiles_on_demand(T):
+    H, I, E, k = 10240, 5120, 2, 1
+    inp = make_mxfp8_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=4, device="cuda")
+    out, _ = run_mx(inp)
+    tokens = np.unique(np.concatenate([[0, T - 1], np.arange(3, T, T // 6)]))
+    experts = {e: tuple(inp[n][e].cpu().numpy() for n in ("w13_q", "w13_s", "w2_q", "w2_s")) for e in range(E)}
+    ref = moe_oracle.get("f32").forward_mxfp8_sampled(bf16_bits(inp["x"]), inp["router_logits"].cpu().numpy(), experts, I, k, tokens)
+    assert_close_out(bf16_to_f64(out[torch.from_numpy(tokens).long().cuda()]), ref, "mxfp8 sampled out")
+    again, _ = run_mx(inp)
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
 @pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
 def test_mxfp8_few_down_tiles_with_two_ctas_each(T, H, I, E, k):
     """Two CTAs per tile of the down GEMM, half of its rows each (2176: 17 slots); the same bits as with one CTA per tile,
