@@ -38,6 +38,7 @@
 #include <string.h>
 
 #include "gqa_decode.h"
+#include "moe_internal.cuh"
 
 namespace moe {
 namespace tc {
@@ -49,8 +50,6 @@ bool encode_kv_cache_map(CUtensorMap *map, const void *cache, uint64_t num_pages
 // (moe_tc_host.cu) cudaFuncAttributeMaxDynamicSharedMemorySize, set once per kernel and device, under a mutex.
 bool set_max_dynamic_smem_once(const void *kernel, int bytes);
 }  // namespace tc
-// (moe_api.cu) MOE_OK when the current device has compute capability 10.x (cached per device), else an error code.
-int check_device();
 }  // namespace moe
 
 namespace gqa {
@@ -97,8 +96,11 @@ struct Params {
 
 // ---- the launches of a call --------------------------------------------------------------------------------------
 // Where parts of sequences may have to be counted, a memset in front of the kernel zeroes the status word and the counters.
-// Where no sequence is split there is nothing to count, and the kernel's first block zeroes the status word
-// (Params::own_status): one launch.  In a loop / on the first pass over new inputs: 1 sequence of 100 tokens 8.5 -> 7.6 us / 25.7 ->
+// Where no sequence is split there is nothing to count, and the kernel's first block zeroes the status word: one launch
+// (Params::own_status), with programmatic serialisation (kChained), so that a kernel's start overlaps the end of the one in front (behind a
+// memset it cannot).
+// Loops without / with: 40 sequences of 31..251 tokens 8.2 / 7.3 us, 162 of 410..821 43.6 / 41.7, 256 of 256..2048 102.5 / 100.7.
+// Memset / one launch, in a loop / on the first pass over new inputs: 1 sequence of 100 tokens 8.5 -> 7.6 us / 25.7 ->
 // 21.7, 256 of 256..2048 105.5 -> 102.8 / 138 -> 133.  A wait gives up after 4 million polls, long after that block has started.
 // (A small kernel that zeroed the words beside a decode kernel launched with programmatic serialisation made loops 0.7 to 2
 // us shorter, but first passes 2.3 longer, memset / small kernel: 1 sequence of 65 536 tokens 36.9 / 36.2 and 58.3 / 61.3, 1 of
@@ -330,7 +332,7 @@ __global__ void __launch_bounds__(kThreads) gqa_wait_timeout_selftest_kernel(int
     if (any_compute(!ok) && (threadIdx.x & 31) == 0) atomicAdd(status + 3, 1);
 }
 
-// By the first block, before it waits for anything.  (In the row gather within the barrier's set-up, as one store by one thread:
+// By the first block of a kernel that is alone.  (In the row gather within the barrier's set-up, as one store by one thread:
 // first thing in the kernel, by four threads, it cost the row gather 2 %, 70 sequences of 1087..2175 131.3 -> 134.6 us.)
 __device__ __forceinline__ void zero_own_status(const Params &p, bool first_block, int tid) {
     if (p.own_status && first_block && tid == 0) *reinterpret_cast<uint4 *>(p.status) = make_uint4(0, 0, 0, 0);
@@ -570,6 +572,7 @@ __device__ __forceinline__ void count_and_merge(const Params &p, BlockParts &s, 
 // The row gather, for page sizes TMA boxes cannot follow: one 256-byte bulk copy per token row, issued by the 128 compute
 // threads themselves, two stages in three blocks per SM, a block barrier per chunk; one block per (sequence split,
 // key-value head, item).
+template <bool kChained>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
 gqa_row_decode_kernel(const Params p) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -580,6 +583,10 @@ gqa_row_decode_kernel(const Params p) {
     const int split = blockIdx.x, kvh = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool first_block = (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
+    if (kChained) {
+        moe::chain_release();
+        moe::chain_wait();
+    }
     const int L = cached_tokens(p, b);
     const int head0 = kvh * p.group;
 
@@ -723,7 +730,7 @@ __device__ __forceinline__ bool balanced_is_faster(long long total, int longest_
     return fmaxf(stream, 0.9f * longest) + 0.15f * (longest - average) + merge > stream + 11.f;
 }
 
-template <bool kAdaptive>
+template <bool kAdaptive, bool kChained>
 __global__ void __launch_bounds__(kThreads + 32, 2)
 gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap v_map) {
     extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -736,7 +743,8 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t smem_base = smem_u32(smem), full_base = smem_u32(full_bar), empty_base = smem_u32(empty_bar);
     const int sh = 31 - __clz(p.box_rows);  // log2 of the rows of a box
-    if (!kAdaptive) zero_own_status(p, blockIdx.x == 0, tid);
+    static_assert(!kAdaptive || !kChained, "parts may be counted");
+    if (kChained) moe::chain_release();
     if (tid == 0) {
         for (int s = 0; s < kTiledStages; ++s) {
             mbar_init(full_base + s * 8, 32);       // the copy warp's lanes
@@ -746,6 +754,11 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         parts.part[0].n_parts = parts.part[1].n_parts = 1;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+
+    if (kChained) {
+        moe::chain_wait();  // (the set-up above overlaps the end of what is in front)
+        zero_own_status(p, blockIdx.x == 0, tid);
     }
 
     // ---- this block's piece: w_end - w chunks, the first of them chunk c of sequence (b, kvh) ----
@@ -1131,20 +1144,23 @@ int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, co
     if (tiled && (!moe::tc::encode_kv_cache_map(&k_map, k_cache, (uint64_t)num_pages, (uint32_t)page_size, (uint32_t)Hkv, (uint32_t)p.box_rows) ||
                   !moe::tc::encode_kv_cache_map(&v_map, v_cache, (uint64_t)num_pages, (uint32_t)page_size, (uint32_t)Hkv, (uint32_t)p.box_rows)))
         return MOE_ERR_CUDA;
-    auto launch = [&](auto kernel, dim3 grid, int threads, int smem_bytes, const auto &...args) {
-        if (!moe::tc::set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), smem_bytes)) return MOE_ERR_CUDA;
-        if (!p.own_status && cudaMemsetAsync(p.status, 0, 256 + bh * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
-        kernel<<<grid, threads, smem_bytes, st>>>(args...);
-        return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
-    };
     const unsigned shares = (unsigned)(bh * p.n_splits);
     // Two slots per balanced block: where the workspace has them, and the fixed shares fill the machine at most twice.
     const bool adaptive = tiled && bh * slots >= 2 * kBalancedBlocks && bh * p.n_splits <= 2 * kBalancedBlocks;
     p.own_status = p.n_splits == 1 && !adaptive;  // (no part is ever counted)
-    if (!tiled) return launch(gqa_row_decode_kernel, dim3(p.n_splits, Hkv, B), kThreads, kSmemBytes, p);
+    // The row gather's loop is at the limit of its registers, and the wait in front of it cost sequences of 1059..2118 tokens 3 % (27 over 8
+    // heads, pages of one token, 75.2 / 77.5 us); short ones gain the launch (14 of 119..239 12.3 / 11.3).
+    const bool chained = p.own_status && (tiled || max_kv_len <= 512);
+    auto launch = [&](auto kernel, dim3 grid, int threads, int smem_bytes, const auto &...args) {
+        if (!moe::tc::set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), smem_bytes)) return MOE_ERR_CUDA;
+        if (!p.own_status && cudaMemsetAsync(p.status, 0, 256 + bh * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
+        return moe::launch_clusters(kernel, chained, 1, grid, threads, smem_bytes, st, args...) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+    };
+    if (!tiled)
+        return launch(chained ? gqa_row_decode_kernel<true> : gqa_row_decode_kernel<false>, dim3(p.n_splits, Hkv, B), kThreads, kSmemBytes, p);
     if (adaptive)
-        return launch(gqa_tiled_decode_kernel<true>, shares > kBalancedBlocks ? shares : kBalancedBlocks, kThreads + 32, kSmemBytesTiled, p, k_map, v_map);
-    return launch(gqa_tiled_decode_kernel<false>, shares, kThreads + 32, kSmemBytesTiled, p, k_map, v_map);
+        return launch(gqa_tiled_decode_kernel<true, false>, shares > kBalancedBlocks ? shares : kBalancedBlocks, kThreads + 32, kSmemBytesTiled, p, k_map, v_map);
+    return launch(chained ? gqa_tiled_decode_kernel<false, true> : gqa_tiled_decode_kernel<false, false>, shares, kThreads + 32, kSmemBytesTiled, p, k_map, v_map);
 }
 
 }  // extern "C"
