@@ -7,6 +7,7 @@
 //   warps 8..    converters: a thread owns one weight row (= its lane of tensor memory)
 //   warp 1       MMA (leader CTA): A from the tensor memory of both CTAs, B halves from both CTAs' token slots
 //   warps 2..5   epilogue (SwiGLU or plain, two accumulators)
+//   warp 7       draws tiles (on demand)
 //
 // What bounded the one-CTA kernel at 64 rows per tile and more: a slot of 96 rows takes in 16 KiB of codes and 24 KiB of
 // tokens, 640 cycles at 64 bytes per cycle, and three token slots, tied to the three converted ones, do not cover the
@@ -57,6 +58,7 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
 // 333-token Mixtral-shaped layer 342 -> 324 us, 4096 tokens of 128 experts 1531 -> 1493 us.  (The other GEMMs, whose
 // producers run a ring of six slots or more ahead, lost up to 1 % by the same copy; their short tiles are decoded ahead by a warp
 // of its own, TileQueue.)
+constexpr int kLookAheadSlots = 16;  // of a tile drawn on demand: so many slots before the end its successor is asked for
 constexpr int kScheduleInts = 3 * kMaxExperts + 2;
 struct Schedule {
     const int *prefix, *offsets;  // [E+1] token tiles before a schedule position; first row of an expert
@@ -101,6 +103,11 @@ __device__ __forceinline__ Tile decode_tile(int tile, const KernelParams &p, con
     return t;
 }
 
+// Tiles on demand: the queue's entries are numbers, which every role looks up in its CTA's copy of the schedule.
+struct TileNumber {
+    int e, tile;  // e = -1: the end of the work
+};
+
 // Rings of one instance: converted slots beside two accumulators in tensor memory, a converter group for each; shared memory
 // is split between codes (from HBM: at least 96 KiB in flight) and token slots (from L2).  With 128 rows per tile, converted
 // slots / weight stages / token stages of 3 / 6 / 6 took 328 us on the 333-token Mixtral-shaped layer, 4 / 8 / 4 339 us and
@@ -121,11 +128,12 @@ struct Fp8PairSmem {
     static constexpr int kTmemSlot = kBars + kNumBars * 8;
     static constexpr int kAbort = kTmemSlot + 4;
     static constexpr int kSchedule = kAbort + 4;
-    static constexpr int kBytes = kSchedule + kScheduleInts * 4;
+    static constexpr int kTiles = (kSchedule + kScheduleInts * 4 + 15) / 16 * 16;  // PairTileQueue
+    static constexpr int kBytes = kTiles + PairTileQueue::kBytes;
     static constexpr int kDynamicBytes = kPairDynamicSmemBytes;  // (kBytes + 1024 of it are used)
 };
 
-template <int NT_MAX, bool SWIGLU>
+template <int NT_MAX, bool SWIGLU, int QUEUE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__((Fp8PairSmem<NT_MAX>::kThreads), 1)
 grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> maps, const KernelParams p) {
     using L = Fp8PairSmem<NT_MAX>;
@@ -151,7 +159,10 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
     auto wait = [&](uint32_t bar, uint32_t parity, int site) {
         return pair_wait(bar, parity, abort_flag, peer_abort, p.status, site + kSiteOffset);
     };
+    const PairTileQueue tiles(base_ptr, base, L::kTiles);
+    auto queue_wait = [&](uint32_t bar, uint32_t parity) { return wait(bar, parity, kSiteProducerEmpty); };
     if (threadIdx.x == 0) {
+        if constexpr (QUEUE == kOnDemand) tiles.init((rank == 0 ? 3 : 2) + kEpilogueWarps + L::kConv * kGroupWarps);
         for (int s = 0; s < kStagesQ; ++s) {
             mbar_init(bar_q_full + s * 8, 1);
             mbar_init(bar_q_empty + s * 8, kGroupWarps);
@@ -188,6 +199,14 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
     const Schedule sched = stage_schedule(p, reinterpret_cast<int *>(base_ptr + L::kSchedule), started);
     const int total_tiles = sched.total_token_tiles * p.n_feature_tiles;
     const int n_pairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
+    // The tile of a round (by a whole warp), or total_tiles at the end of the work (also of a CTA that is aborting).
+    auto tile_at = [&](int round) {
+        if constexpr (QUEUE == kOnDemand) {
+            TileNumber t;
+            return tiles.take(t, round, lane, queue_wait) && t.e >= 0 ? t.tile : total_tiles;
+        }
+        return tile_of_round(round, pair, n_pairs);
+    };
 
     if (warp == 0) {
         // ---------------- weight TMA (both CTAs, each its own rows) ----------------
@@ -195,7 +214,7 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
         uint32_t phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, pair, n_pairs);
+            const int tile = tile_at(round);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p, sched);
             const int feat0 = (2 * t.f + (int)rank) * kFeatPerCta;
@@ -222,7 +241,7 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
         uint32_t phase = 0;
         bool ok = true, gate_up_done = false;
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, pair, n_pairs);
+            const int tile = tile_at(round);
             if (tile >= total_tiles) break;
             const Tile t = decode_tile(tile, p, sched);
             const int n_mma = (t.n_valid + 15) & ~15, my_rows = n_mma >> 1;
@@ -257,7 +276,7 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
             bool ok = true;
             const uint64_t b_desc0 = smem_desc_k_major_sw128(base + L::kB);
             for (int round = 0; ok; ++round) {
-                const int tile = tile_of_round(round, pair, n_pairs);
+                const int tile = tile_at(round);
                 if (tile >= total_tiles) break;
                 const Tile t = decode_tile(tile, p, sched);
                 const int n_mma = (t.n_valid + 15) & ~15, my_rows = n_mma >> 1;
@@ -327,17 +346,21 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
             const int block = !SWIGLU ? 2 * t.f + (int)rank : ((row & 16) ? p.n_out + gate_row : gate_row) >> 7;
             return p.w_scale + ((size_t)t.e * row_blocks + block) * p.n_k_blocks;
         };
-        int tile = tile_of_round(0, pair, n_pairs), kb = group;
+        int tile = tile_at(0), kb = group;
         const float *scale = tile < total_tiles ? scale_row(tile) : nullptr;
         float next = scale && kb < p.n_k_blocks ? __ldg(scale + kb) : 0.f;
         for (int round = 0; ok && tile < total_tiles; ++round) {
-            const int tile_ahead = tile_of_round(round + 1, pair, n_pairs);
+            int tile_ahead = QUEUE == kOnDemand ? -1 : tile_of_round(round + 1, pair, n_pairs);
             turn = (turn + p.n_k_blocks) % kConv;
             const int kb_ahead = (group - turn + kConv) % kConv;  // first slot of the next tile that is this group's
             const float *scale_ahead = nullptr;
             float next_ahead = 0.f;
             auto look_ahead = [&]() {
                 if (scale_ahead || tile_ahead >= total_tiles) return;
+                if (QUEUE == kOnDemand) {
+                    tile_ahead = tile_at(round + 1);
+                    if (tile_ahead >= total_tiles) return;
+                }
                 scale_ahead = scale_row(tile_ahead);
                 if (kb_ahead < p.n_k_blocks) next_ahead = __ldg(scale_ahead + kb_ahead);
             };
@@ -385,7 +408,8 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
                 if (op >= kStagesT) { op = group; op_phase ^= 1u; }
                 stage += kConv;
                 if (stage >= kStagesQ) { stage = group; phase ^= 1u; }
-                look_ahead();  // (behind the tile's first slot of this group)
+                // (behind the tile's first slot of this group; a tile still to be drawn is not waited for until the last slots)
+                if (QUEUE != kOnDemand || kb + kLookAheadSlots >= p.n_k_blocks) look_ahead();
             }
             look_ahead();
             tile = tile_ahead;
@@ -401,12 +425,14 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
         uint32_t acc_phase = 0;
         bool ok = true;
         for (int round = 0; ok; ++round) {
-            const int tile = tile_of_round(round, pair, n_pairs);
-            if (tile >= total_tiles) break;
-            const Tile t = decode_tile(tile, p, sched);
+            const int tile = tile_at(round);
+            if (QUEUE != kOnDemand && tile >= total_tiles) break;
+            ok = tile < total_tiles;  // (on demand the four warps leave at the end as if they gave up: together)
+            Tile t = {};
+            if (ok) t = decode_tile(tile, p, sched);
             const int n_mma = (t.n_valid + 15) & ~15;
             const int feat0 = (2 * t.f + (int)rank) * kFeatPerCta;
-            ok = wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
+            ok = ok && wait(bar_acc_full + acc * 8, acc_phase, kSiteEpilogueTmemFull);
             if (epilogue_any(!ok)) break;  // the four warps meet inside the tile: they leave together
             tcgen05_fence_after();
             drain_staged<SWIGLU>(tmem_base + ((uint32_t)(q * 32) << 16) + acc * NT_MAX, n_mma, t.n_valid,
@@ -417,6 +443,12 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
             handover_count_tile(p.handover_role, p.handover, t.e, lane);  // (after the accumulator is handed back)
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
+    } else if (QUEUE == kOnDemand && warp == 7) {
+        // ---------------- decoder ----------------
+        tiles.fill_pair_on_demand<TileNumber>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane,
+                                              [](int tile) { return TileNumber{0, tile}; }, queue_wait, [&](uint32_t bar, uint32_t parity) {
+            return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
+        });
     }
 
     // ---------------- teardown ----------------
@@ -434,7 +466,8 @@ template <int NT_MAX, bool SWIGLU>
 int launch_fp8w_pair_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = Fp8PairSmem<NT_MAX>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "rings do not fit in shared memory");
-    auto kernel = grouped_gemm_tc_fp8w_pair_kernel<NT_MAX, SWIGLU>;
+    auto kernel = pair_tiles_on_demand(p.n_k_blocks) ? grouped_gemm_tc_fp8w_pair_kernel<NT_MAX, SWIGLU, kOnDemand>
+                                                     : grouped_gemm_tc_fp8w_pair_kernel<NT_MAX, SWIGLU, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, L::kThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;

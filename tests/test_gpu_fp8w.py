@@ -159,6 +159,29 @@ def test_fp8w_with_unit_scales_equals_the_bf16_layer_bit_for_bit():
     assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
 
 
+def test_fp8w_pair_tiles_on_demand():
+    """80 slots of K and 80 tiles of the down GEMM on 74 pairs, against the bf16 layer on the same values (unit scales: the same
+    bits), and again in the same workspace."""
+    g = torch.Generator(device="cuda").manual_seed(1)
+    T, H, I, E, k = 300, 2560, 10240, 8, 2
+    table = torch.arange(256, dtype=torch.uint8).view(torch.float8_e4m3fn).float()
+    finite = torch.nonzero(~torch.isnan(table) & (table.abs() <= 0.125)).flatten().to(torch.uint8).cuda()
+    codes = lambda *shape: finite[torch.randint(len(finite), shape, generator=g, device="cuda")]
+    c13, c2 = codes(E, 2 * I, H), codes(E, H, I)
+    inp = dict(x=(torch.randn(T, H, generator=g, device="cuda") * 0.1).to(torch.bfloat16),
+               router_logits=torch.randn(T, E, generator=g, device="cuda"), top_k=k, w13_q=c13, w2_q=c2,
+               w13_scale=torch.ones(E, 2 * I // 128, H // 128, device="cuda"), w2_scale=torch.ones(E, H // 128, I // 128, device="cuda"))
+    out, ws = run_fp8w(inp)
+    values = table.to(torch.bfloat16).cuda()
+    ref = torch.empty_like(out)
+    moe.moe_forward(inp["x"], inp["router_logits"], torch.stack([values[c.int()] for c in c13]), torch.stack([values[c.int()] for c in c2]), k, ref,
+                    moe.alloc_workspace(moe.moe_workspace_bytes(T, H, I, E, k), "cuda"), flags=moe.MOE_FLAG_SINGLE_CTA_GEMM)
+    torch.cuda.synchronize()
+    assert torch.isfinite(ref.float()).all() and torch.equal(out.view(torch.int16), ref.view(torch.int16))
+    again, _ = run_fp8w(inp)
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
 def test_fp8w_rejects_shapes_outside_its_envelope():
     inp = make_fp8w_inputs(dict(T=8, H=128, I=128, E=2, top_k=1, skew=False), seed=1, device="cuda")
     out = torch.zeros((8, 128), dtype=torch.bfloat16, device="cuda")
