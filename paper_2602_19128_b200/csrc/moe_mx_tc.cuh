@@ -143,7 +143,8 @@ __device__ __forceinline__ void store_swiglu_mx(const float (&v)[G][16], int lef
     for (int g = 0; g < G; ++g) {
         // The two lanes that hold a column's maximum make its scale, and the sixteen fetch all eight by shuffles.  (Every lane had made
         // all eight, 68 instructions against 17, and where K is short the epilogue is what a tile takes: 4096 tokens of 32 experts of 1024 x
-        // 1024, top 4, 150.2 -> 136.1 us, 2244 skewed ones of 160 of 768 x 3584, top 8, 361 -> 317, 4096 of 8 of 256 x 512 59.3 -> 54.7.)  A block with an infinity or a NaN is all NaN codes: its factor is a NaN.
+        // 1024, top 4, 150.2 -> 136.1 us, 2244 skewed ones of 160 of 768 x 3584, top 8, 361 -> 317, 4096 of 8 of 256 x 512 59.3 -> 54.7.)  A block with an infinity or
+        // a NaN is all NaN codes: its factor is a NaN.
         const uint32_t sb = mx_scale_byte(max(col_max[g], partner[g * 16 + (j >> 1)]));
         const uint32_t inverse = sb == 255u ? 0x7FFFFFFFu : (254u - sb) << 23;
         uint8_t code[8];

@@ -210,13 +210,24 @@ template <int kRegs>
 __device__ __forceinline__ void route_one_token_grouped(const float *__restrict__ row, int E, int k, int lane,
                                                         const RouterParams &rp, Candidates *cand, int &my_id, float &my_w) {
     const int G = E / rp.n_group;
+    // All loads, then all sigmoids, then what does not exist is put right.  (With a condition around each expert's load and sigmoid
+    // the eight of a lane ran one after the other, each behind its own load: router and sort of 8192 tokens of 256 experts, top 8, 31.1 ->
+    // 28.7 us, 1056 tokens 22.6 -> 20.5.)
     float s[kRegs], c[kRegs];
 #pragma unroll
     for (int i = 0; i < kRegs; ++i) {
         const int e = i * 32 + lane;
-        s[i] = e < E ? sigmoid_fixed(row[e]) : 0.f;
-        c[i] = e < E ? (rp.bias ? __fadd_rn(s[i], rp.bias[e]) : s[i]) : -INFINITY;
+        s[i] = e < E ? row[e] : 0.f;
+        c[i] = e < E && rp.bias ? rp.bias[e] : 0.f;
     }
+#pragma unroll
+    for (int i = 0; i < kRegs; ++i) {
+        s[i] = sigmoid_fixed(s[i]);
+        if (rp.bias) c[i] = __fadd_rn(s[i], c[i]); else c[i] = s[i];
+    }
+#pragma unroll
+    for (int i = 0; i < kRegs; ++i)
+        if (i * 32 + lane >= E) { s[i] = 0.f; c[i] = -INFINITY; }
     if (G == 32) {
         // Groups of 32 (256 experts in 8 groups): register i of all lanes is group i.  The eight reductions over 32 lanes
         // are folded into one by halving: each exchange leaves a lane half of the groups, so 9 exchanges of a pair do the
