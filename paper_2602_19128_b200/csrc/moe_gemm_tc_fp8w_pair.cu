@@ -445,8 +445,8 @@ grouped_gemm_tc_fp8w_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 1
         }
     } else if (QUEUE == kOnDemand && warp == 7) {
         // ---------------- decoder ----------------
-        tiles.fill_pair_on_demand<TileNumber>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane,
-                                              [](int tile) { return TileNumber{0, tile}; }, queue_wait, [&](uint32_t bar, uint32_t parity) {
+        tiles.fill_pair_on_demand<TileNumber>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, 1,
+                                              InOrder{}, [](int tile) { return TileNumber{0, tile}; }, queue_wait, [&](uint32_t bar, uint32_t parity) {
             return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
         });
     }

@@ -284,7 +284,7 @@ grouped_gemm_tc_mx_pair_kernel(const __grid_constant__ MxPairMapsOf<NT_MAX / 16>
     } else if (warp == 7) {
         // ---------------- decoder ----------------
         if constexpr (QUEUE == kOnDemand)
-            tiles.fill_pair_on_demand<MxTile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+            tiles.fill_pair_on_demand<MxTile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, 1, InOrder{}, decode, queue_wait,
                                           [&](uint32_t bar, uint32_t parity) {
                 return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
             });

@@ -362,7 +362,7 @@ grouped_gemm_tc_mx_ring_kernel(const __grid_constant__ MxRingMaps maps, const Mx
     } else if (warp == 7) {
         // ---------------- decoder ----------------
         if constexpr (QUEUE == kOnDemand)
-            tiles.fill_pair_on_demand<MxTile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+            tiles.fill_pair_on_demand<MxTile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, 1, InOrder{}, decode, queue_wait,
                                           [&](uint32_t bar, uint32_t parity) {
                 return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
             });

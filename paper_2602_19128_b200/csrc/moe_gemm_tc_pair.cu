@@ -270,7 +270,8 @@ grouped_gemm_tc_pair_kernel(const __grid_constant__ TensorMapsOf<NT_MAX / 16> ma
     } else if (warp == 7) {
         // ---------------- decoder ----------------
         if constexpr (QUEUE == kOnDemand)
-            tiles.fill_pair_on_demand<Tile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+            tiles.fill_pair_on_demand<Tile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane,
+                                            pair_tiles_ahead(p.n_k_blocks), LightTiles(p, total_tiles, n_pairs, lane), decode, queue_wait,
                                           [&](uint32_t bar, uint32_t parity) {
                 return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
             });
@@ -294,7 +295,7 @@ template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED>
 int launch_pair_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = PairSmem<NT_MAX, STAGES, SLABS, STAGED ? kStageBytes : 0>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
+    const bool on_demand = wide_pair_tiles_on_demand(p.n_k_blocks, NT_MAX);
     auto kernel = on_demand ? grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kOnDemand> : grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;

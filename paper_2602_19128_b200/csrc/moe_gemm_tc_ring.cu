@@ -23,10 +23,8 @@
 //    both reading the same weight slab.  Each CTA still stages ONE contiguous half of the token tile with ONE copy;
 //    part p reads rows [o_p, o_p + n_p / 2) of both halves, so its accumulator columns [0, n_p / 2) are tile rows
 //    o_p.., and columns [n_p / 2, n_p) are tile rows N / 2 + o_p...  The epilogue applies that map.
-//  * The MMA warp decodes nothing: the leader's weight producer, which runs ahead by the depth of the ring, writes
-//    each tile's column count into a small queue in shared memory before it arms the tile's first slot, and the
-//    MMA warp reads it after that slot's barrier (release / acquire through the barrier).  Between two tiles the
-//    tensor pipe therefore waits for no global load.
+//  * The MMA warp decodes nothing: warp 7 decodes tiles ahead and hands them, widths included, to every role through a
+//    queue in shared memory.  Between two tiles the tensor pipe therefore waits for no global load.
 //
 // Roles, barriers and the bounded waits are those of moe_gemm_tc_pair.cu.
 #include "moe_tc_pair.cuh"
@@ -366,7 +364,8 @@ grouped_gemm_tc_ring_kernel(const __grid_constant__ RingMaps maps, const KernelP
     } else if (warp == 7) {
         // ---------------- decoder ----------------
         if constexpr (QUEUE == kOnDemand)
-            tiles.fill_pair_on_demand<Tile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane, decode, queue_wait,
+            tiles.fill_pair_on_demand<Tile>(rank, pair, n_pairs, total_tiles, p.status + kTileCounterInt + (SWIGLU ? 0 : 1), lane,
+                                            pair_tiles_ahead(p.n_k_blocks), LightTiles(p, total_tiles, n_pairs, lane), decode, queue_wait,
                                           [&](uint32_t bar, uint32_t parity) {
                 return pair_wait_acquire(bar, parity, abort_flag, peer_abort, p.status, kSiteProducerEmpty + kSiteOffset);
             });
@@ -390,7 +389,7 @@ template <int NT_MAX, int STAGES, bool SWIGLU>
 int launch_ring_instance(const RingMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = RingSmem<NT_MAX, STAGES>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
+    const bool on_demand = wide_pair_tiles_on_demand(p.n_k_blocks, NT_MAX);
     auto kernel = on_demand ? grouped_gemm_tc_ring_kernel<NT_MAX, STAGES, SWIGLU, kOnDemand> : grouped_gemm_tc_ring_kernel<NT_MAX, STAGES, SWIGLU, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;

@@ -317,16 +317,17 @@ struct TileQueue {
         }
         __syncwarp();
     }
-    // The decoder warp, static assignment: all tiles of this worker, up to kDepth ahead.
+    // The decoder warp, static assignment: the tiles of this worker from its n-th on, up to kDepth ahead.  Returns their end.
     template <typename Decode, typename Wait>
-    __device__ __forceinline__ void fill(int worker, int n_workers, int total_tiles, int lane, Decode decode, Wait wait) const {
-        for (int n = 0;; ++n) {
+    __device__ __forceinline__ int fill(int worker, int n_workers, int total_tiles, int lane, Decode decode, Wait wait, int n = 0) const {
+        for (;; ++n) {
             const int tile = tile_of_round(n, worker, n_workers);
             if (tile >= total_tiles) break;
             const auto t = decode(tile);
             if (!__all_sync(0xffffffffu, wait(empty + (n & (kDepth - 1)) * 8, ((n / kDepth) & 1) ^ 1))) break;
             publish(t, n, lane);
         }
+        return n;
     }
     // The same for tiles of very few slots, which one walk after the other holds up: after the first, 32 tiles at a time are
     // decoded, one per lane.

@@ -116,10 +116,67 @@ __device__ __forceinline__ bool pair_wait_acquire(uint32_t bar, uint32_t parity,
 // Which pair GEMMs draw their tiles: those with K loops of 80 slots and more, whose tiles are so long that the static assignment's
 // rounds show (512 Mixtral-shaped tokens: 128 tiles of the down GEMM on 74 pairs, which began up to 30 us apart).  Static / on demand,
 // medians of alternating runs: that call 534 / 519 us, 1024 MX tokens of the same shape 436 / 409, MX prefill on 32 of 256 experts
-// 495 / 475..520 / 518, 333 FP8-weight tokens of the Mixtral shape 386 / 369.  With shorter loops the next tile is wanted before the epilogue, which is then most of a tile behind, lets it be
-// drawn: at 32 slots 4096 MX tokens of 128 experts of 4096 x 1536, top 8, 860 / 884 us, skewed 731 / 775; 2000 tokens of 64 of 2048 x
-// 2048, top 4, 346 / 353.  (Drawn two ahead those are level, but 512 Mixtral-shaped tokens take 575.)
-inline bool pair_tiles_on_demand(int slots_per_tile) { return slots_per_tile >= 80; }
+// 495 / 475..520 / 518, 333 FP8-weight tokens of the Mixtral shape 386 / 369.  With shorter loops the next tile is wanted before the
+// epilogue, which is then most of a tile behind, lets it be drawn: at 32 slots 4096 MX tokens of 128 experts of 4096 x 1536, top 8,
+// 860 / 884 us, skewed 731 / 775; 2000 tokens of 64 of 2048 x 2048, top 4, 346 / 353.  Drawn two ahead those are level, but 512
+// Mixtral-shaped tokens take 575.
+__host__ __device__ __forceinline__ bool pair_tiles_on_demand(int slots_per_tile) { return slots_per_tile >= 80; }
+
+// The bf16 kernels with token tiles of 256 rows and more are built to draw from 20 slots on, where they do so, two ahead, if LightTiles
+// finds the routing skewed; otherwise their decoders keep to the static assignment (drawn all the same, 700 tokens of 12 experts of
+// 4096 x 4096, top 2, take 239.5 us instead of 237.2, 512 Mixtral-shaped ones 507 instead of 502).  Below 20 slots not measured; a
+// tile is then too short for its draw.
+inline bool wide_pair_tiles_on_demand(int slots_per_tile, int nt_max) { return slots_per_tile >= (nt_max >= 256 ? 20 : 80); }
+__host__ __device__ __forceinline__ int pair_tiles_ahead(int slots_per_tile) { return slots_per_tile >= 80 ? 1 : 2; }
+
+// Tiles drawn in the schedule's order.
+struct InOrder {
+    static constexpr bool drawn = true;
+    __device__ __forceinline__ void prepare() {}
+    __device__ __forceinline__ int operator()(int n) const { return n; }
+};
+
+// Tiles drawn so that the light ones run beside the heavy ones.  With experts of most rows first a GEMM over skewed routing is two
+// phases: full tiles, bound by matrix work while the memory idles, then tiles of few rows, bound by the stream of their weights while
+// the tensor cores idle (4096 tokens of 128 experts of 4096 x 1536, top 8, Zipf: 14 experts have 96 % of the rows, 29 others bring two
+// thirds of the weights; the larger of both times, summed over the experts, is 1.03 ms, the larger of both sums 0.89).  A pair takes in
+// its slab faster than its share of the memory's rate when the others compute.  So tiles of at most kLightRows, half of the 230 or so
+// rows at which both take as long, are dealt evenly among the heavy ones, if the first expert has more than twice as many rows.  The
+// first draws of all pairs stay in order (the search for the first light tile runs beside the first tile), and the last n_pairs light
+// tiles stay last, where short tiles even out the end.  Both GEMMs deal alike, so the down GEMM asks for experts in the order in which
+// the gate/up GEMM finishes them.  In order / dealt, alternating under the power cap: that case 1225 / 1209 us (another part 1290 /
+// 1244), 2048 tokens of 64 experts of 4096 x 4096, top 4, 886 / 855 (935 / 872), 1500 of 64 of 7168 x 2048, top 6, 942 / 919, 4096 of 64 of
+// 2048 x 1024, top 8, 458 / 453.  A line at 64 or 144 rows and none or three times n_pairs kept for the end are within the spread.
+struct LightTiles {
+    static constexpr int kLightRows = 112;
+    const KernelParams &p;
+    int total_tiles, n_pairs, begin, lane;  // numbers below `begin` are in order
+    bool drawn = true;
+    int first = 0, spread = 0, end = 0;     // numbers begin .. end - 1 hold the `spread` tiles from tile `first` on among the others
+    __device__ __forceinline__ LightTiles(const KernelParams &p, int total_tiles, int n_pairs, int lane)
+        : p(p), total_tiles(total_tiles), n_pairs(n_pairs), begin(pair_tiles_ahead(p.n_k_blocks) * n_pairs), lane(lane) {}
+    __device__ __forceinline__ void prepare() {  // by a whole warp
+        int heavy = 0;  // the schedule ranks experts by rows, and an expert of more than one tile has no light ones: heavy ones come first
+#pragma unroll 4
+        for (int i = 0; i < p.E; i += 32) {
+            const bool mine = i + lane < p.E;
+            heavy += __popc(__ballot_sync(0xffffffffu, mine && p.tile_rows[p.tile_order[mine ? i + lane : 0]] > kLightRows));
+        }
+        first = p.tile_prefix[heavy] * p.n_feature_tiles;
+        spread = total_tiles - n_pairs - first;
+        const int top = p.tile_order[0];
+        const bool skewed = p.expert_offsets[top + 1] - p.expert_offsets[top] > 2 * kLightRows;
+        end = skewed && first > begin && spread > 0 ? first + spread : 0;
+        drawn = end > 0 || pair_tiles_on_demand(p.n_k_blocks);
+    }
+    __device__ __forceinline__ int operator()(int n) const {
+        if (n < begin || n >= end) return n;
+        const unsigned long long numbers = end - begin;
+        const int before = (int)((unsigned long long)(n - begin) * spread / numbers);
+        const int after = (int)((unsigned long long)(n - begin + 1) * spread / numbers);
+        return after > before ? first + before : n - before;
+    }
+};
 
 // Tiles on demand for a CTA pair: the leader's decoder draws them and passes each on to the peer's decoder through one entry in the
 // peer's shared memory; both publish them in their own CTA's queue.
@@ -137,26 +194,40 @@ struct PairTileQueue : TileQueue {
         mbar_init(inbox_full, 1);
         mbar_init(inbox_empty, 1);
     }
+    // ahead: a pair's first `ahead` tiles are assigned, and tile n is drawn once tile n - ahead has been taken by every role.
+    // order: prepare() by a whole warp after the first tile, then the tile of a drawn number.
     // wait / wait_acquire(bar, parity): bounded waits, the second acquiring at cluster scope.
-    template <typename T, typename Decode, typename Wait, typename WaitAcquire>
-    __device__ __forceinline__ void fill_pair_on_demand(uint32_t rank, int pair, int n_pairs, int total_tiles, int *counter, int lane,
-                                                        Decode decode, Wait wait, WaitAcquire wait_acquire) const {
+    template <typename T, typename Order, typename Decode, typename Wait, typename WaitAcquire>
+    __device__ __forceinline__ void fill_pair_on_demand(uint32_t rank, int pair, int n_pairs, int total_tiles, int *counter, int lane, int ahead,
+                                                        Order order, Decode decode, Wait wait, WaitAcquire wait_acquire) const {
         constexpr int kWords = (int)(sizeof(T) / 4);
-        for (int n = 0;; ++n) {
-            T t;
+        T t;
+        t.e = -1;
+        if (pair < total_tiles) t = decode(pair);
+        publish(t, 0, lane);
+        if (t.e < 0) return;
+        order.prepare();
+        if (!order.drawn) {
+            const int n = fill(pair, n_pairs, total_tiles, lane, decode, wait, 1);
+            t.e = -1;
+            if (__all_sync(0xffffffffu, wait(empty + (n & (kDepth - 1)) * 8, ((n / kDepth) & 1) ^ 1))) publish(t, n, lane);
+            return;
+        }
+        for (int n = 1; t.e >= 0; ++n) {
             int *w = reinterpret_cast<int *>(&t);
             if (rank == 0) {
-                int tile = pair;
-                if (n > 0) {
-                    const int m = n - 1;
+                int tile = n * n_pairs + pair;
+                if (n >= ahead) {
+                    const int m = n - ahead;
                     if (!__all_sync(0xffffffffu, wait(empty + (m & (kDepth - 1)) * 8, (m / kDepth) & 1))) break;
-                    if (lane == 0) tile = n_pairs + atomicAdd(counter, 1);
+                    if (lane == 0) tile = ahead * n_pairs + atomicAdd(counter, 1);
                     tile = __shfl_sync(0xffffffffu, tile, 0);
+                    if (tile < total_tiles) tile = order(tile);
                 }
                 t.e = -1;
                 if (tile < total_tiles) t = decode(tile);
                 publish(t, n, lane);
-                if (n > 0 && !__all_sync(0xffffffffu, wait(inbox_empty, (n - 1) & 1))) break;
+                if (n > 1 && !__all_sync(0xffffffffu, wait(inbox_empty, n & 1))) break;
                 if (lane == 0) {
                     const uint32_t dst = map_to_cta(inbox_addr, 1);
 #pragma unroll
@@ -165,7 +236,7 @@ struct PairTileQueue : TileQueue {
                 }
                 __syncwarp();
             } else {
-                if (!__all_sync(0xffffffffu, wait_acquire(inbox_full, n & 1))) break;
+                if (!__all_sync(0xffffffffu, wait_acquire(inbox_full, (n - 1) & 1))) break;
                 const volatile int *in = inbox;
 #pragma unroll
                 for (int k = 0; k < kWords; ++k) w[k] = in[k];
@@ -174,7 +245,6 @@ struct PairTileQueue : TileQueue {
                 if (!__all_sync(0xffffffffu, wait(empty + (n & (kDepth - 1)) * 8, ((n / kDepth) & 1) ^ 1))) break;
                 publish(t, n, lane);
             }
-            if (t.e < 0) break;
         }
     }
 };

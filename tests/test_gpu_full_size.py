@@ -89,6 +89,27 @@ def test_full_size_workload(name):
     close_on_device(out, out_v, f"{name} out")
 
 
+@pytest.mark.parametrize("T,H,I,E,k", [(1400, 3840, 3840, 16, 1),    # 256-row tiles, 60 slots of K: 6 full token tiles, 4 light ones
+                                       (2000, 3840, 3840, 12, 1),    # wide tiles: 8 and 4
+                                       (1400, 5120, 5120, 16, 1),    # 80 slots, light tiles in both GEMMs
+                                       (2100, 1280, 5120, 16, 1),    # 20 slots in the gate/up GEMM
+                                       (500, 4096, 2048, 4, 1)])     # no light tile beyond the kept ones: static all the same
+def test_light_tiles_among_heavy_ones(T, H, I, E, k):
+    """Skewed routing with enough token tiles on both sides: the experts of few rows are dealt among the others, every tile is
+    computed once (all elements against the CUDA-core validation kernels) and the bits are those of every run."""
+    inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=True), seed=2)
+    out, views, ws = run_forward(inp)
+    h, y = views["h"].clone(), views["y"].clone()
+    for _ in range(3):
+        again = torch.empty_like(out)
+        moe.moe_forward(inp["x"], inp["router_logits"], inp["w13"], inp["w2"], k, again, ws)
+        assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+    out_v, views_v, _ = run_forward(inp, flags=moe.MOE_FLAG_VALIDATION_GEMM)
+    close_on_device(h, views_v["h"], "h")
+    close_on_device(y, views_v["y"], "y")
+    close_on_device(out, out_v, "out")
+
+
 @pytest.mark.parametrize("name", ["mixtral", "dsv3_decode", "skewed", "dsv3_prefill"])
 def test_full_size_workload_mxfp8(name):
     """The MX FP8 layer at full size (wide-tile CTA-pair kernel for the prefill-sized batches, 160-row pair tiles
