@@ -83,10 +83,12 @@ def test_route_one_block_cluster_and_many_blocks(T, E, k):
 
 
 @pytest.mark.parametrize("T,E,k", [(3, 32, 5), (40, 33, 7), (300, 128, 8), (300, 129, 8), (1024, 256, 8), (1024, 33, 9),
-                                   (1024, 256, 32), (1100, 32, 2), (1100, 128, 8), (5000, 129, 3)])
+                                   (1024, 256, 32), (1100, 32, 2), (1100, 128, 8), (5000, 129, 3),
+                                   (1024, 8, 8), (650, 40, 13), (1000, 32, 32)])
 def test_route_registers_per_lane_and_spans(T, E, k):
     """The edges of one, four and eight registers of logits per lane (32 / 33, 128 / 129 experts), one and 32 sorting warps,
-    and ids past the 8192 that the sorting block keeps in shared memory (9216, 32768)."""
+    and ids past the 8192 that the sorting block keeps in shared memory (none, 258, 1024, 23808 and 24576 of them: part of a
+    warp's span, whole spans, groups in fours and what is left)."""
     g = torch.Generator().manual_seed(T + 7 * E)
     check_against_oracle(torch.randn(T, E, generator=g), k)
 
