@@ -99,7 +99,7 @@ struct Params {
 // Where no sequence is split there is nothing to count, and the kernel's first block zeroes the status word: one launch
 // (Params::own_status), with programmatic serialisation (kChained), so that a kernel's start overlaps the end of the one in front (behind a
 // memset it cannot).
-// Loops without / with: 40 sequences of 31..251 tokens 8.2 / 7.3 us, 162 of 410..821 43.6 / 41.7, 256 of 256..2048 102.5 / 100.7.
+// Loops without / with: 40 sequences of 31..251 tokens 8.2 / 7.6 us, 162 of 410..821 44.3 / 43.4, 256 of 256..2048 102.8 / 101.3.
 // Memset / one launch, in a loop / on the first pass over new inputs: 1 sequence of 100 tokens 8.5 -> 7.6 us / 25.7 ->
 // 21.7, 256 of 256..2048 105.5 -> 102.8 / 138 -> 133.  A wait gives up after 4 million polls, long after that block has started.
 // (A small kernel that zeroed the words beside a decode kernel launched with programmatic serialisation made loops 0.7 to 2
@@ -338,9 +338,21 @@ __device__ __forceinline__ void zero_own_status(const Params &p, bool first_bloc
     if (p.own_status && first_block && tid == 0) *reinterpret_cast<uint4 *>(p.status) = make_uint4(0, 0, 0, 0);
 }
 
+// A word of the page table.  __ldg is for memory that nothing writes while the kernel lives, and a chained kernel lives before what
+// is in front of it, which may write the table, is done: its loads are ordinary ones, behind the wait.
+template <bool kChained>
+__device__ __forceinline__ int load_index(const int *at) { return kChained ? *at : __ldg(at); }
+// The wait of a chained kernel for what is in front.  That may have written the caches through the generic proxy: the threads
+// that copy them into shared memory link the two by a fence, here, where nothing of theirs is under way yet.
+__device__ __forceinline__ void wait_for_inputs(bool copies) {
+    moe::chain_wait();
+    if (copies) asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+
+template <bool kChained>
 __device__ __forceinline__ int cached_tokens(const Params &p, int b) {
-    const int first = __ldg(&p.kv_indptr[b]), behind = __ldg(&p.kv_indptr[b + 1]);
-    const int last = __ldg(&p.kv_last_page_len[b]);  // (all three in flight: one round trip)
+    const int first = load_index<kChained>(&p.kv_indptr[b]), behind = load_index<kChained>(&p.kv_indptr[b + 1]);
+    const int last = load_index<kChained>(&p.kv_last_page_len[b]);  // (all three in flight: one round trip)
     return behind > first ? (behind - first - 1) * p.page_size + last : 0;
 }
 // out = 0, lse = -inf for the heads of one key-value head (all 128 compute threads call).
@@ -585,9 +597,9 @@ gqa_row_decode_kernel(const Params p) {
     const bool first_block = (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
     if (kChained) {
         moe::chain_release();
-        moe::chain_wait();
+        wait_for_inputs(true);
     }
-    const int L = cached_tokens(p, b);
+    const int L = cached_tokens<kChained>(p, b);
     const int head0 = kvh * p.group;
 
     if (L <= 0) {  // nothing cached: out = 0, lse = -inf (written by the first split's block)
@@ -625,7 +637,7 @@ gqa_row_decode_kernel(const Params p) {
     auto locate = [&](int chunk) -> int {
         const int tok = begin + chunk * kChunk + my_row;
         if (chunk >= n_chunks || tok >= end) return -1;
-        return __ldg(&page_list[tok / p.page_size]) * p.page_size + tok % p.page_size;
+        return load_index<kChained>(&page_list[tok / p.page_size]) * p.page_size + tok % p.page_size;
     };
     int next_loc = locate(0);
     auto issue_chunk = [&](int chunk) {  // called for chunk 0, 1, 2, ... in order
@@ -757,7 +769,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
     }
 
     if (kChained) {
-        moe::chain_wait();  // (the set-up above overlaps the end of what is in front)
+        wait_for_inputs(warp == kWarps);  // (the set-up above overlaps the end of what is in front)
         zero_own_status(p, blockIdx.x == 0, tid);
     }
 
@@ -772,7 +784,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         int sum = 0, longest = 0, sequence = 0, shares = 0;
         if (tid < kThreads)
             for (int i = tid * per; i < min(p.B, (tid + 1) * per); ++i) {
-                const int n = (cached_tokens(p, i) + kChunk - 1) / kChunk;
+                const int n = (cached_tokens<kChained>(p, i) + kChunk - 1) / kChunk;
                 if (n <= 0) continue;  // an item without tokens has no share
                 const int parts_of = min(p.n_splits, (n + split_chunks - 1) / split_chunks);
                 sum += n;
@@ -814,7 +826,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         // items without tokens are dealt out to the blocks
         if (tid < kThreads)
             for (int i = blockIdx.x; i < p.B; i += gridDim.x)
-                if (cached_tokens(p, i) <= 0)
+                if (cached_tokens<kChained>(p, i) <= 0)
                     for (int h = 0; h < p.Hkv; ++h) write_empty(p, i, h * p.group, tid);
         // The blocks' work starts at a chunk of the line (balanced) or at a share; both lie item after item, head after head.
         int n_blocks = shares * p.Hkv;
@@ -840,7 +852,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         int at = range_start[r], units;  // `units`: the item's chunks or shares per head
         b = r * per - 1;
         do {
-            L = cached_tokens(p, ++b);
+            L = cached_tokens<kChained>(p, ++b);
             n_chunks = (L + kChunk - 1) / kChunk;
             units = balanced ? n_chunks : min(p.n_splits, (n_chunks + split_chunks - 1) / split_chunks);
             at += max(units, 0);
@@ -858,7 +870,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         const int split = blockIdx.x % p.n_splits;
         kvh = (blockIdx.x / p.n_splits) % p.Hkv;
         b = blockIdx.x / p.n_splits / p.Hkv;
-        L = cached_tokens(p, b);
+        L = cached_tokens<kChained>(p, b);
         n_chunks = (L + kChunk - 1) / kChunk;
         if (L <= 0) {
             if (split == 0 && tid < kThreads) write_empty(p, b, kvh * p.group, tid);
@@ -876,7 +888,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         if (++kvh == p.Hkv) {
             kvh = 0;
             do {
-                L = cached_tokens(p, ++b);  // (there is one: the line goes on)
+                L = cached_tokens<kChained>(p, ++b);  // (there is one: the line goes on)
             } while (L <= 0);
             n_chunks = (L + kChunk - 1) / kChunk;
         }
@@ -891,11 +903,11 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         const int my_row = (lane >> 1) << sh;
         const CUtensorMap *map = my_values ? &v_map : &k_map;
         const uint32_t my_dst = (my_values ? (uint32_t)kTiledTileBytes : 0u) + (uint32_t)(my_row * kRowBytes);
-        const int *page_list = p.kv_indices + __ldg(&p.kv_indptr[b]);
+        const int *page_list = p.kv_indices + load_index<kChained>(&p.kv_indptr[b]);
         int page, slot, head;
         auto locate = [&]() {
             const int tok = c * kChunk + my_row;
-            page = has_box && tok < L ? __ldg(&page_list[tok / p.page_size]) : -1;
+            page = has_box && tok < L ? load_index<kChained>(&page_list[tok / p.page_size]) : -1;
             slot = tok & (p.page_size - 1);
             head = kvh;
         };
@@ -916,7 +928,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
                 if (++c == n_chunks) {
                     const int old_b = b;
                     next_sequence();
-                    if (b != old_b) page_list = p.kv_indices + __ldg(&p.kv_indptr[b]);
+                    if (b != old_b) page_list = p.kv_indices + load_index<kChained>(&p.kv_indptr[b]);
                 }
                 locate();
             }
@@ -1149,7 +1161,7 @@ int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, co
     const bool adaptive = tiled && bh * slots >= 2 * kBalancedBlocks && bh * p.n_splits <= 2 * kBalancedBlocks;
     p.own_status = p.n_splits == 1 && !adaptive;  // (no part is ever counted)
     // The row gather's loop is at the limit of its registers, and the wait in front of it cost sequences of 1059..2118 tokens 3 % (27 over 8
-    // heads, pages of one token, 75.2 / 77.5 us); short ones gain the launch (14 of 119..239 12.3 / 11.3).
+    // heads, pages of one token, 75.2 / 77.5 us); short ones gain the launch (14 of 119..239 12.3 / 11.8).
     const bool chained = p.own_status && (tiled || max_kv_len <= 512);
     auto launch = [&](auto kernel, dim3 grid, int threads, int smem_bytes, const auto &...args) {
         if (!moe::tc::set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), smem_bytes)) return MOE_ERR_CUDA;

@@ -259,6 +259,103 @@ def test_a_sequence_longer_than_the_hint_is_still_computed_in_full():
     check(inp, max_kv_len=1024)     # the last split runs to the end of the sequence
 
 
+def _rewritten_inputs(B, Hq, Hkv, P, length):
+    """A decode call whose every input is written by kernels before each pass (256 pages): the passes' sources, what writes one
+    into the buffers on the current stream (the page table by the library's router, whose kernel lets the next one start
+    early), and the call."""
+    pages, n = 256, B * -(-length // P)
+    g = torch.Generator(device="cuda").manual_seed(B + P)
+    bf16 = lambda *shape: torch.randn(*shape, generator=g, device="cuda").to(torch.bfloat16)
+    sources = []
+    for i in range(3):
+        table = torch.randint(pages, (n,), generator=g, device="cuda")
+        last = torch.randint(1, P + 1, (B,), generator=g, device="cuda", dtype=torch.int32)
+        sources.append(dict(k=bf16(pages, P, Hkv, 128), v=bf16(pages, P, Hkv, 128), q=bf16(B, Hq, 128), last=last, table=table,
+                            logits=torch.nn.functional.one_hot(table, pages).float()))
+    k, v, q, last = (torch.zeros_like(sources[0][name]) for name in ("k", "v", "q", "last"))
+    indptr = torch.arange(B + 1, dtype=torch.int32, device="cuda") * (n // B)
+    ids, w = torch.zeros((n, 1), dtype=torch.int32, device="cuda"), torch.empty((n, 1), device="cuda")
+    offsets, order = torch.empty(pages + 1, dtype=torch.int32, device="cuda"), torch.empty((2, n), dtype=torch.int32, device="cuda")
+    route_ws = moe.alloc_workspace(moe.moe_route_workspace_bytes(n, pages, 1), "cuda")
+    def write(src, last_writer):
+        s = torch.cuda.current_stream()
+        writers = [lambda: torch.add(src["last"], 0, out=last),
+                   lambda: torch.mul(src["q"], 1, out=q),
+                   lambda: torch.mul(src["v"], 1, out=v),
+                   lambda: torch.mul(src["k"], 1, out=k),
+                   lambda: moe.moe_route(src["logits"], 1, ids, w, offsets, order[0], order[1], route_ws, stream=s)]
+        for i in range(len(writers)):
+            writers[(i + last_writer + 1) % len(writers)]()
+    def call(out, ws):
+        moe.gqa_paged_decode(q, k, v, indptr, ids.view(-1), last, length, 0.09, out, ws, stream=torch.cuda.current_stream())
+    nbytes = moe.gqa_decode_workspace_bytes(B, Hq, Hkv, 128, length)
+    refs = []
+    for src in sources:   # nothing overlaps
+        refs.append(torch.empty_like(q))
+        write(src, 0)
+        torch.cuda.synchronize()
+        assert torch.equal(ids.view(-1).long(), src["table"])
+        ws = moe.alloc_workspace(nbytes, "cuda")
+        call(refs[-1], ws)
+        assert moe.moe_last_status(ws) == 0
+    assert not torch.equal(refs[0], refs[1]) and not torch.equal(refs[1], refs[2])
+    return sources, write, call, refs, nbytes
+
+
+# the launch forms of a call that splits nothing, by blocks and tokens: on SMs of their own, short ones, a full machine,
+# and in between (not started early); the row gather's the same; and a call with parts
+REWRITTEN = [(3, 32, 4, 16, 400), (24, 32, 4, 16, 250), (80, 32, 4, 16, 100), (25, 32, 4, 16, 640), (3, 32, 4, 12, 300),
+             (24, 32, 4, 12, 120), (120, 32, 4, 1, 8), (20, 32, 4, 12, 480), (2, 32, 4, 16, 8000)]
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,P,length", REWRITTEN)
+def test_inputs_written_by_the_kernels_directly_in_front(B, Hq, Hkv, P, length):
+    """Every input anew before every pass, each of them by the kernel directly in front of the call in turn, all queued before
+    the first one runs: no pass sees what an input held before."""
+    sources, write, call, refs, nbytes = _rewritten_inputs(B, Hq, Hkv, P, length)
+    ws = moe.alloc_workspace(nbytes, "cuda")
+    outs = [torch.empty_like(refs[0]) for _ in range(30)]
+    torch.cuda.synchronize()
+    torch.cuda._sleep(40_000_000)
+    for i, out in enumerate(outs):
+        write(sources[i % 3], i % 5)
+        call(out, ws)
+    assert moe.moe_last_status(ws) == 0
+    for i, out in enumerate(outs):
+        assert torch.equal(out.view(torch.int16), refs[i % 3].view(torch.int16)), i
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,P,length", REWRITTEN[:2] + REWRITTEN[4:5] + REWRITTEN[-1:])
+def test_a_captured_call_behind_joined_streams_reads_what_both_wrote(B, Hq, Hkv, P, length):
+    """Captured behind a fork and a join (two nodes in front), and behind a kernel that lets it start early."""
+    sources, write, call, refs, nbytes = _rewritten_inputs(B, Hq, Hkv, P, length)
+    ws = moe.alloc_workspace(nbytes, "cuda")
+    outs = [torch.empty_like(refs[0]) for _ in range(2)]
+    src = {name: t.clone() for name, t in sources[0].items()}
+    fork, s = torch.cuda.Stream(), torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        fork.wait_stream(torch.cuda.current_stream())
+        write(src, 0)
+        with torch.cuda.stream(fork):
+            scratch = src["q"] + 1
+        torch.cuda.current_stream().wait_stream(fork)
+        call(outs[0], ws)
+        write(src, 4)
+        call(outs[1], ws)
+    for i in (1, 2, 0, 1):
+        for name, t in sources[i].items():
+            src[name].copy_(t)
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        assert moe.moe_last_status(ws) == 0
+        for out in outs:
+            assert torch.equal(out.view(torch.int16), refs[i].view(torch.int16))
+    del scratch
+
+
 def test_results_do_not_depend_on_which_block_finishes_last():
     inp = make_gqa_inputs(dict(B=3, Hq=32, Hkv=4, D=128, page_size=16, lengths=[9000, 4000, 12345]), seed=4, device="cuda")
     first, lse0 = run_gpu(inp)
