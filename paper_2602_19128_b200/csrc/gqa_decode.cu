@@ -97,14 +97,26 @@ struct Params {
 // ---- the launches of a call --------------------------------------------------------------------------------------
 // Where parts of sequences may have to be counted, a memset in front of the kernel zeroes the status word and the counters.
 // Where no sequence is split there is nothing to count, and the kernel's first block zeroes the status word: one launch
-// (Params::own_status), with programmatic serialisation (kChained), so that a kernel's start overlaps the end of the one in front (behind a
-// memset it cannot).
+// (Params::own_status), and where that is faster with programmatic serialisation (kChained), so that a kernel's start overlaps the end of the
+// one in front (behind a memset it cannot).
 // Loops without / with: 40 sequences of 31..251 tokens 8.2 / 7.6 us, 162 of 410..821 44.3 / 43.4, 256 of 256..2048 102.8 / 101.3.
 // Memset / one launch, in a loop / on the first pass over new inputs: 1 sequence of 100 tokens 8.5 -> 7.6 us / 25.7 ->
 // 21.7, 256 of 256..2048 105.5 -> 102.8 / 138 -> 133.  A wait gives up after 4 million polls, long after that block has started.
 // (A small kernel that zeroed the words beside a decode kernel launched with programmatic serialisation made loops 0.7 to 2
 // us shorter, but first passes 2.3 longer, memset / small kernel: 1 sequence of 65 536 tokens 36.9 / 36.2 and 58.3 / 61.3, 1 of
 // 4000 14.3 / 13.2 and 32.4 / 34.8, 16 of 8000 51.1 / 50.2 and 73.7 / 75.6.)
+// Chained or not: the blocks of a chained call are placed while those of the call in front still sit on their SMs.  Few find SMs of their
+// own, and a grid that fills the machine is placed evenly all the same; in between several land on one SM, and long ones wait for
+// it.  Equal lengths over 4 heads, plain / chained, loops: tiled, 108 blocks of 300 tokens 8.2 / 7.5 us, 800 14.4 / 15.0, 915 16.4 / 17.2;
+// 32 of 600 12.3 / 10.7; 68 of 700 12.6 / 12.8; 152 of 700 16.2 / 14.9, of 1100 21.8 / 20.8; row gather, 108 blocks of 128 8.2 /
+// 7.2, of 256 12.3 / 12.7, of 512 19.0 / 21.1; 32 of 384 15.6 / 14.0; 68 of 384 15.9 / 16.7; 240 of 256 12.6 / 12.8; 480 of 128 14.4 /
+// 13.3, of 384 34.5 / 33.4.  (The row gather's loop is at the limit of its registers: the wait in front of it cost 216 sequences
+// of 1059..2118 tokens 3 %, 75.2 / 77.5.)
+constexpr unsigned kSms = 148;
+static bool chaining_is_faster(bool tiled, unsigned blocks, int max_kv_len) {
+    if (max_kv_len <= (tiled ? 384 : 128)) return true;
+    return 4 * blocks <= kSms || (tiled ? blocks >= kSms : blocks >= 3 * kSms && max_kv_len <= 384);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -717,7 +729,7 @@ gqa_row_decode_kernel(const Params p) {
 // i-th of the shares that have tokens, not the i-th of the grid: blocks that found their share empty only after reading all
 // lengths had already made the others share an SM (one sequence of 20 000 tokens, an empty one and a hint of 40 000:
 // 28.6 -> 26.7 us).  Batches of more blocks than that balance themselves.
-constexpr int kBalancedBlocks = 148 * 2;  // as many as are resident
+constexpr int kBalancedBlocks = (int)kSms * 2;  // as many as are resident
 constexpr int kMinPiece = 4;              // chunks a balanced block takes at least
 constexpr int kSmemBytesTiled = kTiledStages * kTiledStageBytes + kMergeBytes + 1024;
 static_assert(kSmemBytesTiled + 1024 <= 113 * 1024, "two blocks per SM");
@@ -757,6 +769,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
     const int sh = 31 - __clz(p.box_rows);  // log2 of the rows of a box
     static_assert(!kAdaptive || !kChained, "parts may be counted");
     if (kChained) moe::chain_release();
+    else if (!kAdaptive) zero_own_status(p, blockIdx.x == 0, tid);
     if (tid == 0) {
         for (int s = 0; s < kTiledStages; ++s) {
             mbar_init(full_base + s * 8, 32);       // the copy warp's lanes
@@ -1160,9 +1173,7 @@ int gqa_paged_decode(const void *q, const void *k_cache, const void *v_cache, co
     // Two slots per balanced block: where the workspace has them, and the fixed shares fill the machine at most twice.
     const bool adaptive = tiled && bh * slots >= 2 * kBalancedBlocks && bh * p.n_splits <= 2 * kBalancedBlocks;
     p.own_status = p.n_splits == 1 && !adaptive;  // (no part is ever counted)
-    // The row gather's loop is at the limit of its registers, and the wait in front of it cost sequences of 1059..2118 tokens 3 % (27 over 8
-    // heads, pages of one token, 75.2 / 77.5 us); short ones gain the launch (14 of 119..239 12.3 / 11.8).
-    const bool chained = p.own_status && (tiled || max_kv_len <= 512);
+    const bool chained = p.own_status && chaining_is_faster(tiled, shares, max_kv_len);
     auto launch = [&](auto kernel, dim3 grid, int threads, int smem_bytes, const auto &...args) {
         if (!moe::tc::set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), smem_bytes)) return MOE_ERR_CUDA;
         if (!p.own_status && cudaMemsetAsync(p.status, 0, 256 + bh * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
