@@ -125,7 +125,7 @@ __host__ __device__ __forceinline__ bool pair_tiles_on_demand(int slots_per_tile
 // The bf16 kernels with token tiles of 256 rows and more are built to draw from 20 slots on, where they do so, two ahead, if LightTiles
 // finds the routing skewed; otherwise their decoders keep to the static assignment (drawn all the same, 700 tokens of 12 experts of
 // 4096 x 4096, top 2, take 239.5 us instead of 237.2, 512 Mixtral-shaped ones 507 instead of 502).  Below 20 slots not measured; a
-// tile is then too short for its draw.
+// tile is then too short for its draw.  With 128 rows they draw from 80 slots on, and deal light tiles there too.
 inline bool wide_pair_tiles_on_demand(int slots_per_tile, int nt_max) { return slots_per_tile >= (nt_max >= 256 ? 20 : 80); }
 __host__ __device__ __forceinline__ int pair_tiles_ahead(int slots_per_tile) { return slots_per_tile >= 80 ? 1 : 2; }
 
@@ -144,9 +144,11 @@ struct InOrder {
 // rows at which both take as long, are dealt evenly among the heavy ones, if the first expert has more than twice as many rows.  The
 // first draws of all pairs stay in order (the search for the first light tile runs beside the first tile), and the last n_pairs light
 // tiles stay last, where short tiles even out the end.  Both GEMMs deal alike, so the down GEMM asks for experts in the order in which
-// the gate/up GEMM finishes them.  In order / dealt, alternating under the power cap: that case 1225 / 1209 us (another part 1290 /
-// 1244), 2048 tokens of 64 experts of 4096 x 4096, top 4, 886 / 855 (935 / 872), 1500 of 64 of 7168 x 2048, top 6, 942 / 919, 4096 of 64 of
-// 2048 x 1024, top 8, 458 / 453.  A line at 64 or 144 rows and none or three times n_pairs kept for the end are within the spread.
+// the gate/up GEMM finishes them.  "Light" is an expert of at most kLightRows rows: with a bound of 128 rows an expert of more may
+// have tiles of fewer (410 rows: four of 112), which stay in order.  In order / dealt, alternating under the power cap: that case
+// 1225 / 1209 us (another part 1290 / 1244), 2048 tokens of 64 experts of 4096 x 4096, top 4, 886 / 855 (935 / 872), 1500 of 64 of
+// 7168 x 2048, top 6, 942 / 919, 4096 of 64 of 2048 x 1024, top 8, 458 / 453; with 128-row tiles 600 of 16 of 5120 x 5120, top 2,
+// 332 / 317, 1024 of 64 of 7168 x 2048, top 4, 538 / 518, 800 of 16 of 7168 x 7168, top 1, 424 / 393.  A line at 64 or 144 rows and none or three times n_pairs kept for the end are within the spread.
 struct LightTiles {
     static constexpr int kLightRows = 112;
     const KernelParams &p;
@@ -156,11 +158,12 @@ struct LightTiles {
     __device__ __forceinline__ LightTiles(const KernelParams &p, int total_tiles, int n_pairs, int lane)
         : p(p), total_tiles(total_tiles), n_pairs(n_pairs), begin(pair_tiles_ahead(p.n_k_blocks) * n_pairs), lane(lane) {}
     __device__ __forceinline__ void prepare() {  // by a whole warp
-        int heavy = 0;  // the schedule ranks experts by rows, and an expert of more than one tile has no light ones: heavy ones come first
+        int heavy = 0;  // the schedule ranks experts by rows: those of more than kLightRows come first
 #pragma unroll 4
         for (int i = 0; i < p.E; i += 32) {
             const bool mine = i + lane < p.E;
-            heavy += __popc(__ballot_sync(0xffffffffu, mine && p.tile_rows[p.tile_order[mine ? i + lane : 0]] > kLightRows));
+            const int e = p.tile_order[mine ? i + lane : 0];
+            heavy += __popc(__ballot_sync(0xffffffffu, mine && p.expert_offsets[e + 1] - p.expert_offsets[e] > kLightRows));
         }
         first = p.tile_prefix[heavy] * p.n_feature_tiles;
         spread = total_tiles - n_pairs - first;

@@ -93,7 +93,8 @@ def test_full_size_workload(name):
                                        (2000, 3840, 3840, 12, 1),    # wide tiles: 8 and 4
                                        (1400, 5120, 5120, 16, 1),    # 80 slots, light tiles in both GEMMs
                                        (2100, 1280, 5120, 16, 1),    # 20 slots in the gate/up GEMM
-                                       (500, 4096, 2048, 4, 1)])     # no light tile beyond the kept ones: static all the same
+                                       (500, 4096, 2048, 4, 1),      # no light tile beyond the kept ones: static all the same
+                                       (600, 5120, 5120, 16, 2)])    # 128-row tiles, 80 slots: heavy experts of several tiles of 112 and fewer
 def test_light_tiles_among_heavy_ones(T, H, I, E, k):
     """Skewed routing with enough token tiles on both sides: the experts of few rows are dealt among the others, every tile is
     computed once (all elements against the CUDA-core validation kernels) and the bits are those of every run."""
