@@ -208,21 +208,21 @@ int forward_impl(const void *x, const float *logits, const void *w13, const void
         // skewed workloads they are 5 % resp. 25 % slower than one slab, because the accumulators then
         // fill TMEM and the epilogue no longer overlaps the next tile's MMAs.
         const bool single = (flags & MOE_FLAG_SINGLE_CTA_GEMM) != 0;
-        auto run = [&](const GroupedGemmArgs &g, bool allow_two_slabs) {
+        auto run = [&](const GroupedGemmArgs &g) {
             if (!single && grouped_gemm_tc_ring_applies(g)) return launch_grouped_gemm_tc_ring(g, stream);
             int slabs = single ? 0 : grouped_gemm_tc_pair_slabs(g);
-            if (slabs == 2 && !(dense_tiles && allow_two_slabs)) slabs = grouped_gemm_tc_pair_slabs(g) >= 1 ? 1 : 0;
-            if (slabs == 2 || slabs == 1) {
+            if (slabs == 2 && !dense_tiles) slabs = 1;
+            if (slabs >= 1) {
                 // a one-slab launch needs its own divisibility (256 resp. 128 features)
                 const int st = launch_grouped_gemm_tc_pair(g, slabs, stream);
                 if (st != MOE_ERR_UNSUPPORTED) return st;
             }
             return launch_grouped_gemm_tc(g, stream);
         };
-        int st = run(g1, true);
+        int st = run(g1);
         if (st != MOE_OK) return st;
         if (!mark(3)) return MOE_ERR_CUDA;
-        st = run(g2, false);
+        st = run(g2);
         if (st != MOE_OK) return st;
     }
     if (!mark(4)) return MOE_ERR_CUDA;

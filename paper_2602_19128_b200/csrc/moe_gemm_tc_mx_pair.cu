@@ -308,8 +308,11 @@ int launch_pair_instance(const MxPairMaps &maps, const MxParams &p, int grid, cu
     using L = MxPairSmem<NT_MAX, STAGES, !STAGED ? 0 : SWIGLU ? 2 * kMxStageBytes : Stage<false>::kBytes>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
     const MxPairMapsOf<NT_MAX / 16> own = {TensorMapsOf<NT_MAX / 16>(maps.ops), maps.w_sf, maps.act_sf};
-    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
-    auto kernel = on_demand ? grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kOnDemand> : grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kStaticQueue>;
+    // (160-row tiles are staged where K is short: such an instance never draws its tiles)
+    constexpr bool kShortTiles = NT_MAX == 160 && STAGED && !pair_tiles_on_demand((kDirectFromK - 1) / kMxSlotK);
+    auto kernel = grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kStaticQueue>;
+    if constexpr (!kShortTiles)
+        if (pair_tiles_on_demand(p.n_k_blocks)) kernel = grouped_gemm_tc_mx_pair_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kOnDemand>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, own, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;

@@ -385,8 +385,11 @@ template <int NT_MAX, int STAGES, bool SWIGLU, bool STAGED = true>
 int launch_mx_ring_instance(const MxRingMaps &maps, const MxParams &p, int grid, cudaStream_t stream) {
     using L = MxRingSmem<NT_MAX, STAGES, SWIGLU, STAGED>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    const bool on_demand = pair_tiles_on_demand(p.n_k_blocks);
-    auto kernel = on_demand ? grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kOnDemand> : grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kStaticQueue>;
+    // (gate/up tiles of 304 rows are staged where K is short: such an instance never draws its tiles)
+    constexpr bool kShortTiles = NT_MAX == 304 && SWIGLU && STAGED && !pair_tiles_on_demand((kDirectFromK - 1) / kMxSlotK);
+    auto kernel = grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kStaticQueue>;
+    if constexpr (!kShortTiles)
+        if (pair_tiles_on_demand(p.n_k_blocks)) kernel = grouped_gemm_tc_mx_ring_kernel<NT_MAX, STAGES, SWIGLU, STAGED, kOnDemand>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kMxRingThreads, L::kDynamicBytes, stream, maps, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;

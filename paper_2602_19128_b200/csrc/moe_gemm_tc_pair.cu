@@ -295,8 +295,11 @@ template <int NT_MAX, int STAGES, int SLABS, bool SWIGLU, bool STAGED>
 int launch_pair_instance(const TensorMaps &maps, const KernelParams &p, int grid, cudaStream_t stream) {
     using L = PairSmem<NT_MAX, STAGES, SLABS, STAGED ? kStageBytes : 0>;
     static_assert(L::kBytes + 1024 <= L::kDynamicBytes, "ring does not fit in shared memory");
-    const bool on_demand = wide_pair_tiles_on_demand(p.n_k_blocks, NT_MAX);
-    auto kernel = on_demand ? grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kOnDemand> : grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kStaticQueue>;
+    // (one-slab tiles are stored directly where K is long: such an instance always draws its tiles)
+    constexpr bool kLongTiles = SLABS == 1 && !STAGED && wide_pair_tiles_on_demand(kDirectFromK / kBlockK, NT_MAX);
+    auto kernel = grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kOnDemand>;
+    if constexpr (!kLongTiles)
+        if (!wide_pair_tiles_on_demand(p.n_k_blocks, NT_MAX)) kernel = grouped_gemm_tc_pair_kernel<NT_MAX, STAGES, SLABS, SWIGLU, STAGED, kStaticQueue>;
     if (!set_max_dynamic_smem_once(reinterpret_cast<const void *>(kernel), L::kDynamicBytes))
         return MOE_ERR_CUDA;
     return launch_chained(kernel, grid, kPairThreads, L::kDynamicBytes, stream, TensorMapsOf<NT_MAX / 16>(maps), p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
@@ -306,10 +309,10 @@ int features_per_pair_tile(const GroupedGemmArgs &a, int slabs) { return slabs *
 
 }  // namespace
 
-// Largest number of weight slabs per CTA (2, 1) the pair kernel supports for this GEMM, 0 if none.
+// Largest number of weight slabs per CTA (2, 1) the pair kernel supports for this GEMM, 0 if none.  Two: the gate/up GEMM only.
 int grouped_gemm_tc_pair_slabs(const GroupedGemmArgs &a) {
     if (!(a.nt_max == 128 || a.nt_max == 256) || a.K % kBlockK != 0 || a.A <= 0) return 0;
-    if (a.nt_max == 256 && a.n_out % features_per_pair_tile(a, 2) == 0) return 2;
+    if (a.nt_max == 256 && a.swiglu && a.n_out % features_per_pair_tile(a, 2) == 0) return 2;
     return a.n_out % features_per_pair_tile(a, 1) == 0 ? 1 : 0;
 }
 
@@ -343,9 +346,7 @@ int launch_grouped_gemm_tc_pair(const GroupedGemmArgs &a, int slabs, cudaStream_
     const int pairs_on_device = sm_count() / 2;
     const int n_pairs = (int)(max_tiles < pairs_on_device ? max_tiles : pairs_on_device);
     const int grid = 2 * (n_pairs > 0 ? n_pairs : 1);
-    if (slabs == 2)
-        return a.swiglu ? launch_pair_instance<256, 4, 2, true, false>(maps, p, grid, stream)
-                        : launch_pair_instance<256, 4, 2, false, false>(maps, p, grid, stream);
+    if (slabs == 2) return launch_pair_instance<256, 4, 2, true, false>(maps, p, grid, stream);
     // 256-row tiles: seven slots leave no room for the epilogue's buffers (kDirectFromK).
     if (a.nt_max == 256 && a.K >= kDirectFromK)
         return a.swiglu ? launch_pair_instance<256, 7, 1, true, false>(maps, p, grid, stream)

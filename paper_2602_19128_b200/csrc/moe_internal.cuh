@@ -187,7 +187,7 @@ int launch_grouped_gemm_tc(const GroupedGemmArgs &args, cudaStream_t stream);  /
 
 // The same GEMM on CTA pairs (cta_group::2): 256 x N tiles (one weight slab per CTA) or 512 x N tiles
 // (two slabs per CTA sharing one token tile).  grouped_gemm_tc_pair_slabs gives the largest slab count
-// usable for this GEMM: 2, 1, or 0 when the pair kernel does not apply (token-tile bound below 128, or a
+// usable for this GEMM: 2 (gate/up only), 1, or 0 when the pair kernel does not apply (token-tile bound below 128, or a
 // feature count the pair tile does not divide).
 int grouped_gemm_tc_pair_slabs(const GroupedGemmArgs &args);
 int launch_grouped_gemm_tc_pair(const GroupedGemmArgs &args, int slabs, cudaStream_t stream);

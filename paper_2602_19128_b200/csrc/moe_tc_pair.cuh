@@ -120,13 +120,13 @@ __device__ __forceinline__ bool pair_wait_acquire(uint32_t bar, uint32_t parity,
 // epilogue, which is then most of a tile behind, lets it be drawn: at 32 slots 4096 MX tokens of 128 experts of 4096 x 1536, top 8,
 // 860 / 884 us, skewed 731 / 775; 2000 tokens of 64 of 2048 x 2048, top 4, 346 / 353.  Drawn two ahead those are level, but 512
 // Mixtral-shaped tokens take 575.
-__host__ __device__ __forceinline__ bool pair_tiles_on_demand(int slots_per_tile) { return slots_per_tile >= 80; }
+__host__ __device__ constexpr bool pair_tiles_on_demand(int slots_per_tile) { return slots_per_tile >= 80; }
 
 // The bf16 kernels with token tiles of 256 rows and more are built to draw from 20 slots on, where they do so, two ahead, if LightTiles
 // finds the routing skewed; otherwise their decoders keep to the static assignment (drawn all the same, 700 tokens of 12 experts of
 // 4096 x 4096, top 2, take 239.5 us instead of 237.2, 512 Mixtral-shaped ones 507 instead of 502).  Below 20 slots not measured; a
 // tile is then too short for its draw.  With 128 rows they draw from 80 slots on, and deal light tiles there too.
-inline bool wide_pair_tiles_on_demand(int slots_per_tile, int nt_max) { return slots_per_tile >= (nt_max >= 256 ? 20 : 80); }
+__host__ __device__ constexpr bool wide_pair_tiles_on_demand(int slots_per_tile, int nt_max) { return slots_per_tile >= (nt_max >= 256 ? 20 : 80); }
 __host__ __device__ __forceinline__ int pair_tiles_ahead(int slots_per_tile) { return slots_per_tile >= 80 ? 1 : 2; }
 
 // Tiles drawn in the schedule's order.
