@@ -427,6 +427,24 @@ __device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
     return v;
 }
 
+// The schedule's row quantum with ceil(2^32 / q): the rows of a tile are rounded up without a division.  n / q is the upper half of
+// n * inverse for every n with n q < 2^32, tiles and quanta being 384 at most; a quantum of 1 has no 32-bit inverse (launch_route
+// refuses it).
+constexpr int kMaxTileRows = 384;
+struct RowQuantum {
+    int q;
+    unsigned inverse;
+    constexpr explicit RowQuantum(int quantum) : q(quantum), inverse((unsigned)(((1ull << 32) + quantum - 1) / quantum)) {}
+    static constexpr bool valid(int quantum) { return quantum >= 2 && quantum <= kMaxTileRows; }
+};
+constexpr bool divides_exactly(int quantum) {
+    for (unsigned n = 0; n < 2 * kMaxTileRows; ++n)
+        if ((unsigned)(((unsigned long long)n * RowQuantum(quantum).inverse) >> 32) != n / quantum) return false;
+    return true;
+}
+static_assert(divides_exactly(2) && divides_exactly(16) && divides_exactly(32) && divides_exactly(64) && divides_exactly(128) &&
+              divides_exactly(160) && divides_exactly(240) && divides_exactly(kMaxTileRows), "rounding a tile's rows");
+
 // Schedule phase, run by one block of 1024 threads: exclusive scan over the experts' row counts and the token-tile
 // schedule.  `count` is expert threadIdx.x's rows in threads 0..E-1 and 0 in the others; `started(row)` is called by
 // thread e < E with expert e's first row, and what it writes is visible to the block on return.  The schedule's flag is
@@ -436,12 +454,6 @@ __device__ __forceinline__ int warp_inclusive_scan(int v, int lane) {
 // barrier per step -- twelve -- and a thousand threads counting spans of a few ids, the tiny layer's 32 ids took 3.9 us
 // from the last id to the flag; now 2.5.)  Every instruction runs once or a few times per call, so what is not a loop costs its
 // fetch more than its issue: loops are unrolled only where loads have to overlap.
-// The schedule's row quantum with ceil(2^32 / q): the rows of a tile (384 at most) are rounded up without a division.
-struct RowQuantum {
-    int q;
-    unsigned inverse;
-    explicit RowQuantum(int quantum) : q(quantum), inverse((unsigned)(((1ull << 32) + quantum - 1) / quantum)) {}
-};
 struct ScheduleShared {
     int warp_sums[kMaxExperts / 32];
     __align__(16) unsigned keys[kMaxExperts];
@@ -1021,6 +1033,7 @@ cudaError_t launch_route(const float *logits, int T, int E, int k, LocalExperts 
                          float *topk_w, int *expert_offsets, int *sorted_to_flat, int *flat_to_sorted,
                          RouteScratch scratch, int *status, cudaStream_t stream, int row_quantum, RouterParams router,
                          size_t status_bytes) {
+    if (!RowQuantum::valid(row_quantum)) return cudaErrorInvalidValue;
     const int A = T * k;
     if (scratch.n_chunks <= kFusedMaxChunks) {
         // One block, a cluster of eight, or up to 64 blocks of at least four tokens (the comment at kFusedOneBlockTokens).
