@@ -112,6 +112,25 @@ def run_forward(inp: dict, flags: int = 0, poison: bool = True, x_perm_written: 
     return out, moe.workspace_views(ws, T, H, I, E, k), ws
 
 
+# Ints 10 and 11 of a layer's status region: the counters that the gate/up and the down GEMM draw tiles from.
+TILE_COUNTERS = slice(40, 48)
+
+
+def assert_same_bits_again(call, out: torch.Tensor, ws: torch.Tensor, status_bytes: int):
+    """`call(result, workspace)` gives the bits of `out` again, and MOE_OK, in a workspace that holds none of its results: NaN
+    behind the status region, and in that region what the call before left, or counters far beyond the last tile.  A tile that
+    was not computed shows as NaN."""
+    for drawn in (None, 1 << 20, None):
+        ws[status_bytes:].fill_(POISON)
+        if drawn is not None:
+            ws[TILE_COUNTERS].view(torch.int32).fill_(drawn)
+        again = torch.full_like(out, float("nan"))
+        call(again, ws)
+        status = moe.moe_last_status(ws)
+        assert status == moe.MOE_OK, moe.moe_status_string(status)
+        assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+
+
 def to_host_case(inp: dict) -> dict:
     return dict(x=bf16_bits(inp["x"]), logits=inp["router_logits"].cpu().numpy(), w13=bf16_bits(inp["w13"]),
                 w2=bf16_bits(inp["w2"]), k=inp["top_k"])

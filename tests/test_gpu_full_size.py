@@ -13,8 +13,8 @@ import paper_2602_19128_b200 as moe
 from oracle import moe_oracle
 from paper_2602_19128_b200.inputs import CONFIGS, bf16_bits
 from tests.weight_quantizers import quantize_mxfp8
-from tests.gpu_common import (OUT_TOL, Guarded, assert_close_out, assert_routing_exact, bf16_to_f64, check_guards,
-                              gpu_inputs, guarded_out, mx_regions, run_forward)
+from tests.gpu_common import (OUT_TOL, Guarded, assert_close_out, assert_routing_exact, assert_same_bits_again, bf16_to_f64,
+                              check_guards, gpu_inputs, guarded_out, mx_regions, run_forward)
 
 pytestmark = pytest.mark.gpu
 
@@ -98,13 +98,27 @@ def test_full_size_workload(name):
 def test_light_tiles_among_heavy_ones(T, H, I, E, k):
     """Skewed routing with enough token tiles on both sides: the experts of few rows are dealt among the others, every tile is
     computed once (all elements against the CUDA-core validation kernels) and the bits are those of every run."""
-    inp = gpu_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=True), seed=2)
-    out, views, ws = run_forward(inp)
+    check_every_element_and_every_run(dict(T=T, H=H, I=I, E=E, top_k=k, skew=True))
+
+
+@pytest.mark.parametrize("flag,T,H,I,E,skew", [
+    (moe.MOE_FLAG_TWO_SLAB_GEMM, 1400, 3840, 3840, 16, True),     # 60 slots of K, light tiles dealt
+    (moe.MOE_FLAG_TWO_SLAB_GEMM, 1100, 5120, 2560, 8, False),     # 80 slots, 80 gate/up tiles on 74 pairs
+    (moe.MOE_FLAG_GATHER_IN_LOAD, 2000, 3840, 3840, 12, True),
+    (moe.MOE_FLAG_GATHER_IN_LOAD, 1000, 5120, 2560, 5, False)], ids=["two_slab_skew", "two_slab", "gather_skew", "gather"])
+def test_opt_in_forms_with_tiles_on_demand(flag, T, H, I, E, skew):
+    """Two weight slabs per CTA, and token rows fetched from x by the load warp, on tiles long enough to be drawn."""
+    rows = moe.moe_token_tile_rows(T, H, I, E, 1, flag)
+    assert rows == 256 if flag == moe.MOE_FLAG_TWO_SLAB_GEMM else rows in (320, 384)
+    check_every_element_and_every_run(dict(T=T, H=H, I=I, E=E, top_k=1, skew=skew), flag)
+
+
+def check_every_element_and_every_run(cfg, flags=0):
+    inp, k = gpu_inputs(cfg, seed=2), cfg["top_k"]
+    out, views, ws = run_forward(inp, flags=flags, x_perm_written=not flags & moe.MOE_FLAG_GATHER_IN_LOAD)
     h, y = views["h"].clone(), views["y"].clone()
-    for _ in range(3):
-        again = torch.empty_like(out)
-        moe.moe_forward(inp["x"], inp["router_logits"], inp["w13"], inp["w2"], k, again, ws)
-        assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+    assert_same_bits_again(lambda o, w: moe.moe_forward(inp["x"], inp["router_logits"], inp["w13"], inp["w2"], k, o, w, flags=flags),
+                           out, ws, moe.moe_workspace_layout(cfg["T"], cfg["H"], cfg["I"], cfg["E"], k).topk_ids)
     out_v, views_v, _ = run_forward(inp, flags=moe.MOE_FLAG_VALIDATION_GEMM)
     close_on_device(h, views_v["h"], "h")
     close_on_device(y, views_v["y"], "y")

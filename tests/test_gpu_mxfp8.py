@@ -9,8 +9,8 @@ import paper_2602_19128_b200 as moe
 from oracle import moe_oracle
 from paper_2602_19128_b200.inputs import bf16_bits
 from tests.weight_quantizers import make_mxfp8_inputs
-from tests.gpu_common import (Guarded, assert_close_out, assert_routing_exact, bf16_to_f64, check_guards, guarded_out,
-                              mx_regions, widen_hidden)
+from tests.gpu_common import (Guarded, assert_close_out, assert_routing_exact, assert_same_bits_again, bf16_to_f64, check_guards,
+                              guarded_out, mx_regions, widen_hidden)
 
 pytestmark = pytest.mark.gpu
 
@@ -46,6 +46,14 @@ def unpack_act_scales(atoms: np.ndarray, offsets: np.ndarray, n_blocks: int, til
             for b in range(n_blocks):
                 plain[begin + i, b] = atoms[b // 4, a, atom_byte(r % 128, b % 4)]
     return plain
+
+
+def assert_mx_same_bits_again(inp, out):
+    (T, H), (E, I2, _), k = inp["x"].shape, inp["w13_q"].shape, inp["top_k"]
+    sf = moe.moe_mxfp8_pack_scales(inp["w13_s"], gate_up=True), moe.moe_mxfp8_pack_scales(inp["w2_s"], gate_up=False)
+    ws = moe.alloc_workspace(moe.moe_mxfp8_workspace_bytes(T, H, I2 // 2, E, k), "cuda")
+    assert_same_bits_again(lambda o, w: moe.moe_forward_mxfp8(inp["x"], inp["router_logits"], inp["w13_q"], sf[0], inp["w2_q"], sf[1], k, o, w),
+                           out, ws, moe.moe_mxfp8_workspace_layout(T, H, I2 // 2, E, k).topk_ids)
 
 
 def run_mx(inp, local_offset=0):
@@ -201,8 +209,7 @@ def test_mxfp8_tiles_on_demand(T, H, I, E, k, skew):
     inp = make_mxfp8_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=skew), seed=3, device="cuda")
     out, _ = run_mx(inp)
     assert_close_out(bf16_to_f64(out), oracle_mx(inp), "mxfp8 out")
-    again, _ = run_mx(inp)
-    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+    assert_mx_same_bits_again(inp, out)
 
 
 @pytest.mark.parametrize("T", [100, 520])  # 128-row tiles and wide ones, 80 slots of K, 80 tiles of the gate/up GEMM on 74 pairs
@@ -214,14 +221,13 @@ def test_mxfp8_pair_tiles_on_demand(T):
     experts = {e: tuple(inp[n][e].cpu().numpy() for n in ("w13_q", "w13_s", "w2_q", "w2_s")) for e in range(E)}
     ref = moe_oracle.get("f32").forward_mxfp8_sampled(bf16_bits(inp["x"]), inp["router_logits"].cpu().numpy(), experts, I, k, tokens)
     assert_close_out(bf16_to_f64(out[torch.from_numpy(tokens).long().cuda()]), ref, "mxfp8 sampled out")
-    again, _ = run_mx(inp)
-    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+    assert_mx_same_bits_again(inp, out)
 
 
 @pytest.mark.parametrize("T,H,I,E,k", [(1, 512, 2048, 4, 2), (3, 256, 2176, 2, 2), (30, 384, 2304, 4, 2)])
 def test_mxfp8_few_down_tiles_with_two_ctas_each(T, H, I, E, k):
-    """Two CTAs per tile of the down GEMM, half of its rows each (2176: 17 slots); the same bits as with one CTA per tile,
-    which the layer has with its hidden dimension padded (tests/test_gpu_forward.py)."""
+    """Down GEMMs of a few tiles with a long K (2176: 17 slots), whose tiles the bf16 layer cuts in two and this one does not;
+    the same bits with the hidden dimension padded (tests/test_gpu_forward.py), where there are many tiles."""
     inp = make_mxfp8_inputs(dict(T=T, H=H, I=I, E=E, top_k=k, skew=False), seed=2, device="cuda")
     out, _ = run_mx(inp)
     assert_close_out(bf16_to_f64(out), oracle_mx(inp), "mxfp8 out")
