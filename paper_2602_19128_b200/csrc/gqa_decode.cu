@@ -99,7 +99,7 @@ struct Params {
 // Where no sequence is split there is nothing to count, and the kernel's first block zeroes the status word: one launch
 // (Params::own_status), and where that is faster with programmatic serialisation (kChained), so that a kernel's start overlaps the end of the
 // one in front (behind a memset it cannot).
-// Loops without / with: 40 sequences of 31..251 tokens 8.2 / 7.6 us, 162 of 410..821 44.3 / 43.4, 256 of 256..2048 102.8 / 101.3.
+// Loops without / with: 40 sequences of 31..251 tokens 8.2 / 7.5 us, 162 of 410..821 44.3 / 42.8, 256 of 256..2048 105.9 / 103.5.
 // Memset / one launch, in a loop / on the first pass over new inputs: 1 sequence of 100 tokens 8.5 -> 7.6 us / 25.7 ->
 // 21.7, 256 of 256..2048 105.5 -> 102.8 / 138 -> 133.  A wait gives up after 4 million polls, long after that block has started.
 // (A small kernel that zeroed the words beside a decode kernel launched with programmatic serialisation made loops 0.7 to 2
@@ -107,10 +107,10 @@ struct Params {
 // 4000 14.3 / 13.2 and 32.4 / 34.8, 16 of 8000 51.1 / 50.2 and 73.7 / 75.6.)
 // Chained or not: the blocks of a chained call are placed while those of the call in front still sit on their SMs.  Few find SMs of their
 // own, and a grid that fills the machine is placed evenly all the same; in between several land on one SM, and long ones wait for
-// it.  Equal lengths over 4 heads, plain / chained, loops: tiled, 108 blocks of 300 tokens 8.2 / 7.5 us, 800 14.4 / 15.0, 915 16.4 / 17.2;
-// 32 of 600 12.3 / 10.7; 68 of 700 12.6 / 12.8; 152 of 700 16.2 / 14.9, of 1100 21.8 / 20.8; row gather, 108 blocks of 128 8.2 /
-// 7.2, of 256 12.3 / 12.7, of 512 19.0 / 21.1; 32 of 384 15.6 / 14.0; 68 of 384 15.9 / 16.7; 240 of 256 12.6 / 12.8; 480 of 128 14.4 /
-// 13.3, of 384 34.5 / 33.4.  (The row gather's loop is at the limit of its registers: the wait in front of it cost 216 sequences
+// it.  Equal lengths over 4 heads, plain / chained, loops: tiled, 108 blocks of 300 tokens 8.2 / 7.6 us, 800 14.4 / 14.8, 915 16.4 / 17.0;
+// 32 of 600 12.3 / 10.5; 68 of 700 12.6 / 12.7; 152 of 700 15.8 / 14.4, of 1100 22.2 / 21.0; row gather, 120 blocks of 128 8.2 /
+// 7.2, of 256 12.3 / 12.5; 108 of 512 19.0 / 20.9; 32 of 384 15.6 / 13.9; 68 of 384 15.9 / 16.5; 240 of 256 12.6 / 12.7; 480 of 128
+// 14.4 / 12.9, of 384 34.5 / 33.1.  (The row gather's loop is at the limit of its registers: the wait in front of it cost 216 blocks
 // of 1059..2118 tokens 3 %, 75.2 / 77.5.)
 constexpr unsigned kSms = 148;
 static bool chaining_is_faster(bool tiled, unsigned blocks, int max_kv_len) {
@@ -351,9 +351,16 @@ __device__ __forceinline__ void zero_own_status(const Params &p, bool first_bloc
 }
 
 // A word of the page table.  __ldg is for memory that nothing writes while the kernel lives, and a chained kernel lives before what
-// is in front of it, which may write the table, is done: its loads are ordinary ones, behind the wait.
+// is in front of it, which may write the table, is done: its loads are ordinary ones, behind the wait.  (They cost what __ldg
+// costs; as plain C++ loads, whose order to each other and to the copies the compiler chose anew, they cost a call 0.1 to 0.5 us:
+// 40 sequences of 700 tokens 15.4 / 15.8, 256 of 256..2048 103.5 / 104.2.)
 template <bool kChained>
-__device__ __forceinline__ int load_index(const int *at) { return kChained ? *at : __ldg(at); }
+__device__ __forceinline__ int load_index(const int *at) {
+    if (!kChained) return __ldg(at);
+    int v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(at) : "memory");
+    return v;
+}
 // The wait of a chained kernel for what is in front.  That may have written the caches through the generic proxy: the threads
 // that copy them into shared memory link the two by a fence, here, where nothing of theirs is under way yet.
 __device__ __forceinline__ void wait_for_inputs(bool copies) {
@@ -361,11 +368,18 @@ __device__ __forceinline__ void wait_for_inputs(bool copies) {
     if (copies) asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// Cached tokens of an item; its first entry in the page table, which a chained kernel would otherwise load twice.
 template <bool kChained>
-__device__ __forceinline__ int cached_tokens(const Params &p, int b) {
-    const int first = load_index<kChained>(&p.kv_indptr[b]), behind = load_index<kChained>(&p.kv_indptr[b + 1]);
+__device__ __forceinline__ int cached_tokens(const Params &p, int b, int &first) {
+    first = load_index<kChained>(&p.kv_indptr[b]);
+    const int behind = load_index<kChained>(&p.kv_indptr[b + 1]);
     const int last = load_index<kChained>(&p.kv_last_page_len[b]);  // (all three in flight: one round trip)
     return behind > first ? (behind - first - 1) * p.page_size + last : 0;
+}
+template <bool kChained>
+__device__ __forceinline__ int cached_tokens(const Params &p, int b) {
+    int first;
+    return cached_tokens<kChained>(p, b, first);
 }
 // out = 0, lse = -inf for the heads of one key-value head (all 128 compute threads call).
 __device__ __forceinline__ void write_empty(const Params &p, int b, int head0, int tid) {
@@ -611,7 +625,8 @@ gqa_row_decode_kernel(const Params p) {
         moe::chain_release();
         wait_for_inputs(true);
     }
-    const int L = cached_tokens<kChained>(p, b);
+    int first_page;
+    const int L = cached_tokens<kChained>(p, b, first_page);
     const int head0 = kvh * p.group;
 
     if (L <= 0) {  // nothing cached: out = 0, lse = -inf (written by the first split's block)
@@ -629,7 +644,7 @@ gqa_row_decode_kernel(const Params p) {
 
     // Thread i brings ONE token row per chunk -- row i % 64 of the keys (i < 64) or of the values -- and arrives on the
     // stage's barrier once per chunk, with its bytes when its row exists.
-    const int *page_list = p.kv_indices + p.kv_indptr[b];
+    const int *page_list = p.kv_indices + (kChained ? first_page : p.kv_indptr[b]);
     const size_t token_stride = (size_t)p.Hkv * kD;  // elements between consecutive slots of a page
     const uint32_t smem_base = smem_u32(smem), bar_base = smem_u32(full_bar);
     const int my_row = tid & (kChunk - 1);
@@ -788,6 +803,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
 
     // ---- this block's piece: w_end - w chunks, the first of them chunk c of sequence (b, kvh) ----
     int b, kvh, c, L, n_chunks;  // the sequence the cursor is in, its tokens and chunks
+    int first_page = 0;          // (chained: of the block's only sequence)
     long long w = 0, w_end = 0;
     const int split_chunks = p.split_tokens / kChunk;
     bool balanced = false;
@@ -883,7 +899,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         const int split = blockIdx.x % p.n_splits;
         kvh = (blockIdx.x / p.n_splits) % p.Hkv;
         b = blockIdx.x / p.n_splits / p.Hkv;
-        L = cached_tokens<kChained>(p, b);
+        L = cached_tokens<kChained>(p, b, first_page);
         n_chunks = (L + kChunk - 1) / kChunk;
         if (L <= 0) {
             if (split == 0 && tid < kThreads) write_empty(p, b, kvh * p.group, tid);
@@ -916,7 +932,7 @@ gqa_tiled_decode_kernel(const Params p, const __grid_constant__ CUtensorMap k_ma
         const int my_row = (lane >> 1) << sh;
         const CUtensorMap *map = my_values ? &v_map : &k_map;
         const uint32_t my_dst = (my_values ? (uint32_t)kTiledTileBytes : 0u) + (uint32_t)(my_row * kRowBytes);
-        const int *page_list = p.kv_indices + load_index<kChained>(&p.kv_indptr[b]);
+        const int *page_list = p.kv_indices + (kChained ? first_page : __ldg(&p.kv_indptr[b]));
         int page, slot, head;
         auto locate = [&]() {
             const int tok = c * kChunk + my_row;
