@@ -39,8 +39,8 @@ __device__ __forceinline__ unsigned ordered_key(float f) {
 }
 
 // k rounds of a warp arg-max under the strict order (larger key first, ties to the lower expert index).  Expert
-// e = 32 i + lane has key[i] in its lane (kRegs = ceil(E / 32), rounded up to 1, 4 or 8); entries with e >= E must hold key 0 and are never selected while a real
-// candidate is left.  Each round: every lane finds its best remaining entry, one warp reduction gives the largest
+// e = 32 i + lane has key[i] in its lane (kRegs = ceil(E / 32), rounded up to 1, 4 or 8); entries with e >= E must hold key 0 and are
+// never selected while a real candidate is left.  Each round: every lane finds its best remaining entry, one warp reduction gives the largest
 // key, a second one the lowest expert index among the lanes that hold it.  Lane j < k returns rank j's expert.
 template <int kRegs>
 __device__ __forceinline__ int select_top_k(const unsigned (&key)[kRegs], int E, int k, int lane) {
@@ -112,7 +112,7 @@ __device__ __forceinline__ void select_candidates(const unsigned (&key)[kRegs], 
         n = 0;
 #pragma unroll
         for (int i = 0; i < kRegs; ++i) {
-            const bool in = key[i] >= bound;  // (a bound of 0 takes all 256 slots: the fallback)
+            const bool in = key[i] >= bound;  // (a bound of 0 takes all slots, 128 or 256: the fallback)
             const unsigned mask = __ballot_sync(kFullMask, in);
             const int at = n + __popc(mask & ((1u << lane) - 1u));
             if (in && at < 32) { c->key[at] = key[i]; c->e[at] = i * 32 + lane; c->score[at] = score[i]; }
@@ -148,7 +148,7 @@ __device__ __forceinline__ void select_candidates(const unsigned (&key)[kRegs], 
     __syncwarp();  // (the next token of this warp writes here)
 }
 
-// Router for one token by one warp: top-k of the E logits (8 per lane) under the strict order, then the
+// Router for one token by one warp: top-k of the E logits (kRegs per lane) under the strict order, then the
 // renormalised softmax weights.  Softmax's normaliser cancels in the renormalisation, so only the k selected
 // logits are exponentiated: w_j = exp(l_j - l_0) / sum_j' exp(l_j' - l_0), the sum in rank order.
 // Lane j < k returns rank j's expert and weight.
@@ -704,7 +704,7 @@ route_scatter_kernel(const int *topk_ids, const int *chunk_starts, const int *ex
 constexpr int kFusedThreads = 1024;
 constexpr int kFusedMaxChunks = 32;  // of kRouteTokensPerBlock tokens
 constexpr int kFusedWarps = kFusedThreads / 32;
-// Two ways from the blocks to the one that sorts.  Up to 16 tokens: one block.  Up to 256 (and kFusedIds ids): the blocks are
+// Two ways from the blocks to the one that sorts.  Up to 16 tokens: one block.  Up to 256 (and kFusedClusterIds ids): the blocks are
 // a cluster of eight, which leave their ids in the first one's shared memory and meet at the cluster's barrier; that
 // block also zeroes the call's status region, so the call needs neither a memset in front nor an atomic count and a trip of
 // the ids through L2.  Beyond, eight SMs would have more than a token per warp, and up to 64 blocks count themselves.
