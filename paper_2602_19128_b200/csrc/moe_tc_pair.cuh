@@ -115,9 +115,9 @@ __device__ __forceinline__ bool pair_wait_acquire(uint32_t bar, uint32_t parity,
 
 // Which pair GEMMs draw their tiles: those with K loops of 80 slots and more, whose tiles are so long that the static assignment's
 // rounds show (512 Mixtral-shaped tokens: 128 tiles of the down GEMM on 74 pairs, which began up to 30 us apart).  Static / on demand,
-// medians of alternating runs: that call 565 / 543 us, 1024 MX tokens of the same shape 460 / 429, 333 FP8-weight tokens of it 390 /
-// 370.  With shorter loops the next tile is wanted before the
-// epilogue, which is then most of a tile behind, lets it be drawn: at 32 slots 4096 MX tokens of 128 experts of 4096 x 1536, top 8,
+// medians of alternating bursts of 40 ms, all else alike: that call 519 / 507 us, 1024 tokens 722 / 700, 333 FP8-weight tokens 354 / 343
+// (1024 MX tokens 421 / 411, no more than two runs of the static form differ; the power cap evens it out in longer runs).  With shorter
+// loops the next tile is wanted before the epilogue, which is then most of a tile behind, lets it be drawn: at 32 slots 4096 MX tokens of 128 experts of 4096 x 1536, top 8,
 // 860 / 884 us, skewed 731 / 775; 2000 tokens of 64 of 2048 x 2048, top 4, 346 / 353.  Drawn two ahead those are level, but 512
 // Mixtral-shaped tokens take 575.
 __host__ __device__ constexpr bool pair_tiles_on_demand(int slots_per_tile) { return slots_per_tile >= 80; }
