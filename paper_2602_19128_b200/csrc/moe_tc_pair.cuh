@@ -117,9 +117,9 @@ __device__ __forceinline__ bool pair_wait_acquire(uint32_t bar, uint32_t parity,
 // rounds show (512 Mixtral-shaped tokens: 128 tiles of the down GEMM on 74 pairs, which began up to 30 us apart).  Static / on demand,
 // medians of alternating bursts of 40 ms, all else alike: that call 519 / 507 us, 1024 tokens 722 / 700, 333 FP8-weight tokens 354 / 343
 // (1024 MX tokens 421 / 411, no more than two runs of the static form differ; the power cap evens it out in longer runs).  With shorter
-// loops the next tile is wanted before the epilogue, which is then most of a tile behind, lets it be drawn: at 32 slots 4096 MX tokens of 128 experts of 4096 x 1536, top 8,
-// 860 / 884 us, skewed 731 / 775; 2000 tokens of 64 of 2048 x 2048, top 4, 346 / 353.  Drawn two ahead those are level, but 512
-// Mixtral-shaped tokens take 575.
+// loops the next tile is wanted before the epilogue, which is then most of a tile behind, lets it be drawn: at 32 slots 4096 MX
+// tokens of 128 experts of 4096 x 1536, top 8, 860 / 884 us, skewed 731 / 775; 2000 tokens of 64 of 2048 x 2048, top 4, 346 / 353.  Drawn
+// two ahead those are level, but 512 Mixtral-shaped tokens took 8 % longer.
 __host__ __device__ constexpr bool pair_tiles_on_demand(int slots_per_tile) { return slots_per_tile >= 80; }
 
 // The bf16 kernels with token tiles of 256 rows and more are built to draw from 20 slots on, where they do so, two ahead, if LightTiles
@@ -148,7 +148,8 @@ struct InOrder {
 // have tiles of fewer (410 rows: four of 112), which stay in order.  In order / dealt, alternating under the power cap: that case
 // 1225 / 1209 us (another part 1290 / 1244), 2048 tokens of 64 experts of 4096 x 4096, top 4, 886 / 855 (935 / 872), 1500 of 64 of
 // 7168 x 2048, top 6, 942 / 919, 4096 of 64 of 2048 x 1024, top 8, 458 / 453; with 128-row tiles 600 of 16 of 5120 x 5120, top 2,
-// 332 / 317, 1024 of 64 of 7168 x 2048, top 4, 538 / 518, 800 of 16 of 7168 x 7168, top 1, 424 / 393.  A line at 64 or 144 rows and none or three times n_pairs kept for the end are within the spread.
+// 332 / 317, 1024 of 64 of 7168 x 2048, top 4, 538 / 518, 800 of 16 of 7168 x 7168, top 1, 424 / 393.  A line at 64 or 144 rows and
+// none or three times n_pairs kept for the end are within the spread.
 struct LightTiles {
     static constexpr int kLightRows = 112;
     const KernelParams &p;
